@@ -279,7 +279,7 @@ hdd_status hdd_autotune(hdd_ctx *ctx, const hdd_solve_params *prm, void *stream,
 /*   op 6: out = A_j⁻¹ in      (fine → fine, direct solve; needs hdd_setup_exact)            */
 /* prec: 64 runs the fine arithmetic of ops 0, 1, 2, 4 in complex64 (inputs rounded to FP32, */
 /* outputs widened back) and the banded solves of ops 3 and 6 in double-FP32 arithmetic (the  */
-/* form the complex64 inner iteration uses, HDD_OPT_COARSE_DF); 128: complex128 / FP64. */
+/* banded form of the complex64 inner iteration, HDD_OPT_COARSE_DF); 128: complex128 / FP64. */
 hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void *out_dev,
                         void *stream);
 
@@ -387,6 +387,13 @@ long long hdd_launch_count(const hdd_ctx *ctx);
 /* in the pass, those dots within a few 1e-12 of Σ|v w| instead of about 1e-15 (1, the        */
 /* default: the delayed second pass, which keeps the two-sum, measures and removes what the   */
 /* first pass left) or the two-sum for both (0).                                              */
+/* HDD_OPT_COARSE_DENSE (9): the coarse solves E_j⁻¹ of the inner iteration and of the training */
+/* loss run as products with the explicit inverses of the distinct E_j on the tensor cores, in  */
+/* exact integer arithmetic on 56-bit fixed-point copies of the FP64 entries (1, the default,   */
+/* where the shapes and tasks make that the faster form; the inverses are formed at             */
+/* hdd_setup_deflation, or at hdd_setup_batch when the batch makes it pay) or by the banded     */
+/* kernels the options 1, 6 and 7 describe (0).  hdd_local_op always applies the banded ones.   */
+/* With HDD_OPT_COARSE_LOOKAHEAD 0, or HDD_OPT_COARSE_DF 0 in complex64, the banded kernels run. */
 /* HDD_ERR_INVALID_ARG for an unknown key or a value other than 0 or 1.  Takes effect from the  */
 /* next call that solves.                                                                       */
 #define HDD_OPT_COARSE_LOOKAHEAD 1
@@ -397,6 +404,7 @@ long long hdd_launch_count(const hdd_ctx *ctx);
 #define HDD_OPT_COARSE_DF 6
 #define HDD_OPT_COARSE_SPIKE 7
 #define HDD_OPT_OUTER_DOTS_BIASED 8
+#define HDD_OPT_COARSE_DENSE 9
 hdd_status hdd_set_option(hdd_ctx *ctx, int key, int value);
 
 /* ---------------------------------------------------------------------------------------- */

@@ -47,7 +47,23 @@ struct FactorSet {            // banded FP64 factors of one matrix per shape, bl
     BlockSolveCfg cfg;              // shared-memory plan of the blocked solve
     bool re2 = false;               // factors of real-equivalent systems (complex matrices)
     bool ready = false;
-    void clear() { G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
+    // the explicit inverses as base-256 digits (kernels_dense.cu) and the plans of their products
+    // for the task table and for the doubled one
+    struct DenseOp { long long aoff, soff; int m, mt, kseg, kc; };
+    DevMem dA, drs;
+    std::vector<DenseOp> dop;       // empty: no dense form
+    std::vector<int4> meta;         // host copy of Meta and the operators' length (for the spike matrices)
+    long long mo = 0;
+    bool spike_tried = false;       // the SPIKE plans were formed, or were not wanted at set-up
+    bool dense_on = false;          // the dense form pays for the tasks there are
+    int digits32 = 6;               // digits of the complex64 iteration
+    struct Plan {
+        DevMem sh, recs, tabs, tcoff, B, cs, ws, part;  // tabs: sunits, items, then tlist and tshape (ntask each)
+        int ntask = 0, ntmax = 0, nst = 0, nitem = 0;
+        double bytes = 0, flops = 0;
+        void clear() { sh.release(); recs.release(); tabs.release(); tcoff.release(); B.release(); cs.release(); ws.release(); part.release(); ntask = 0; }
+    } plan[4];                      // {task table, doubled table} with 6 digits, with 7
+    void clear() { dA.release(); drs.release(); dop.clear(); for (auto &P : plan) P.clear(); meta.clear(); mo = 0; spike_tried = dense_on = false; G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
                    M.release(); Mdf.release(); P.release(); Meta.release(); table.release(); h.clear(); fma_col.clear(); cfg = BlockSolveCfg{}; re2 = false; ready = false; }
 };
 
@@ -62,15 +78,15 @@ template <typename R> struct InnerWork {   // inner GMRES buffers for one precis
 // Kernel families timed by the profiler (CUDA events around every launch on the launching
 // stream).  bound: 0 = memory (HBM bytes), 1 = FP64 arithmetic.
 enum Fam { F_ZT, F_COARSE, F_PS, F_CGS, F_GIVENS, F_LMISC, F_OCGS, F_OMISC, F_CNN, F_OREORTH, F_STEP, F_ODF,
-           F_CGRID, F_OUDF, F_CDF, F_CSPK, NFAM };
+           F_CGRID, F_OUDF, F_CDF, F_CSPK, F_CDENSE, NFAM };
 const char *kFamName[NFAM] = {"local_stencil_zt", "coarse_solve_fp64", "local_prolong_stencil_dots",
                               "local_cgs2_update", "local_givens_normalize", "local_misc",
                               "outer_cgs2_fp64", "outer_misc_fp64", "warm_start_cnn",
                               "outer_reorth_fp32", "local_arnoldi_step", "outer_dots_df32",
                               "two_level_grid_coarse", "outer_update_df32", "coarse_solve_df32",
-                              "coarse_solve_df32_spike"};
+                              "coarse_solve_df32_spike", "coarse_solve_dense"};
 // (2: FP32 pipe; for the double-FP32 families the flop counts are FP32 instructions)
-const int kFamBound[NFAM] = {0, 1, 0, 0, 0, 0, 1, 0, 2, 0, 0, 2, 0, 2, 2, 2};
+const int kFamBound[NFAM] = {0, 1, 0, 0, 0, 0, 1, 0, 2, 0, 0, 2, 0, 2, 2, 2, 0};
 
 struct Prof {
     bool on = false;
@@ -164,8 +180,8 @@ struct hdd_ctx {
     CnnState cnn;
     DevMem tmp_a, tmp_b, tmp_c;                // staging for test hooks
     DevMem d_alist;                            // active tasks of a SPIKE coarse solve, compacted
-    int *h_counter = nullptr;                  // pinned
-    DevMem d_counter;
+    int *h_counter = nullptr;                  // pinned copy of d_counter
+    DevMem d_counter;                          // {tasks still running, error flag of the dense solves}
     std::vector<double> hist;
     std::vector<int> h_its;
     Prof prof;
@@ -178,6 +194,7 @@ struct hdd_ctx {
     int coarse_df = 1;                         // HDD_OPT_COARSE_DF
     int coarse_spike = 1;                      // HDD_OPT_COARSE_SPIKE
     int outer_bias = 1;                        // HDD_OPT_OUTER_DOTS_BIASED
+    int coarse_dense = 1;                      // HDD_OPT_COARSE_DENSE
     int step_C[2] = {-1, -1};                  // fused-step cluster size per inner precision (0: off, -1: unplanned)
     size_t step_smem[2] = {0, 0};
     bool poisoned = false;                     // a device wait gave up with work in flight
@@ -252,16 +269,28 @@ template <typename R> LocalArgs<R> local_args(hdd_ctx *ctx) {
     return a;
 }
 
-hdd_status read_counter(hdd_ctx *ctx, cudaStream_t s, int *out) {
-    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    ctx->prof.harvest();
-    *out = *ctx->h_counter;
-    return HDD_OK;
+// The error flag of the dense coarse solves, read beside the counter (e: its value).
+hdd_status dense_error(hdd_ctx *ctx, int e, cudaStream_t s) {
+    if (!e) return HDD_OK;
+    if (e == 2) {
+        ctx->poisoned = true;
+        FAIL(HDD_ERR_TIMEOUT, "a dense coarse solve's wait and its drain timed out; work still in flight may have "
+                              "written freed memory, so this context refuses further work (discard it and its CUDA context)");
+    }
+    CK(cudaMemsetAsync(ctx->d_counter.as<int>() + 1, 0, sizeof(int), s));
+    for (auto &P : ctx->E.plan)
+        if (P.ws.p) CK(cudaMemsetAsync(P.ws.p, 0, P.ws.bytes, s));
+    FAIL(HDD_ERR_TIMEOUT, "a dense coarse solve's wait timed out");
 }
 
-// E_j (or A_j) factors for every distinct shape, FP64, on the device: banded LU with partial
-// pivoting, then the blocked solve operators.
+hdd_status read_counter(hdd_ctx *ctx, cudaStream_t s, int *out) {
+    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    ctx->prof.harvest();
+    *out = ctx->h_counter[0];
+    return dense_error(ctx, ctx->h_counter[1], s);
+}
+
 // ---- SPIKE plans of a factor set (the double-FP32 coarse solve split over P parts) ----------
 // Forward / backward sweeps of blocks [J0, J1) of one shape emulated in FP64 on the host with the
 // device's own block operators, for W unit window vectors at once (zero inputs): Y holds rows
@@ -380,6 +409,227 @@ hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &met
     return HDD_OK;
 }
 
+
+// ---- the coarse solve as a product with explicit inverses (kernels_dense.cu) ------------------
+// Whether it is the faster form for `per` tasks of each shape.  Dense: three kernels, about 12 us
+// where nothing else counts, and the operators' digits at 5.5 TB/s with the MMAs under them (28
+// products of nt columns per 16-column unit, nt/2 clocks each).  Banded: 0.77 us per 16-row block
+// and sweep (164 us for the 106 blocks of m = 1681), one chain per SM, or 1.7 times that for two
+// per SM.  Measured: four shapes, 64 tasks (k=200) 164 us against 45; 256 uneven shapes of
+// N = 1280 with 32 right-hand sides 15.2 ms against 2.3, while for one right-hand side the banded
+// form stays ahead (0.5 against 2 ms: every operator is read for one task); m = 64, 4 tasks, 15 us
+// against 17.
+bool dense_pays(const hdd_ctx *ctx, const FactorSet &F, const std::vector<int> &per) {
+    double bytes = 0, mma = 0, chain = 0, chains = 0;
+    for (size_t q = 0; q < F.h.size(); q++) {
+        const int m = F.re2 ? F.h[q].m / 2 : F.h[q].m;
+        const double units = (double)((m + 127) / 128) * ((m + 15) / 16) * (F.re2 ? 2 : 1);
+        bytes += units * DENSE_ABYTES;
+        mma += units * 28.0 * 0.5 * std::max(16.0, 2.0 * per[q]);
+        chain = std::max(chain, 2.0 * F.h[q].nblk * 0.77e-6);
+        chains += (F.re2 ? 1.0 : 2.0) * per[q];
+    }
+    const double td = 12e-6 + std::max(bytes / 5.5e12, mma / (ctx->nsm * 1.9e9));
+    const double tb = chains <= ctx->nsm ? chain : 1.7 * chain * std::ceil(chains / (2.0 * ctx->nsm));
+    return td < 0.8 * tb;
+}
+
+std::vector<int> tasks_per_shape(const hdd_ctx *ctx) {
+    std::vector<int> per(ctx->shapes.size(), 0);
+    for (const Task &T : ctx->h_tasks) per[T.shape]++;
+    return per;
+}
+
+// Tables and buffers of the product with ds digits for the task table (which = 0) or the doubled
+// one (1).
+hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_t s) {
+    FactorSet::Plan &P = F.plan[which + (ds == 7 ? 2 : 0)];
+    const int ntm = dense_nt(ds);
+    const int nt1 = (int)ctx->h_tasks.size(), nt = which ? 2 * nt1 : nt1, ns = (int)F.dop.size();
+    if (P.ntask == nt) return HDD_OK;
+    P.ntask = 0;
+    std::vector<std::vector<int>> by(ns);
+    for (int t = 0; t < nt; t++) by[ctx->h_tasks[t % nt1].shape].push_back(t);
+    std::vector<DenseShape> sh(ns);
+    std::vector<DenseTask> recs(nt);
+    std::vector<int> tlist, tshape(nt);
+    std::vector<int4> units(ns), items;
+    std::vector<long long> tcoff(nt);
+    for (int t = 0; t < nt; t++) {
+        tshape[t] = ctx->h_tasks[t % nt1].shape;
+        tcoff[t] = ctx->h_tasks[t % nt1].coff + (t < nt1 ? 0 : ctx->ldc);
+    }
+    long long bo = 0, wo = 0;
+    P.ntmax = 16; P.bytes = P.flops = 0;
+    for (int q = 0; q < ns; q++) {
+        const FactorSet::DenseOp &o = F.dop[q];
+        DenseShape &S = sh[q];
+        S.aoff = o.aoff; S.soff = o.soff; S.m = o.m; S.mt = o.mt; S.kseg = o.kseg; S.kc = o.kc; S.re2 = F.re2 ? 1 : 0;
+        const int cols = 2 * (int)by[q].size();
+        // column tiles of equal width: a multiple of 16 up to dense_nt
+        S.nct = std::max(1, (cols + ntm - 1) / ntm);
+        S.nt = std::max(16, ((cols + S.nct - 1) / S.nct + 15) / 16 * 16);
+        S.nct = std::max(1, (cols + S.nt - 1) / S.nt);
+        S.boff = bo;
+        bo += (long long)S.nct * S.kc * 2 * ds * S.nt * 16;
+        S.t0 = (int)tlist.size(); S.ntask = (int)by[q].size();
+        for (int r = 0; r < S.ntask; r++) {
+            const int t = by[q][r], ct = 2 * r / S.nt, col = 2 * r - ct * S.nt;
+            recs[t] = DenseTask{tcoff[t], S.boff / 16 + (long long)ct * S.kc * 2 * ds * S.nt + col, S.m, S.kseg, S.nt, S.re2};
+            tlist.push_back(t);
+        }
+        S.acc0 = wo;
+        wo += (long long)S.mt * S.nct * 128 * S.nt;
+        units[q] = make_int4(S.mt * S.nct, S.kc, (ds * (4096 + 32 * S.nt) + 1023) / 1024, 0);
+        for (int t = 0; t < S.mt * S.nct; t++)
+            for (int pr = 0; pr < S.nt / 2; pr += 8) items.push_back(make_int4(q, t, pr, 0));
+        P.ntmax = std::max(P.ntmax, S.nt);
+        P.bytes += (double)S.kc * 16 * S.m * 2 * ds;
+        P.flops += 2.0 * (ds * (ds + 1) / 2) * S.kc * 16 * S.m * cols;
+    }
+    P.nst = dense_stages(ds, ns, P.ntmax);
+    CK(dense_set_smem());
+    CK(P.sh.ensure(ns * sizeof(DenseShape)));
+    P.nitem = (int)items.size();
+    const size_t b4 = (size_t)(ns + P.nitem) * sizeof(int4), b1 = (size_t)nt * sizeof(int);
+    CK(P.tabs.ensure(b4 + 2 * b1));
+    CK(P.part.ensure((size_t)(ns + 2) * sizeof(int2)));
+    CK(P.tcoff.ensure(tcoff.size() * sizeof(long long)));
+    CK(P.B.ensure((size_t)bo));
+    CK(P.cs.ensure(2 * (size_t)nt * sizeof(int)));
+    CK(P.ws.ensure((size_t)wo * sizeof(unsigned long long)));
+    CK(P.recs.ensure(recs.size() * sizeof(DenseTask)));
+    CK(cudaMemcpy(P.recs.p, recs.data(), recs.size() * sizeof(DenseTask), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(P.sh.p, sh.data(), ns * sizeof(DenseShape), cudaMemcpyHostToDevice));
+    char *tb = P.tabs.as<char>();
+    CK(cudaMemcpy(tb, units.data(), ns * sizeof(int4), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(tb + ns * sizeof(int4), items.data(), P.nitem * sizeof(int4), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(tb + b4, tlist.data(), b1, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(tb + b4 + b1, tshape.data(), b1, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(P.tcoff.p, tcoff.data(), tcoff.size() * sizeof(long long), cudaMemcpyHostToDevice));
+    CK(cudaMemsetAsync(P.ws.p, 0, P.ws.bytes, s));
+    P.ntask = nt;
+    return HDD_OK;
+}
+
+// Explicit inverses of every shape as digits, where the product pays and fits (a quarter of the
+// free memory, 8192 operator columns, the set-up kernel's shared memory); else F.dop stays empty.
+hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
+    const int ns = (int)F.h.size();
+    const int re2 = F.re2 ? 1 : 0, cw = std::max(F.cfg.cwx, F.cfg.cwy);
+    if (ns > DENSE_MAXNS || inv_cols_smem(F.cfg.maxK, cw) > 226 * 1024) return HDD_OK;
+    std::vector<FactorSet::DenseOp> op(ns);
+    std::vector<long long> wsz(ns);
+    long long ao = 0, so = 0;
+    for (int q = 0; q < ns; q++) {
+        FactorSet::DenseOp &o = op[q];
+        o.m = F.h[q].m / (re2 ? 2 : 1);
+        if (F.h[q].m > 8192) return HDD_OK;
+        o.mt = (o.m + 127) / 128; o.kseg = (o.m + 15) / 16; o.kc = o.kseg * (re2 ? 2 : 1);
+        o.aoff = ao; o.soff = so;
+        ao += (long long)o.mt * o.kc * DENSE_ABYTES;
+        so += (long long)o.mt * 128;
+        wsz[q] = (long long)o.kseg * 16 * F.h[q].nblk * BNB;       // 16 columns x all rows per column block
+    }
+    size_t fr = 0, tot = 0;
+    CK(cudaMemGetInfo(&fr, &tot));
+    if ((size_t)ao > fr / 4) return HDD_OK;
+    CK(F.dA.ensure((size_t)ao));
+    CK(F.drs.ensure((size_t)so * sizeof(int)));
+    // shapes in groups of up to 1 GB of workspace
+    DevMem W, jobs, shs, rmax;
+    for (int q0 = 0; q0 < ns;) {
+        int q1 = q0;
+        long long w = 0;
+        std::vector<InvShape> sh;
+        std::vector<InvJob> jb;
+        int mmax = 0, kmax = 0, tmax = 0;
+        while (q1 < ns && (q1 == q0 || w + wsz[q1] <= (1LL << 27))) {
+            const FactorSet::DenseOp &o = op[q1];
+            const long long rows = (long long)F.h[q1].nblk * BNB;
+            sh.push_back(InvShape{w, o.soff, o.soff, o.aoff, rows, o.m, o.mt, o.kseg, o.kc, re2});
+            for (int jc = 0; jc < o.kseg; jc++) jb.push_back(InvJob{q1, jc, w + (long long)jc * 16 * rows});
+            w += wsz[q1];
+            mmax = std::max(mmax, o.m); kmax = std::max(kmax, o.kseg); tmax = std::max(tmax, o.mt);
+            q1++;
+        }
+        // the longest jobs (first columns) first
+        std::stable_sort(jb.begin(), jb.end(), [&](const InvJob &a, const InvJob &b) {
+            return op[a.shape].kseg - a.jc > op[b.shape].kseg - b.jc;
+        });
+        CK(W.ensure((size_t)w * sizeof(double)));
+        CK(jobs.ensure(jb.size() * sizeof(InvJob)));
+        CK(shs.ensure(sh.size() * sizeof(InvShape)));
+        CK(rmax.ensure((size_t)so * sizeof(unsigned long long)));
+        if (q0 == 0) CK(cudaMemsetAsync(rmax.p, 0, (size_t)so * sizeof(unsigned long long), s));
+        CK(cudaMemcpyAsync(jobs.p, jb.data(), jb.size() * sizeof(InvJob), cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(shs.p, sh.data(), sh.size() * sizeof(InvShape), cudaMemcpyHostToDevice, s));
+        CK(launch_inv(jobs.as<InvJob>(), (int)jb.size(), shs.as<InvShape>(), (int)sh.size(), mmax, kmax, tmax,
+                      F.table.as<BlockFactor>(), F.M.as<double>(), F.P.as<int>(), F.Meta.as<int4>(), W.as<double>(),
+                      F.cfg.maxK, cw, re2, rmax.as<unsigned long long>(), F.drs.as<int>(), F.dA.as<uint8_t>(), s));
+        CK(cudaStreamSynchronize(s));           // the tables and the workspace are used again
+        q0 = q1;
+    }
+    F.dop = op;
+    // Against the exact inverse, 6 digits leave 1e-13 of the solution where the double-FP32 banded
+    // solve leaves 1e-12 to 2e-11 (36 geometries, m = 625 to 2401), but 5.5e-14 against 3.5e-14 at
+    // m = 64, where nothing is gained by the shorter operator: 7 digits below 256
+    F.digits32 = 6;
+    for (const FactorSet::DenseOp &o : op) if (o.m < 256) F.digits32 = 7;
+    return HDD_OK;
+}
+
+// E⁻¹ in for the flagged tasks by the product; ds and which as in dense_plan.
+hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
+    hdd_status st = dense_plan(ctx, F, ds, which, s);
+    if (st != HDD_OK) return st;
+    FactorSet::Plan &P = F.plan[which + (ds == 7 ? 2 : 0)];
+    DensePlanArgs a;
+    a.recs = P.recs.as<DenseTask>();
+    a.ntask = P.ntask;
+    a.sh = P.sh.as<DenseShape>(); a.ns = (int)F.dop.size();
+    a.sunits = P.tabs.as<int4>(); a.items = a.sunits + a.ns; a.nitem = P.nitem;
+    a.tlist = reinterpret_cast<const int *>(a.items + P.nitem); a.tshape = a.tlist + P.ntask;
+    a.tcoff = P.tcoff.as<long long>();
+    a.A = F.dA.as<uint8_t>(); a.rexp = F.drs.as<int>();
+    a.B = P.B.as<uint8_t>(); a.cexp = P.cs.as<int>(); a.ws = P.ws.as<unsigned long long>(); a.part = P.part.as<int2>();
+    a.ntmax = P.ntmax; a.nst = P.nst; a.grid = ctx->nsm;
+    a.err = ctx->d_counter.as<int>() + 1;
+    KL(F_CDENSE, P.bytes, P.flops, launch_dense_solve(ds, a, in, out, flag, s));
+    ctx->prof.launches += 2;
+    return HDD_OK;
+}
+
+// SPIKE plans of the coarse factors (their double-FP32 solves), where the host emulation that
+// forms the spike matrices stays cheap (about m·(wf² + wb²) multiply-adds per shape).
+hdd_status spike_build(hdd_ctx *ctx, FactorSet &F) {
+    F.spike_tried = true;
+    double cost = 0.0;
+    for (const BlockFactor &b : F.h) cost += (double)b.m * ((double)b.wl * b.wl + (double)b.wu * b.wu);
+    return cost <= 1.5e9 ? build_spikes(ctx, F, F.meta, F.mo) : HDD_OK;
+}
+
+// The form the inner iteration's coarse solves take, chosen by the tasks there are: the product
+// with explicit inverses, or the banded kernels with their SPIKE plans.
+hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
+    hdd_status st = HDD_OK;
+    F.dense_on = dense_pays(ctx, F, tasks_per_shape(ctx));
+    if (ctx->coarse_dense && F.dense_on && F.dop.empty()) st = dense_build(ctx, F, s);
+    if (!ctx->coarse_spike) F.spike_tried = true;
+    if (st == HDD_OK && !F.spike_tried && !(F.dense_on && !F.dop.empty())) {
+        CK(cudaStreamSynchronize(s));
+        st = spike_build(ctx, F);
+    }
+    return st;
+}
+
+// Whether the coarse solves of the inner iteration and of the training loss run as that product.
+bool use_dense(const hdd_ctx *ctx) {
+    return ctx->coarse_dense && ctx->coarse_la && ctx->E.dense_on && !ctx->E.dop.empty();
+}
+
+// E_j (or A_j) factors for every distinct shape, FP64, on the device: banded LU with partial
+// pivoting, then the blocked solve operators.
 hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s) {
     F.clear();
     const int ns = (int)ctx->shapes.size();
@@ -504,18 +754,6 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     CK(F.Mdf.ensure((size_t)std::max(mo, 1LL) * sizeof(float2)));
     launch_ops_to_df(mo, F.M.as<double>(), F.Mdf.as<float2>(), s);
     CKL();
-    // SPIKE plans of the coarse factors (their double-FP32 solves), where the host emulation that
-    // forms the spike matrices stays cheap (about m·(wf² + wb²) multiply-adds per shape)
-    if (coarse && ctx->coarse_spike) {
-        CK(cudaStreamSynchronize(s));
-        double cost = 0.0;
-        for (int q = 0; q < ns; q++)
-            cost += (double)F.h[q].m * ((double)F.h[q].wl * F.h[q].wl + (double)F.h[q].wu * F.h[q].wu);
-        if (cost <= 1.5e9) {
-            hdd_status sst = build_spikes(ctx, F, meta, mo);
-            if (sst != HDD_OK) return sst;
-        }
-    }
     CK(F.table.ensure(ns * sizeof(BlockFactor)));
     CK(cudaMemcpyAsync(F.table.p, F.h.data(), ns * sizeof(BlockFactor), cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
@@ -524,6 +762,12 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     if (set_block_solve_smem(F.cfg) != cudaSuccess)
         FAIL(HDD_ERR_INVALID_ARG, "factor panels of width %d exceed the shared-memory solve", F.cfg.maxK);
     F.re2 = re2;
+    if (coarse) {
+        F.meta = std::move(meta);
+        F.mo = mo;
+        hdd_status dst = coarse_forms(ctx, F, s);
+        if (dst != HDD_OK) return dst;
+    }
     F.ready = true;
     return HDD_OK;
 }
@@ -733,16 +977,22 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     float2 *Fh = C.Fh.as<float2>(), *Q = C.Q.as<float2>(), *T2 = C.T2.as<float2>();
     float2 *Rr = reinterpret_cast<float2 *>(C.Rr.as<float>());
     double2 *Yc = C.Yc.as<double2>(), *Sc = C.Sc.as<double2>();
+    hdd_status st = HDD_OK;
+    auto coarse = [&](const double2 *in, double2 *out) -> hdd_status {
+        if (use_dense(ctx)) return dense_solve(ctx, ctx->E, 7, 0, in, out, nullptr, s);
+        band_solve(ctx, ctx->E, in, out, false, nullptr, s);
+        return HDD_OK;
+    };
     KL(F_CNN, 0, 0, launch_zt<float>(a, Fh, Yc, 0, nullptr, s));
-    band_solve(ctx, ctx->E, Yc, Sc, false, nullptr, s);
+    if ((st = coarse(Yc, Sc)) != HDD_OK) return st;
     KL(F_CNN, 0, 0, launch_prolong_stencil<float>(a, 1, Fh, Sc, T2, nullptr, 0, C.Pf.as<float2>(), nullptr, s));
     KL(F_CNN, 0, 0, launch_cnn_resid(T, ft, nft, ctx->st, C.X0.as<float>(), C.A4.as<float>(), C.Rr.as<float>(),
                                        C.lpart.as<float>(), s));
     KL(F_CNN, 0, 0, launch_zt<float>(a, Rr, Yc, 0, nullptr, s));
-    band_solve(ctx, ctx->E, Yc, Sc, false, nullptr, s);
+    if ((st = coarse(Yc, Sc)) != HDD_OK) return st;
     KL(F_CNN, 0, 0, launch_prolong_stencil<float>(a, 1, Rr, Sc, Q, nullptr, 0, C.Pr.as<float2>(), nullptr, s));
     KL(F_CNN, 0, 0, launch_zt<float>(a, Q, Yc, 1, nullptr, s));
-    band_solve(ctx, ctx->E, Yc, Sc, false, nullptr, s);
+    if ((st = coarse(Yc, Sc)) != HDD_OK) return st;
     KL(F_CNN, 0, 0, launch_z<float>(a, Sc, Q, T2, nullptr, s, -1.0f));
     KL(F_CNN, 0, 0, launch_cnn_task_scale(T, nt, C.Pf.as<float2>(), C.scale.as<float>(), s));
     KL(F_CNN, 0, 0, launch_cnn_task_loss(T, nt, C.Pr.as<float2>(), C.Pf.as<float2>(), C.tloss.as<float>(), s));
@@ -770,8 +1020,8 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     CKL();
     std::vector<float> lt(nt);
     CK(cudaMemcpyAsync(lt.data(), C.tloss.p, nt * sizeof(float), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    ctx->prof.harvest();
+    int unused = 0;
+    if ((st = read_counter(ctx, s, &unused)) != HDD_OK) return st;
     double L = 0;
     for (int t = 0; t < nt; t++) L += lt[t];
     if (loss) *loss = L / nt;
@@ -880,6 +1130,16 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     const int maxit = prm->inner_maxit;
     // the complex64 inner iteration takes its coarse solves in double-FP32 (HDD_OPT_COARSE_DF)
     const bool cdf = sizeof(R) == 4 && ctx->coarse_df;
+    // E⁻¹ in for the flagged tasks: the product with explicit inverses (FP64 accuracy, so it serves
+    // both precisions), or the banded kernels; without coarse_df the complex64 iteration asks for those
+    const bool dense = use_dense(ctx) && (cdf || sizeof(R) == 8);
+    const int ds = sizeof(R) == 8 ? 7 : ctx->E.digits32;
+    if (!dense && cdf && ctx->coarse_spike && !ctx->E.spike_tried && (st = spike_build(ctx, ctx->E)) != HDD_OK) return st;
+    auto coarse = [&](const double2 *in, double2 *out, const int *flag, int n) -> hdd_status {
+        if (dense) return dense_solve(ctx, ctx->E, ds, 0, in, out, flag, s);
+        band_solve(ctx, ctx->E, in, out, false, flag, s, n, cdf);
+        return HDD_OK;
+    };
 
     const int *all = mask ? mask : ones;
     KL(F_LMISC, ld * (16 + cs), 0, launch_restrict<R>(a, v, ctx->nglob, f, mask, s));
@@ -893,7 +1153,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         CK(cudaMemsetAsync(u, 0, ld * sizeof(c2<R>), s));
         // first cycle from ũ = 0: r0 = P f̃ = f̃ - A Z E⁻¹ Zᵀ f̃, and ref = ||P f̃||
         KL(F_ZT, ld * cs + ldc * 16, 0, launch_zt<R>(a, f, y, 0, mask, s));
-        band_solve(ctx, ctx->E, y, sc, false, mask, s, -1, cdf);
+        if ((st = coarse(y, sc, mask, -1)) != HDD_OK) return st;
         KL(F_PS, 2 * ld * cs + ldc * 16, 0, launch_prolong_stencil<R>(a, 1, f, sc, V, nullptr, 0, p3, mask, s));
     } else {
         // learned initial guess ũ₀ = σ·CNN(f̃/σ) (tensor-core inference); ref = ||P f̃|| and
@@ -915,7 +1175,8 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         KL(F_LMISC, 3 * ld * cs, 0, launch_local_A<R>(a, u, t, f, mask, s));
         KL(F_ZT, ld * cs + ldc * 16, 0, launch_zt<R>(a, f, yy, 0, mask, s));
         KL(F_ZT, ld * cs + ldc * 16, 0, launch_zt<R>(a, t, yy + ldc, 0, mask, s));
-        band_solve2(ctx, ctx->E, yy, ss, m2, s, cdf);
+        if (!dense) band_solve2(ctx, ctx->E, yy, ss, m2, s, cdf);
+        else if ((st = dense_solve(ctx, ctx->E, ds, 1, yy, ss, m2, s)) != HDD_OK) return st;
         CK(cudaMemcpyAsync(sc, ss + ldc, ldc * sizeof(double2), cudaMemcpyDeviceToDevice, s));
         KL(F_PS, 2 * ld * cs + ldc * 16, 0, launch_prolong_stencil<R>(a, 1, f, ss, x, nullptr, 0, p3, mask, s));
         KL(F_LMISC, 0, 0, launch_set_ref<R>(a, S, p3, mask, s));
@@ -942,7 +1203,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
             const double fa = (double)nact / nt;            // fraction of tasks still iterating
             double2 *si = sc + (long long)(i + 1) * ldc;  // E⁻¹ Zᵀ A v_i, kept for the completion
             if (stepC > 0) {
-                band_solve(ctx, ctx->E, y, si, false, ain, s, nact, cdf);
+                if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
                 CK(cudaMemsetAsync(aout, 0, nt * sizeof(int), s));
                 CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
                 // algorithmic bytes of the fused schedule: 3 passes over V_0..V_i, v_i, v_{i+1}
@@ -951,7 +1212,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
                    CK(launch_arnoldi_step<R>(a, stepC, i, RST, V, si, y, S, ain, aout, cnt, tol, maxit, step_sm, s)));
             } else {
                 KL(F_ZT, fa * (ld * cs + ldc * 16), 0, launch_zt<R>(a, vi, y, 1, ain, s));
-                band_solve(ctx, ctx->E, y, si, false, ain, s, nact, cdf);
+                if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
                 KL(F_PS, fa * ((i + 3) * ld * cs + ldc * 16), fa * 8.0 * (i + 1) * ld,
                    launch_prolong_stencil<R>(a, 0, vi, si, vn, V, i + 1, p1, ain, s));
                 KL(F_CGS, fa * (i + 3) * ld * cs, fa * 16.0 * (i + 1) * ld,
@@ -980,7 +1241,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         // restart: r = P(f̃ - A ũ) → v0
         KL(F_LMISC, 0, 0, launch_local_A<R>(a, u, t, f, rs, s));
         KL(F_ZT, 0, 0, launch_zt<R>(a, t, y, 0, rs, s));
-        band_solve(ctx, ctx->E, y, sc, false, rs, s, nrs, cdf);
+        if ((st = coarse(y, sc, rs, nrs)) != HDD_OK) return st;
         KL(F_PS, 0, 0, launch_prolong_stencil<R>(a, 1, t, sc, V, nullptr, 0, p3, rs, s));
         CK(cudaMemsetAsync(act[cur], 0, nt * sizeof(int), s));
         CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
@@ -1280,6 +1541,7 @@ hdd_status build_tasks(hdd_ctx *ctx, int nrhs) {
     const int ns = (int)ctx->subs.size();
     // a fine tile holds at most LOCAL_THREADS·FINE_EPT nodes (one register slot per thread each)
     while (ctx->frows > 1 && ctx->frows * ctx->max_nx > LOCAL_THREADS * FINE_EPT) ctx->frows--;
+    for (auto &P : ctx->E.plan) P.ntask = 0;
     ctx->h_tasks.clear(); ctx->h_ftiles.clear(); ctx->h_ctiles.clear(); ctx->h_tct.clear();
     ctx->step_C[0] = ctx->step_C[1] = -1;
     ctx->foffs.assign(1, 0); ctx->coffs.assign(1, 0);
@@ -1395,7 +1657,9 @@ hdd_status hdd_create(hdd_ctx **out, int device) {
     ctx->device = device;
     if (cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || ctx->nsm < 1)
         ctx->nsm = 152;
-    if (cudaMallocHost(&ctx->h_counter, sizeof(int)) != cudaSuccess || ctx->d_counter.ensure(sizeof(int)) != cudaSuccess) {
+    if (cudaMallocHost(&ctx->h_counter, 2 * sizeof(int)) != cudaSuccess ||
+        ctx->d_counter.ensure(2 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_counter.p, 0, 2 * sizeof(int)) != cudaSuccess) {
         delete ctx;
         return HDD_ERR_OOM;
     }
@@ -2071,7 +2335,11 @@ hdd_status hdd_setup_batch(hdd_ctx *ctx, int nrhs) {
     if (!ctx->dd) FAIL(HDD_ERR_STATE, "hdd_setup_dd first");
     if (nrhs < 1 || nrhs > 4096) FAIL(HDD_ERR_INVALID_ARG, "nrhs must be in 1..4096");
     CK(cudaSetDevice(ctx->device));
-    return build_tasks(ctx, nrhs);
+    hdd_status st = build_tasks(ctx, nrhs);
+    if (st != HDD_OK || !ctx->E.ready) return st;
+    st = coarse_forms(ctx, ctx->E, 0);
+    CK(cudaStreamSynchronize(0));
+    return st;
 }
 
 int hdd_num_rhs(const hdd_ctx *ctx) { return ctx && ctx->dd ? ctx->nrhs : 0; }
@@ -2285,6 +2553,7 @@ hdd_status hdd_set_option(hdd_ctx *ctx, int key, int value) {
     else if (key == HDD_OPT_COARSE_DF) ctx->coarse_df = value;
     else if (key == HDD_OPT_COARSE_SPIKE) ctx->coarse_spike = value;
     else if (key == HDD_OPT_OUTER_DOTS_BIASED) ctx->outer_bias = value;
+    else if (key == HDD_OPT_COARSE_DENSE) ctx->coarse_dense = value;
     else FAIL(HDD_ERR_INVALID_ARG, "unknown option %d", key);
     return HDD_OK;
 }
@@ -2336,6 +2605,11 @@ hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void
     const double2 *in = (const double2 *)in_dev;
     double2 *out = (double2 *)out_dev;
     if (op == 3) {
+        // the hook applies the banded kernels, whichever form the inner iteration takes
+        if (prec == 64 && ctx->coarse_spike && !ctx->E.spike_tried) {
+            hdd_status st = spike_build(ctx, ctx->E);
+            if (st != HDD_OK) return st;
+        }
         band_solve(ctx, ctx->E, in, out, false, nullptr, s, -1, prec == 64);
         CKL(); CK(cudaStreamSynchronize(s)); return HDD_OK;
     }

@@ -311,6 +311,52 @@ void launch_block_solve(const Task *tasks, int ntasks, const BlockFactor *shapes
                         const float2 *Mdf = nullptr);
 void launch_ops_to_df(long long n, const double *M, float2 *Mdf, cudaStream_t s);
 
+// ---- the coarse solve as a product with the explicit E⁻¹ (kernels_dense.cu) ----------------
+constexpr int DSL = 7;                       // base-256 digits per entry (56 bits)
+constexpr int DENSE_ABYTES = DSL * 128 * 16 * 2;   // operator digits of 128 rows x 16 columns
+// most columns of a column tile: 6 sums x 80, 7 sums x 64 of the 512 TMEM columns, 256 per MMA
+constexpr int dense_nt(int ds) { return ds == 6 ? 80 : 64; }
+constexpr int DENSE_MAXST = 7;               // stages of the shared-memory ring
+constexpr int DENSE_MINU = 4;                // fewest units (16 operator columns) a CTA is given
+constexpr int DENSE_TILEW = 6;               // units that a tile's own cost is worth in the split of the work
+constexpr int DENSE_MAXNS = 1024;            // shapes the kernel's unit table takes
+struct InvJob { int shape, jc; long long woff; };   // 16 columns of one shape's E⁻¹ and their workspace
+struct InvShape {                            // one shape at set-up
+    long long woff, roff, soff, aoff;        // workspace (doubles), row maxima, row exponents, operator (bytes)
+    long long rows;                          // workspace rows per column block: 16·nblk
+    int m, mt, kseg, kc, re2;                // order of E, row tiles, chunks per part and in all
+};
+struct DenseShape {                          // one shape of a solve plan
+    long long aoff, soff, boff, acc0;        // operator (bytes), row exponents, right-hand-side digits (bytes), sums
+    int m, mt, kseg, kc, re2;
+    int nt, nct;                             // columns per column tile (multiple of 16), column tiles
+    int t0, ntask;                           // its tasks in the plan's list
+};
+struct DenseTask {                           // one task of a solve plan
+    long long coff, b0;                      // its packed coarse offset; its first column's records in B
+    int m, kseg, nt, re2;                    // of its shape
+};
+struct DensePlanArgs {
+    const DenseTask *recs; int ntask;
+    const DenseShape *sh; int ns;
+    const int *tlist;                        // tasks by shape
+    const int4 *sunits;                      // per shape {tiles, units of one, weight of a unit, 0}
+    const int4 *items; int nitem;            // {shape, tile, first column pair, 0}: 8 pairs of a tile
+    const int *tshape;                       // task → shape
+    const long long *tcoff;                  // task → its packed coarse offset
+    const uint8_t *A; const int *rexp;       // operator digits, row exponents
+    uint8_t *B; int *cexp; unsigned long long *ws; int2 *part;
+    int ntmax, nst, grid;
+    int *err;
+};
+size_t inv_cols_smem(int maxK, int cw);
+cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns, int mmax, int ksegmax, int mtmax,
+                       const BlockFactor *shapes, const double *Mall, const int *Pall, const int4 *Meta, double *W,
+                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, cudaStream_t s);
+int dense_stages(int ds, int ns, int ntmax);
+cudaError_t dense_set_smem();
+void launch_dense_solve(int ds, const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s);
+
 // SPIKE partition of one factor's blocked solve (Polizzi & Sameh's SPIKE algorithm for banded
 // systems, on the blocked operators): the block range [0, nblk) split into P parts solved at
 // once by a cluster of P CTAs, each part with zero values outside it; the exact solution follows

@@ -67,6 +67,32 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
         "}\n" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
 }
 
+// The same with descriptors given by their low words and one high word for both.
+__device__ __forceinline__ void mma_bf16_lohi(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
+                                              uint32_t acc) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        ".reg .b64 a, b;\n"
+        "mov.b64 a, {%1, %3};\n"
+        "mov.b64 b, {%2, %3};\n"
+        "setp.ne.b32 p, %5, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n"
+        "}\n" ::"r"(tmem_d), "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
+}
+
+// True in one lane of a fully active warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n" : "=r"(e));
+    return e != 0;
+}
+
 // Arrive on the mbarrier once every tcgen05 operation issued so far by this thread completes.
 __device__ __forceinline__ void commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
@@ -92,6 +118,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, int m
         if (done) return true;
     }
     return false;
+}
+
+// Wait for the given phase parity for at most `limit` nanoseconds; also gives up when *stop (may be
+// null) becomes non-zero.
+__device__ __forceinline__ bool mbar_wait_ns(uint64_t *mbar, uint32_t parity, unsigned long long limit,
+                                             volatile int *stop) {
+    unsigned long long t0 = 0;
+    for (unsigned it = 0;; it++) {
+        if (mbar_wait(mbar, parity, 1)) return true;
+        if ((it & 63u) != 63u) continue;
+        if (stop && *stop) return false;
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;\n" : "=l"(t));
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > limit) return false;
+    }
+}
+
+// One arrival on the mbarrier.
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 // Expect `bytes` of asynchronous-copy completions on the mbarrier and arrive once.
