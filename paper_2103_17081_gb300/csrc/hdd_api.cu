@@ -850,7 +850,7 @@ hdd_status cnn_buffers(hdd_ctx *ctx) {
     CK(C.A3.ensure(ld * 32 * sizeof(float))); CK(C.A4.ensure(ld * 2 * sizeof(float)));
     CK(C.dA4.ensure(ld * 2 * sizeof(float))); CK(C.Rr.ensure(ld * 2 * sizeof(float)));
     CK(C.dB1.ensure(ld * 32 * sizeof(float))); CK(C.dB2.ensure(ld * 32 * sizeof(float)));
-    CK(C.part.ensure((size_t)nft * (CNN_OFF[2] - CNN_OFF[1]) * sizeof(float)));
+    CK(C.part.ensure((size_t)conv_bwd_w_parts(nft) * (CNN_OFF[2] - CNN_OFF[1]) * sizeof(float)));
     CK(C.lpart.ensure(nft * sizeof(float)));
     CK(C.Fh.ensure(ld * sizeof(float2))); CK(C.Q.ensure(ld * sizeof(float2))); CK(C.T2.ensure(ld * sizeof(float2)));
     CK(C.Yc.ensure(ctx->ldc * sizeof(double2))); CK(C.Sc.ensure(ctx->ldc * sizeof(double2)));
@@ -876,7 +876,7 @@ void cnn_forward(hdd_ctx *ctx, const c2<R> *f, cudaStream_t s) {
     for (int l = 0; l < 4; l++) {
         const int nw = COUT[l] * 9 * CIN[l];
         KL(F_CNN, px * 4.0 * (CIN[l] + COUT[l]), 2.0 * px * nw,
-           launch_conv_fwd(l, T, ft, nft, Wb + CNN_OFF[l], P + CNN_OFF[l] + nw, acts[l], acts[l + 1], s));
+           launch_conv_fwd(l, T, ft, nft, ctx->max_nx, ctx->frows, Wb + CNN_OFF[l], P + CNN_OFF[l] + nw, acts[l], acts[l + 1], s));
     }
 }
 
@@ -1008,11 +1008,11 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     for (int l = 3; l >= 0; l--) {
         const float *mask = l == 3 ? nullptr : acts[l + 1];            // ReLU of this layer's output
         const int nw = CNN_OFF[l + 1] - CNN_OFF[l];
-        KL(F_CNN, 0, 0, launch_conv_bwd_w(l, T, ft, nft, dY, mask, acts[l], part, s));
-        KL(F_CNN, 0, 0, launch_sum_partials(part, nft, nw, 1.0f, G + CNN_OFF[l], s));
+        KL(F_CNN, 0, 0, launch_conv_bwd_w(l, T, ft, nft, ctx->max_nx, dY, mask, acts[l], part, s));
+        KL(F_CNN, 0, 0, launch_sum_partials(part, conv_bwd_w_parts(nft), nw, 1.0f, G + CNN_OFF[l], s));
         if (l > 0) {
             float *dX = bufs[l & 1];
-            KL(F_CNN, 0, 0, launch_conv_bwd_data(l, T, ft, nft, Wb + CNN_OFF[l], dY, mask, dX, s));
+            KL(F_CNN, 0, 0, launch_conv_bwd_data(l, T, ft, nft, ctx->max_nx, ctx->frows, Wb + CNN_OFF[l], dY, mask, dX, s));
             dY = dX;
         }
         (void)CIN; (void)COUT;

@@ -400,14 +400,15 @@ void launch_cnn_task_loss(const Task *tasks, int ntasks, const float2 *p3r, cons
 template <typename R> void launch_cnn_output(const Task *tasks, const Tile *tiles, int ntiles,
                                              const float *sigma, const float *Y4, c2<R> *x0,
                                              const int *flag, cudaStream_t s);
-void launch_conv_fwd(int layer, const Task *tasks, const Tile *tiles, int ntiles, const __nv_bfloat16 *W,
-                     const float *b, const float *X, float *Y, cudaStream_t s);
-void launch_conv_bwd_data(int layer, const Task *tasks, const Tile *tiles, int ntiles,
-                          const __nv_bfloat16 *W, const float *dY, const float *act_out, float *dX,
-                          cudaStream_t s);
-void launch_conv_bwd_w(int layer, const Task *tasks, const Tile *tiles, int ntiles, const float *dY,
+// (max_nx, frows: the widest box and the tallest fine tile, for shared memory)
+void launch_conv_fwd(int layer, const Task *tasks, const Tile *tiles, int ntiles, int max_nx, int frows,
+                     const __nv_bfloat16 *W, const float *b, const float *X, float *Y, cudaStream_t s);
+void launch_conv_bwd_data(int layer, const Task *tasks, const Tile *tiles, int ntiles, int max_nx, int frows,
+                          const __nv_bfloat16 *W, const float *dY, const float *act_out, float *dX, cudaStream_t s);
+int conv_bwd_w_parts(int ntiles);            // partial sums per weight
+void launch_conv_bwd_w(int layer, const Task *tasks, const Tile *tiles, int ntiles, int max_nx, const float *dY,
                        const float *act_out, const float *X, float *part, cudaStream_t s);
-void launch_sum_partials(const float *part, int ntiles, int nw, float scale, float *grad, cudaStream_t s);
+void launch_sum_partials(const float *part, int npart, int nw, float scale, float *grad, cudaStream_t s);
 void launch_cnn_resid(const Task *tasks, const Tile *tiles, int ntiles, const Stencil &st, const float *X0,
                       const float *Y4, float *Rr, float *lpart, cudaStream_t s);
 void launch_cnn_out_grad(const Task *tasks, const Tile *tiles, int ntiles, const Stencil &st, const float *Rr,
