@@ -71,8 +71,8 @@ template <typename R> struct InnerWork {   // inner GMRES buffers for one precis
     int restart = 0;
     DevMem f, u, x, t, V, y, s, p1, p2, p3;
     DevMem y2, s2;                              // two coarse vectors per task (warm start)
-    DevMem H, cs, sn, g, ref, its, kcols, conv, rsf;
-    DevMem act0, act1, flagA, flagB;
+    DevMem H, cs, sn, g, ref, rsf;
+    DevMem ints;                                // per task: its, conv, kcols, two active sets, two restart sets
 };
 
 // Kernel families timed by the profiler (CUDA events around every launch on the launching
@@ -1047,21 +1047,19 @@ template <typename R> hdd_status ensure_inner(hdd_ctx *ctx, int R_) {
     CK(W.sn.ensure((size_t)nt * R_ * cs));
     CK(W.g.ensure((size_t)nt * (R_ + 1) * cs));
     CK(W.ref.ensure(nt * sizeof(R)));
-    CK(W.its.ensure(nt * sizeof(int))); CK(W.kcols.ensure(nt * sizeof(int)));
-    CK(W.conv.ensure(nt * sizeof(int))); CK(W.rsf.ensure(nt * sizeof(int)));
-    CK(W.act0.ensure(nt * sizeof(int))); CK(W.act1.ensure(nt * sizeof(int)));
-    CK(W.flagA.ensure(nt * sizeof(int))); CK(W.flagB.ensure(nt * sizeof(int)));
+    CK(W.rsf.ensure(nt * sizeof(int)));
+    CK(W.ints.ensure(7 * nt * sizeof(int)));
     W.restart = R_;
     size_t smem = local_max_dynamic_smem(ctx->max_nx, (int)cs, ctx->frows, ctx->crows);
     if (smem > 48 * 1024) CK(set_local_smem_limits<R>(smem));
     return HDD_OK;
 }
 
-template <typename R> InnerState<R> inner_state(InnerWork<R> &W) {
+template <typename R> InnerState<R> inner_state(InnerWork<R> &W, int nt) {
     InnerState<R> S;
     S.H = W.H.template as<c2<R>>(); S.cs = W.cs.template as<R>(); S.sn = W.sn.template as<c2<R>>();
-    S.g = W.g.template as<c2<R>>(); S.ref = W.ref.template as<R>(); S.its = W.its.template as<int>();
-    S.kcols = W.kcols.template as<int>(); S.conv = W.conv.template as<int>(); S.restart = W.rsf.template as<int>();
+    S.g = W.g.template as<c2<R>>(); S.ref = W.ref.template as<R>(); S.its = W.ints.template as<int>();
+    S.conv = S.its + nt; S.kcols = S.its + 2 * nt; S.restart = W.rsf.template as<int>();
     return S;
 }
 
@@ -1113,17 +1111,16 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     if (st != HDD_OK) return st;
     if (prm->warm_start && ctx->cnn.ready && (st = cnn_buffers(ctx)) != HDD_OK) return st;
     InnerWork<R> &W = work<R>(ctx);
-    InnerState<R> S = inner_state<R>(W);
     LocalArgs<R> a = local_args<R>(ctx);
     const long long ld = ctx->ld, ldc = ctx->ldc;
     const double cs = (double)sizeof(c2<R>);
     const int nt = (int)ctx->h_tasks.size();
+    InnerState<R> S = inner_state<R>(W, nt);
     c2<R> *f = W.f.template as<c2<R>>(), *u = W.u.template as<c2<R>>(), *x = W.x.template as<c2<R>>();
     c2<R> *t = W.t.template as<c2<R>>(), *V = W.V.template as<c2<R>>();
     double2 *y = W.y.template as<double2>(), *sc = W.s.template as<double2>();
     c2<R> *p1 = W.p1.template as<c2<R>>(), *p2 = W.p2.template as<c2<R>>(), *p3 = W.p3.template as<c2<R>>();
-    int *act[2] = {W.act0.template as<int>(), W.act1.template as<int>()};
-    int *cyc = W.flagA.template as<int>(), *rs = W.flagB.template as<int>();
+    int *act[2] = {S.its + 3 * nt, S.its + 4 * nt}, *rs = S.its + 5 * nt, *rs2 = S.its + 6 * nt;
     int *cnt = ctx->d_counter.as<int>();
     const int *ones = ctx->d_ones.as<int>();
     const R tol = (R)prm->inner_tol;
@@ -1143,14 +1140,9 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
 
     const int *all = mask ? mask : ones;
     KL(F_LMISC, ld * (16 + cs), 0, launch_restrict<R>(a, v, ctx->nglob, f, mask, s));
-    CK(cudaMemsetAsync(W.its.p, 0, nt * sizeof(int), s));
-    CK(cudaMemsetAsync(W.conv.p, 0, nt * sizeof(int), s));
-    CK(cudaMemsetAsync(W.kcols.p, 0, nt * sizeof(int), s));
-    CK(cudaMemsetAsync(act[0], 0, nt * sizeof(int), s));
-    CK(cudaMemsetAsync(act[1], 0, nt * sizeof(int), s));
+    CK(cudaMemsetAsync(W.ints.p, 0, 7 * nt * sizeof(int), s));
     const bool warm = prm->warm_start && ctx->cnn.ready;
     if (!warm) {
-        CK(cudaMemsetAsync(u, 0, ld * sizeof(c2<R>), s));
         // first cycle from ũ = 0: r0 = P f̃ = f̃ - A Z E⁻¹ Zᵀ f̃, and ref = ||P f̃||
         KL(F_ZT, ld * cs + ldc * 16, 0, launch_zt<R>(a, f, y, 0, mask, s));
         if ((st = coarse(y, sc, mask, -1)) != HDD_OK) return st;
@@ -1185,7 +1177,9 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
     KL(F_LMISC, 2 * ld * cs, 0, launch_init_cycle<R>(a, S, RST, V, p3, all, act[0], cnt, tol, maxit, warm ? 0 : 1, s));
     CKL();
-    CK(cudaMemcpyAsync(cyc, all, nt * sizeof(int), cudaMemcpyDeviceToDevice, s));
+    const int *cyc = all;                       // tasks of this cycle
+    bool first = !warm;                         // ũ is still zero (and not in memory)
+    double2 *scomp = sc + (long long)(RST + 1) * ldc;
     int cur = 0, nact = 0;
     st = read_counter(ctx, s, &nact);
     if (st != HDD_OK) return st;
@@ -1204,7 +1198,6 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
             double2 *si = sc + (long long)(i + 1) * ldc;  // E⁻¹ Zᵀ A v_i, kept for the completion
             if (stepC > 0) {
                 if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
-                CK(cudaMemsetAsync(aout, 0, nt * sizeof(int), s));
                 CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
                 // algorithmic bytes of the fused schedule: 3 passes over V_0..V_i, v_i, v_{i+1}
                 // written and read back for the next Zᵀ A, s read and y written
@@ -1229,11 +1222,15 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
             st = read_counter(ctx, s, &nact);
             if (st != HDD_OK) return st;
         }
-        // end of cycle: ũ += V y for the tasks of this cycle; flag the ones needing a restart
+        // end of cycle for its tasks: ũ += V y, and for those that are done the completion
+        // x = ũ + Z E⁻¹ Zᵀ (f̃ - A ũ), E⁻¹ Zᵀ (f̃ - A ũ) = s₀ - Σ y_i s_{i+1} (linearity; every term
+        // was solved during the cycle), into z = Σ R_jᵀ D_j x_j; flag the ones needing a restart
         CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
-        CK(cudaMemsetAsync(rs, 0, nt * sizeof(int), s));
-        KL(F_LMISC, 0, 0, launch_update_u<R>(a, S, RST, u, V, cyc, rs, cnt, maxit, s));
+        KL(F_LMISC, (RST + 2) * ldc * 16.0, 0, launch_coarse_combine<R>(a, S, RST, sc, scomp, cyc, s));
+        KL(F_LMISC, ld * (5 * cs + 16) + ldc * 16, 0,
+           launch_finish<R>(a, S, RST, first ? 1 : 0, u, V, scomp, cyc, rs, cnt, maxit, ctx->nglob, z, s));
         CKL();
+        first = false;
         int nrs = 0;
         st = read_counter(ctx, s, &nrs);
         if (st != HDD_OK) return st;
@@ -1247,19 +1244,14 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
         KL(F_LMISC, 0, 0, launch_init_cycle<R>(a, S, RST, V, p3, rs, act[cur], cnt, tol, maxit, 0, s));
         CKL();
-        std::swap(cyc, rs);
+        cyc = rs;
+        std::swap(rs, rs2);
+        CK(cudaMemsetAsync(rs, 0, nt * sizeof(int), s));
         st = read_counter(ctx, s, &nact);
         if (st != HDD_OK) return st;
     }
-    // completion x = ũ + Z E⁻¹ Zᵀ (f̃ - A ũ) with E⁻¹ Zᵀ (f̃ - A ũ) = s₀ - Σ y_i s_{i+1}
-    // (linearity; every term was solved during the last cycle), then z = Σ R_jᵀ D_j x_j
-    double2 *scomp = sc + (long long)(RST + 1) * ldc;
-    KL(F_LMISC, (RST + 2) * ldc * 16.0, 0, launch_coarse_combine<R>(a, S, RST, sc, scomp, mask, s));
-    KL(F_LMISC, 2 * ld * cs + ldc * 16, 0, launch_z<R>(a, scomp, u, x, mask, s));
-    KL(F_LMISC, ld * (cs + 16), 0, launch_scatter<R>(a, x, z, ctx->nglob, mask, s));
-    CKL();
     ctx->h_its.resize(nt);
-    CK(cudaMemcpyAsync(ctx->h_its.data(), W.its.p, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(ctx->h_its.data(), S.its, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     ctx->prof.harvest();
     long long tot = 0, nh = 0;

@@ -255,9 +255,10 @@ template <typename R> void launch_init_cycle(const LocalArgs<R> &a, const InnerS
                                              c2<R> *v0, const c2<R> *p3, const int *flag,
                                              int *act_out, int *counter, R tol, int maxit,
                                              int set_ref, cudaStream_t s);
-template <typename R> void launch_update_u(const LocalArgs<R> &a, const InnerState<R> &S, int restart,
-                                           c2<R> *u, const c2<R> *V, const int *flag, int *rs_out,
-                                           int *counter, int maxit, cudaStream_t s);
+template <typename R> void launch_finish(const LocalArgs<R> &a, const InnerState<R> &S, int restart, int first,
+                                         c2<R> *u, const c2<R> *V, const double2 *sc, const int *flag,
+                                         int *rs_out, int *counter, int maxit, long long nglob, double2 *glob,
+                                         cudaStream_t s);
 template <typename R> cudaError_t set_local_smem_limits(size_t bytes);
 template <typename R> void launch_set_ref(const LocalArgs<R> &a, const InnerState<R> &S, const c2<R> *p3,
                                           const int *flag, cudaStream_t s);

@@ -608,34 +608,54 @@ k_coarse_combine(LocalArgs<R> a, InnerState<R> S, int restart, const double2 *__
     }
 }
 
-// u += V y with y = H⁻¹ g (each tile solves the small triangle itself); the first tile of a
-// task flags it for another cycle when it neither converged nor ran out of iterations.
+// End of a cycle for its tasks: ũ += V y with y = H⁻¹ g (each tile solves the small triangle
+// itself; first: ũ was zero and is not read), and for a task that is done the completed solution
+// ũ + Z s straight into the owned nodes of the global vector, z = Σ_j R_jᵀ D_j x_j (every owned
+// node is written by exactly one task, no atomics).  A task that neither converged nor ran out of
+// iterations keeps ũ and is flagged for another cycle.  One pass over V and z where the update,
+// the prolongation and the scatter made three, with ũ and x through memory in between: FIN_US us
+// for the three kernels' SEP_US at k=200.
 template <typename R>
 __global__ void __launch_bounds__(LOCAL_THREADS)
-k_update_u(LocalArgs<R> a, InnerState<R> S, int restart, c2<R> *__restrict__ u,
-           const c2<R> *__restrict__ V, const int *__restrict__ flag, int *__restrict__ rs_out,
-           int *__restrict__ counter, int maxit) {
+k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restrict__ u, const c2<R> *__restrict__ V,
+         const double2 *__restrict__ s, const int *__restrict__ flag, int *__restrict__ rs_out,
+         int *__restrict__ counter, int maxit, long long nglob, double2 *__restrict__ glob) {
+    extern __shared__ unsigned char smem_raw[];
     __shared__ c2<R> y[MAX_RESTART];
     const Tile tl = a.ftiles[blockIdx.x];
-    if (!flag[tl.task]) return;
-    const Task T = a.tasks[tl.task];
     const int t = tl.task;
+    if (!flag[t]) return;
+    const Task T = a.tasks[t];
     const int k = S.kcols[t];
+    const bool again = !S.conv[t] && S.its[t] < maxit;
     if (threadIdx.x == 0) {
         solve_small<R>(S, restart, t, k, y);
         if (blockIdx.x == T.tile0) {
-            const bool again = !S.conv[t] && S.its[t] < maxit;
             rs_out[t] = again ? 1 : 0;
             if (again) atomicAdd(counter, 1);
         }
     }
-    __syncthreads();
-    if (k == 0) return;
+    const int maxc = prolong_max_cy(tl.nr);
+    c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
+    c2<R> *px = sc + maxc * T.mx;
+    c2<R> *zs = px + maxc * T.nx;
+    if (!again) prolong_rows<R>(T, s, tl.r0, tl.nr, sc, px, zs);       // ends with a barrier
+    else __syncthreads();
+    const BoxDiv dnx(T.nx);
     const long long base = T.foff + (long long)tl.r0 * T.nx;
     for (int e = threadIdx.x; e < tl.nr * T.nx; e += blockDim.x) {
-        c2<R> x = u[base + e];
+        const int yy = dnx.q(e), gx = T.ix0 + e - yy * T.nx, gy = T.iy0 + tl.r0 + yy;
+        const bool own = gx >= T.ox0 && gx <= T.ox1 && gy >= T.oy0 && gy <= T.oy1;
+        if (!again && !own) continue;
+        c2<R> x = first ? mk<R>(0, 0) : u[base + e];
         for (int l = 0; l < k; l++) caxpy<R>(x, y[l], V[(long long)l * a.ld + base + e]);
-        u[base + e] = x;
+        if (again) {
+            u[base + e] = x;
+        } else {
+            x = cadd<R>(x, zs[e]);
+            glob[(long long)(gx - a.glo) + (long long)(gy - a.glo) * a.gw + (long long)T.rhs * nglob] =
+                make_double2((double)x.x, (double)x.y);
+        }
     }
 }
 
@@ -733,7 +753,10 @@ k_arnoldi_step(StepArgs<R> a) {
     const int C = a.C;
     const int t = (int)blockIdx.x / C;
     const unsigned rank = cluster_rank();
-    if (!a.act_in[t]) return;                     // the same flag for every CTA of the cluster
+    if (!a.act_in[t]) {                           // the same flag for every CTA of the cluster
+        if (rank == 0 && threadIdx.x == 0) a.act_out[t] = 0;
+        return;
+    }
     const Task T = a.tasks[t];
     const int nx = T.nx, ny = T.ny, mx = T.mx, my = T.my;
     const BoxDiv dnx(nx), dmx(mx);
@@ -977,11 +1000,14 @@ void launch_zt(const LocalArgs<R> &a, const c2<R> *in, double2 *y, int apply_A, 
     else k_zt<R, false><<<a.nctiles, LOCAL_THREADS, zt_smem(a, apply_A), s>>>(a, in, y, apply_A, flag);
 }
 template <typename R>
+size_t z_smem(const LocalArgs<R> &a) {
+    const int maxc = prolong_max_cy(a.frows);
+    return ((size_t)maxc * (a.max_nx / 2 + 1) + (size_t)maxc * a.max_nx + (size_t)a.frows * a.max_nx) * csz<R>();
+}
+template <typename R>
 void launch_z(const LocalArgs<R> &a, const double2 *sc, const c2<R> *add, c2<R> *out,
               const int *flag, cudaStream_t s, R sign) {
-    int maxc = prolong_max_cy(a.frows);
-    size_t sm = ((size_t)maxc * (a.max_nx / 2 + 1) + (size_t)maxc * a.max_nx + (size_t)a.frows * a.max_nx) * csz<R>();
-    k_z<R><<<a.nftiles, LOCAL_THREADS, sm, s>>>(a, sc, add, out, flag, sign);
+    k_z<R><<<a.nftiles, LOCAL_THREADS, z_smem(a), s>>>(a, sc, add, out, flag, sign);
 }
 template <typename R>
 size_t ps_smem(const LocalArgs<R> &a) {
@@ -1021,10 +1047,11 @@ void launch_init_cycle(const LocalArgs<R> &a, const InnerState<R> &S, int restar
                                                          tol, maxit, set_ref);
 }
 template <typename R>
-void launch_update_u(const LocalArgs<R> &a, const InnerState<R> &S, int restart, c2<R> *u,
-                     const c2<R> *V, const int *flag, int *rs_out, int *counter, int maxit,
-                     cudaStream_t s) {
-    k_update_u<R><<<a.nftiles, LOCAL_THREADS, 0, s>>>(a, S, restart, u, V, flag, rs_out, counter, maxit);
+void launch_finish(const LocalArgs<R> &a, const InnerState<R> &S, int restart, int first, c2<R> *u, const c2<R> *V,
+                   const double2 *sc, const int *flag, int *rs_out, int *counter, int maxit, long long nglob,
+                   double2 *glob, cudaStream_t s) {
+    k_finish<R><<<a.nftiles, LOCAL_THREADS, z_smem(a), s>>>(a, S, restart, first, u, V, sc, flag, rs_out, counter, maxit,
+                                                            nglob, glob);
 }
 template <typename R>
 void launch_set_ref(const LocalArgs<R> &a, const InnerState<R> &S, const c2<R> *p3, const int *flag,
@@ -1115,6 +1142,7 @@ template <typename R> cudaError_t set_local_smem_limits(size_t bytes) {
     if ((e = cudaFuncSetAttribute(k_zt<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_zt<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_z<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_finish<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_local_A<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_local_A<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     return cudaSuccess;
@@ -1130,7 +1158,7 @@ template <typename R> cudaError_t set_local_smem_limits(size_t bytes) {
     template void launch_cgs_update<R>(const LocalArgs<R> &, int, c2<R> *, const c2<R> *, int, const c2<R> *, c2<R> *, const int *, cudaStream_t); \
     template void launch_givens_normalize<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const c2<R> *, const c2<R> *, const int *, int *, int *, R, int, cudaStream_t); \
     template void launch_init_cycle<R>(const LocalArgs<R> &, const InnerState<R> &, int, c2<R> *, const c2<R> *, const int *, int *, int *, R, int, int, cudaStream_t); \
-    template void launch_update_u<R>(const LocalArgs<R> &, const InnerState<R> &, int, c2<R> *, const c2<R> *, const int *, int *, int *, int, cudaStream_t); \
+    template void launch_finish<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const double2 *, const int *, int *, int *, int, long long, double2 *, cudaStream_t); \
     template cudaError_t set_local_smem_limits<R>(size_t); \
     template void launch_coarse_combine<R>(const LocalArgs<R> &, const InnerState<R> &, int, const double2 *, double2 *, const int *, cudaStream_t); \
     template void launch_set_ref<R>(const LocalArgs<R> &, const InnerState<R> &, const c2<R> *, const int *, cudaStream_t); \
