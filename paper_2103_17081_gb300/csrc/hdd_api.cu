@@ -140,6 +140,8 @@ struct OuterWork {
 
 }  // namespace
 
+constexpr int CNT_N = MAX_RESTART + 3;         // error flag, counts before step 0 .. MAX_RESTART, tasks to restart
+
 struct hdd_ctx {
     int device = 0;
     std::string err;
@@ -181,9 +183,12 @@ struct hdd_ctx {
     DevMem tmp_a, tmp_b, tmp_c;                // staging for test hooks
     DevMem d_alist;                            // active tasks of a SPIKE coarse solve, compacted
     int *h_counter = nullptr;                  // pinned copy of d_counter
-    DevMem d_counter;                          // {tasks still running, error flag of the dense solves}
+    DevMem d_counter;                          // error flag of the dense solves, then the tasks still running
+                                               // before each inner step of a cycle and after it (CNT_*)
+    cudaEvent_t ev[2] = {nullptr, nullptr};    // the copies of d_counter that are under way
+    int *h_its = nullptr;                      // pinned: step counts of the tasks
+    size_t h_its_n = 0;
     std::vector<double> hist;
-    std::vector<int> h_its;
     Prof prof;
     int nsm = 152;                             // SMs of the device
     int coarse_la = 1;                         // HDD_OPT_COARSE_LOOKAHEAD
@@ -205,7 +210,11 @@ struct hdd_ctx {
         int c = 0, Nc = 0, m = 0;
         DevMem S64, S32, D64, D32, bufA, bufB, z0, t;
     } cg;
-    ~hdd_ctx() { if (h_counter) cudaFreeHost(h_counter); }
+    ~hdd_ctx() {
+        if (h_counter) cudaFreeHost(h_counter);
+        if (h_its) cudaFreeHost(h_its);
+        for (cudaEvent_t e : ev) if (e) cudaEventDestroy(e);
+    }
 };
 
 #define FAIL(code, ...)                                                                            \
@@ -277,18 +286,18 @@ hdd_status dense_error(hdd_ctx *ctx, int e, cudaStream_t s) {
         FAIL(HDD_ERR_TIMEOUT, "a dense coarse solve's wait and its drain timed out; work still in flight may have "
                               "written freed memory, so this context refuses further work (discard it and its CUDA context)");
     }
-    CK(cudaMemsetAsync(ctx->d_counter.as<int>() + 1, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(ctx->d_counter.p, 0, sizeof(int), s));
     for (auto &P : ctx->E.plan)
         if (P.ws.p) CK(cudaMemsetAsync(P.ws.p, 0, P.ws.bytes, s));
     FAIL(HDD_ERR_TIMEOUT, "a dense coarse solve's wait timed out");
 }
 
-hdd_status read_counter(hdd_ctx *ctx, cudaStream_t s, int *out) {
-    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+// Synchronises the stream; the error flag of the dense coarse solves so far.
+hdd_status sync_checked(hdd_ctx *ctx, cudaStream_t s) {
+    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, CNT_N * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     ctx->prof.harvest();
-    *out = ctx->h_counter[0];
-    return dense_error(ctx, ctx->h_counter[1], s);
+    return dense_error(ctx, ctx->h_counter[0], s);
 }
 
 // ---- SPIKE plans of a factor set (the double-FP32 coarse solve split over P parts) ----------
@@ -594,7 +603,7 @@ hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const doub
     a.A = F.dA.as<uint8_t>(); a.rexp = F.drs.as<int>();
     a.B = P.B.as<uint8_t>(); a.cexp = P.cs.as<int>(); a.ws = P.ws.as<unsigned long long>(); a.part = P.part.as<int2>();
     a.ntmax = P.ntmax; a.nst = P.nst; a.grid = ctx->nsm;
-    a.err = ctx->d_counter.as<int>() + 1;
+    a.err = ctx->d_counter.as<int>();
     KL(F_CDENSE, P.bytes, P.flops, launch_dense_solve(ds, a, in, out, flag, s));
     ctx->prof.launches += 2;
     return HDD_OK;
@@ -1020,8 +1029,7 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     CKL();
     std::vector<float> lt(nt);
     CK(cudaMemcpyAsync(lt.data(), C.tloss.p, nt * sizeof(float), cudaMemcpyDeviceToHost, s));
-    int unused = 0;
-    if ((st = read_counter(ctx, s, &unused)) != HDD_OK) return st;
+    if ((st = sync_checked(ctx, s)) != HDD_OK) return st;
     double L = 0;
     for (int t = 0; t < nt; t++) L += lt[t];
     if (loss) *loss = L / nt;
@@ -1121,7 +1129,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     double2 *y = W.y.template as<double2>(), *sc = W.s.template as<double2>();
     c2<R> *p1 = W.p1.template as<c2<R>>(), *p2 = W.p2.template as<c2<R>>(), *p3 = W.p3.template as<c2<R>>();
     int *act[2] = {S.its + 3 * nt, S.its + 4 * nt}, *rs = S.its + 5 * nt, *rs2 = S.its + 6 * nt;
-    int *cnt = ctx->d_counter.as<int>();
+    int *cnt = ctx->d_counter.as<int>() + 1;     // cnt[i]: tasks before step i; cnt[RST + 1]: tasks to restart
     const int *ones = ctx->d_ones.as<int>();
     const R tol = (R)prm->inner_tol;
     const int maxit = prm->inner_maxit;
@@ -1136,6 +1144,29 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         if (dense) return dense_solve(ctx, ctx->E, ds, 0, in, out, flag, s);
         band_solve(ctx, ctx->E, in, out, false, flag, s, n, cdf);
         return HDD_OK;
+    };
+
+    if (ctx->h_its_n < (size_t)nt) {
+        if (ctx->h_its) { cudaFreeHost(ctx->h_its); ctx->h_its = nullptr; ctx->h_its_n = 0; }
+        CK(cudaMallocHost(&ctx->h_its, nt * sizeof(int)));
+        ctx->h_its_n = nt;
+    }
+    // Progress: each step counts the tasks that go on into a slot of its own, and the slots are
+    // copied to the host after every step.  The host launches a step before it has seen whether any
+    // task needs it, then waits for the count before that step: the device always has the next step
+    // queued, and one step at the end finds no task (a few microseconds against a round trip to the
+    // host per step, 10 to 15).  A split (SPIKE) banded solve is launched for a given number of
+    // tasks, so there the host waits first.
+    const bool ahead = dense || !(cdf && ctx->coarse_spike && ctx->E.spike_levels_built);
+    auto post = [&](int slot) -> hdd_status {
+        CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, CNT_N * sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaEventRecord(ctx->ev[slot & 1], s));
+        return HDD_OK;
+    };
+    auto seen = [&](int slot, int *n) -> hdd_status {
+        CK(cudaEventSynchronize(ctx->ev[slot & 1]));
+        *n = ctx->h_counter[1 + slot];
+        return dense_error(ctx, ctx->h_counter[0], s);
     };
 
     const int *all = mask ? mask : ones;
@@ -1174,23 +1205,27 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         KL(F_LMISC, 0, 0, launch_set_ref<R>(a, S, p3, mask, s));
         KL(F_PS, 2 * ld * cs + ldc * 16, 0, launch_prolong_stencil<R>(a, 1, t, sc, V, nullptr, 0, p3, mask, s));
     }
-    CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(cnt, 0, (RST + 2) * sizeof(int), s));
     KL(F_LMISC, 2 * ld * cs, 0, launch_init_cycle<R>(a, S, RST, V, p3, all, act[0], cnt, tol, maxit, warm ? 0 : 1, s));
     CKL();
+    if ((st = post(0)) != HDD_OK) return st;
     const int *cyc = all;                       // tasks of this cycle
     bool first = !warm;                         // ũ is still zero (and not in memory)
     double2 *scomp = sc + (long long)(RST + 1) * ldc;
-    int cur = 0, nact = 0;
-    st = read_counter(ctx, s, &nact);
-    if (st != HDD_OK) return st;
+    int cur = 0, nact = nt;                     // nact: at most so many tasks run
     // one launch per Arnoldi step between the coarse solves (cluster per task), or the separate
     // stencil, CGS and Givens kernels
     const int stepC = ctx->fused_inner ? step_plan<R>(ctx) : 0;
     const size_t step_sm = ctx->step_smem[sizeof(R) == 4 ? 0 : 1];
     for (;;) {
-        if (stepC > 0 && nact > 0)                        // y = Zᵀ A v_0 of this cycle's tasks
+        if (stepC > 0)                                    // y = Zᵀ A v_0 of this cycle's tasks
             KL(F_ZT, (double)nact / nt * (ld * cs + ldc * 16), 0, launch_zt<R>(a, V, y, 1, act[cur], s));
-        for (int i = 0; i < RST && nact > 0; i++) {
+        for (int i = 0; i < RST; i++) {
+            if (!ahead) {
+                if ((st = seen(i, &nact)) != HDD_OK) return st;
+                if (nact == 0) break;
+            }
+            int *next = cnt + i + 1;
             const int *ain = act[cur];
             int *aout = act[cur ^ 1];
             c2<R> *vi = V + (long long)i * ld, *vn = V + (long long)(i + 1) * ld;
@@ -1198,11 +1233,10 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
             double2 *si = sc + (long long)(i + 1) * ldc;  // E⁻¹ Zᵀ A v_i, kept for the completion
             if (stepC > 0) {
                 if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
-                CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
                 // algorithmic bytes of the fused schedule: 3 passes over V_0..V_i, v_i, v_{i+1}
                 // written and read back for the next Zᵀ A, s read and y written
                 KL(F_STEP, fa * ((3.0 * i + 7) * ld * cs + 2.0 * ldc * 16), fa * 40.0 * (i + 1) * ld,
-                   CK(launch_arnoldi_step<R>(a, stepC, i, RST, V, si, y, S, ain, aout, cnt, tol, maxit, step_sm, s)));
+                   CK(launch_arnoldi_step<R>(a, stepC, i, RST, V, si, y, S, ain, aout, next, tol, maxit, step_sm, s)));
             } else {
                 KL(F_ZT, fa * (ld * cs + ldc * 16), 0, launch_zt<R>(a, vi, y, 1, ain, s));
                 if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
@@ -1213,27 +1247,28 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
                 KL(F_CGS, fa * (i + 3) * ld * cs, fa * 8.0 * (i + 1) * ld,
                    launch_cgs_update<R>(a, 3, vn, V, i + 1, p2, p3, ain, s));
                 CK(cudaMemsetAsync(aout, 0, nt * sizeof(int), s));
-                CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
                 KL(F_GIVENS, fa * 2 * ld * cs, 0,
-                   launch_givens_normalize<R>(a, S, RST, i, vn, p1, p2, p3, ain, aout, cnt, tol, maxit, s));
+                   launch_givens_normalize<R>(a, S, RST, i, vn, p1, p2, p3, ain, aout, next, tol, maxit, s));
             }
             CKL();
             cur ^= 1;
-            st = read_counter(ctx, s, &nact);
-            if (st != HDD_OK) return st;
+            if ((st = post(i + 1)) != HDD_OK) return st;
+            if (ahead) {
+                if ((st = seen(i, &nact)) != HDD_OK) return st;
+                if (nact == 0) break;
+            }
         }
         // end of cycle for its tasks: ũ += V y, and for those that are done the completion
         // x = ũ + Z E⁻¹ Zᵀ (f̃ - A ũ), E⁻¹ Zᵀ (f̃ - A ũ) = s₀ - Σ y_i s_{i+1} (linearity; every term
         // was solved during the cycle), into z = Σ R_jᵀ D_j x_j; flag the ones needing a restart
-        CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
         KL(F_LMISC, (RST + 2) * ldc * 16.0, 0, launch_coarse_combine<R>(a, S, RST, sc, scomp, cyc, s));
         KL(F_LMISC, ld * (5 * cs + 16) + ldc * 16, 0,
-           launch_finish<R>(a, S, RST, first ? 1 : 0, u, V, scomp, cyc, rs, cnt, maxit, ctx->nglob, z, s));
+           launch_finish<R>(a, S, RST, first ? 1 : 0, u, V, scomp, cyc, rs, cnt + RST + 1, maxit, ctx->nglob, z, s));
         CKL();
         first = false;
-        int nrs = 0;
-        st = read_counter(ctx, s, &nrs);
-        if (st != HDD_OK) return st;
+        CK(cudaMemcpyAsync(ctx->h_its, S.its, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
+        if ((st = sync_checked(ctx, s)) != HDD_OK) return st;
+        const int nrs = ctx->h_counter[1 + RST + 1];
         if (nrs == 0) break;
         // restart: r = P(f̃ - A ũ) → v0
         KL(F_LMISC, 0, 0, launch_local_A<R>(a, u, t, f, rs, s));
@@ -1241,19 +1276,15 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         if ((st = coarse(y, sc, rs, nrs)) != HDD_OK) return st;
         KL(F_PS, 0, 0, launch_prolong_stencil<R>(a, 1, t, sc, V, nullptr, 0, p3, rs, s));
         CK(cudaMemsetAsync(act[cur], 0, nt * sizeof(int), s));
-        CK(cudaMemsetAsync(cnt, 0, sizeof(int), s));
+        CK(cudaMemsetAsync(cnt, 0, (RST + 2) * sizeof(int), s));
         KL(F_LMISC, 0, 0, launch_init_cycle<R>(a, S, RST, V, p3, rs, act[cur], cnt, tol, maxit, 0, s));
         CKL();
+        if ((st = post(0)) != HDD_OK) return st;
+        nact = nrs;
         cyc = rs;
         std::swap(rs, rs2);
         CK(cudaMemsetAsync(rs, 0, nt * sizeof(int), s));
-        st = read_counter(ctx, s, &nact);
-        if (st != HDD_OK) return st;
     }
-    ctx->h_its.resize(nt);
-    CK(cudaMemcpyAsync(ctx->h_its.data(), S.its, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    ctx->prof.harvest();
     long long tot = 0, nh = 0;
     int mx = 0;
     for (int q = 0; q < nt; q++) {
@@ -1264,7 +1295,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     if (its_total) *its_total = tot;
     if (its_max) *its_max = mx;
     if (hits) *hits = nh;
-    if (its_out) std::copy(ctx->h_its.begin(), ctx->h_its.end(), its_out);
+    if (its_out) std::copy(ctx->h_its, ctx->h_its + nt, its_out);
     return HDD_OK;
 }
 
@@ -1649,9 +1680,11 @@ hdd_status hdd_create(hdd_ctx **out, int device) {
     ctx->device = device;
     if (cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || ctx->nsm < 1)
         ctx->nsm = 152;
-    if (cudaMallocHost(&ctx->h_counter, 2 * sizeof(int)) != cudaSuccess ||
-        ctx->d_counter.ensure(2 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_counter.p, 0, 2 * sizeof(int)) != cudaSuccess) {
+    if (cudaMallocHost(&ctx->h_counter, CNT_N * sizeof(int)) != cudaSuccess ||
+        ctx->d_counter.ensure(CNT_N * sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_counter.p, 0, CNT_N * sizeof(int)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev[1], cudaEventDisableTiming) != cudaSuccess) {
         delete ctx;
         return HDD_ERR_OOM;
     }
