@@ -91,10 +91,18 @@ __global__ void k_cg_prolong(CGrid g, const c2<T> *__restrict__ xH, double2 *__r
 // Dinv, for an m x m complex matrix `in` (row j, column x) and the real symmetric S:
 // out[x][i] = Dinv[x][i] · Σ_j S[i][j] in[j][x].  Two passes give S X S; the solve is
 // A_H⁻¹ Y = S (D⁻¹ ∘ (S Y S)) S (S orthonormal and symmetric, D symmetric), four passes.
-// CTA: a DT x DT output tile, the j range in chunks of DKC staged in shared memory (coalesced
-// along x for `in` and along i for S, which is read as S[j][i] = S[i][j]); each of the 128
-// threads accumulates 2 rows x 4 columns (i = i0 + ti + 8q, x = x0 + tx + 16p).
-constexpr int DT = 32, DKC = 32, DTHREADS = 128;
+// The sines of row i are even (i odd, counted from 1) or odd (i even) about the middle of the range,
+// S[i][Nc-j] = ±S[i][j], so with e± = in[j] ± in[Nc-j] (the middle entry of an even Nc alone)
+// the sum runs over j <= Nc/2 only: half the products.  CTA: a DT x DT output tile (rows i sorted
+// by parity in shared memory), four groups of 64 threads that each take a quarter of the j range,
+// 4 rows of one parity x 4 columns per thread (16 complex sums for three 16-byte loads); the
+// groups' sums are added up through shared memory in a fixed order.  Bound by latency: at m = 319
+// there are 100 CTAs, one per SM, so a CTA brings its whole operands (DKC pairs of rows at a time)
+// in one go and its eight warps share one tile: 13 us per pass (29 with chunks of 32 rows, four
+// warps and all 319 products per output; 0.8 us at the FP32 peak).
+constexpr int DT = 32, DTHREADS = 256, DGROUPS = 4;
+template <typename T> constexpr int DKC = sizeof(T) == 4 ? 160 : 80;     // pairs of rows staged at a time
+template <typename T> constexpr size_t dst_smem() { return (size_t)DKC<T> * DT * (2 * sizeof(c2<T>) + sizeof(T)); }
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS)
 k_dst_pass(int m, long long ldh, const T *__restrict__ S, const T *__restrict__ Dinv,
@@ -102,57 +110,73 @@ k_dst_pass(int m, long long ldh, const T *__restrict__ S, const T *__restrict__ 
     if (active && !active[blockIdx.z]) return;
     in += blockIdx.z * ldh;
     out += blockIdx.z * ldh;
-    __shared__ c2<T> Xs[DKC][DT];
-    __shared__ T Ss[DKC][DT];
-    const int tid = threadIdx.x, ti = tid & 7, tx = tid >> 3;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    c2<T> *E = reinterpret_cast<c2<T> *>(dsm);                           // [parity][pair][column]
+    T *Ss = reinterpret_cast<T *>(E + (size_t)2 * DKC<T> * DT);          // [pair][parity · 16 + row / 2]
+    const int tid = threadIdx.x, grp = tid >> 6, ti = tid & 7, tx = (tid >> 3) & 7, par = ti >> 2;
     const int i0 = blockIdx.x * DT, x0 = blockIdx.y * DT;
-    c2<T> acc[2][4];
+    const int Nc = m + 1, K = Nc / 2;                                    // pairs 1..K (the last without partner if Nc is even)
+    c2<T> acc[4][4];                                                     // [column][row]
 #pragma unroll
-    for (int p = 0; p < 2; p++)
+    for (int p = 0; p < 4; p++)
 #pragma unroll
         for (int q = 0; q < 4; q++) acc[p][q] = mk<T>((T)0, (T)0);
-    for (int j0 = 0; j0 < m; j0 += DKC) {
-        for (int e = tid; e < DKC * DT; e += DTHREADS) {
-            const int kk = e / DT, cc = e % DT, j = j0 + kk;
-            const bool okj = j < m;
-            Xs[kk][cc] = (okj && x0 + cc < m) ? in[(long long)j * m + x0 + cc] : mk<T>((T)0, (T)0);
-            Ss[kk][cc] = (okj && i0 + cc < m) ? S[(long long)j * m + i0 + cc] : (T)0;
+    for (int k0 = 0; k0 < K; k0 += DKC<T>) {
+        const int nk = min(DKC<T>, K - k0);
+        if (k0) __syncthreads();
+#pragma unroll 4
+        for (int e = tid; e < nk * DT; e += DTHREADS) {
+            const int kk = e / DT, cc = e % DT, j = k0 + kk + 1, x = x0 + cc, i = i0 + cc;
+            c2<T> u = mk<T>((T)0, (T)0), v = u;
+            if (x < m) {
+                u = in[(long long)(j - 1) * m + x];
+                if (2 * j != Nc) v = in[(long long)(Nc - j - 1) * m + x];
+            }
+            // row index i counts from 0: sine number i + 1, even about the middle for even i
+            E[(size_t)kk * DT + cc] = cadd<T>(u, v);
+            E[(size_t)(DKC<T> + kk) * DT + cc] = 2 * j != Nc ? csub<T>(u, v) : mk<T>((T)0, (T)0);
+            Ss[kk * DT + (cc & 1) * 16 + (cc >> 1)] = i < m ? S[(long long)(j - 1) * m + i] : (T)0;
         }
         __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < DKC; kk++) {
+        // (i0 is a multiple of DT, so a row's parity is that of its place in the tile)
+        const c2<T> *Ep = E + (size_t)par * DKC<T> * DT + 4 * tx;
+        const T *Sp = Ss + par * 16 + 4 * (ti & 3);
+        const int ka = grp * nk / DGROUPS, kb = (grp + 1) * nk / DGROUPS;
+#pragma unroll 4
+        for (int kk = ka; kk < kb; kk++) {
             T sv[4];
-            c2<T> xv[2];
+            c2<T> xv[4];
 #pragma unroll
-            for (int q = 0; q < 4; q++) sv[q] = Ss[kk][ti + 8 * q];
+            for (int q = 0; q < 4; q++) { sv[q] = Sp[kk * DT + q]; xv[q] = Ep[(size_t)kk * DT + q]; }
 #pragma unroll
-            for (int p = 0; p < 2; p++) xv[p] = Xs[kk][tx + 16 * p];
-#pragma unroll
-            for (int p = 0; p < 2; p++)
+            for (int p = 0; p < 4; p++)
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
                     acc[p][q].x = fma(sv[q], xv[p].x, acc[p][q].x);
                     acc[p][q].y = fma(sv[q], xv[p].y, acc[p][q].y);
                 }
         }
-        __syncthreads();
     }
+    __syncthreads();                                                     // the operands' space takes the groups' sums
+    c2<T> *R = E;                                                        // [group][column][row], rows padded to 33
+    constexpr int RP = DT + 1;
 #pragma unroll
-    for (int p = 0; p < 2; p++) {
-        const int x = x0 + tx + 16 * p;
-        if (x >= m) continue;
+    for (int p = 0; p < 4; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int i = i0 + ti + 8 * q;
-            if (i >= m) continue;
-            c2<T> r = acc[p][q];
-            if (Dinv) {
-                const T d = Dinv[(long long)x * m + i];
-                r.x *= d;
-                r.y *= d;
-            }
-            out[(long long)x * m + i] = r;
+        for (int q = 0; q < 4; q++) R[((size_t)grp * DT + 4 * tx + p) * RP + 2 * (4 * (ti & 3) + q) + par] = acc[p][q];
+    __syncthreads();
+    for (int e = tid; e < DT * DT; e += DTHREADS) {
+        const int cx = e / DT, ci = e % DT, x = x0 + cx, i = i0 + ci;
+        if (x >= m || i >= m) continue;
+        c2<T> r = R[(size_t)cx * RP + ci];
+#pragma unroll
+        for (int g = 1; g < DGROUPS; g++) r = cadd<T>(r, R[((size_t)g * DT + cx) * RP + ci]);
+        if (Dinv) {
+            const T d = Dinv[(long long)x * m + i];
+            r.x *= d;
+            r.y *= d;
         }
+        out[(long long)x * m + i] = r;
     }
 }
 
@@ -189,7 +213,9 @@ template <typename T>
 void launch_dst_pass(int m, const T *S, const T *Dinv, const c2<T> *in, c2<T> *out, int nrhs, long long ldh,
                      const int *active, cudaStream_t s) {
     const int t = (m + DT - 1) / DT;
-    k_dst_pass<T><<<dim3(t, t, nrhs), DTHREADS, 0, s>>>(m, ldh, S, Dinv, in, out, active);
+    static_assert((size_t)DGROUPS * DT * (DT + 1) * sizeof(c2<T>) <= dst_smem<T>(), "the groups' sums fit");
+    cudaFuncSetAttribute(k_dst_pass<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dst_smem<T>());
+    k_dst_pass<T><<<dim3(t, t, nrhs), DTHREADS, dst_smem<T>(), s>>>(m, ldh, S, Dinv, in, out, active);
 }
 void launch_cg_widen(long long n, const float2 *in, double2 *out, cudaStream_t s) {
     k_cg_convert<float2, double2><<<cg_grid(n), 256, 0, s>>>(n, in, out);
