@@ -652,35 +652,29 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
         else { m[q] = nx * ny; kl[q] = ku[q] = nx + 1; }
         if (re2) { m[q] *= 2; kl[q] = ku[q] = 2 * kl[q] + 1; }
     }
-    std::vector<DevMem> ab(ns), piv(ns);
-    std::vector<double *> abp(ns);
-    std::vector<int *> pivp(ns);
+    std::vector<LuShape> lu(ns);
+    long long nab = 0, nlp = 0, totP = 0;
+    int max_m = 0, max_kl = 0, max_ku = 0, max_nodes = 0;
     for (int q = 0; q < ns; q++) {
-        size_t W = 2 * kl[q] + ku[q] + 1;
-        CK(ab[q].ensure((size_t)m[q] * W * sizeof(double)));
-        CK(cudaMemsetAsync(ab[q].p, 0, (size_t)m[q] * W * sizeof(double), s));
-        CK(piv[q].ensure((size_t)m[q] * sizeof(int)));
-        abp[q] = ab[q].as<double>();
-        pivp[q] = piv[q].as<int>();
-        int nx = ctx->shapes[q].first, ny = ctx->shapes[q].second;
-        const int gx0 = ctx->shape_org[q].first, gy0 = ctx->shape_org[q].second;
-        if (re2 && coarse) launch_assemble_E_re2(ctx->st, nx, ny, gx0, gy0, kl[q], ku[q], abp[q], s);
-        else if (re2) launch_assemble_Aloc_re2(ctx->st, nx, ny, gx0, gy0, kl[q], ku[q], abp[q], s);
-        else if (coarse) launch_assemble_E(ctx->st, nx, ny, kl[q], ku[q], abp[q], s);
-        else launch_assemble_Aloc(ctx->st, nx, ny, kl[q], ku[q], abp[q], s);
-        CKL();
+        const int nx = ctx->shapes[q].first, ny = ctx->shapes[q].second;
+        lu[q] = LuShape{nx, ny, ctx->shape_org[q].first, ctx->shape_org[q].second, m[q], kl[q], ku[q], nab, nlp, totP, 0};
+        nab += (long long)m[q] * (2 * kl[q] + ku[q] + 1);
+        nlp += (long long)m[q] * 3 * kl[q];
+        totP += m[q];
+        max_m = std::max(max_m, m[q]); max_kl = std::max(max_kl, kl[q]); max_ku = std::max(max_ku, ku[q]);
+        max_nodes = std::max(max_nodes, nx * ny);
     }
-    DevMem dm, dkl, dku, dab, dpiv, dinfo;
-    CK(dm.ensure(ns * sizeof(int))); CK(dkl.ensure(ns * sizeof(int))); CK(dku.ensure(ns * sizeof(int)));
-    CK(dab.ensure(ns * sizeof(double *))); CK(dpiv.ensure(ns * sizeof(int *))); CK(dinfo.ensure(ns * sizeof(int)));
-    CK(cudaMemcpyAsync(dm.p, m.data(), ns * sizeof(int), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(dkl.p, kl.data(), ns * sizeof(int), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(dku.p, ku.data(), ns * sizeof(int), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(dab.p, abp.data(), ns * sizeof(double *), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(dpiv.p, pivp.data(), ns * sizeof(int *), cudaMemcpyHostToDevice, s));
-    launch_band_lu(ns, dm.as<int>(), dkl.as<int>(), dku.as<int>(), dab.as<double *>(), dpiv.as<int *>(),
-                   dinfo.as<int>(), s);
+    DevMem AB, LP, ints, dlu, dinfo, derr;              // ints: pivots, L and U extents of every row
+    CK(AB.ensure((size_t)nab * sizeof(double)));
+    CK(ints.ensure(3 * (size_t)std::max(totP, 1LL) * sizeof(int)));
+    CK(dlu.ensure(ns * sizeof(LuShape)));
+    CK(dinfo.ensure(ns * sizeof(int)));
+    int *piv = ints.as<int>(), *lext = piv + totP, *uext = lext + totP;
+    CK(cudaMemsetAsync(AB.p, 0, (size_t)nab * sizeof(double), s));
+    CK(cudaMemcpyAsync(dlu.p, lu.data(), ns * sizeof(LuShape), cudaMemcpyHostToDevice, s));
+    launch_assemble(ctx->st, dlu.as<LuShape>(), ns, max_nodes, coarse ? 1 : 0, re2 ? 1 : 0, AB.as<double>(), s);
     CKL();
+    CK(launch_band_lu(dlu.as<LuShape>(), ns, max_kl, max_ku, AB.as<double>(), piv, dinfo.as<int>(), s));
     std::vector<int> info(ns);
     CK(cudaMemcpyAsync(info.data(), dinfo.p, ns * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -692,27 +686,15 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     // permuted L, extents, permutation; then the panel widths (index bookkeeping on the host)
     F.h.resize(ns);
     F.fma_col.assign(ns, 0.0);
-    long long totP = 0;
-    std::vector<DevMem> Lp(ns), lext(ns), uext(ns);
-    std::vector<int> KLW(ns);
-    DevMem perm_all, derr;
-    for (int q = 0; q < ns; q++) totP += m[q];
     CK(F.P.ensure((size_t)std::max(totP, 1LL) * sizeof(int)));
+    CK(LP.ensure((size_t)nlp * sizeof(double)));
     CK(derr.ensure(sizeof(int)));
     CK(cudaMemsetAsync(derr.p, 0, sizeof(int), s));
-    long long po = 0;
-    for (int q = 0; q < ns; q++) {
-        KLW[q] = 3 * kl[q];
-        CK(Lp[q].ensure((size_t)m[q] * KLW[q] * sizeof(double)));
-        CK(lext[q].ensure(m[q] * sizeof(int)));
-        CK(uext[q].ensure(m[q] * sizeof(int)));
-        launch_factor_prepare(m[q], kl[q], ku[q], abp[q], pivp[q], KLW[q], Lp[q].as<double>(),
-                              lext[q].as<int>(), uext[q].as<int>(), F.P.as<int>() + po, derr.as<int>(), s);
-        CKL();
-        F.h[q].m = m[q];
-        F.h[q].perm_off = po;
-        po += m[q];
-    }
+    CK(launch_factor_prepare(dlu.as<LuShape>(), ns, max_m, AB.as<double>(), piv, LP.as<double>(), lext, uext,
+                             F.P.as<int>(), derr.as<int>(), s));
+    for (int q = 0; q < ns; q++) { F.h[q].m = m[q]; F.h[q].perm_off = lu[q].row; }
+    std::vector<int> ext(2 * (size_t)totP);
+    CK(cudaMemcpyAsync(ext.data(), lext, ext.size() * sizeof(int), cudaMemcpyDeviceToHost, s));
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, derr.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -720,9 +702,7 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     long long mo = 0;
     std::vector<int4> meta;
     for (int q = 0; q < ns; q++) {
-        std::vector<int> le(m[q]), ue(m[q]);
-        CK(cudaMemcpy(le.data(), lext[q].p, m[q] * sizeof(int), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(ue.data(), uext[q].p, m[q] * sizeof(int), cudaMemcpyDeviceToHost));
+        const int *le = ext.data() + lu[q].row, *ue = le + totP, KLW = 3 * kl[q];
         const int nbk = (m[q] + BNB - 1) / BNB;
         BlockFactor &b = F.h[q];
         b.nblk = nbk; b.wl = 0; b.wu = 0;
@@ -732,7 +712,7 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
         for (int J = 0; J < nbk; J++) {
             const int r0 = J * BNB, r1 = std::min(m[q], r0 + BNB) - 1;
             int wl = 0, wu = 0;
-            for (int c = std::max(0, r0 - KLW[q]); c < r0; c++)             // left panel
+            for (int c = std::max(0, r0 - KLW); c < r0; c++)             // left panel
                 if (c + le[c] >= r0) { wl = r0 - c; break; }
             for (int c = std::min(m[q] - 1, r1 + kl[q] + ku[q]); c > r1; c--)  // right panel
                 if (c - ue[c] <= r1) { wu = c - r1; break; }
@@ -755,11 +735,11 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     CK(F.M.ensure((size_t)std::max(mo, 1LL) * sizeof(double)));
     CK(F.Meta.ensure(meta.size() * sizeof(int4)));
     CK(cudaMemcpy(F.Meta.p, meta.data(), meta.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    for (int q = 0; q < ns; q++) {
-        launch_block_operators(m[q], kl[q], ku[q], abp[q], KLW[q], Lp[q].as<double>(),
-                               F.Meta.as<int4>() + F.h[q].meta_off, F.M.as<double>(), s);
-        CKL();
-    }
+    for (int q = 0; q < ns; q++) lu[q].meta = F.h[q].meta_off;
+    CK(cudaMemcpyAsync(dlu.p, lu.data(), ns * sizeof(LuShape), cudaMemcpyHostToDevice, s));
+    launch_block_operators(dlu.as<LuShape>(), ns, max_m, AB.as<double>(), LP.as<double>(), F.Meta.as<int4>(),
+                           F.M.as<double>(), s);
+    CKL();
     CK(F.Mdf.ensure((size_t)std::max(mo, 1LL) * sizeof(float2)));
     launch_ops_to_df(mo, F.M.as<double>(), F.Mdf.as<float2>(), s);
     CKL();

@@ -278,21 +278,24 @@ void launch_cast(long long n, const void *in, int in_double, void *out, int out_
 constexpr int LOCAL_LDP = MAX_RESTART + 2;   // partial-sum slots per fine tile
 
 // coarse / banded FP64
-void launch_assemble_E(const Stencil &st, int nx, int ny, int kl, int ku, double *ab, cudaStream_t s);
-void launch_assemble_Aloc(const Stencil &st, int nx, int ny, int kl, int ku, double *ab, cudaStream_t s);
-// complex E (resp. A_j) of a box with origin (gx0, gy0) under the impedance condition, written as
-// its real equivalent: unknowns (Re x_0, Im x_0, Re x_1, ...), i.e. the complex vector read as
-// doubles; order 2m, half-bandwidths kl2 = ku2 = 2·kl + 1 of the complex band kl
-void launch_assemble_E_re2(const Stencil &st, int nx, int ny, int gx0, int gy0, int kl2, int ku2, double *ab,
+// One matrix (E_j or A_j of a box shape) at set-up; all shapes go through a stage in one launch.
+struct LuShape {
+    int nx, ny, gx0, gy0;      // box and origin (impedance: which of its sides lie on the square's)
+    int m, kl, ku;             // order and half-bandwidths (of the real equivalent under bc = 1)
+    long long ab, lp;          // offsets (doubles) of its band storage and of its permuted L, 3·kl per column
+    long long row, meta;       // offsets of its rows' arrays (pivots, extents, permutation) and of its block table
+};
+// E (coarse) or A_j of every shape into zeroed band storage.  re2: the complex matrix of the
+// impedance condition as its real equivalent: unknowns (Re x_0, Im x_0, Re x_1, ...), i.e. the
+// complex vector read as doubles; order 2m, half-bandwidths kl = ku = 2·kl_c + 1 of the complex kl_c
+void launch_assemble(const Stencil &st, const LuShape *sh, int ns, int max_nodes, int coarse, int re2, double *AB,
+                     cudaStream_t s);
+cudaError_t launch_band_lu(const LuShape *sh, int ns, int max_kl, int max_ku, double *AB, int *PIV, int *info,
                            cudaStream_t s);
-void launch_assemble_Aloc_re2(const Stencil &st, int nx, int ny, int gx0, int gy0, int kl2, int ku2, double *ab,
-                              cudaStream_t s);
-void launch_band_lu(int nmat, const int *m, const int *kl, const int *ku, double *const *ab,
-                    int *const *piv, int *info, cudaStream_t s);
-void launch_factor_prepare(int m, int kl, int ku, const double *ab, const int *piv, int KLW,
-                           double *Lp, int *lext, int *uext, int *perm, int *err, cudaStream_t s);
-void launch_block_operators(int m, int kl, int ku, const double *ab, int KLW, const double *Lp,
-                            const int4 *meta, double *Mall, cudaStream_t s);
+cudaError_t launch_factor_prepare(const LuShape *sh, int ns, int max_m, const double *AB, const int *PIV, double *LP,
+                                  int *LEXT, int *UEXT, int *PERM, int *err, cudaStream_t s);
+void launch_block_operators(const LuShape *sh, int ns, int max_m, const double *AB, const double *LP, const int4 *Meta,
+                            double *Mall, cudaStream_t s);
 struct BlockSolveCfg {       // shared-memory plan of the blocked solve over a set of factors
     int maxK = 0;          // widest operator row stride: op_stride(panel width)
     int cwy = 0, cwx = 0;  // circular y / x windows, powers of two >= BNB + widest left / right panel
