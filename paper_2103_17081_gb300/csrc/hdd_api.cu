@@ -2014,7 +2014,7 @@ hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_sol
     float2 *V32L = df ? O.V32L.as<float2>() : nullptr;
     // delayed CGS2 (two passes over the basis per step) with the double-FP32 dots and update
     const bool dc = df && ctx->outer_udf && ctx->outer_dcgs;
-    const int Gc = oupdate_dcgs_grid(n);        // partials of its update
+    const int Gc = std::max(oupdate_dcgs_grid(n, 0), oupdate_dcgs_grid_max(n));   // most partials of its update
     if (dc) {
         CK(O.part2.ensure((size_t)nr * G * ldp * sizeof(double2)));
         CK(O.invs.ensure(nr * sizeof(double)));
@@ -2124,9 +2124,8 @@ hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_sol
                     KL(F_ODF, fa * (nv * 16 + 32) * n, fa * (ctx->outer_bias ? 72 : 96) * nv * n,
                        CK(launch_odots2_df(B, V32, V32L, j + 1, V32 + (long long)j * B.ld32,
                                            V32L + (long long)j * B.ld32, w, O.part.as<double2>(),
-                                           O.part2.as<double2>(), O.vmax.as<unsigned>(), ctx->outer_bias, s)));
-                    KL(F_OMISC, 0, 0, launch_oreduce(B, O.part.as<double2>(), j + 1, P1, s));
-                    KL(F_OMISC, 0, 0, launch_oreduce(B, O.part2.as<double2>(), j + 1, P2, s));
+                                           O.part2.as<double2>(), O.vmax.as<unsigned>(), ctx->outer_bias, P1, P2, s)));
+                    ctx->prof.launches++;
                 }
                 KL(F_OMISC, 0, 0,
                    launch_dcgs_col(B, O.H.as<double2>(), O.cs.as<double>(), O.sn.as<double2>(), O.g.as<double2>(),
@@ -2142,7 +2141,7 @@ hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_sol
                                        O.npart1.as<double>(), O.vmax.as<unsigned>(), s));
                 KL(F_OMISC, 0, 0,
                    launch_dcgs_tent(B, O.H.as<double2>(), O.g.as<double2>(), O.Wq.as<double2>(), j,
-                                    O.npart1.as<double>(), Gc, O.fnorm.as<double>(), prm->outer_tol,
+                                    O.npart1.as<double>(), oupdate_dcgs_grid(n, j), O.fnorm.as<double>(), prm->outer_tol,
                                     O.hn.as<double>(), O.flag.as<int>(), O.hist.as<double>(), hstride, total, s));
                 KL(F_OMISC, 2.0 * fa * n * 16 + fa * n * 16.0, 0,
                    launch_oscale(B, V + (long long)(j + 1) * B.ld, V32 + (long long)(j + 1) * B.ld32,

@@ -449,10 +449,11 @@ void launch_oupdate2(const OuterBatch &B, const double2 *V, const float2 *V32, i
 // first CGS pass update in double-FP32 from the hi/lo FP32 basis; norm partials on its own grid
 int oupdate_df_grid(long long n);
 // delayed CGS2: fused dots of the pending vector and w, per-RHS coefficient kernels, fused update
-int oupdate_dcgs_grid(long long n);
+int oupdate_dcgs_grid(long long n, int j);
+int oupdate_dcgs_grid_max(long long n);
 cudaError_t launch_odots2_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int nv, const float2 *x1h,
                              const float2 *x1l, const double2 *w, double2 *part1, double2 *part2,
-                             const unsigned *vmax, int bias, cudaStream_t s);
+                             const unsigned *vmax, int bias, double2 *out1, double2 *out2, cudaStream_t s);
 void launch_dcgs_col(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                      const double2 *P1, double2 *P2, const double *hn, double *invs, const double *fnorm,
                      double *hist, int hstride, int it, int *err, unsigned *vmax, cudaStream_t s);

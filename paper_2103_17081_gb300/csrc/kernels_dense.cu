@@ -631,38 +631,51 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
                const int *__restrict__ rexp, const int *__restrict__ cexp, double2 *__restrict__ out,
                unsigned long long *__restrict__ ws, const int2 *__restrict__ part) {
     const int tid = threadIdx.x, row = tid & 127;
-    int4 it = blockIdx.x < nitem ? items[blockIdx.x] : make_int4(0, 0, 0, 0);    // shape, tile (rt·nct + ct), first pair
-    DenseShape S = sh[it.x];
-    int4 n = sunits[it.x];
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    const long long G = part[ns + 1].x, Wt = part[ns].y;
+    bool waited = false;
     for (int b = blockIdx.x; b < nitem; b += gridDim.x) {
-        if (b != (int)blockIdx.x) { it = items[b]; S = sh[it.x]; n = sunits[it.x]; }
-        const int2 p0 = part[it.x];
-        if (part[it.x + 1].x == p0.x) continue;                                  // no task of this shape
-        const long long w0 = p0.y + (long long)it.y * (n.y + DENSE_TILEW) * n.z + DENSE_TILEW * n.z,
-                        w1 = w0 + (long long)(n.y - 1) * n.z;
-        if (((w0 + 1) * G - 1) / Wt == ((w1 + 1) * G - 1) / Wt) continue;        // one CTA had it all
+        // everything but the sums and exponents is there before the products are done
+        const int4 it = items[b];                                                // shape, tile (rt·nct + ct), first pair
+        const DenseShape S = sh[it.x];
+        const int4 n = sunits[it.x];
         const int rt = it.y / S.nct, ct = it.y - rt * S.nct, i = rt * 128 + row;
-        unsigned long long *acc = ws + S.acc0 + (size_t)it.y * 128 * S.nt + row;
         const int re = i < S.m ? rexp[S.soff + i] : 0;
-        unsigned long long x[8];
         int t[4];
+        long long o[4];
 #pragma unroll
         for (int e = 0; e < 4; e++) {
-            const int pr = it.z + (tid >> 7) + 2 * e, task = ct * (S.nt / 2) + pr;
-            t[e] = task < S.ntask ? tlist[S.t0 + task] : -1;
+            const int task = ct * (S.nt / 2) + it.z + (tid >> 7) + 2 * e;
+            t[e] = task < S.ntask && i < S.m ? tlist[S.t0 + task] : -1;
+            if (t[e] >= 0 && flag && !flag[t[e]]) t[e] = -1;
+            o[e] = t[e] >= 0 ? tcoff[t[e]] + i : 0;
+        }
+        if (!waited) {
+            asm volatile("griddepcontrol.wait;\n" ::: "memory");
+            waited = true;
+        }
+        unsigned long long *acc = ws + S.acc0 + (size_t)it.y * 128 * S.nt + row;
+        unsigned long long x[8];
+        int2 ce[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int pr = it.z + (tid >> 7) + 2 * e;
             x[2 * e] = __ldcg(acc + (size_t)(2 * pr) * 128);
             x[2 * e + 1] = __ldcg(acc + (size_t)(2 * pr + 1) * 128);
+            ce[e] = t[e] >= 0 ? make_int2(cexp[2 * t[e]], cexp[2 * t[e] + 1]) : make_int2(0, 0);
         }
+        const int2 p0 = part[it.x], p1 = part[it.x + 1];
+        const unsigned G = (unsigned)part[ns + 1].x, Wt = (unsigned)part[ns].y;
+        if (p1.x == p0.x) continue;                                              // no task of this shape
+        // the CTAs that hold the tile's first and last unit: one and the same wrote it out itself
+        const unsigned long long w0 = (unsigned)(p0.y + it.y * (n.y + DENSE_TILEW) * n.z + DENSE_TILEW * n.z),
+                                 w1 = w0 + (unsigned)((n.y - 1) * n.z);
+        if (((w0 + 1) * G - 1) / Wt == ((w1 + 1) * G - 1) / Wt) continue;
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const int pr = it.z + (tid >> 7) + 2 * e;
             __stcg(acc + (size_t)(2 * pr) * 128, 0ull);
             __stcg(acc + (size_t)(2 * pr + 1) * 128, 0ull);
-            if (t[e] < 0 || i >= S.m || (flag && !flag[t[e]])) continue;
-            out[tcoff[t[e]] + i] = make_double2(from_fixed((long long)x[2 * e], re + cexp[2 * t[e]]),
-                                                from_fixed((long long)x[2 * e + 1], re + cexp[2 * t[e] + 1]));
+            if (t[e] < 0) continue;
+            out[o[e]] = make_double2(from_fixed((long long)x[2 * e], re + ce[e].x), from_fixed((long long)x[2 * e + 1], re + ce[e].y));
         }
     }
 }

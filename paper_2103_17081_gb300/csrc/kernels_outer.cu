@@ -4,6 +4,8 @@
 //
 // Reductions are two-stage and deterministic: OUTER_CTAS CTAs each own a fixed contiguous chunk
 // and write one partial per basis vector; a second kernel adds the partials in CTA order.
+#include <algorithm>
+
 #include "hdd_common.cuh"
 
 namespace hdd {
@@ -587,13 +589,16 @@ __global__ void __launch_bounds__(OT) k_onorm(OuterBatch B, const double2 *__res
 
 // out[r][l] = Σ_q part[r][q][l]: one warp per l, lane i adds q = i, i+32, ... in order, then a
 // fixed shuffle tree (deterministic).
-__global__ void k_oreduce(OuterBatch B, const double2 *__restrict__ part, int nv, double2 *__restrict__ out) {
+__global__ void k_oreduce(OuterBatch B, const double2 *__restrict__ part, int nv, double2 *__restrict__ out,
+                          const double2 *__restrict__ part_b, double2 *__restrict__ out_b) {
     const int r = blockIdx.y;
     if (B.active && !B.active[r]) return;
+    if (blockIdx.z) { part = part_b; out = out_b; }       // two sets of partials in one launch
     const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (l >= nv) return;
     part += (long long)r * B.G * B.ldp;
     double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
     for (int q = lane; q < B.G; q += 32) { double2 v = part[(long long)q * B.ldp + l]; s.x += v.x; s.y += v.y; }
     for (int o = 16; o > 0; o >>= 1) { s.x += shfl_xor(s.x, o); s.y += shfl_xor(s.y, o); }
     if (lane == 0) out[(long long)r * B.ldp + l] = s;
@@ -694,8 +699,9 @@ k_ogivens(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double
 // or at once when the cycle ends, the column then keeping its first-pass coefficients).
 // ------------------------------------------------------------------------------------------
 
-// Warp q forms the partial dots of vectors l = q, q + 8, ... with the two staged vectors s1, s2
-// (double-FP32, as warp_dots_df; four element groups per pass, the next group's basis loads
+// Warp q of nw forms the partial dots of the vector pairs q, q + nw, ... (l = 2q, 2q + 1, ...) with
+// the two staged vectors s1, s2 (double-FP32, as warp_dots_df; two vectors and two element groups
+// of 32 at a time, so a staged element is read once for two vectors, the next group's basis loads
 // issued before the current group's arithmetic).  BIAS: the dots with w (s2, the first pass of
 // the new vector) take the biased sums of df_acc_biased (6 FP32 instructions per product instead
 // of 12).  Their error (a few 1e-12 of Σ|v w| instead of about 1e-15) needs no care: the first
@@ -703,115 +709,153 @@ k_ogivens(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double
 // left, V^H ṽ, exactly and adds it to the column (the Arnoldi relation w = V h + ν σ v holds
 // whatever the first-pass coefficients were).  The dots with s1 (that second pass, which sets
 // the orthogonality of the basis) keep the two-sum.  The bias of vector l is the power of two
-// M >= 4·T·vm_l·xm, T = 2·(len/128 + 4) the products one accumulator takes (len/128 whole
-// groups plus at most four tail elements, two products each per component), vm_l >= |hi part|
+// M >= 4·T·vm_l·xm, T = 2·(D2_FLUSH + 2) the products one accumulator takes before its sum moves
+// to an unbiased pair (two per element and component), vm_l >= |hi part|
 // of every entry of V_l (vms[l] for the final slots, recorded by the update that wrote them; the
 // chunk maximum of s1 for the last slot, which is s1) and xm the chunk maximum of w's hi parts.
+// The 8 sums of a pair are spread over the lanes while they are reduced (18 shuffles and 9
+// additions instead of 80 and 40).
+constexpr int D2_FLUSH = 10;             // groups of 64 elements a biased sum takes
 template <bool BIAS>
 __device__ __forceinline__ void warp_dots2_df(const float2 *__restrict__ Vh, const float2 *__restrict__ Vl,
                                               long long ld32, int nv, const float4 *__restrict__ s1,
                                               const float4 *__restrict__ s2, long long b, int len,
-                                              double2 *__restrict__ part1, double2 *__restrict__ part2, int ldp,
-                                              const float *__restrict__ vms, float xm1, float xm2) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float Tb = 4.001f * (float)(2 * ((len >> 7) + 4));
-    for (int l = warp; l < nv; l += OT / 32) {
-        const float2 *hp = Vh + (long long)l * ld32 + b, *lp = Vl + (long long)l * ld32 + b;
-        const float M2 = BIAS ? pow2_ceil(Tb * (l < nv - 1 ? vms[l] : xm1) * xm2) : 0.f;
-        float ah[4][2], al[4][2], bh[4][2], bl[4][2];
+                                              double2 *__restrict__ part1, double2 *__restrict__ part2,
+                                              const float *__restrict__ vms, float xm1, float xm2, int q0, int nw) {
+    const int lane = threadIdx.x & 31;
+    const float Tb = 4.001f * (float)(2 * (min(D2_FLUSH, len >> 6) + 2));
+    const int full = len & ~63;
+    for (int l = 2 * q0; l < nv; l += 2 * nw) {
+        const int l2 = min(l + 1, nv - 1);                // an odd last vector is its own partner
+        const float2 *hp[2] = {Vh + (long long)l * ld32 + b, Vh + (long long)l2 * ld32 + b};
+        const float2 *lp[2] = {Vl + (long long)l * ld32 + b, Vl + (long long)l2 * ld32 + b};
+        float M[2] = {0.f, 0.f};
+        if (BIAS) {
+            M[0] = pow2_ceil(Tb * (l < nv - 1 ? vms[l] : xm1) * xm2);
+            M[1] = pow2_ceil(Tb * (l2 < nv - 1 ? vms[l2] : xm1) * xm2);
+        }
+        float ah[2][2][2], al[2][2][2], bh[2][2][2], bl[2][2][2];     // [vector][group][component]
+        float th[2][2], tl[2][2];                                      // sums moved out of the biased pairs
 #pragma unroll
-        for (int u = 0; u < 4; u++)
+        for (int v = 0; v < 2; v++)
 #pragma unroll
-            for (int c = 0; c < 2; c++) { ah[u][c] = al[u][c] = bl[u][c] = 0.f; bh[u][c] = M2; }
-        auto acc1 = [](float &sh, float &sl, float xh, float xl, float yh, float yl) {
-            df_acc(sh, sl, xh, xl, yh, yl);
-        };
+            for (int c = 0; c < 2; c++) {
+                th[v][c] = tl[v][c] = 0.f;
+#pragma unroll
+                for (int u = 0; u < 2; u++) { ah[v][u][c] = al[v][u][c] = bl[v][u][c] = 0.f; bh[v][u][c] = M[v]; }
+            }
         auto acc2 = [](float &sh, float &sl, float xh, float xl, float yh, float yl) {
             if (BIAS) df_acc_biased(sh, sl, xh, xl, yh, yl);
             else df_acc(sh, sl, xh, xl, yh, yl);
         };
-        auto step = [&](int u, float2 h, float2 q, float4 x, float4 y) {
+        auto step = [&](int v, int u, float2 h, float2 q, float4 x, float4 y) {
             // conj(v)·x = (vr xr + vi xi) + i (vr xi - vi xr), the same for y
-            acc1(ah[u][0], al[u][0], h.x, q.x, x.x, x.y);
-            acc1(ah[u][1], al[u][1], h.x, q.x, x.z, x.w);
-            acc1(ah[u][0], al[u][0], h.y, q.y, x.z, x.w);
-            acc1(ah[u][1], al[u][1], -h.y, -q.y, x.x, x.y);
-            acc2(bh[u][0], bl[u][0], h.x, q.x, y.x, y.y);
-            acc2(bh[u][1], bl[u][1], h.x, q.x, y.z, y.w);
-            acc2(bh[u][0], bl[u][0], h.y, q.y, y.z, y.w);
-            acc2(bh[u][1], bl[u][1], -h.y, -q.y, y.x, y.y);
+            df_acc(ah[v][u][0], al[v][u][0], h.x, q.x, x.x, x.y);
+            df_acc(ah[v][u][1], al[v][u][1], h.x, q.x, x.z, x.w);
+            df_acc(ah[v][u][0], al[v][u][0], h.y, q.y, x.z, x.w);
+            df_acc(ah[v][u][1], al[v][u][1], -h.y, -q.y, x.x, x.y);
+            acc2(bh[v][u][0], bl[v][u][0], h.x, q.x, y.x, y.y);
+            acc2(bh[v][u][1], bl[v][u][1], h.x, q.x, y.z, y.w);
+            acc2(bh[v][u][0], bl[v][u][0], h.y, q.y, y.z, y.w);
+            acc2(bh[v][u][1], bl[v][u][1], -h.y, -q.y, y.x, y.y);
         };
-        const int full = len & ~127;
-        float2 vh[4], vl[4];
-        int i = lane;
+        auto flush = [&]() {   // sh in [3M/4, 5M/4], so sh - M is exact
+#pragma unroll
+            for (int v = 0; v < 2; v++)
+#pragma unroll
+                for (int u = 0; u < 2; u++)
+#pragma unroll
+                    for (int c = 0; c < 2; c++) {
+                        df_add(th[v][c], tl[v][c], __fsub_rn(bh[v][u][c], M[v]), bl[v][u][c]);
+                        bh[v][u][c] = M[v];
+                        bl[v][u][c] = 0.f;
+                    }
+        };
+        float2 vh[2][2], vl[2][2];
+        int i = lane, room = D2_FLUSH;
         if (i < full) {
 #pragma unroll
-            for (int u = 0; u < 4; u++) { vh[u] = hp[i + 32 * u]; vl[u] = lp[i + 32 * u]; }
-        }
-        for (; i < full; i += 128) {
-            float2 nh[4], nl[4];
-            const bool more = i + 128 < full;
+            for (int v = 0; v < 2; v++)
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                nh[u] = more ? hp[i + 128 + 32 * u] : make_float2(0.f, 0.f);
-                nl[u] = more ? lp[i + 128 + 32 * u] : make_float2(0.f, 0.f);
+                for (int u = 0; u < 2; u++) { vh[v][u] = hp[v][i + 32 * u]; vl[v][u] = lp[v][i + 32 * u]; }
+        }
+        for (; i < full; i += 64) {
+            float2 nh[2][2], nl[2][2];
+            const bool more = i + 64 < full;
+#pragma unroll
+            for (int v = 0; v < 2; v++)
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    nh[v][u] = more ? hp[v][i + 64 + 32 * u] : make_float2(0.f, 0.f);
+                    nl[v][u] = more ? lp[v][i + 64 + 32 * u] : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const float4 x = s1[i + 32 * u], y = s2[i + 32 * u];
+#pragma unroll
+                for (int v = 0; v < 2; v++) step(v, u, vh[v][u], vl[v][u], x, y);
             }
 #pragma unroll
-            for (int u = 0; u < 4; u++) step(u, vh[u], vl[u], s1[i + 32 * u], s2[i + 32 * u]);
+            for (int v = 0; v < 2; v++)
 #pragma unroll
-            for (int u = 0; u < 4; u++) { vh[u] = nh[u]; vl[u] = nl[u]; }
+                for (int u = 0; u < 2; u++) { vh[v][u] = nh[v][u]; vl[v][u] = nl[v][u]; }
+            if (BIAS && --room == 0) { flush(); room = D2_FLUSH; }
         }
-        for (i = full + lane; i < len; i += 32) step(0, hp[i], lp[i], s1[i], s2[i]);
-        if (BIAS) {            // remove the bias: sh in [3M/4, 5M/4], so sh - M is exact
+        for (i = full + lane; i < len; i += 32) {         // at most two elements per lane
+            const float4 x = s1[i], y = s2[i];
 #pragma unroll
-            for (int u = 0; u < 4; u++)
-#pragma unroll
-                for (int c = 0; c < 2; c++) bh[u][c] = __fsub_rn(bh[u][c], M2);
+            for (int v = 0; v < 2; v++) step(v, 0, hp[v][i], lp[v][i], x, y);
         }
+        flush();                                          // (without BIAS: M = 0, the groups' sums together)
+        float h[8], q[8];                                 // [vector][with s1, with s2][component]
 #pragma unroll
-        for (int u = 1; u < 4; u++)
+        for (int v = 0; v < 2; v++)
 #pragma unroll
             for (int c = 0; c < 2; c++) {
-                df_add(ah[0][c], al[0][c], ah[u][c], al[u][c]);
-                df_add(bh[0][c], bl[0][c], bh[u][c], bl[u][c]);
+                df_add(ah[v][0][c], al[v][0][c], ah[v][1][c], al[v][1][c]);
+                h[4 * v + c] = ah[v][0][c]; q[4 * v + c] = al[v][0][c];
+                h[4 * v + 2 + c] = th[v][c]; q[4 * v + 2 + c] = tl[v][c];
             }
-        for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-            for (int c = 0; c < 2; c++) {
-                const float x1 = __shfl_xor_sync(0xffffffffu, ah[0][c], o), x2 = __shfl_xor_sync(0xffffffffu, al[0][c], o);
-                const float y1 = __shfl_xor_sync(0xffffffffu, bh[0][c], o), y2 = __shfl_xor_sync(0xffffffffu, bl[0][c], o);
-                df_add(ah[0][c], al[0][c], x1, x2);
-                df_add(bh[0][c], bl[0][c], y1, y2);
+        for (int half = 4; half > 0; half >>= 1) {        // lanes 16, 8, 4 apart: each keeps one half of the sums
+            const int o = 4 * half;
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int k = 0; k < half; k++) {
+                const float x = __shfl_xor_sync(0xffffffffu, up ? h[k] : h[k + half], o);
+                const float y = __shfl_xor_sync(0xffffffffu, up ? q[k] : q[k + half], o);
+                if (up) { h[k] = h[k + half]; q[k] = q[k + half]; }
+                df_add(h[k], q[k], x, y);
             }
         }
-        if (lane == 0) {
-            part1[(long long)blockIdx.x * ldp + l] = make_double2((double)ah[0][0] + (double)al[0][0],
-                                                                  (double)ah[0][1] + (double)al[0][1]);
-            part2[(long long)blockIdx.x * ldp + l] = make_double2((double)bh[0][0] + (double)bl[0][0],
-                                                                  (double)bh[0][1] + (double)bl[0][1]);
+#pragma unroll
+        for (int o = 2; o > 0; o >>= 1) {
+            const float x = __shfl_xor_sync(0xffffffffu, h[0], o), y = __shfl_xor_sync(0xffffffffu, q[0], o);
+            df_add(h[0], q[0], x, y);
         }
+        const int v = lane >> 4;
+        if ((lane & 3) == 0 && l + v < nv)
+            reinterpret_cast<double *>((lane & 8 ? part2 : part1) + l + v)[(lane >> 2) & 1] = (double)h[0] + (double)q[0];
     }
 }
 
-// Partials part1[r][cta][l] = Σ conj(V_l) x1 and part2[r][cta][l] = Σ conj(V_l) w for l < nv
+// Partials part1[r][chunk][l] = Σ conj(V_l) x1 and part2[r][chunk][l] = Σ conj(V_l) w for l < nv
 // (x1: hi/lo copies of basis slot nv-1; w: FP64).  vmax[r·ldp + l], l < nv-1: max |hi part| of
-// slot l as float bits (BIAS only).  Dynamic shared memory: 2 · chunk float4, then nv - 1 floats
-// (BIAS).
+// slot l as float bits (BIAS only).  CTA: one of B.G chunks of the vectors, one of ng shares of the
+// basis (odots2_plan).  Dynamic shared memory: 2 · chunk float4, then nv - 1 floats (BIAS).
 template <bool BIAS>
 __global__ void __launch_bounds__(OT, 2)
-k_odots2_df(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__restrict__ Vl, int nv,
+k_odots2_df(OuterBatch B, int ng, const float2 *__restrict__ Vh, const float2 *__restrict__ Vl, int nv,
             const float2 *__restrict__ x1h, const float2 *__restrict__ x1l, const double2 *__restrict__ w,
             double2 *__restrict__ part1, double2 *__restrict__ part2, const unsigned *__restrict__ vmax) {
     extern __shared__ float4 st2[];
     __shared__ float mx[2][OT / 32];
-    const int r = blockIdx.y;
+    const int r = blockIdx.y, ch = blockIdx.x / ng, sh = blockIdx.x - ch * ng;
     if (B.active && !B.active[r]) return;
     Vh += r * B.n32; Vl += r * B.n32; x1h += r * B.n32; x1l += r * B.n32; w += r * B.n;
-    part1 += (long long)r * B.G * B.ldp; part2 += (long long)r * B.G * B.ldp;
-    long long b, e;
-    chunk_of(B.n, b, e);
-    const int len = (int)(e > b ? e - b : 0);
-    const long long chunk = (B.n + gridDim.x - 1) / gridDim.x;
+    part1 += ((long long)r * B.G + ch) * B.ldp; part2 += ((long long)r * B.G + ch) * B.ldp;
+    const long long chunk = (B.n + B.G - 1) / B.G, b = min((long long)ch * chunk, B.n);
+    const int len = (int)(min(b + chunk, B.n) - b);
     float4 *s1 = st2, *s2 = st2 + len;
     float *vms = reinterpret_cast<float *>(st2 + 2 * chunk);
     float m1 = 0.f, m2 = 0.f;
@@ -839,7 +883,8 @@ k_odots2_df(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__restric
 #pragma unroll
         for (int q = 0; q < OT / 32; q++) { xm1 = fmaxf(xm1, mx[0][q]); xm2 = fmaxf(xm2, mx[1][q]); }
     }
-    warp_dots2_df<BIAS>(Vh, Vl, B.ld32, nv, s1, s2, b, len, part1, part2, B.ldp, vms, xm1, xm2);
+    warp_dots2_df<BIAS>(Vh, Vl, B.ld32, nv, s1, s2, b, len, part1, part2, vms, xm1, xm2,
+                        sh * (OT / 32) + (int)(threadIdx.x >> 5), ng * (OT / 32));
 }
 
 // Block reductions of the small per-RHS kernels (OG threads)
@@ -1007,12 +1052,16 @@ k_dcgs_close(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, dou
 // largest |hi part| of the final v_j (an atomic maximum on float bits into vmax[r·ldp + j],
 // which k_dcgs_col cleared) for the biased dot products of the later steps.
 // Dynamic shared memory: j · (float4 + float2).
+// KS > 1: the CTA's threads are KS groups that share the vectors (blocks of 32 in turn) for
+// OTU / KS element pairs, for vectors too short to fill the SMs with a pair per thread.
+template <int KS>
 __global__ void __launch_bounds__(OTU, 3)
 k_oupdate_dcgs(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__restrict__ Vl, int j, int corr,
                double2 *__restrict__ Vj, double *__restrict__ Dj, float2 *__restrict__ Vjh, float2 *__restrict__ Vjl,
                const double2 *__restrict__ acoef, const double2 *__restrict__ bcoef, const double *__restrict__ invs,
                double2 *__restrict__ w, double *__restrict__ part_norm, unsigned *__restrict__ vmax) {
     extern __shared__ float4 dq[];
+    __shared__ double part[KS > 1 ? KS - 1 : 1][8][KS > 1 ? OTU / KS : 1];
     float4 *bq = dq;                                      // (Re hi, Re lo, Im hi, Im lo) of b_l
     float2 *aq = reinterpret_cast<float2 *>(dq + j);      // a_l in FP32
     __shared__ double red[OTU / 32];
@@ -1031,16 +1080,18 @@ k_oupdate_dcgs(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__rest
     __syncthreads();
     const double2 hj = bcoef[j];
     const double is = corr ? invs[r] : 1.0;
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x, i = 2 * p;
+    const int tp = KS > 1 ? OTU / KS : (int)blockDim.x, tx = KS > 1 ? (int)threadIdx.x % tp : (int)threadIdx.x,
+              grp = KS > 1 ? (int)threadIdx.x / tp : 0;
+    const long long p = (long long)blockIdx.x * tp + tx, i = 2 * p;
     double nrm = 0.0;
     float vm = 0.f;
+    double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;            // Σ V b (elements a, b of the pair)
+    double cx = 0.0, cy = 0.0, ex = 0.0, ey = 0.0;            // Σ V a
+    const bool two = i + 1 < B.n;
     if (i < B.n) {
-        const bool two = i + 1 < B.n;
         const float4 *hp = reinterpret_cast<const float4 *>(Vh) + p;
         const float4 *lp = reinterpret_cast<const float4 *>(Vl) + p;
         const long long ld4 = B.ld32 / 2;
-        double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;        // Σ V b (elements a, b of the pair)
-        double cx = 0.0, cy = 0.0, ex = 0.0, ey = 0.0;        // Σ V a
         float axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f, bxh = 0.f, bxl = 0.f, byh = 0.f, byl = 0.f;
         float cxf = 0.f, cyf = 0.f, exf = 0.f, eyf = 0.f;
         auto acc = [&](const float4 vh, const float4 vl, const float4 c, const float2 a) {
@@ -1057,7 +1108,9 @@ k_oupdate_dcgs(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__rest
             exf = fmaf(vh.z, a.x, fmaf(-vh.w, a.y, exf));
             eyf = fmaf(vh.z, a.y, fmaf(vh.w, a.x, eyf));
         };
-        for (int l0 = 0; l0 < j; l0 += 32) {
+        // last vectors first: the dots pass just before this one ended with them, and what is left of
+        // it in L2 (some 100 MB of the basis) is read from there
+        for (int l0 = ((j - 1) / 32 - grp) * 32; l0 >= 0; l0 -= 32 * KS) {
             const int l1 = l0 + 32 < j ? l0 + 32 : j;
             int l = l0;
             for (; l + 4 <= l1; l += 4) {
@@ -1077,6 +1130,22 @@ k_oupdate_dcgs(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__rest
             axh = axl = ayh = ayl = bxh = bxl = byh = byl = 0.f;
             cxf = cyf = exf = eyf = 0.f;
         }
+    }
+    if (KS > 1) {                                             // the groups' sums to group 0, in their order
+        if (grp > 0) {
+            double (*d)[KS > 1 ? OTU / KS : 1] = part[grp - 1];
+            d[0][tx] = ax; d[1][tx] = ay; d[2][tx] = bx; d[3][tx] = by;
+            d[4][tx] = cx; d[5][tx] = cy; d[6][tx] = ex; d[7][tx] = ey;
+        }
+        __syncthreads();
+        if (grp == 0)
+#pragma unroll
+            for (int g = 0; g < KS - 1; g++) {
+                ax += part[g][0][tx]; ay += part[g][1][tx]; bx += part[g][2][tx]; by += part[g][3][tx];
+                cx += part[g][4][tx]; cy += part[g][5][tx]; ex += part[g][6][tx]; ey += part[g][7][tx];
+            }
+    }
+    if (i < B.n && grp == 0) {
         auto finish = [&](long long k, double sbx, double sby, double sax, double say) {
             double2 v = Vj[k];
             float2 hi;
@@ -1310,20 +1379,56 @@ int oupdate_df_grid(long long n) {
     pair_plan(k_oupdate_df, plan_udf, n, t, g);
     return g;
 }
-int oupdate_dcgs_grid(long long n) {
+// Groups of threads per element pair: one from 64 k pairs on (two thirds of what the SMs hold at
+// three CTAs each), two, or four below 32 k; one while there is nothing to share.  By the vectors'
+// length and not the batch, as the groups set the order of the sums.  n = 101 k at 161 vectors on
+// average: 79 us with two against 87 (63 with the vectors taken from the last).
+static int dcgs_groups(long long n, int j) {
+    const long long P = (n + 1) / 2;
+    const int k = P >= 64 * 1024 ? 1 : P >= 32 * 1024 ? 2 : 4;
+    return j >= 32 * k ? k : j >= 64 ? 2 : 1;
+}
+int oupdate_dcgs_grid(long long n, int j) {
+    const int k = dcgs_groups(n, j);
+    if (k > 1) return (int)(((n + 1) / 2 + OTU / k - 1) / (OTU / k));
     int t = 0, g = 0;
-    pair_plan(k_oupdate_dcgs, plan_dcgs, n, t, g);
+    pair_plan(k_oupdate_dcgs<1>, plan_dcgs, n, t, g);
     return g;
 }
+int oupdate_dcgs_grid_max(long long n) { return (int)(((n + 1) / 2 + OTU / 4 - 1) / (OTU / 4)); }
 void launch_oupdate_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int nv, const double2 *h,
                        double2 *w, double *part_norm, cudaStream_t s) {
     int t = 0, g = 0;
     pair_plan(k_oupdate_df, plan_udf, B.n, t, g);
     k_oupdate_df<<<dim3(g, B.nrhs), t, (size_t)nv * sizeof(float4), s>>>(B, Vh, Vl, nv, h, w, part_norm);
 }
-cudaError_t launch_odots2_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int nv, const float2 *x1h,
+// Chunks of the vectors and shares of the basis of the fused dots.  The chunks set the order of the
+// sums, so they depend on the vectors' length alone (the same bits of the dots in any batch): the
+// fewest of 304, 152, 76 or 38 (two per SM and halves of that) that fit shared memory, as a pair's
+// reduction costs as much as 50 elements.  The shares then fill two CTAs per SM: waves of CTAs
+// times a CTA's warp instructions, per round of its warps' vector pairs 4.5 an element and about
+// 250, and some 2 an element for the staging.  With both reductions: n = 101 k, 161 vectors on
+// average, 87 us against 106 + 11 for 304 chunks of 335 elements; n = 37 k with four right-hand
+// sides 49 against 97; n = 229 k, 368 vectors, 324 against 376 + 12.
+static void odots2_plan(const OuterBatch &B, int nv, int &nchunk, int &ng) {
+    const int pairs = (nv + 1) / 2, per = OT / 32;
+    nchunk = B.G;
+    while (nchunk % 2 == 0 && nchunk > OUTER_CTAS / 8 && B.n <= (long long)OCH * (nchunk / 2)) nchunk /= 2;
+    const double len = (double)((B.n + nchunk - 1) / nchunk);
+    double best = 1e300;
+    ng = 1;
+    for (int g = 1; g <= 16; g *= 2) {
+        const double waves = (double)(((long long)nchunk * g * B.nrhs + OUTER_CTAS - 1) / OUTER_CTAS);
+        const double cost = waves * (((pairs + per * g - 1) / (per * g)) * (len * 4.5 + 250.0) + len * 2.0 + 600.0);
+        if (cost < best * 0.999) { best = cost; ng = g; }
+    }
+}
+cudaError_t launch_odots2_df(const OuterBatch &B0, const float2 *Vh, const float2 *Vl, int nv, const float2 *x1h,
                              const float2 *x1l, const double2 *w, double2 *part1, double2 *part2,
-                             const unsigned *vmax, int bias, cudaStream_t s) {
+                             const unsigned *vmax, int bias, double2 *out1, double2 *out2, cudaStream_t s) {
+    OuterBatch B = B0;
+    int ng = 1;
+    odots2_plan(B0, nv, B.G, ng);
     const long long chunk = (B.n + B.G - 1) / B.G;
     const size_t smem = (size_t)(2 * chunk) * sizeof(float4) + (bias ? (size_t)nv * sizeof(float) : 0);
     // the largest dynamic shared memory requested so far, per device and variant (the attribute
@@ -1335,16 +1440,17 @@ cudaError_t launch_odots2_df(const OuterBatch &B, const float2 *Vh, const float2
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= MAXDEV) return cudaErrorInvalidDevice;
     bias = bias ? 1 : 0;
-    void (*const kern[2])(OuterBatch, const float2 *, const float2 *, int, const float2 *, const float2 *,
+    void (*const kern[2])(OuterBatch, int, const float2 *, const float2 *, int, const float2 *, const float2 *,
                           const double2 *, double2 *, double2 *, const unsigned *) = {k_odots2_df<false>,
                                                                                       k_odots2_df<true>};
-    if (smem > 48 * 1024 && smem > set[dev][bias]) {
+    if (smem > 47 * 1024 && smem > set[dev][bias]) {         // (48 KB with the kernel's static part)
         e = cudaFuncSetAttribute(kern[bias], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         set[dev][bias] = smem;
     }
-    kern[bias]<<<dim3(B.G, B.nrhs), OT, smem, s>>>(B, Vh, Vl, nv, x1h, x1l, w, part1, part2, vmax);
-    return cudaSuccess;
+    kern[bias]<<<dim3(B.G * ng, B.nrhs), OT, smem, s>>>(B, ng, Vh, Vl, nv, x1h, x1l, w, part1, part2, vmax);
+    k_oreduce<<<dim3((nv + 7) / 8, B.nrhs, 2), 256, 0, s>>>(B, part1, nv, out1, part2, out2);
+    return cudaGetLastError();
 }
 void launch_dcgs_col(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                      const double2 *P1, double2 *P2, const double *hn, double *invs, const double *fnorm,
@@ -1363,10 +1469,20 @@ void launch_dcgs_close(const OuterBatch &B, double2 *H, double *cs, double2 *sn,
 void launch_oupdate_dcgs(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int j, int corr, double2 *Vj,
                          double *Dj, float2 *Vjh, float2 *Vjl, const double2 *acoef, const double2 *bcoef,
                          const double *invs, double2 *w, double *part_norm, unsigned *vmax, cudaStream_t s) {
-    int t = 0, g = 0;
-    pair_plan(k_oupdate_dcgs, plan_dcgs, B.n, t, g);
-    k_oupdate_dcgs<<<dim3(g, B.nrhs), t, (size_t)j * (sizeof(float4) + sizeof(float2)), s>>>(
-        B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w, part_norm, vmax);
+    const size_t sm = (size_t)j * (sizeof(float4) + sizeof(float2));
+    const int k = dcgs_groups(B.n, j), grid = oupdate_dcgs_grid(B.n, j);
+    if (k == 4)
+        k_oupdate_dcgs<4><<<dim3(grid, B.nrhs), OTU, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+                                                              part_norm, vmax);
+    else if (k == 2)
+        k_oupdate_dcgs<2><<<dim3(grid, B.nrhs), OTU, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+                                                              part_norm, vmax);
+    else {
+        int t = 0, g = 0;
+        pair_plan(k_oupdate_dcgs<1>, plan_dcgs, B.n, t, g);
+        k_oupdate_dcgs<1><<<dim3(g, B.nrhs), t, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+                                                         part_norm, vmax);
+    }
 }
 void launch_oupdate2(const OuterBatch &B, const double2 *V, const float2 *V32, int nv, const double2 *h,
                      double2 *w, const double *npart1, int g1, double *part_norm, int allow32, int *fallbacks,
@@ -1378,7 +1494,7 @@ void launch_onorm(const OuterBatch &B, const double2 *x, double *part, cudaStrea
     k_onorm<<<dim3(B.G, B.nrhs), OT, 0, s>>>(B, x, part);
 }
 void launch_oreduce(const OuterBatch &B, const double2 *part, int nv, double2 *out, cudaStream_t s) {
-    k_oreduce<<<dim3((nv + 7) / 8, B.nrhs), 256, 0, s>>>(B, part, nv, out);
+    k_oreduce<<<dim3((nv + 7) / 8, B.nrhs), 256, 0, s>>>(B, part, nv, out, nullptr, nullptr);
 }
 void launch_ogivens(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                     const double2 *h1, const double2 *h2, const double *npart, const double *fnorm,
@@ -1412,7 +1528,9 @@ cudaError_t set_outer_smem_limits(size_t bytes) {
     if ((e = cudaFuncSetAttribute(k_oupdate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_oupdate2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_oupdate_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_otrisolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_oaxpy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     return cudaSuccess;
