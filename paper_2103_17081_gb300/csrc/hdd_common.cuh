@@ -105,6 +105,7 @@ template <typename R> __device__ __forceinline__ void caxpy(c2<R> &acc, c2<R> h,
 }
 
 template <typename R> __device__ __forceinline__ R shfl_xor(R v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+template <typename R> __device__ __forceinline__ R shfl(R v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
 
 // Division by a box dimension d (1 <= d <= 256) of an index 0 <= e < 2^24, as the high word of
 // e·M with M = ceil(2^32/d): with M·d = 2^32 + r (0 <= r < d) the excess over e/d is
@@ -113,7 +114,7 @@ template <typename R> __device__ __forceinline__ R shfl_xor(R v, int m) { return
 struct BoxDiv {
     unsigned m;
     __device__ __forceinline__ explicit BoxDiv(int d)
-        : m(d > 1 ? (unsigned)((0x100000000ull + (unsigned)d - 1) / (unsigned)d) : 0u) {}
+        : m(d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u) {}        // ceil(2^32 / d) by a 32-bit division
     __device__ __forceinline__ int q(int e) const { return m ? (int)__umulhi((unsigned)e, m) : e; }
 };
 

@@ -6,6 +6,8 @@
 // tile table; the host sizes shared memory for the largest heights.
 // Reductions are two-stage and deterministic: each tile writes its partial sums to a slot of
 // its own, and every consumer adds the partials of a task in tile order.
+#include <type_traits>
+
 #include "hdd_common.cuh"
 
 namespace hdd {
@@ -20,6 +22,31 @@ __device__ __forceinline__ float zw_f(int t) {
     return t == 0 || t == 4 ? 0.125f : (t == 2 ? 0.75f : 0.5f);
 }
 template <typename R> __device__ __forceinline__ R zw(int t) { return (R)zw_f(t); }
+
+// double -> R and R -> double.  A float conversion runs on the FP64 pipe, which holds a scheduler for
+// 64 clocks a warp whatever the operands; with FP32 vectors it is done on the bits instead (round to
+// nearest even; values that are no normal floats take the conversion).
+__device__ __forceinline__ float narrow_f(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 254u) {                                // a normal float, up to rounding to infinity
+        const unsigned b = (hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+        return __uint_as_float(b + (((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    return (float)x;
+}
+__device__ __forceinline__ double widen_f(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    return (double)x;
+}
+template <typename R> __device__ __forceinline__ c2<R> narrow_c(double2 v);
+template <> __device__ __forceinline__ c2<float> narrow_c<float>(double2 v) { return mk<float>(narrow_f(v.x), narrow_f(v.y)); }
+template <> __device__ __forceinline__ c2<double> narrow_c<double>(double2 v) { return v; }
+__device__ __forceinline__ double2 widen_c(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
+__device__ __forceinline__ double2 widen_c(double2 v) { return v; }
 
 template <typename R> __device__ __forceinline__ c2<R> load_c(const c2<R> *p) { return *p; }
 
@@ -62,6 +89,23 @@ __device__ __forceinline__ c2<R> stencil_smem(const Stencil &st, const c2<R> *u,
         const int cls = node_class(st.N, gx0 + x, gy0 + y);
         if (cls != 4) return boundary_row<R>(st.bcoef + cls * 7, cc, e, wv, n, s, d1, d2);
     }
+    r.x = c0 * cc.x + c1 * (((e.x + wv.x) + n.x) + s.x) + c2v * (d1.x + d2.x);
+    r.y = c0 * cc.y + c1 * (((e.y + wv.y) + n.y) + s.y) + c2v * (d1.y + d2.y);
+    return r;
+}
+
+// The same on a tile whose rows carry zeros beside and around the box (pitch elements a row): p is
+// the centre node, no bounds to check.
+template <typename R, bool IMP>
+__device__ __forceinline__ c2<R> stencil_padded(const Stencil &st, R c0, R c1, R c2v, const c2<R> *p, int pitch,
+                                                int gx, int gy) {
+    const int dd = st.diag == 0 ? pitch + 1 : 1 - pitch;
+    const c2<R> cc = p[0], e = p[1], wv = p[-1], n = p[pitch], s = p[-pitch], d1 = p[dd], d2 = p[-dd];
+    if (IMP) {
+        const int cls = node_class(st.N, gx, gy);
+        if (cls != 4) return boundary_row<R>(st.bcoef + cls * 7, cc, e, wv, n, s, d1, d2);
+    }
+    c2<R> r;
     r.x = c0 * cc.x + c1 * (((e.x + wv.x) + n.x) + s.x) + c2v * (d1.x + d2.x);
     r.y = c0 * cc.y + c1 * (((e.y + wv.y) + n.y) + s.y) + c2v * (d1.y + d2.y);
     return r;
@@ -229,61 +273,69 @@ k_zt(LocalArgs<R> a, const c2<R> *__restrict__ in, double2 *__restrict__ yout, i
     }
 }
 
-// Z s for box rows [F0, F0+nF): s (FP64 coarse) → px (x-interpolated coarse rows) → zs.
-// Shared buffers: sc[ncy*mx], px[ncy*nx].  Returns via zs[nF*nx].
-template <typename R>
-__device__ void prolong_rows(const Task &T, const double2 *__restrict__ s, int F0, int nF,
-                             c2<R> *sc, c2<R> *px, c2<R> *zs) {
-    const int nx = T.nx, ny = T.ny, mx = T.mx, my = T.my;
-    // coarse rows cy with 2cy-1 <= f <= 2cy+3 for some f in [F0, F0+nF)
-    int C0 = (F0 - 3) >= 0 ? (F0 - 3 + 1) / 2 : -((3 - F0) / 2);
-    int C1 = (F0 + nF - 1 + 1) / 2;
-    if (C0 < 0) C0 = 0;
-    if (C1 > my - 1) C1 = my - 1;
-    const int ncy = C1 - C0 + 1;
-    const BoxDiv dmx(mx), dnx(nx);
-    for (int e = threadIdx.x; e < ncy * mx; e += blockDim.x) {
-        const int rr = dmx.q(e);
-        double2 v = s[T.coff + (long long)(C0 + rr) * mx + (e - rr * mx)];
-        sc[e] = mk<R>((R)v.x, (R)v.y);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < ncy * nx; e += blockDim.x) {
-        const int r = dnx.q(e), fx = e - r * nx;
-        c2<R> acc = mk<R>(0, 0);
-        int cx0 = (fx - 3) >= 0 ? (fx - 3 + 1) / 2 : 0;
-        int cx1 = (fx + 1) / 2;
-        if (cx1 > mx - 1) cx1 = mx - 1;
-        for (int cx = cx0; cx <= cx1; cx++) {
-            R wgt = zw<R>(fx - 2 * cx + 1);
-            c2<R> v = sc[r * mx + cx];
-            acc.x = fma(wgt, v.x, acc.x);
-            acc.y = fma(wgt, v.y, acc.y);
-        }
-        px[e] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nF * nx; e += blockDim.x) {
-        const int qy = dnx.q(e);
-        int fy = F0 + qy, fx = e - qy * nx;
-        c2<R> acc = mk<R>(0, 0);
-        if (fy >= 0 && fy < ny) {
-            int cy0 = (fy - 3) >= 0 ? (fy - 3 + 1) / 2 : 0;
-            int cy1 = (fy + 1) / 2;
-            if (cy1 > my - 1) cy1 = my - 1;
-            for (int cy = cy0; cy <= cy1; cy++) {
-                R wgt = zw<R>(fy - 2 * cy + 1);
-                c2<R> v = px[(cy - C0) * nx + fx];
-                acc.x = fma(wgt, v.x, acc.x);
-                acc.y = fma(wgt, v.y, acc.y);
-            }
-        }
-        zs[e] = acc;
-    }
-    __syncthreads();
-}
+// Z s for box rows [F0, F0+nF): s (FP64 coarse) → px (x-interpolated coarse rows) → out(row - F0,
+// column, value) for the rows inside the box.  Fine indices go in pairs (2m, 2m + 1), which take the
+// coarse entries m-1, m, m+1 with the weights (1/2, 1/2, 0) and (1/8, 3/4, 1/8): a thread makes both
+// from three loads, and entries outside the coarse box are staged as zeros, so nothing is selected
+// or checked per tap (the sums in the order of the taps).  Shared buffers: sc[rows·((nx+1)/2 + 2)],
+// px[rows·nx], rows = prolong_max_cy(nF).  Waits for the thread's asynchronous copies before the
+// last barrier; ends without one.
+__host__ __device__ inline int prolong_max_cy(int nrows_fine) { return nrows_fine / 2 + 3; }
+__host__ __device__ inline int prolong_pitch(int nx) { return (nx + 1) / 2 + 2; }
 
-__host__ __device__ inline int prolong_max_cy(int nrows_fine) { return nrows_fine / 2 + 4; }
+__device__ __forceinline__ void async_copy(float2 *dst, const float2 *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_copy(double2 *dst, const double2 *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+template <typename R, typename Out>
+__device__ __forceinline__ void prolong_rows(const Task &T, const double2 *__restrict__ s, int F0, int nF,
+                                             c2<R> *sc, c2<R> *px, Out out) {
+    const int nx = T.nx, ny = T.ny, mx = T.mx, my = T.my;
+    const int hx = (nx + 1) / 2, P = prolong_pitch(nx);
+    const int M0 = max(F0, 0) >> 1, M1 = (min(F0 + nF, ny) - 1) >> 1, nm = M1 - M0 + 1;
+    const BoxDiv dP(P), dhx(hx), dnx(nx);
+    auto mix2 = [](c2<R> p, c2<R> q) {
+        return mk<R>(fma((R)0.5, q.x, (R)0.5 * p.x), fma((R)0.5, q.y, (R)0.5 * p.y));
+    };
+    auto mix3 = [](c2<R> p, c2<R> q, c2<R> r) {
+        return mk<R>(fma((R)0.125, r.x, fma((R)0.75, q.x, (R)0.125 * p.x)),
+                     fma((R)0.125, r.y, fma((R)0.75, q.y, (R)0.125 * p.y)));
+    };
+#pragma unroll 2
+    for (int e = threadIdx.x; e < (nm + 2) * P; e += blockDim.x) {
+        const int rr = dP.q(e), cx = e - rr * P - 1, cy = M0 - 1 + rr;
+        c2<R> v = mk<R>(0, 0);
+        if ((unsigned)cx < (unsigned)mx && (unsigned)cy < (unsigned)my)
+            v = narrow_c<R>(s[T.coff + (long long)cy * mx + cx]);
+        sc[e] = v;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int e = threadIdx.x; e < (nm + 2) * hx; e += blockDim.x) {
+        const int r = dhx.q(e), q = e - r * hx;
+        const c2<R> *p = sc + r * P + q;
+        const c2<R> va = p[0], vb = p[1], vc = p[2];
+        c2<R> *o = px + r * nx + 2 * q;
+        o[0] = mix2(va, vb);
+        if (2 * q + 1 < nx) o[1] = mix3(va, vb, vc);
+    }
+    async_wait();
+    __syncthreads();
+#pragma unroll 1
+    for (int e = threadIdx.x; e < nm * nx; e += blockDim.x) {
+        const int m = dnx.q(e), fx = e - m * nx, f = 2 * (M0 + m) - F0;
+        const c2<R> *p = px + m * nx + fx;
+        const c2<R> va = p[0], vb = p[nx], vc = p[2 * nx];
+        if (f >= 0) out(f, fx, mix2(va, vb));
+        if (f + 1 < nF && f + 1 + F0 < ny) out(f + 1, fx, mix3(va, vb, vc));
+    }
+}
 
 // out = add + Z s on fine tiles (add may be null)
 template <typename R>
@@ -296,9 +348,10 @@ k_z(LocalArgs<R> a, const double2 *__restrict__ s, const c2<R> *__restrict__ add
     const Task T = a.tasks[tl.task];
     const int maxc = prolong_max_cy(tl.nr);
     c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
-    c2<R> *px = sc + maxc * T.mx;
+    c2<R> *px = sc + maxc * prolong_pitch(T.nx);
     c2<R> *zs = px + maxc * T.nx;
-    prolong_rows<R>(T, s, tl.r0, tl.nr, sc, px, zs);
+    prolong_rows<R>(T, s, tl.r0, tl.nr, sc, px, [&](int r, int fx, c2<R> v) { zs[r * T.nx + fx] = v; });
+    __syncthreads();
     for (int e = threadIdx.x; e < tl.nr * T.nx; e += blockDim.x) {
         long long gi = T.foff + (long long)tl.r0 * T.nx + e;
         c2<R> v = cscale<R>(sign, zs[e]);
@@ -323,10 +376,12 @@ k_prolong_stencil(LocalArgs<R> a, int mode, const c2<R> *__restrict__ in,
     const int F0 = tl.r0 - 1, nF = tl.nr + 2;
     const int maxc = prolong_max_cy(nF);
     c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
-    c2<R> *px = sc + maxc * T.mx;
+    c2<R> *px = sc + maxc * prolong_pitch(nx);
     c2<R> *u = px + maxc * nx;                     // nF*nx
     c2<R> *red = u + nF * nx;                      // NWARP*LDP
-    prolong_rows<R>(T, s, F0, nF, sc, px, u);      // u = Z s on rows F0..F0+nF-1
+    prolong_rows<R>(T, s, F0, nF, sc, px,          // u = Z s on the box's rows of F0..F0+nF-1
+                    [&](int r, int fx, c2<R> v) { u[r * nx + fx] = v; });
+    __syncthreads();
     if (mode == 0) {
         for (int e = threadIdx.x; e < nF * nx; e += blockDim.x) {
             int yy = F0 + e / nx;
@@ -637,10 +692,10 @@ k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restr
     }
     const int maxc = prolong_max_cy(tl.nr);
     c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
-    c2<R> *px = sc + maxc * T.mx;
+    c2<R> *px = sc + maxc * prolong_pitch(T.nx);
     c2<R> *zs = px + maxc * T.nx;
-    if (!again) prolong_rows<R>(T, s, tl.r0, tl.nr, sc, px, zs);       // ends with a barrier
-    else __syncthreads();
+    if (!again) prolong_rows<R>(T, s, tl.r0, tl.nr, sc, px, [&](int r, int fx, c2<R> v) { zs[r * T.nx + fx] = v; });
+    __syncthreads();
     const BoxDiv dnx(T.nx);
     const long long base = T.foff + (long long)tl.r0 * T.nx;
     for (int e = threadIdx.x; e < tl.nr * T.nx; e += blockDim.x) {
@@ -654,7 +709,7 @@ k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restr
         } else {
             x = cadd<R>(x, zs[e]);
             glob[(long long)(gx - a.glo) + (long long)(gy - a.glo) * a.gw + (long long)T.rhs * nglob] =
-                make_double2((double)x.x, (double)x.y);
+                widen_c(x);
         }
     }
 }
@@ -682,8 +737,8 @@ __global__ void k_cast(long long n, const c2<RI> *__restrict__ in, c2<RO> *__res
 // ------------------------------------------------------------------------------------------
 // One inner Arnoldi step in one launch (every phase between two coarse solves), one cluster of
 // C CTAs per task: CTA `rank` holds box rows [rank·ny/C, (rank+1)·ny/C) and coarse rows
-// [rank·my/C, (rank+1)·my/C).  The new vector w stays in registers from the stencil to the
-// normalisation; the three task-wide sums (first CGS dots, second CGS dots, ||w||²) are
+// [rank·my/C, (rank+1)·my/C).  The new vector w stays in shared memory from the stencil to
+// the normalisation; the two sets of task-wide sums (first CGS dots; second CGS dots and ||w||²) are
 // all-gathered through distributed shared memory, one cluster barrier each, and every CTA adds
 // the C partials in rank order (deterministic, bitwise the same in every CTA).  Steps:
 //   A  w = A_j(v_i - Z_j s_{i+1}) (s_{i+1} = E_j⁻¹ Z_jᵀ A_j v_i from the coarse solve), h1 = V^H w
@@ -712,6 +767,7 @@ template <typename R> struct StepArgs {
     int *counter;
     R tol;
     int maxit;
+    R c0, c1, c2v;          // the interior stencil in the inner precision
 };
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -730,186 +786,312 @@ template <typename T> __device__ __forceinline__ T *cluster_map(T *p, unsigned r
 }
 
 size_t step_smem_bytes(int max_nx, int max_ny, int C, int bytes_per_c) {
-    const int nr = (max_ny + C - 1) / C, nF = nr + 2, maxc = nF / 2 + 4;
-    const int mx = max_nx / 2 + 1, my = max_ny / 2;
-    const int ncy = (my + C - 1) / C, nFz = 2 * ncy + 3, nVz = nFz + 2;
-    const size_t a = (size_t)maxc * mx + (size_t)maxc * max_nx + (size_t)nF * max_nx;
-    const size_t e = (size_t)nVz * max_nx + (size_t)nFz * max_nx + (size_t)nFz * mx;
+    const int nr = (max_ny + C - 1) / C, nF = nr + 2, maxc = prolong_max_cy(nF);
+    const int my = max_ny / 2, ncy = (my + C - 1) / C, nFz = 2 * ncy + 3, nVz = nFz + 2;
+    const size_t px = (size_t)maxc * prolong_pitch(max_nx) + (size_t)maxc * max_nx, w = (size_t)nr * max_nx;
+    const size_t a = (px > w ? px : w) + (size_t)nF * (max_nx + 3);
+    const size_t e = (size_t)(nVz + nFz) * (max_nx + 3);
     return (a > e ? a : e) * bytes_per_c;
 }
 
+// sqrt(x² + y²) without overflow or underflow: for doubles scaled by a power of two (some 15 FP64
+// instructions, at 64 clocks each, where hypot takes several times that), hypot's own rounding kept
+// for what the scale does not reach
+__device__ __forceinline__ float hyp(float x, float y) { return hypotf(x, y); }
+__device__ __forceinline__ double hyp(double x, double y) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu, ey = ((unsigned)__double2hiint(y) >> 20) & 0x7ffu;
+    const unsigned e = ex > ey ? ex : ey;
+    if (e - 64u > 1900u) return hypot(x, y);
+    const double sc = __hiloint2double((int)((2046u - e) << 20), 0);
+    const double xs = x * sc, ys = y * sc;
+    return sqrt(fma(xs, xs, ys * ys)) * __hiloint2double((int)(e << 20), 0);
+}
+
+// Bound: with FP64 vectors by the FP64 pipe (64 clocks a warp instruction, whatever its lanes do),
+// with FP32 by the chain of phases and by fetching instructions that run once or twice each.  So w is
+// kept in shared memory, where loops over a thread's elements need no unrolling and end with the box
+// (70 KB of code; with w in registers and every loop unrolled 126 KB and 23 us for 17 at k=100); up
+// to four basis vectors go through a pass together (w read and written once, the second dots in the
+// pass of the first update); the eight sums of four vectors are reduced by halves across the lanes
+// (9 additions for 40); ||w||² after the second pass is ||w'||² - ||h2||², both known from the second
+// all-gather (V is orthonormal; where h2 is not small against w' and the difference could cancel, it
+// is summed directly); tiles in shared memory carry a frame of zeros instead of bounds checks; the
+// column's rotations run in one warp, real components, divisions and products spread over its lanes,
+// beside the other warps' scaling of v.  Per step: k=100 FP32 21.2 -> 17.0 us, k=200 25 -> 19.8,
+// 8192 boxes of 84 x 84 2392 -> 1329; FP64 k=20 49 -> 19.3, k=100 82 -> 60.
 template <typename R, bool IMP>
-__global__ void __launch_bounds__(LOCAL_THREADS)
+__global__ void __launch_bounds__(LOCAL_THREADS, sizeof(R) == 4 ? 4 : 2)
 k_arnoldi_step(StepArgs<R> a) {
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ c2<R> red[NWARP * LDP];            // per-warp partials
-    __shared__ c2<R> gat[2][STEP_CMAX][LDP];      // cluster all-gather slots (written remotely)
-    __shared__ c2<R> h1s[LDP], h2s[LDP], nrm_s[1];   // task sums: the two CGS passes, ||w||²
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ R red[NWARP][2 * LDP];                // per-warp partials (real components)
+    __shared__ R gat[2][STEP_CMAX][2 * LDP];         // cluster all-gather slots (written remotely)
+    __shared__ c2<R> h1s[LDP], h2s[LDP], hcs[LDP];   // task sums of the two CGS passes, the column
     __shared__ R cs_s[MAX_RESTART];
     __shared__ c2<R> sn_s[MAX_RESTART];
     __shared__ c2<R> g_s;
-    __shared__ R ref_s, hn_s;
-    __shared__ int its_s, stop_s;
+    __shared__ R ref_s, hn_s, inv_s;
+    __shared__ int its_s, stop_s, direct_s;
     const int C = a.C;
     const int t = (int)blockIdx.x / C;
     const unsigned rank = cluster_rank();
-    if (!a.act_in[t]) {                           // the same flag for every CTA of the cluster
+    const int act = a.act_in[t];                     // the same flag for every CTA of the cluster
+    const Task T = a.tasks[t];
+    if (!act) {
         if (rank == 0 && threadIdx.x == 0) a.act_out[t] = 0;
         return;
     }
-    const Task T = a.tasks[t];
     const int nx = T.nx, ny = T.ny, mx = T.mx, my = T.my;
-    const BoxDiv dnx(nx), dmx(mx);
+    const BoxDiv dnx(nx);
     const int i = a.i, nv = i + 1;
     const int r0 = (int)(rank * ny) / C, r1 = (int)((rank + 1) * ny) / C, nr = r1 - r0;
     const int cnt = nr * nx;
     const long long base = T.foff + (long long)r0 * nx;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // ---- A: u = v_i - Z s on rows [r0-1, r1], w = A u on own rows ----
+    c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
+    const int F0 = r0 - 1, nF = nr + 2, maxc = prolong_max_cy(nF), PU = nx + 2;
+    c2<R> *px = sc + maxc * prolong_pitch(nx);
+    c2<R> *u = sc + max(maxc * (prolong_pitch(nx) + nx), cnt);   // nF rows of nx + 2, a zero on each side
+    c2<R> *const ws = sc;                            // w on own rows, once sc and px are used up
+    // rows [y0, y0 + n) of vector v into a framed tile (asynchronously)
+    auto stage = [&](const c2<R> *v, c2<R> *tile, int y0, int n, int pitch) {
+        const BoxDiv dp(pitch);
+#pragma unroll 2
+        for (int e = tid; e < n * pitch; e += LOCAL_THREADS) {
+            const int q = dp.q(e), x = e - q * pitch - 1, yy = y0 + q;
+            if ((unsigned)x < (unsigned)nx && (unsigned)yy < (unsigned)ny) async_copy(tile + e, v + (long long)yy * nx + x);
+            else tile[e] = mk<R>(0, 0);
+        }
+    };
+    const c2<R> *const Vt = a.V + T.foff;
+    if (nr > 0) stage(Vt + (long long)i * a.ld, u, F0, nF, PU);
     // Givens state of earlier steps (written by earlier launches; rank 0 rewrites it below, after
     // every CTA has passed the first cluster barrier)
     if (tid < i) {
         cs_s[tid] = a.S.cs[(long long)t * a.restart + tid];
         sn_s[tid] = a.S.sn[(long long)t * a.restart + tid];
     }
-    if (tid == 0) {
+    if (tid == LOCAL_THREADS - 1) {
         g_s = a.S.g[(long long)t * (a.restart + 1) + i];
         ref_s = a.S.ref[t];
         its_s = a.S.its[t];
     }
-    // ---- A: u = v_i - Z s on rows [r0-1, r1], w = A u on own rows, partial h1 ----
-    c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
-    const int F0 = r0 - 1, nF = nr + 2, maxc = prolong_max_cy(nF);
-    c2<R> *px = sc + maxc * mx;
-    c2<R> *u = px + maxc * nx;
-    const c2<R> *vi = a.V + (long long)i * a.ld;
-    c2<R> wv[EPT];
-#pragma unroll
-    for (int k = 0; k < EPT; k++) wv[k] = mk<R>(0, 0);
+    const int nw = min(NWARP, (cnt + 31) / 32);      // warps that hold any of the elements tid + 256 k
     if (nr > 0) {
-        prolong_rows<R>(T, a.s, F0, nF, sc, px, u);
-        for (int e = tid; e < nF * nx; e += blockDim.x) {
-            const int qy = dnx.q(e), yy = F0 + qy;
-            if (yy >= 0 && yy < ny) u[e] = csub<R>(vi[T.foff + (long long)yy * nx + (e - qy * nx)], u[e]);
-        }
+        prolong_rows<R>(T, a.s, F0, nF, sc, px, [&](int r, int fx, c2<R> z) {
+            c2<R> *p = u + r * PU + 1 + fx;
+            *p = csub<R>(*p, z);
+        });
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < EPT; k++) {
-            const int e = tid + k * LOCAL_THREADS;
-            if (e < cnt) {
-                const int qy = dnx.q(e), yy = r0 + qy, xx = e - qy * nx;
-                wv[k] = stencil_smem<R, IMP>(a.st, u, F0, nF, nx, ny, xx, yy, T.ix0, T.iy0);
-            }
+#pragma unroll 1
+        for (int e = tid; e < cnt; e += LOCAL_THREADS) {
+            const int qy = dnx.q(e), xx = e - qy * nx;
+            ws[e] = stencil_padded<R, IMP>(a.st, a.c0, a.c1, a.c2v, u + (qy + 1) * PU + 1 + xx, PU, T.ix0 + xx,
+                                           T.iy0 + r0 + qy);
         }
     }
-    // task-wide sums of n values: the per-warp partials in red[warp][l] are added per CTA and
-    // sent to slot gat[b][rank][l] of every CTA, then one cluster barrier, then each CTA adds
-    // the C slots in rank order into out[l]
-    const int lane = tid & 31, warp = tid >> 5;
-    auto gather = [&](int b, int n, c2<R> *out) {
+    // task-wide sums of n real values: the warps' partials red[warp][j] are added per CTA and sent to
+    // slot gat[b][rank][j] of every CTA, then one cluster barrier, then each CTA adds the C slots in
+    // rank order: get(j, sum)
+    auto gather = [&](int b, int n, auto get) {
         __syncthreads();
-        for (int idx = tid; idx < n * C; idx += blockDim.x) {
-            const int l = idx % n, dst = idx / n;
-            c2<R> sum = mk<R>(0, 0);
-            for (int q = 0; q < NWARP; q++) sum = cadd<R>(sum, red[q * LDP + l]);
-            *cluster_map(&gat[b][rank][l], (unsigned)dst) = sum;
-        }
+        for (int j = lane; j < n; j += 32)
+            for (int dst = warp; dst < C; dst += NWARP) {
+                R sum = 0;
+#pragma unroll 1
+                for (int q = 0; q < nw; q++) sum += red[q][j];
+                *cluster_map(&gat[b][rank][j], (unsigned)dst) = sum;
+            }
         cluster_barrier();
-        for (int l = tid; l < n; l += blockDim.x) {
-            c2<R> sum = mk<R>(0, 0);
-            for (int q = 0; q < C; q++) sum = cadd<R>(sum, gat[b][q][l]);
-            out[l] = sum;
+        for (int j = tid; j < n; j += LOCAL_THREADS) {
+            R sum = gat[b][0][j];
+#pragma unroll 1
+            for (int q = 1; q < C; q++) sum += gat[b][q][j];
+            get(j, sum);
         }
         __syncthreads();
     };
-    auto warp_store = [&](int l, c2<R> v) {
+    // one pass of basis vectors l0 .. l0 + 3 over the thread's elements: UPD subtracts h_l v_l from w,
+    // DOT adds conj(v_l)·w to acc[l]; both: also |w|² to nrm
+    const c2<R> *const Vb = a.V + base;
+    R nrm = 0;
+    c2<R> acc[4];
+    auto pass = [&](auto upd, auto dot, int l0, const c2<R> *h) {
+        constexpr bool UPD = decltype(upd)::value, DOT = decltype(dot)::value;
+        const int nl = min(4, nv - l0);
+        const c2<R> *const vp = Vb + (long long)l0 * a.ld;
+        c2<R> hl[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) { v.x += shfl_xor(v.x, o); v.y += shfl_xor(v.y, o); }
-        if (lane == 0) red[warp * LDP + l] = v;
-    };
-    // h = V^H w over the task (per-warp partials, then the cluster gather)
-    auto reduce_dots = [&](int b, c2<R> *out) {
-        for (int l = 0; l < nv; l++) {
-            c2<R> acc = mk<R>(0, 0);
-            const c2<R> *vl = a.V + (long long)l * a.ld + base;
-#pragma unroll
-            for (int k = 0; k < EPT; k++) {
-                const int e = tid + k * LOCAL_THREADS;
-                if (e < cnt) cdotc_acc<R>(acc, vl[e], wv[k]);
-            }
-            warp_store(l, acc);
+        for (int q = 0; q < 4; q++) {
+            if (UPD) hl[q] = h[l0 + min(q, nl - 1)];
+            if (DOT) acc[q] = mk<R>(0, 0);
         }
-        gather(b, nv, out);
-    };
-    // w -= V h
-    auto update = [&](const c2<R> *h) {
-        for (int l = 0; l < nv; l++) {
-            const c2<R> hl = h[l];
-            const c2<R> *vl = a.V + (long long)l * a.ld + base;
+#pragma unroll 2
+        for (int e = tid; e < cnt; e += LOCAL_THREADS) {
+            c2<R> v[4], w = ws[e];
 #pragma unroll
-            for (int k = 0; k < EPT; k++) {
-                const int e = tid + k * LOCAL_THREADS;
-                if (e < cnt) caxpy_neg<R>(wv[k], hl, vl[e]);
+            for (int q = 0; q < 4; q++)
+                if (q == 0 || q < nl) v[q] = vp[q * a.ld + e];
+            if (UPD) {
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (q == 0 || q < nl) caxpy_neg<R>(w, hl[q], v[q]);
+                ws[e] = w;
             }
+            if (DOT) {
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (q == 0 || q < nl) cdotc_acc<R>(acc[q], v[q], w);
+            }
+            if (UPD && DOT) nrm = fma(w.x, w.x, fma(w.y, w.y, nrm));
         }
     };
-    reduce_dots(0, h1s);
-    // ---- B: w -= V h1, partial h2 ----
-    update(h1s);
-    reduce_dots(1, h2s);
-    // ---- C: w -= V h2, ||w||² ----
-    update(h2s);
-    {
-        R nrm = 0;
+    // the eight sums of four vectors over the warp: lanes 16, 8, 4 apart keep one half each
+    auto reduce4 = [&](int l0) {
+        R v[8];
 #pragma unroll
-        for (int k = 0; k < EPT; k++) nrm = fma(wv[k].x, wv[k].x, fma(wv[k].y, wv[k].y, nrm));
-        warp_store(0, mk<R>(nrm, 0));
-        gather(0, 1, nrm_s);
+        for (int q = 0; q < 4; q++) { v[2 * q] = acc[q].x; v[2 * q + 1] = acc[q].y; }
+#pragma unroll
+        for (int half = 4; half > 0; half >>= 1) {
+            const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+            for (int q = 0; q < half; q++) {
+                const R x = shfl_xor(up ? v[q] : v[q + half], 4 * half);
+                v[q] = (up ? v[q + half] : v[q]) + x;
+            }
+        }
+        v[0] += shfl_xor(v[0], 2);
+        v[0] += shfl_xor(v[0], 1);
+        const int j = 2 * l0 + (lane >> 2);
+        if ((lane & 3) == 0 && j < 2 * LDP) red[warp][j] = v[0];
+    };
+    using yes = std::true_type;
+    using no = std::false_type;
+    // h1 = V^H w
+    if (warp < nw)
+#pragma unroll 1
+        for (int l0 = 0; l0 < nv; l0 += 4) {
+            pass(no(), yes(), l0, nullptr);
+            reduce4(l0);
+        }
+    gather(0, 2 * nv, [&](int j, R v) { reinterpret_cast<R *>(h1s)[j] = v; });
+    // ---- B: w -= V h1 and, in the pass of the last vectors, h2 = V^H w; slot nv of the sums: ||w||² ----
+    if (warp < nw) {
+        const int ll = (nv - 1) & ~3;
+#pragma unroll 1
+        for (int l0 = 0; l0 < ll; l0 += 4) pass(yes(), no(), l0, h1s);
+        pass(yes(), yes(), ll, h1s);
+        // (in a free place among the last four)
+#pragma unroll 1
+        for (int l0 = ll; l0 <= nv; l0 += 4) {
+            if (l0 > ll) acc[0] = acc[1] = acc[2] = acc[3] = mk<R>(0, 0);
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (l0 + q == nv) acc[q] = mk<R>(nrm, 0);
+            reduce4(l0);
+        }
+#pragma unroll 1
+        for (int l0 = 0; l0 < ll; l0 += 4) {
+            pass(no(), yes(), l0, nullptr);
+            reduce4(l0);
+        }
     }
-    if (tid == 0) hn_s = sqrt(nrm_s[0].x);
+    gather(1, 2 * nv + 1, [&](int j, R v) { reinterpret_cast<R *>(h2s)[j] = v; });
+    // ---- C: w -= V h2; the last warp first forms ||w|| ----
+    if (warp == NWARP - 1) {
+        R hh = 0;
+        for (int j = lane; j < 2 * nv; j += 32) { const R x = reinterpret_cast<const R *>(h2s)[j]; hh = fma(x, x, hh); }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) hh += shfl_xor(hh, o);
+        const R n2 = h2s[nv].x, hn = sqrt(n2 - hh);
+        if (lane == 0) {
+            direct_s = hh > (R)0.0625 * n2;
+            hn_s = hn;
+            inv_s = (R)1 / hn;
+        }
+    }
+    if (warp < nw)
+#pragma unroll 1
+        for (int l0 = 0; l0 < nv; l0 += 4) pass(yes(), no(), l0, h2s);
     __syncthreads();
+    if (direct_s) {                                  // (the same decision in every CTA)
+        nrm = 0;
+        for (int e = tid; e < cnt; e += LOCAL_THREADS) nrm = fma(ws[e].x, ws[e].x, fma(ws[e].y, ws[e].y, nrm));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) nrm += shfl_xor(nrm, o);
+        if (lane == 0) red[warp][0] = nrm;
+        gather(0, 1, [&](int, R v) { hn_s = sqrt(v); inv_s = (R)1 / sqrt(v); });
+    }
     const R hn = hn_s;
     // ---- D: v_{i+1} = w/||w||; Givens rotation and stop test ----
-    c2<R> *vn = a.V + (long long)(i + 1) * a.ld + base;
     if (hn > (R)0) {
-        const R inv = (R)1 / hn;
-#pragma unroll
-        for (int k = 0; k < EPT; k++) {
-            const int e = tid + k * LOCAL_THREADS;
-            if (e < cnt) vn[e] = mk<R>(wv[k].x * inv, wv[k].y * inv);
-        }
+        const R inv = inv_s;
+        c2<R> *vn = a.V + (long long)(i + 1) * a.ld + base;
+#pragma unroll 1
+        for (int e = tid; e < cnt; e += LOCAL_THREADS) vn[e] = mk<R>(ws[e].x * inv, ws[e].y * inv);
     }
-    if (tid == 0) {
-        c2<R> hc[MAX_RESTART + 1];
-        for (int l = 0; l <= i; l++) hc[l] = cadd<R>(h1s[l], h2s[l]);
+    if (warp == NWARP - 1) {
+        for (int l = lane; l <= i; l += 32) hcs[l] = cadd<R>(h1s[l], h2s[l]);
+        __syncwarp();
+        // earlier rotations: lanes 0, 1 form c x + s y, lanes 2, 3 c y - conj(s) x
+        c2<R> x = hcs[0];
+        __syncwarp();
+        const bool second = (lane & 2) != 0, im = (lane & 1) != 0;
         for (int l = 0; l < i; l++) {
-            const c2<R> x = hc[l], yv = hc[l + 1], sx = sn_s[l];
-            hc[l] = cadd<R>(cscale<R>(cs_s[l], x), cmul<R>(sx, yv));
-            hc[l + 1] = csub<R>(cscale<R>(cs_s[l], yv), cmul<R>(mk<R>(sx.x, -sx.y), x));
+            const c2<R> yv = hcs[l + 1], sx = sn_s[l];
+            const R p = second ? (im ? yv.y : yv.x) : (im ? x.y : x.x);
+            const R q = second ? (im ? -x.y : -x.x) : (im ? yv.y : yv.x);
+            const R r = second ? (im ? x.x : -x.y) : (im ? yv.x : -yv.y);
+            const R o = fma(cs_s[l], p, fma(sx.x, q, sx.y * r));
+            if (lane < 2) reinterpret_cast<R *>(hcs)[2 * l + lane] = o;
+            x = mk<R>(shfl(o, 2), shfl(o, 3));
         }
-        R c; c2<R> sv, rr;
-        givens<R>(hc[i], mk<R>(hn, 0), c, sv, rr);
-        hc[i] = rr;
-        hc[i + 1] = mk<R>(0, 0);
+        // the new rotation of (x, ||w||): c = |x|/t, s = (x/|x|)·||w||/t, r = (x/|x|)·t
+        R c = 1;
+        c2<R> sv = mk<R>(0, 0), rr = x;
+        const R aa = hyp(x.x, x.y), bb = hn;
+        if (bb != (R)0) {
+            if (aa == (R)0) {
+                c = 0;
+                sv = mk<R>(1, 0);
+                rr = mk<R>(bb, 0);
+            } else {
+                const R tt = hyp(aa, bb);
+                const R qv = (second ? (im ? bb : aa) : (im ? x.y : x.x)) / (second ? tt : aa);
+                const c2<R> ph = mk<R>(shfl(qv, 0), shfl(qv, 1));
+                const R cb = shfl(qv, 3);
+                c = shfl(qv, 2);
+                sv = mk<R>(ph.x * cb, ph.y * cb);
+                rr = mk<R>(ph.x * tt, ph.y * tt);
+            }
+        }
         const c2<R> gi = g_s;
         const c2<R> gn = mk<R>(-(sv.x * gi.x + sv.y * gi.y), -(sv.x * gi.y - sv.y * gi.x));   // -conj(s) g_i
         const int its = its_s + 1;
-        const R res = hypot(gn.x, gn.y);
+        const R res = hyp(gn.x, gn.y);
         const bool conv = res <= a.tol * ref_s || !(hn > (R)0);
         const bool stop = conv || its >= a.maxit || i + 1 >= a.restart;
-        stop_s = stop ? 1 : 0;
+        if (lane == 0) {
+            stop_s = stop ? 1 : 0;
+            hcs[i] = rr;
+            hcs[i + 1] = mk<R>(0, 0);
+        }
+        __syncwarp();
         if (rank == 0) {
             c2<R> *Hc = a.S.H + (long long)t * (a.restart + 1) * a.restart + (long long)i * (a.restart + 1);
-            for (int l = 0; l <= i + 1; l++) Hc[l] = hc[l];
-            a.S.cs[(long long)t * a.restart + i] = c;
-            a.S.sn[(long long)t * a.restart + i] = sv;
-            c2<R> *g = a.S.g + (long long)t * (a.restart + 1);
-            g[i] = cscale<R>(c, gi);
-            g[i + 1] = gn;
-            a.S.its[t] = its;
-            a.S.kcols[t] = i + 1;
-            if (conv || its >= a.maxit) a.S.conv[t] = 1;
-            a.act_out[t] = stop ? 0 : 1;
-            if (!stop) atomicAdd(a.counter, 1);
+            for (int l = lane; l <= i + 1; l += 32) Hc[l] = hcs[l];
+            if (lane == 0) {
+                a.S.cs[(long long)t * a.restart + i] = c;
+                a.S.sn[(long long)t * a.restart + i] = sv;
+                c2<R> *g = a.S.g + (long long)t * (a.restart + 1);
+                g[i] = cscale<R>(c, gi);
+                g[i + 1] = gn;
+                a.S.its[t] = its;
+                a.S.kcols[t] = i + 1;
+                if (conv || its >= a.maxit) a.S.conv[t] = 1;
+                a.act_out[t] = stop ? 0 : 1;
+                if (!stop) atomicAdd(a.counter, 1);
+            }
         }
     }
     __syncthreads();
@@ -918,51 +1100,48 @@ k_arnoldi_step(StepArgs<R> a) {
     cluster_barrier();                            // v_{i+1} of every CTA written and visible
     const int c0 = (int)(rank * my) / C, c1 = (int)((rank + 1) * my) / C;
     if (c1 <= c0) return;
-    const int G0 = 2 * c0 - 1, G1 = 2 * (c1 - 1) + 3, nG = G1 - G0 + 1;
-    const int W0 = G0 - 1, nW = nG + 2;
-    c2<R> *vin = reinterpret_cast<c2<R> *>(smem_raw);
-    c2<R> *tt = vin + nW * nx;
-    c2<R> *sx = tt + nG * nx;
-    const c2<R> *vnf = a.V + (long long)(i + 1) * a.ld + T.foff;
-    for (int e = tid; e < nW * nx; e += blockDim.x) {
-        const int qy = dnx.q(e), yy = W0 + qy;
-        vin[e] = (yy >= 0 && yy < ny) ? vnf[(long long)yy * nx + (e - qy * nx)] : mk<R>(0, 0);
+    const int G0 = 2 * c0 - 1, G1 = 2 * (c1 - 1) + 3, nG = G1 - G0 + 1, nW = nG + 2, PE = nx + 3;
+    c2<R> *vin = reinterpret_cast<c2<R> *>(smem_raw);                 // rows G0 - 1 .. G1 + 1
+    c2<R> *tt = vin + nW * PE;
+    stage(Vt + (long long)(i + 1) * a.ld, vin, G0 - 1, nW, PE);
+#pragma unroll 1
+    for (int e = tid; e < 3 * nG; e += LOCAL_THREADS) {               // columns -1, nx, nx + 1 of A v
+        const int q = e / 3, b = e - 3 * q;
+        tt[q * PE + (b ? nx + b : 0)] = mk<R>(0, 0);
+    }
+    async_wait();
+    __syncthreads();
+#pragma unroll 1
+    for (int e = tid; e < nG * nx; e += LOCAL_THREADS) {
+        const int q = dnx.q(e), yy = G0 + q, xx = e - q * nx;
+        c2<R> v = mk<R>(0, 0);
+        if ((unsigned)yy < (unsigned)ny)
+            v = stencil_padded<R, IMP>(a.st, a.c0, a.c1, a.c2v, vin + (q + 1) * PE + 1 + xx, PE, T.ix0 + xx, T.iy0 + yy);
+        tt[q * PE + 1 + xx] = v;
     }
     __syncthreads();
-    for (int e = tid; e < nG * nx; e += blockDim.x) {
-        const int qy = dnx.q(e), yy = G0 + qy, xx = e - qy * nx;
-        tt[e] = (yy >= 0 && yy < ny) ? stencil_smem<R, IMP>(a.st, vin, W0, nW, nx, ny, xx, yy, T.ix0, T.iy0)
-                                     : mk<R>(0, 0);
-    }
-    __syncthreads();
-    for (int e = tid; e < nG * mx; e += blockDim.x) {
+    auto five = [](const c2<R> *p, int step) {    // Σ (1,4,6,4,1)/8 · p[q·step]
+        c2<R> s = mk<R>(0, 0);
+#pragma unroll
+        for (int q = 0; q < 5; q++) {
+            const c2<R> v = p[q * step];
+            s.x = fma(zw<R>(q), v.x, s.x);
+            s.y = fma(zw<R>(q), v.y, s.y);
+        }
+        return s;
+    };
+    const BoxDiv dmx(mx);
+    c2<R> *sx = vin;                              // (A v is done with v)
+#pragma unroll 1
+    for (int e = tid; e < nG * mx; e += LOCAL_THREADS) {
         const int fr = dmx.q(e), cx = e - fr * mx;
-        c2<R> acc = mk<R>(0, 0);
-#pragma unroll
-        for (int qq = 0; qq < 5; qq++) {
-            const int fx = 2 * cx - 1 + qq;
-            if (fx >= 0 && fx < nx) {
-                const c2<R> v = tt[fr * nx + fx];
-                acc.x = fma(zw<R>(qq), v.x, acc.x);
-                acc.y = fma(zw<R>(qq), v.y, acc.y);
-            }
-        }
-        sx[e] = acc;
+        sx[e] = five(tt + fr * PE + 2 * cx, 1);
     }
     __syncthreads();
-    for (int e = tid; e < (c1 - c0) * mx; e += blockDim.x) {
-        const int qc = dmx.q(e), cy = c0 + qc, cx = e - qc * mx;
-        c2<R> acc = mk<R>(0, 0);
-#pragma unroll
-        for (int qq = 0; qq < 5; qq++) {
-            const int fy = 2 * cy - 1 + qq;
-            if (fy >= 0 && fy < ny) {
-                const c2<R> v = sx[(fy - G0) * mx + cx];
-                acc.x = fma(zw<R>(qq), v.x, acc.x);
-                acc.y = fma(zw<R>(qq), v.y, acc.y);
-            }
-        }
-        a.y[T.coff + (long long)cy * mx + cx] = make_double2((double)acc.x, (double)acc.y);
+#pragma unroll 1
+    for (int e = tid; e < (c1 - c0) * mx; e += LOCAL_THREADS) {
+        const int qc = dmx.q(e), cx = e - qc * mx;
+        a.y[T.coff + (long long)c0 * mx + e] = widen_c(five(sx + 2 * qc * mx + cx, mx));
     }
 }
 
@@ -1002,7 +1181,7 @@ void launch_zt(const LocalArgs<R> &a, const c2<R> *in, double2 *y, int apply_A, 
 template <typename R>
 size_t z_smem(const LocalArgs<R> &a) {
     const int maxc = prolong_max_cy(a.frows);
-    return ((size_t)maxc * (a.max_nx / 2 + 1) + (size_t)maxc * a.max_nx + (size_t)a.frows * a.max_nx) * csz<R>();
+    return ((size_t)maxc * prolong_pitch(a.max_nx) + (size_t)maxc * a.max_nx + (size_t)a.frows * a.max_nx) * csz<R>();
 }
 template <typename R>
 void launch_z(const LocalArgs<R> &a, const double2 *sc, const c2<R> *add, c2<R> *out,
@@ -1012,7 +1191,7 @@ void launch_z(const LocalArgs<R> &a, const double2 *sc, const c2<R> *add, c2<R> 
 template <typename R>
 size_t ps_smem(const LocalArgs<R> &a) {
     int nF = a.frows + 2, maxc = prolong_max_cy(nF);
-    return ((size_t)maxc * (a.max_nx / 2 + 1) + (size_t)maxc * a.max_nx + (size_t)nF * a.max_nx +
+    return ((size_t)maxc * prolong_pitch(a.max_nx) + (size_t)maxc * a.max_nx + (size_t)nF * a.max_nx +
             (size_t)NWARP * LDP) * csz<R>();
 }
 template <typename R>
@@ -1071,6 +1250,7 @@ cudaError_t launch_arnoldi_step(const LocalArgs<R> &la, int C, int i, int restar
     a.tasks = la.tasks; a.st = la.st; a.ld = la.ld; a.C = C; a.i = i; a.restart = restart;
     a.V = V; a.s = sc; a.y = y; a.S = S; a.act_in = act_in; a.act_out = act_out; a.counter = counter;
     a.tol = tol; a.maxit = maxit;
+    a.c0 = (R)la.st.c0; a.c1 = (R)la.st.c1; a.c2v = (R)la.st.c2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(la.ntasks * C));
     cfg.blockDim = dim3(LOCAL_THREADS);
@@ -1128,7 +1308,7 @@ void launch_cast(long long n, const void *in, int in_double, void *out, int out_
 
 size_t local_max_dynamic_smem(int max_nx, int bytes_per_c, int frows, int crows) {
     int nF = frows + 2, maxc = prolong_max_cy(nF);
-    size_t ps = ((size_t)maxc * (max_nx / 2 + 1) + (size_t)maxc * max_nx + (size_t)nF * max_nx +
+    size_t ps = ((size_t)maxc * prolong_pitch(max_nx) + (size_t)maxc * max_nx + (size_t)nF * max_nx +
                  (size_t)NWARP * LDP) * bytes_per_c;
     int cF = 2 * crows + 3;
     size_t zt = ((size_t)(cF + 2) * max_nx + (size_t)cF * max_nx + (size_t)cF * (max_nx / 2 + 1)) * bytes_per_c;
