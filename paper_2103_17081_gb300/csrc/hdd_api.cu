@@ -140,7 +140,7 @@ struct OuterWork {
 
 }  // namespace
 
-constexpr int CNT_N = MAX_RESTART + 3;         // error flag, counts before step 0 .. MAX_RESTART, tasks to restart
+constexpr int CNT_N = MAX_RESTART + 2;         // error flag, progress of step 0 .. MAX_RESTART
 
 struct hdd_ctx {
     int device = 0;
@@ -182,10 +182,10 @@ struct hdd_ctx {
     CnnState cnn;
     DevMem tmp_a, tmp_b, tmp_c;                // staging for test hooks
     DevMem d_alist;                            // active tasks of a SPIKE coarse solve, compacted
-    int *h_counter = nullptr;                  // pinned copy of d_counter
-    DevMem d_counter;                          // error flag of the dense solves, then the tasks still running
+    int *h_counter = nullptr;                  // pinned copy of the error flag
+    int *h_pub = nullptr;                      // pinned, written by the kernels: tasks before step i (-1: not known yet)
+    DevMem d_counter;                          // error flag of the dense solves, then the steps' progress
                                                // before each inner step of a cycle and after it (CNT_*)
-    cudaEvent_t ev[2] = {nullptr, nullptr};    // the copies of d_counter that are under way
     int *h_its = nullptr;                      // pinned: step counts of the tasks
     size_t h_its_n = 0;
     std::vector<double> hist;
@@ -213,7 +213,7 @@ struct hdd_ctx {
     ~hdd_ctx() {
         if (h_counter) cudaFreeHost(h_counter);
         if (h_its) cudaFreeHost(h_its);
-        for (cudaEvent_t e : ev) if (e) cudaEventDestroy(e);
+        if (h_pub) cudaFreeHost(h_pub);
     }
 };
 
@@ -294,10 +294,10 @@ hdd_status dense_error(hdd_ctx *ctx, int e, cudaStream_t s) {
 
 // Synchronises the stream; the error flag of the dense coarse solves so far.
 hdd_status sync_checked(hdd_ctx *ctx, cudaStream_t s) {
-    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, CNT_N * sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     ctx->prof.harvest();
-    return dense_error(ctx, ctx->h_counter[0], s);
+    return dense_error(ctx, *ctx->h_counter, s);
 }
 
 // ---- SPIKE plans of a factor set (the double-FP32 coarse solve split over P parts) ----------
@@ -1109,7 +1109,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     double2 *y = W.y.template as<double2>(), *sc = W.s.template as<double2>();
     c2<R> *p1 = W.p1.template as<c2<R>>(), *p2 = W.p2.template as<c2<R>>(), *p3 = W.p3.template as<c2<R>>();
     int *act[2] = {S.its + 3 * nt, S.its + 4 * nt}, *rs = S.its + 5 * nt, *rs2 = S.its + 6 * nt;
-    int *cnt = ctx->d_counter.as<int>() + 1;     // cnt[i]: tasks before step i; cnt[RST + 1]: tasks to restart
+    const Progress pr = {ctx->d_counter.as<unsigned long long>() + 1, ctx->h_pub, ctx->d_counter.as<int>(), nt};
     const int *ones = ctx->d_ones.as<int>();
     const R tol = (R)prm->inner_tol;
     const int maxit = prm->inner_maxit;
@@ -1131,27 +1131,32 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         CK(cudaMallocHost(&ctx->h_its, nt * sizeof(int)));
         ctx->h_its_n = nt;
     }
-    // Progress: each step counts the tasks that go on into a slot of its own, and the slots are
-    // copied to the host after every step.  The host launches a step before it has seen whether any
-    // task needs it, then waits for the count before that step: the device always has the next step
-    // queued, and one step at the end finds no task (a few microseconds against a round trip to the
-    // host per step, 10 to 15).  A split (SPIKE) banded solve is launched for a given number of
-    // tasks, so there the host waits first.
+    // Progress: the last task to decide about a step writes the count of those that run it where the
+    // host reads it.  The host launches a step before it has seen whether any task needs it, then
+    // waits for the count before that step: the device always has the next step queued, and one step
+    // at the end finds no task (a few microseconds against a round trip to the host per step, 10 to
+    // 15).  A split (SPIKE) banded solve is launched for a given number of tasks, so there the host
+    // waits first.
     const bool ahead = dense || !(cdf && ctx->coarse_spike && ctx->E.spike_levels_built);
-    auto post = [&](int slot) -> hdd_status {
-        CK(cudaMemcpyAsync(ctx->h_counter, ctx->d_counter.p, CNT_N * sizeof(int), cudaMemcpyDeviceToHost, s));
-        CK(cudaEventRecord(ctx->ev[slot & 1], s));
-        return HDD_OK;
-    };
+    volatile int *pub = ctx->h_pub;
+    std::fill(ctx->h_its, ctx->h_its + nt, 0);
+    for (int i = 0; i <= MAX_RESTART; i++) pub[i] = -1;
     auto seen = [&](int slot, int *n) -> hdd_status {
-        CK(cudaEventSynchronize(ctx->ev[slot & 1]));
-        *n = ctx->h_counter[1 + slot];
-        return dense_error(ctx, ctx->h_counter[0], s);
+        for (long long spin = 1; pub[slot] == -1; spin++)
+            if (spin % 4096 == 0) {                     // the stream must still be running
+                const cudaError_t e = cudaStreamQuery(s);
+                if (e == cudaErrorNotReady) continue;
+                CK(e);
+                if (pub[slot] == -1) FAIL(HDD_ERR_CUDA, "the inner iteration's progress was not reported");
+            }
+        *n = pub[slot];
+        return *n == -2 ? sync_checked(ctx, s) : HDD_OK;
     };
 
     const int *all = mask ? mask : ones;
-    KL(F_LMISC, ld * (16 + cs), 0, launch_restrict<R>(a, v, ctx->nglob, f, mask, s));
     CK(cudaMemsetAsync(W.ints.p, 0, 7 * nt * sizeof(int), s));
+    CK(cudaMemsetAsync(pr.slot, 0, (RST + 1) * sizeof(*pr.slot), s));
+    KL(F_LMISC, ld * (16 + cs), 0, launch_restrict<R>(a, v, ctx->nglob, f, mask, s));
     const bool warm = prm->warm_start && ctx->cnn.ready;
     if (!warm) {
         // first cycle from ũ = 0: r0 = P f̃ = f̃ - A Z E⁻¹ Zᵀ f̃, and ref = ||P f̃||
@@ -1185,10 +1190,8 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         KL(F_LMISC, 0, 0, launch_set_ref<R>(a, S, p3, mask, s));
         KL(F_PS, 2 * ld * cs + ldc * 16, 0, launch_prolong_stencil<R>(a, 1, t, sc, V, nullptr, 0, p3, mask, s));
     }
-    CK(cudaMemsetAsync(cnt, 0, (RST + 2) * sizeof(int), s));
-    KL(F_LMISC, 2 * ld * cs, 0, launch_init_cycle<R>(a, S, RST, V, p3, all, act[0], cnt, tol, maxit, warm ? 0 : 1, s));
+    KL(F_LMISC, 2 * ld * cs, 0, launch_init_cycle<R>(a, S, RST, V, p3, all, act[0], pr, tol, maxit, warm ? 0 : 1, s));
     CKL();
-    if ((st = post(0)) != HDD_OK) return st;
     const int *cyc = all;                       // tasks of this cycle
     bool first = !warm;                         // ũ is still zero (and not in memory)
     double2 *scomp = sc + (long long)(RST + 1) * ldc;
@@ -1205,7 +1208,6 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
                 if ((st = seen(i, &nact)) != HDD_OK) return st;
                 if (nact == 0) break;
             }
-            int *next = cnt + i + 1;
             const int *ain = act[cur];
             int *aout = act[cur ^ 1];
             c2<R> *vi = V + (long long)i * ld, *vn = V + (long long)(i + 1) * ld;
@@ -1216,7 +1218,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
                 // algorithmic bytes of the fused schedule: 3 passes over V_0..V_i, v_i, v_{i+1}
                 // written and read back for the next Zᵀ A, s read and y written
                 KL(F_STEP, fa * ((3.0 * i + 7) * ld * cs + 2.0 * ldc * 16), fa * 40.0 * (i + 1) * ld,
-                   CK(launch_arnoldi_step<R>(a, stepC, i, RST, V, si, y, S, ain, aout, next, tol, maxit, step_sm, s)));
+                   CK(launch_arnoldi_step<R>(a, stepC, i, RST, V, si, y, S, ain, aout, pr, tol, maxit, step_sm, s)));
             } else {
                 KL(F_ZT, fa * (ld * cs + ldc * 16), 0, launch_zt<R>(a, vi, y, 1, ain, s));
                 if ((st = coarse(y, si, ain, nact)) != HDD_OK) return st;
@@ -1228,11 +1230,10 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
                    launch_cgs_update<R>(a, 3, vn, V, i + 1, p2, p3, ain, s));
                 CK(cudaMemsetAsync(aout, 0, nt * sizeof(int), s));
                 KL(F_GIVENS, fa * 2 * ld * cs, 0,
-                   launch_givens_normalize<R>(a, S, RST, i, vn, p1, p2, p3, ain, aout, next, tol, maxit, s));
+                   launch_givens_normalize<R>(a, S, RST, i, vn, p1, p2, p3, ain, aout, pr, tol, maxit, s));
             }
             CKL();
             cur ^= 1;
-            if ((st = post(i + 1)) != HDD_OK) return st;
             if (ahead) {
                 if ((st = seen(i, &nact)) != HDD_OK) return st;
                 if (nact == 0) break;
@@ -1243,12 +1244,12 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         // was solved during the cycle), into z = Σ R_jᵀ D_j x_j; flag the ones needing a restart
         KL(F_LMISC, (RST + 2) * ldc * 16.0, 0, launch_coarse_combine<R>(a, S, RST, sc, scomp, cyc, s));
         KL(F_LMISC, ld * (5 * cs + 16) + ldc * 16, 0,
-           launch_finish<R>(a, S, RST, first ? 1 : 0, u, V, scomp, cyc, rs, cnt + RST + 1, maxit, ctx->nglob, z, s));
+           launch_finish<R>(a, S, RST, first ? 1 : 0, u, V, scomp, cyc, rs, ctx->h_its, maxit, ctx->nglob, z, s));
         CKL();
         first = false;
-        CK(cudaMemcpyAsync(ctx->h_its, S.its, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
         if ((st = sync_checked(ctx, s)) != HDD_OK) return st;
-        const int nrs = ctx->h_counter[1 + RST + 1];
+        int nrs = 0;                                // h_its: iterations, inverted for a task that goes on
+        for (int q = 0; q < nt; q++) nrs += ctx->h_its[q] < 0;
         if (nrs == 0) break;
         // restart: r = P(f̃ - A ũ) → v0
         KL(F_LMISC, 0, 0, launch_local_A<R>(a, u, t, f, rs, s));
@@ -1256,10 +1257,10 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
         if ((st = coarse(y, sc, rs, nrs)) != HDD_OK) return st;
         KL(F_PS, 0, 0, launch_prolong_stencil<R>(a, 1, t, sc, V, nullptr, 0, p3, rs, s));
         CK(cudaMemsetAsync(act[cur], 0, nt * sizeof(int), s));
-        CK(cudaMemsetAsync(cnt, 0, (RST + 2) * sizeof(int), s));
-        KL(F_LMISC, 0, 0, launch_init_cycle<R>(a, S, RST, V, p3, rs, act[cur], cnt, tol, maxit, 0, s));
+        CK(cudaMemsetAsync(pr.slot, 0, (RST + 1) * sizeof(*pr.slot), s));
+        for (int i = 0; i <= MAX_RESTART; i++) pub[i] = -1;      // (the stream is idle)
+        KL(F_LMISC, 0, 0, launch_init_cycle<R>(a, S, RST, V, p3, rs, act[cur], pr, tol, maxit, 0, s));
         CKL();
-        if ((st = post(0)) != HDD_OK) return st;
         nact = nrs;
         cyc = rs;
         std::swap(rs, rs2);
@@ -1660,11 +1661,10 @@ hdd_status hdd_create(hdd_ctx **out, int device) {
     ctx->device = device;
     if (cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || ctx->nsm < 1)
         ctx->nsm = 152;
-    if (cudaMallocHost(&ctx->h_counter, CNT_N * sizeof(int)) != cudaSuccess ||
-        ctx->d_counter.ensure(CNT_N * sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_counter.p, 0, CNT_N * sizeof(int)) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->ev[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ctx->ev[1], cudaEventDisableTiming) != cudaSuccess) {
+    if (cudaMallocHost(&ctx->h_counter, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_pub, (MAX_RESTART + 1) * sizeof(int)) != cudaSuccess ||
+        ctx->d_counter.ensure(CNT_N * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMemset(ctx->d_counter.p, 0, CNT_N * sizeof(unsigned long long)) != cudaSuccess) {
         delete ctx;
         return HDD_ERR_OOM;
     }

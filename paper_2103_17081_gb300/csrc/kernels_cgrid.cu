@@ -23,6 +23,8 @@ __device__ __forceinline__ int hat_num(int dx, int dy, int c, int diag) {
 template <typename T>
 __global__ void k_cg_restrict(CGrid g, const double2 *__restrict__ v, c2<T> *__restrict__ vH,
                               long long ldv, long long ldh, const int *__restrict__ active) {
+    CHAIN_ENTER();
+    LAUNDER(v); LAUNDER(active);
     if (active && !active[blockIdx.y]) return;
     v += blockIdx.y * ldv;
     vH += blockIdx.y * ldh;
@@ -52,6 +54,8 @@ __global__ void k_cg_restrict(CGrid g, const double2 *__restrict__ v, c2<T> *__r
 template <typename T>
 __global__ void k_cg_prolong(CGrid g, const c2<T> *__restrict__ xH, double2 *__restrict__ z, int accumulate,
                              long long ldv, long long ldh, const int *__restrict__ active) {
+    CHAIN_ENTER();
+    LAUNDER(xH); LAUNDER(active);
     if (active && !active[blockIdx.y]) return;
     z += blockIdx.y * ldv;
     xH += blockIdx.y * ldh;
@@ -107,6 +111,8 @@ template <typename T>
 __global__ void __launch_bounds__(DTHREADS)
 k_dst_pass(int m, long long ldh, const T *__restrict__ S, const T *__restrict__ Dinv,
            const c2<T> *__restrict__ in, c2<T> *__restrict__ out, const int *__restrict__ active) {
+    CHAIN_ENTER();
+    LAUNDER(in); LAUNDER(active);
     if (active && !active[blockIdx.z]) return;
     in += blockIdx.z * ldh;
     out += blockIdx.z * ldh;
@@ -201,13 +207,13 @@ static int cg_grid(long long n) {
 template <typename T>
 void launch_cg_restrict(const CGrid &g, const double2 *v, c2<T> *vH, int nrhs, long long ldv, long long ldh,
                         const int *active, cudaStream_t s) {
-    k_cg_restrict<T><<<dim3(cg_grid((long long)g.m * g.m), nrhs), 256, 0, s>>>(g, v, vH, ldv, ldh, active);
+    launch_chained(k_cg_restrict<T>, dim3(cg_grid((long long)g.m * g.m), nrhs), 256, 0, s, g, v, vH, ldv, ldh, active);
 }
 template <typename T>
 void launch_cg_prolong(const CGrid &g, const c2<T> *xH, double2 *z, int accumulate, int nrhs, long long ldv,
                        long long ldh, const int *active, cudaStream_t s) {
     const long long n = (long long)(g.N - 1) * (g.N - 1);
-    k_cg_prolong<T><<<dim3(cg_grid(n), nrhs), 256, 0, s>>>(g, xH, z, accumulate, ldv, ldh, active);
+    launch_chained(k_cg_prolong<T>, dim3(cg_grid(n), nrhs), 256, 0, s, g, xH, z, accumulate, ldv, ldh, active);
 }
 template <typename T>
 void launch_dst_pass(int m, const T *S, const T *Dinv, const c2<T> *in, c2<T> *out, int nrhs, long long ldh,
@@ -215,7 +221,7 @@ void launch_dst_pass(int m, const T *S, const T *Dinv, const c2<T> *in, c2<T> *o
     const int t = (m + DT - 1) / DT;
     static_assert((size_t)DGROUPS * DT * (DT + 1) * sizeof(c2<T>) <= dst_smem<T>(), "the groups' sums fit");
     cudaFuncSetAttribute(k_dst_pass<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dst_smem<T>());
-    k_dst_pass<T><<<dim3(t, t, nrhs), DTHREADS, dst_smem<T>(), s>>>(m, ldh, S, Dinv, in, out, active);
+    launch_chained(k_dst_pass<T>, dim3(t, t, nrhs), DTHREADS, dst_smem<T>(), s, m, ldh, S, Dinv, in, out, active);
 }
 void launch_cg_widen(long long n, const float2 *in, double2 *out, cudaStream_t s) {
     k_cg_convert<float2, double2><<<cg_grid(n), 256, 0, s>>>(n, in, out);

@@ -264,9 +264,10 @@ template <int DS>
 __global__ void __launch_bounds__(128)
 k_dense_slice(const DenseTask *__restrict__ recs, const double2 *__restrict__ in, uint4 *__restrict__ B, int *__restrict__ cexp,
               const int *__restrict__ flag) {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int t = blockIdx.x, tid = threadIdx.x;
     const DenseTask S = recs[t];
+    CHAIN_ENTER();
+    LAUNDER(in); LAUNDER(flag);
     if (flag && !flag[t]) return;
     const double2 *y = in + S.coff;
     __shared__ unsigned long long red[2][4];
@@ -411,7 +412,10 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
         for (int q = tid; q <= ns; q += DE_T) part[q] = pre[q];
         if (tid == 0) part[ns + 1] = make_int2((int)G, 0);
     }
-    if (U == 0 || blockIdx.x >= G) return;
+    if (U == 0 || blockIdx.x >= G) {                 // (waits all the same: the end of this kernel is the end of those before)
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
+        return;
+    }
     // CTA b takes the units that start in [Wt·b/G, Wt·(b+1)/G) of the total weight
     auto shape_of = [&](int v, bool wt) {            // the last shape whose offset is at most v
         int lo = 0, hi = ns;
@@ -650,6 +654,7 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
         }
         if (!waited) {
             asm volatile("griddepcontrol.wait;\n" ::: "memory");
+            asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
             waited = true;
         }
         unsigned long long *acc = ws + S.acc0 + (size_t)it.y * 128 * S.nt + row;
@@ -678,6 +683,7 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
             out[o[e]] = make_double2(from_fixed((long long)x[2 * e], re + ce[e].x), from_fixed((long long)x[2 * e + 1], re + ce[e].y));
         }
     }
+    if (!waited) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 // ------------------------------------------------------------------------------------------
@@ -712,7 +718,7 @@ cudaError_t dense_set_smem() {
 }
 template <int DS>
 static void dense_launch(const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
-    k_dense_slice<DS><<<dim3(p.ntask, DSPLIT), 128, 0, s>>>(p.recs, in, reinterpret_cast<uint4 *>(p.B), p.cexp, flag);
+    launch_chained(k_dense_slice<DS>, dim3(p.ntask, DSPLIT), 128, 0, s, p.recs, in, reinterpret_cast<uint4 *>(p.B), p.cexp, flag);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.grid);
     cfg.blockDim = dim3(DE_T);

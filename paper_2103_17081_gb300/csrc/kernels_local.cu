@@ -150,8 +150,10 @@ __global__ void __launch_bounds__(LOCAL_THREADS)
 k_restrict(LocalArgs<R> a, int gw, long long nglob, const double2 *__restrict__ glob,
            c2<R> *__restrict__ out, const int *__restrict__ flag) {
     const Tile tl = a.ftiles[blockIdx.x];
-    if (flag && !flag[tl.task]) return;
     const Task T = a.tasks[tl.task];
+    CHAIN_ENTER();
+    LAUNDER(glob); LAUNDER(flag);
+    if (flag && !flag[tl.task]) return;
     const int cnt = tl.nr * T.nx;
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
         int y = tl.r0 + e / T.nx, x = e % T.nx;
@@ -213,8 +215,10 @@ k_zt(LocalArgs<R> a, const c2<R> *__restrict__ in, double2 *__restrict__ yout, i
      const int *__restrict__ flag) {
     extern __shared__ unsigned char smem_raw[];
     const Tile tl = a.ctiles[blockIdx.x];
-    if (flag && !flag[tl.task]) return;
     const Task T = a.tasks[tl.task];
+    CHAIN_ENTER();
+    LAUNDER(in); LAUNDER(flag);
+    if (flag && !flag[tl.task]) return;
     const int nx = T.nx, ny = T.ny, mx = T.mx;
     // fine rows feeding coarse rows [r0, r0+nr): 2c-1 .. 2c+3
     const int F0 = 2 * tl.r0 - 1, F1 = 2 * (tl.r0 + tl.nr - 1) + 3;
@@ -370,8 +374,10 @@ k_prolong_stencil(LocalArgs<R> a, int mode, const c2<R> *__restrict__ in,
                   const int *__restrict__ flag) {
     extern __shared__ unsigned char smem_raw[];
     const Tile tl = a.ftiles[blockIdx.x];
-    if (flag && !flag[tl.task]) return;
     const Task T = a.tasks[tl.task];
+    CHAIN_ENTER();
+    LAUNDER(in); LAUNDER(s); LAUNDER(V); LAUNDER(flag);
+    if (flag && !flag[tl.task]) return;
     const int nx = T.nx, ny = T.ny;
     const int F0 = tl.r0 - 1, nF = tl.nr + 2;
     const int maxc = prolong_max_cy(nF);
@@ -527,13 +533,16 @@ __global__ void __launch_bounds__(LOCAL_THREADS)
 k_givens_normalize(LocalArgs<R> a, InnerState<R> S, int restart, int i, c2<R> *__restrict__ w,
                    const c2<R> *__restrict__ p1, const c2<R> *__restrict__ p2,
                    const c2<R> *__restrict__ p3, const int *__restrict__ act_in,
-                   int *__restrict__ act_out, int *__restrict__ counter, R tol, int maxit) {
+                   int *__restrict__ act_out, Progress pr, R tol, int maxit) {
     __shared__ R hn_s;
     __shared__ c2<R> hsum[LDP];
     const Tile tl = a.ftiles[blockIdx.x];
-    if (!act_in[tl.task]) return;
     const Task T = a.tasks[tl.task];
     const bool first = blockIdx.x == T.tile0;          // this tile also updates the task's rotations
+    if (!act_in[tl.task]) {
+        if (first && threadIdx.x == 0) publish(pr, i + 1, 0);
+        return;
+    }
     if (threadIdx.x < 32) {
         const R s = task_norm2_warp<R>(p3, T);
         if (threadIdx.x == 0) hn_s = sqrt(s);
@@ -581,7 +590,7 @@ k_givens_normalize(LocalArgs<R> a, InnerState<R> S, int restart, int i, c2<R> *_
     const bool stop = conv || its >= maxit || i + 1 >= restart;
     if (conv || its >= maxit) S.conv[t] = 1;
     act_out[t] = stop ? 0 : 1;
-    if (!stop) atomicAdd(counter, 1);
+    publish(pr, i + 1, stop ? 0 : 1);
 }
 
 // Start of a cycle: r = P(f̃ - A u) was written into v0 by k_prolong_stencil (mode 1) with its
@@ -590,11 +599,16 @@ template <typename R>
 __global__ void __launch_bounds__(LOCAL_THREADS)
 k_init_cycle(LocalArgs<R> a, InnerState<R> S, int restart, c2<R> *__restrict__ v0,
              const c2<R> *__restrict__ p3, const int *__restrict__ flag, int *__restrict__ act_out,
-             int *__restrict__ counter, R tol, int maxit, int set_ref) {
+             Progress pr, R tol, int maxit, int set_ref) {
     __shared__ R beta_s;
     const Tile tl = a.ftiles[blockIdx.x];
-    if (!flag[tl.task]) return;
     const Task T = a.tasks[tl.task];
+    CHAIN_ENTER();
+    LAUNDER(p3); LAUNDER(flag);
+    if (!flag[tl.task]) {
+        if (blockIdx.x == T.tile0 && threadIdx.x == 0) publish(pr, 0, 0);
+        return;
+    }
     if (threadIdx.x < 32) {
         const R s = task_norm2_warp<R>(p3, T);
         if (threadIdx.x == 0) beta_s = sqrt(s);
@@ -619,7 +633,7 @@ k_init_cycle(LocalArgs<R> a, InnerState<R> S, int restart, c2<R> *__restrict__ v
     const bool done = !(beta > tol * S.ref[t]) || S.its[t] >= maxit;
     if (done) S.conv[t] = 1;
     act_out[t] = done ? 0 : 1;
-    if (!done) atomicAdd(counter, 1);
+    publish(pr, 0, done ? 0 : 1);
 }
 
 // y = H(0:k,0:k)⁻¹ g(0:k) for task t, by one thread (k <= restart <= 64).
@@ -645,8 +659,10 @@ k_coarse_combine(LocalArgs<R> a, InnerState<R> S, int restart, const double2 *__
                  double2 *__restrict__ sc, const int *__restrict__ flag) {
     __shared__ c2<R> y[MAX_RESTART];
     const Tile tl = a.ctiles[blockIdx.x];
-    if (flag && !flag[tl.task]) return;
     const Task T = a.tasks[tl.task];
+    CHAIN_ENTER();
+    LAUNDER(sbuf); LAUNDER(flag);
+    if (flag && !flag[tl.task]) return;
     const int k = S.kcols[tl.task];
     if (threadIdx.x == 0) solve_small<R>(S, restart, tl.task, k, y);
     __syncthreads();
@@ -674,20 +690,22 @@ template <typename R>
 __global__ void __launch_bounds__(LOCAL_THREADS)
 k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restrict__ u, const c2<R> *__restrict__ V,
          const double2 *__restrict__ s, const int *__restrict__ flag, int *__restrict__ rs_out,
-         int *__restrict__ counter, int maxit, long long nglob, double2 *__restrict__ glob) {
+         int *__restrict__ its_out, int maxit, long long nglob, double2 *__restrict__ glob) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ c2<R> y[MAX_RESTART];
     const Tile tl = a.ftiles[blockIdx.x];
     const int t = tl.task;
-    if (!flag[t]) return;
     const Task T = a.tasks[t];
+    CHAIN_ENTER();
+    LAUNDER(V); LAUNDER(s); LAUNDER(flag);
+    if (!flag[t]) return;
     const int k = S.kcols[t];
     const bool again = !S.conv[t] && S.its[t] < maxit;
     if (threadIdx.x == 0) {
         solve_small<R>(S, restart, t, k, y);
         if (blockIdx.x == T.tile0) {
             rs_out[t] = again ? 1 : 0;
-            if (again) atomicAdd(counter, 1);
+            its_out[t] = again ? ~S.its[t] : S.its[t];    // (the host's pinned memory)
         }
     }
     const int maxc = prolong_max_cy(tl.nr);
@@ -764,7 +782,7 @@ template <typename R> struct StepArgs {
     InnerState<R> S;
     const int *act_in;
     int *act_out;
-    int *counter;
+    Progress pr;
     R tol;
     int maxit;
     R c0, c1, c2v;          // the interior stencil in the inner precision
@@ -834,10 +852,13 @@ k_arnoldi_step(StepArgs<R> a) {
     const int C = a.C;
     const int t = (int)blockIdx.x / C;
     const unsigned rank = cluster_rank();
-    const int act = a.act_in[t];                     // the same flag for every CTA of the cluster
     const Task T = a.tasks[t];
-    if (!act) {
-        if (rank == 0 && threadIdx.x == 0) a.act_out[t] = 0;
+    CHAIN_ENTER();
+    if (!a.act_in[t]) {                              // the same flag for every CTA of the cluster
+        if (rank == 0 && threadIdx.x == 0) {
+            a.act_out[t] = 0;
+            publish(a.pr, a.i + 1, 0);
+        }
         return;
     }
     const int nx = T.nx, ny = T.ny, mx = T.mx, my = T.my;
@@ -1090,7 +1111,7 @@ k_arnoldi_step(StepArgs<R> a) {
                 a.S.kcols[t] = i + 1;
                 if (conv || its >= a.maxit) a.S.conv[t] = 1;
                 a.act_out[t] = stop ? 0 : 1;
-                if (!stop) atomicAdd(a.counter, 1);
+                publish(a.pr, i + 1, stop ? 0 : 1);
             }
         }
     }
@@ -1153,7 +1174,7 @@ template <typename R> static size_t csz() { return sizeof(c2<R>); }
 template <typename R>
 void launch_restrict(const LocalArgs<R> &a, const double2 *glob, long long nglob, c2<R> *out,
                      const int *flag, cudaStream_t s) {
-    k_restrict<R><<<a.nftiles, LOCAL_THREADS, 0, s>>>(a, a.gw, nglob, glob, out, flag);
+    launch_chained(k_restrict<R>, a.nftiles, LOCAL_THREADS, 0, s, a, a.gw, nglob, glob, out, flag);
 }
 template <typename R>
 void launch_scatter(const LocalArgs<R> &a, const c2<R> *x, double2 *glob, long long nglob,
@@ -1175,8 +1196,8 @@ size_t zt_smem(const LocalArgs<R> &a, int apply_A) {
 template <typename R>
 void launch_zt(const LocalArgs<R> &a, const c2<R> *in, double2 *y, int apply_A, const int *flag,
                cudaStream_t s) {
-    if (a.st.bc) k_zt<R, true><<<a.nctiles, LOCAL_THREADS, zt_smem(a, apply_A), s>>>(a, in, y, apply_A, flag);
-    else k_zt<R, false><<<a.nctiles, LOCAL_THREADS, zt_smem(a, apply_A), s>>>(a, in, y, apply_A, flag);
+    if (a.st.bc) launch_chained(k_zt<R, true>, a.nctiles, LOCAL_THREADS, zt_smem(a, apply_A), s, a, in, y, apply_A, flag);
+    else launch_chained(k_zt<R, false>, a.nctiles, LOCAL_THREADS, zt_smem(a, apply_A), s, a, in, y, apply_A, flag);
 }
 template <typename R>
 size_t z_smem(const LocalArgs<R> &a) {
@@ -1199,11 +1220,11 @@ void launch_prolong_stencil(const LocalArgs<R> &a, int mode, const c2<R> *in, co
                             c2<R> *out, const c2<R> *V, int nv, c2<R> *part, const int *flag,
                             cudaStream_t s) {
     if (a.st.bc)
-        k_prolong_stencil<R, true><<<a.nftiles, LOCAL_THREADS, ps_smem(a), s>>>(a, mode, in, sc, out, V, nv,
-                                                                                part, flag);
+        launch_chained(k_prolong_stencil<R, true>, a.nftiles, LOCAL_THREADS, ps_smem(a), s, a, mode, in, sc, out, V, nv, part,
+                       flag);
     else
-        k_prolong_stencil<R, false><<<a.nftiles, LOCAL_THREADS, ps_smem(a), s>>>(a, mode, in, sc, out, V, nv,
-                                                                                 part, flag);
+        launch_chained(k_prolong_stencil<R, false>, a.nftiles, LOCAL_THREADS, ps_smem(a), s, a, mode, in, sc, out, V, nv, part,
+                       flag);
 }
 template <typename R>
 void launch_cgs_update(const LocalArgs<R> &a, int pass, c2<R> *w, const c2<R> *V, int nv,
@@ -1213,24 +1234,24 @@ void launch_cgs_update(const LocalArgs<R> &a, int pass, c2<R> *w, const c2<R> *V
 template <typename R>
 void launch_givens_normalize(const LocalArgs<R> &a, const InnerState<R> &S, int restart, int i,
                              c2<R> *w, const c2<R> *p1, const c2<R> *p2, const c2<R> *p3,
-                             const int *act_in, int *act_out, int *counter, R tol, int maxit,
+                             const int *act_in, int *act_out, const Progress &pr, R tol, int maxit,
                              cudaStream_t s) {
     k_givens_normalize<R><<<a.nftiles, LOCAL_THREADS, 0, s>>>(a, S, restart, i, w, p1, p2, p3, act_in,
-                                                               act_out, counter, tol, maxit);
+                                                               act_out, pr, tol, maxit);
 }
 template <typename R>
 void launch_init_cycle(const LocalArgs<R> &a, const InnerState<R> &S, int restart, c2<R> *v0,
-                       const c2<R> *p3, const int *flag, int *act_out, int *counter, R tol,
+                       const c2<R> *p3, const int *flag, int *act_out, const Progress &pr, R tol,
                        int maxit, int set_ref, cudaStream_t s) {
-    k_init_cycle<R><<<a.nftiles, LOCAL_THREADS, 0, s>>>(a, S, restart, v0, p3, flag, act_out, counter,
-                                                         tol, maxit, set_ref);
+    launch_chained(k_init_cycle<R>, a.nftiles, LOCAL_THREADS, 0, s, a, S, restart, v0, p3, flag, act_out, pr, tol, maxit,
+                   set_ref);
 }
 template <typename R>
 void launch_finish(const LocalArgs<R> &a, const InnerState<R> &S, int restart, int first, c2<R> *u, const c2<R> *V,
-                   const double2 *sc, const int *flag, int *rs_out, int *counter, int maxit, long long nglob,
+                   const double2 *sc, const int *flag, int *rs_out, int *its_out, int maxit, long long nglob,
                    double2 *glob, cudaStream_t s) {
-    k_finish<R><<<a.nftiles, LOCAL_THREADS, z_smem(a), s>>>(a, S, restart, first, u, V, sc, flag, rs_out, counter, maxit,
-                                                            nglob, glob);
+    launch_chained(k_finish<R>, a.nftiles, LOCAL_THREADS, z_smem(a), s, a, S, restart, first, u, V, sc, flag, rs_out, its_out,
+                   maxit, nglob, glob);
 }
 template <typename R>
 void launch_set_ref(const LocalArgs<R> &a, const InnerState<R> &S, const c2<R> *p3, const int *flag,
@@ -1240,15 +1261,15 @@ void launch_set_ref(const LocalArgs<R> &a, const InnerState<R> &S, const c2<R> *
 template <typename R>
 void launch_coarse_combine(const LocalArgs<R> &a, const InnerState<R> &S, int restart,
                            const double2 *sbuf, double2 *sc, const int *flag, cudaStream_t s) {
-    k_coarse_combine<R><<<a.nctiles, LOCAL_THREADS, 0, s>>>(a, S, restart, sbuf, sc, flag);
+    launch_chained(k_coarse_combine<R>, a.nctiles, LOCAL_THREADS, 0, s, a, S, restart, sbuf, sc, flag);
 }
 template <typename R>
 cudaError_t launch_arnoldi_step(const LocalArgs<R> &la, int C, int i, int restart, c2<R> *V, const double2 *sc,
                                 double2 *y, const InnerState<R> &S, const int *act_in, int *act_out,
-                                int *counter, R tol, int maxit, size_t smem, cudaStream_t s) {
+                                const Progress &pr, R tol, int maxit, size_t smem, cudaStream_t s) {
     StepArgs<R> a;
     a.tasks = la.tasks; a.st = la.st; a.ld = la.ld; a.C = C; a.i = i; a.restart = restart;
-    a.V = V; a.s = sc; a.y = y; a.S = S; a.act_in = act_in; a.act_out = act_out; a.counter = counter;
+    a.V = V; a.s = sc; a.y = y; a.S = S; a.act_in = act_in; a.act_out = act_out; a.pr = pr;
     a.tol = tol; a.maxit = maxit;
     a.c0 = (R)la.st.c0; a.c1 = (R)la.st.c1; a.c2v = (R)la.st.c2;
     cudaLaunchConfig_t cfg = {};
@@ -1256,13 +1277,15 @@ cudaError_t launch_arnoldi_step(const LocalArgs<R> &la, int C, int i, int restar
     cfg.blockDim = dim3(LOCAL_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (la.st.bc) return cudaLaunchKernelEx(&cfg, k_arnoldi_step<R, true>, a);
     return cudaLaunchKernelEx(&cfg, k_arnoldi_step<R, false>, a);
 }
@@ -1336,13 +1359,13 @@ template <typename R> cudaError_t set_local_smem_limits(size_t bytes) {
     template void launch_z<R>(const LocalArgs<R> &, const double2 *, const c2<R> *, c2<R> *, const int *, cudaStream_t, R); \
     template void launch_prolong_stencil<R>(const LocalArgs<R> &, int, const c2<R> *, const double2 *, c2<R> *, const c2<R> *, int, c2<R> *, const int *, cudaStream_t); \
     template void launch_cgs_update<R>(const LocalArgs<R> &, int, c2<R> *, const c2<R> *, int, const c2<R> *, c2<R> *, const int *, cudaStream_t); \
-    template void launch_givens_normalize<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const c2<R> *, const c2<R> *, const int *, int *, int *, R, int, cudaStream_t); \
-    template void launch_init_cycle<R>(const LocalArgs<R> &, const InnerState<R> &, int, c2<R> *, const c2<R> *, const int *, int *, int *, R, int, int, cudaStream_t); \
+    template void launch_givens_normalize<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const c2<R> *, const c2<R> *, const int *, int *, const Progress &, R, int, cudaStream_t); \
+    template void launch_init_cycle<R>(const LocalArgs<R> &, const InnerState<R> &, int, c2<R> *, const c2<R> *, const int *, int *, const Progress &, R, int, int, cudaStream_t); \
     template void launch_finish<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const double2 *, const int *, int *, int *, int, long long, double2 *, cudaStream_t); \
     template cudaError_t set_local_smem_limits<R>(size_t); \
     template void launch_coarse_combine<R>(const LocalArgs<R> &, const InnerState<R> &, int, const double2 *, double2 *, const int *, cudaStream_t); \
     template void launch_set_ref<R>(const LocalArgs<R> &, const InnerState<R> &, const c2<R> *, const int *, cudaStream_t); \
-    template cudaError_t launch_arnoldi_step<R>(const LocalArgs<R> &, int, int, int, c2<R> *, const double2 *, double2 *, const InnerState<R> &, const int *, int *, int *, R, int, size_t, cudaStream_t); \
+    template cudaError_t launch_arnoldi_step<R>(const LocalArgs<R> &, int, int, int, c2<R> *, const double2 *, double2 *, const InnerState<R> &, const int *, int *, const Progress &, R, int, size_t, cudaStream_t); \
     template int arnoldi_step_max_cluster<R>(size_t, int);
 
 INST(float)

@@ -27,6 +27,8 @@ int outer_grid(long long n) {
 template <bool IMP>
 __global__ void k_gstencil(Stencil st, int N, const double2 *__restrict__ x, double2 *__restrict__ y,
                            const double2 *__restrict__ f, const int *__restrict__ active) {
+    CHAIN_ENTER();
+    LAUNDER(x); LAUNDER(f); LAUNDER(active);
     if (active && !active[blockIdx.y]) return;
     const int w = IMP ? N + 1 : N - 1;
     const long long n = (long long)w * w;
@@ -592,6 +594,8 @@ __global__ void __launch_bounds__(OT) k_onorm(OuterBatch B, const double2 *__res
 __global__ void k_oreduce(OuterBatch B, const double2 *__restrict__ part, int nv, double2 *__restrict__ out,
                           const double2 *__restrict__ part_b, double2 *__restrict__ out_b) {
     const int r = blockIdx.y;
+    CHAIN_ENTER();
+    LAUNDER(part); LAUNDER(part_b);
     if (B.active && !B.active[r]) return;
     if (blockIdx.z) { part = part_b; out = out_b; }       // two sets of partials in one launch
     const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -851,6 +855,8 @@ k_odots2_df(OuterBatch B, int ng, const float2 *__restrict__ Vh, const float2 *_
     extern __shared__ float4 st2[];
     __shared__ float mx[2][OT / 32];
     const int r = blockIdx.y, ch = blockIdx.x / ng, sh = blockIdx.x - ch * ng;
+    CHAIN_ENTER();
+    LAUNDER(Vh); LAUNDER(Vl); LAUNDER(x1h); LAUNDER(x1l); LAUNDER(w); LAUNDER(vmax);
     if (B.active && !B.active[r]) return;
     Vh += r * B.n32; Vl += r * B.n32; x1h += r * B.n32; x1l += r * B.n32; w += r * B.n;
     part1 += ((long long)r * B.G + ch) * B.ldp; part2 += ((long long)r * B.G + ch) * B.ldp;
@@ -957,6 +963,8 @@ k_dcgs_col(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, doubl
     __shared__ double red[OG / 32];
     __shared__ double2 hj_s;
     const int r = blockIdx.x;
+    CHAIN_ENTER();
+    LAUNDER(P1); LAUNDER(hn); LAUNDER(fnorm);
     if (B.active && !B.active[r]) return;
     if (threadIdx.x == 0) vmax[(long long)r * B.ldp + j] = 0u;
     const int R = B.R;
@@ -1010,6 +1018,8 @@ k_dcgs_tent(OuterBatch B, double2 *__restrict__ H, double2 *__restrict__ g, doub
             double *__restrict__ hn_out, int *__restrict__ flag, double *__restrict__ hist, int hstride, int it) {
     __shared__ double red[OG / 32];
     const int r = blockIdx.x;
+    CHAIN_ENTER();
+    LAUNDER(npart); LAUNDER(fnorm);
     if (B.active && !B.active[r]) return;
     const int R = B.R;
     H += (long long)r * (R + 1) * R; g += (long long)r * (R + 1); Wq += (long long)r * (R + 1);
@@ -1067,6 +1077,8 @@ k_oupdate_dcgs(OuterBatch B, const float2 *__restrict__ Vh, const float2 *__rest
     __shared__ double red[OTU / 32];
     __shared__ float redm[OTU / 32];
     const int r = blockIdx.y;
+    CHAIN_ENTER();
+    LAUNDER(Vh); LAUNDER(Vl); LAUNDER(acoef); LAUNDER(bcoef); LAUNDER(invs);
     if (B.active && !B.active[r]) return;
     Vh += r * B.n32; Vl += r * B.n32; w += r * B.n; Vj += r * B.n; Dj += r * B.n;
     Vjh += r * B.n32; Vjl += r * B.n32;
@@ -1205,6 +1217,8 @@ __global__ void k_oscale(OuterBatch B, double2 *__restrict__ out, float2 *__rest
                          float2 *__restrict__ out32L, double *__restrict__ outD, const double2 *__restrict__ w,
                          const double *__restrict__ hn) {
     const int r = blockIdx.y;
+    CHAIN_ENTER();
+    LAUNDER(w); LAUNDER(hn);
     if (B.active && !B.active[r]) return;
     const double h = hn[r];
     if (!(h > 0.0)) return;
@@ -1327,8 +1341,8 @@ void launch_fill_test(long long n, unsigned long long seed, double2 *x, cudaStre
 void launch_gstencil(const Stencil &st, int N, const double2 *x, double2 *y, const double2 *f, int nrhs,
                      const int *active, cudaStream_t s) {
     const long long w = st.bc ? N + 1 : N - 1, n = w * w;
-    if (st.bc) k_gstencil<true><<<dim3(grid_for(n, 256), nrhs), 256, 0, s>>>(st, N, x, y, f, active);
-    else k_gstencil<false><<<dim3(grid_for(n, 256), nrhs), 256, 0, s>>>(st, N, x, y, f, active);
+    if (st.bc) launch_chained(k_gstencil<true>, dim3(grid_for(n, 256), nrhs), 256, 0, s, st, N, x, y, f, active);
+    else launch_chained(k_gstencil<false>, dim3(grid_for(n, 256), nrhs), 256, 0, s, st, N, x, y, f, active);
 }
 void launch_build_rhs(const Stencil &st, int N, double h, int npts, const double *pts, int nb, const double *bumps,
                       double2 *f, cudaStream_t s) {
@@ -1448,19 +1462,19 @@ cudaError_t launch_odots2_df(const OuterBatch &B0, const float2 *Vh, const float
         if (e != cudaSuccess) return e;
         set[dev][bias] = smem;
     }
-    kern[bias]<<<dim3(B.G * ng, B.nrhs), OT, smem, s>>>(B, ng, Vh, Vl, nv, x1h, x1l, w, part1, part2, vmax);
-    k_oreduce<<<dim3((nv + 7) / 8, B.nrhs, 2), 256, 0, s>>>(B, part1, nv, out1, part2, out2);
+    launch_chained(kern[bias], dim3(B.G * ng, B.nrhs), OT, smem, s, B, ng, Vh, Vl, nv, x1h, x1l, w, part1, part2, vmax);
+    launch_chained(k_oreduce, dim3((nv + 7) / 8, B.nrhs, 2), 256, 0, s, B, part1, nv, out1, part2, out2);
     return cudaGetLastError();
 }
 void launch_dcgs_col(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                      const double2 *P1, double2 *P2, const double *hn, double *invs, const double *fnorm,
                      double *hist, int hstride, int it, int *err, unsigned *vmax, cudaStream_t s) {
-    k_dcgs_col<<<B.nrhs, OG, 0, s>>>(B, H, cs, sn, g, Wq, j, P1, P2, hn, invs, fnorm, hist, hstride, it, err, vmax);
+    launch_chained(k_dcgs_col, B.nrhs, OG, 0, s, B, H, cs, sn, g, Wq, j, P1, P2, hn, invs, fnorm, hist, hstride, it, err, vmax);
 }
 void launch_dcgs_tent(const OuterBatch &B, double2 *H, double2 *g, double2 *Wq, int j, const double *npart, int gp,
                       const double *fnorm, double tol, double *hn_out, int *flag, double *hist, int hstride, int it,
                       cudaStream_t s) {
-    k_dcgs_tent<<<B.nrhs, OG, 0, s>>>(B, H, g, Wq, j, npart, gp, fnorm, tol, hn_out, flag, hist, hstride, it);
+    launch_chained(k_dcgs_tent, B.nrhs, OG, 0, s, B, H, g, Wq, j, npart, gp, fnorm, tol, hn_out, flag, hist, hstride, it);
 }
 void launch_dcgs_close(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                        const int *close, cudaStream_t s) {
@@ -1472,15 +1486,15 @@ void launch_oupdate_dcgs(const OuterBatch &B, const float2 *Vh, const float2 *Vl
     const size_t sm = (size_t)j * (sizeof(float4) + sizeof(float2));
     const int k = dcgs_groups(B.n, j), grid = oupdate_dcgs_grid(B.n, j);
     if (k == 4)
-        k_oupdate_dcgs<4><<<dim3(grid, B.nrhs), OTU, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+        launch_chained(k_oupdate_dcgs<4>, dim3(grid, B.nrhs), OTU, sm, s, B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
                                                               part_norm, vmax);
     else if (k == 2)
-        k_oupdate_dcgs<2><<<dim3(grid, B.nrhs), OTU, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+        launch_chained(k_oupdate_dcgs<2>, dim3(grid, B.nrhs), OTU, sm, s, B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
                                                               part_norm, vmax);
     else {
         int t = 0, g = 0;
         pair_plan(k_oupdate_dcgs<1>, plan_dcgs, B.n, t, g);
-        k_oupdate_dcgs<1><<<dim3(g, B.nrhs), t, sm, s>>>(B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
+        launch_chained(k_oupdate_dcgs<1>, dim3(g, B.nrhs), t, sm, s, B, Vh, Vl, j, corr, Vj, Dj, Vjh, Vjl, acoef, bcoef, invs, w,
                                                          part_norm, vmax);
     }
 }
@@ -1494,7 +1508,7 @@ void launch_onorm(const OuterBatch &B, const double2 *x, double *part, cudaStrea
     k_onorm<<<dim3(B.G, B.nrhs), OT, 0, s>>>(B, x, part);
 }
 void launch_oreduce(const OuterBatch &B, const double2 *part, int nv, double2 *out, cudaStream_t s) {
-    k_oreduce<<<dim3((nv + 7) / 8, B.nrhs), 256, 0, s>>>(B, part, nv, out, nullptr, nullptr);
+    launch_chained(k_oreduce, dim3((nv + 7) / 8, B.nrhs), 256, 0, s, B, part, nv, out, nullptr, nullptr);
 }
 void launch_ogivens(const OuterBatch &B, double2 *H, double *cs, double2 *sn, double2 *g, double2 *Wq, int j,
                     const double2 *h1, const double2 *h2, const double *npart, const double *fnorm,
@@ -1509,7 +1523,7 @@ void launch_orotate(const OuterBatch &B, double2 *H, const double *cs, const dou
 }
 void launch_oscale(const OuterBatch &B, double2 *out, float2 *out32, float2 *out32L, double *outD,
                    const double2 *w, const double *hn, cudaStream_t s) {
-    k_oscale<<<dim3(grid_for(B.n, 256), B.nrhs), 256, 0, s>>>(B, out, out32, out32L, outD, w, hn);
+    launch_chained(k_oscale, dim3(grid_for(B.n, 256), B.nrhs), 256, 0, s, B, out, out32, out32L, outD, w, hn);
 }
 void launch_otrisolve(const OuterBatch &B, const double2 *H, const double2 *g, const int *kcols, int kmax,
                       double2 *y, cudaStream_t s) {
