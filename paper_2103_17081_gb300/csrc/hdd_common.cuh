@@ -68,10 +68,30 @@ __device__ __forceinline__ void df_add(float &sh, float &sl, float bh, float bl)
     sl = __fadd_rn(sl, __fadd_rn(err, bl));
 }
 
+// double -> R and R -> double.  A float conversion runs on the FP64 pipe, which holds a scheduler for
+// 64 clocks a warp whatever the operands; with FP32 vectors it is done on the bits instead (round to
+// nearest even; values that are no normal floats take the conversion).
+__device__ __forceinline__ float narrow_f(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 254u) {                                // a normal float, up to rounding to infinity
+        const unsigned b = (hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+        return __uint_as_float(b + (((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    return (float)x;
+}
+__device__ __forceinline__ double widen_f(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    return (double)x;
+}
+
 // the FP64 value x as a pair (hi, lo) with hi + lo = x to about 2^-48 relative
 __device__ __forceinline__ float2 df_split(double x) {
-    const float h = (float)x;
-    return make_float2(h, (float)(x - (double)h));
+    const float h = narrow_f(x);
+    return make_float2(h, narrow_f(x - widen_f(h)));
 }
 
 template <typename R> struct C2;
@@ -104,8 +124,53 @@ template <typename R> __device__ __forceinline__ void caxpy(c2<R> &acc, c2<R> h,
     acc.y = fma(h.x, v.y, acc.y); acc.y = fma(h.y, v.x, acc.y);
 }
 
+template <typename R> __device__ __forceinline__ c2<R> narrow_c(double2 v);
+template <> __device__ __forceinline__ c2<float> narrow_c<float>(double2 v) { return mk<float>(narrow_f(v.x), narrow_f(v.y)); }
+template <> __device__ __forceinline__ c2<double> narrow_c<double>(double2 v) { return v; }
+__device__ __forceinline__ double2 widen_c(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
+__device__ __forceinline__ double2 widen_c(double2 v) { return v; }
+
 template <typename R> __device__ __forceinline__ R shfl_xor(R v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 template <typename R> __device__ __forceinline__ R shfl(R v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
+// sqrt(x² + y²) without overflow or underflow: for doubles scaled by a power of two (some 15 FP64
+// instructions, at 64 clocks each, where hypot takes several times that), hypot's own rounding kept
+// for what the scale does not reach
+__device__ __forceinline__ float hyp(float x, float y) { return hypotf(x, y); }
+__device__ __forceinline__ double hyp(double x, double y) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu, ey = ((unsigned)__double2hiint(y) >> 20) & 0x7ffu;
+    const unsigned e = ex > ey ? ex : ey;
+    if (e - 64u > 1900u) return hypot(x, y);
+    const double sc = __hiloint2double((int)((2046u - e) << 20), 0);
+    const double xs = x * sc, ys = y * sc;
+    return sqrt(fma(xs, xs, ys * ys)) * __hiloint2double((int)(e << 20), 0);
+}
+
+// Givens rotation of (x, b) with b >= 0 real, by a whole warp: c = |x|/t, s = (x/|x|)·b/t,
+// r = (x/|x|)·t, t = sqrt(|x|² + b²); the four divisions in four lanes at once.
+template <typename R>
+__device__ __forceinline__ void rotation_warp(c2<R> x, R b, R &c, c2<R> &s, c2<R> &r) {
+    const int lane = threadIdx.x & 31;
+    c = 1;
+    s = mk<R>(0, 0);
+    r = x;
+    const R aa = hyp(x.x, x.y);
+    if (b == (R)0) return;
+    if (aa == (R)0) {
+        c = 0;
+        s = mk<R>(1, 0);
+        r = mk<R>(b, 0);
+        return;
+    }
+    const R t = hyp(aa, b);
+    const bool second = (lane & 2) != 0, im = (lane & 1) != 0;
+    const R q = (second ? (im ? b : aa) : (im ? x.y : x.x)) / (second ? t : aa);
+    const c2<R> ph = mk<R>(shfl(q, 0), shfl(q, 1));
+    const R bt = shfl(q, 3);
+    c = shfl(q, 2);
+    s = mk<R>(ph.x * bt, ph.y * bt);
+    r = mk<R>(ph.x * t, ph.y * t);
+}
 
 // Launches that follow one another on a stream: a kernel launched by launch_chained may start while
 // the one before it still runs, does what needs no result of it (tables that set-up wrote), and waits

@@ -5,6 +5,8 @@
 //
 // Layouts: fine vectors complex128, (N-1)² interior nodes, x fastest, nrhs consecutive vectors
 // (stride ldv); coarse vectors m² entries (m = N/c - 1), x fastest, stride ldh.
+#include <algorithm>
+
 #include "hdd_common.cuh"
 
 namespace hdd {
@@ -18,77 +20,97 @@ __device__ __forceinline__ int hat_num(int dx, int dy, int c, int diag) {
     return mx < c ? c - mx : 0;
 }
 
+// The weights num / c as a table in shared memory (c below CG_TAB; a division costs some 15 FP64
+// instructions at 64 clocks a warp, the rest of a node's work 8 to 14)
+constexpr int CG_T = 128, CG_TAB = 256;
+__device__ __forceinline__ void hat_table(double *tab, int c) {
+    if (c < CG_TAB)
+        for (int q = threadIdx.x; q <= c; q += CG_T) tab[q] = (double)q / c;
+    __syncthreads();
+}
+__device__ __forceinline__ double hat_weight(const double *tab, int num, int c) {
+    return c < CG_TAB ? tab[num] : (double)num / c;
+}
+
 // vH = Pᵀ v: a coarse node gathers its (2c-1)² fine neighbours weighted by its hat function
-// (all interior nodes for 1 <= I, J <= m), rows of the stencil in increasing fine index.
+// (all interior nodes for 1 <= I, J <= m), rows of the stencil in increasing fine index.  A CTA takes
+// rpb rows of CG_T nodes.  Bound by the FP64 pipe (14 instructions a node at c = 2); N = 640, c = 2:
+// 19 us with a division per weight and 64-bit index divisions, 10 now.
 template <typename T>
-__global__ void k_cg_restrict(CGrid g, const double2 *__restrict__ v, c2<T> *__restrict__ vH,
-                              long long ldv, long long ldh, const int *__restrict__ active) {
+__global__ void __launch_bounds__(CG_T)
+k_cg_restrict(CGrid g, const double2 *__restrict__ v, c2<T> *__restrict__ vH, long long ldv, long long ldh,
+              const int *__restrict__ active, int rpb) {
+    __shared__ double tab[CG_TAB];
+    const int m = g.m, c = g.c, w = g.N - 1;
+    hat_table(tab, c);
     CHAIN_ENTER();
     LAUNDER(v); LAUNDER(active);
-    if (active && !active[blockIdx.y]) return;
-    v += blockIdx.y * ldv;
-    vH += blockIdx.y * ldh;
-    const int m = g.m, c = g.c, w = g.N - 1;
-    const long long mm = (long long)m * m;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < mm;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int I = (int)(e % m) + 1, J = (int)(e / m) + 1;
-        double sx = 0.0, sy = 0.0;
-        for (int dy = 1 - c; dy < c; dy++) {
-            const double2 *row = v + (long long)(c * J + dy - 1) * w + (c * I - 1);
-            for (int dx = 1 - c; dx < c; dx++) {
-                const int num = hat_num(dx, dy, c, g.diag);
-                if (num == 0) continue;
-                const double wt = (double)num / c;
-                const double2 a = row[dx];
-                sx = fma(wt, a.x, sx);
-                sy = fma(wt, a.y, sy);
+    if (active && !active[blockIdx.z]) return;
+    v += blockIdx.z * ldv;
+    vH += blockIdx.z * ldh;
+    const int I = blockIdx.x * CG_T + threadIdx.x + 1;
+    if (I > m) return;
+    for (long long j0 = (long long)blockIdx.y * rpb; j0 < m; j0 += (long long)gridDim.y * rpb)
+        for (int J = (int)j0 + 1; J <= min(m, (int)j0 + rpb); J++) {
+            double sx = 0.0, sy = 0.0;
+            for (int dy = 1 - c; dy < c; dy++) {
+                const double2 *row = v + (long long)(c * J + dy - 1) * w + (c * I - 1);
+#pragma unroll 4
+                for (int dx = 1 - c; dx < c; dx++) {
+                    const int num = hat_num(dx, dy, c, g.diag);
+                    if (num == 0) continue;
+                    const double wt = hat_weight(tab, num, c);
+                    const double2 a = row[dx];
+                    sx = fma(wt, a.x, sx);
+                    sy = fma(wt, a.y, sy);
+                }
             }
+            vH[(I - 1) + (long long)(J - 1) * m] = narrow_c<T>(make_double2(sx, sy));
         }
-        vH[e] = mk<T>((T)sx, (T)sy);
-    }
 }
 
 // z = P xH (accumulate = 0) or z += P xH (1): a fine node interpolates the corners of the coarse
-// cell that contains it (the corner off its triangle has weight 0; boundary corners hold 0).
+// cell that contains it (the corner off its triangle has weight 0; boundary corners hold 0).  CTAs
+// as above; N = 640, c = 2: 32 us before, 13 now.
 template <typename T>
-__global__ void k_cg_prolong(CGrid g, const c2<T> *__restrict__ xH, double2 *__restrict__ z, int accumulate,
-                             long long ldv, long long ldh, const int *__restrict__ active) {
+__global__ void __launch_bounds__(CG_T)
+k_cg_prolong(CGrid g, const c2<T> *__restrict__ xH, double2 *__restrict__ z, int accumulate, long long ldv, long long ldh,
+             const int *__restrict__ active, int rpb) {
+    __shared__ double tab[CG_TAB];
+    const int m = g.m, c = g.c, w = g.N - 1;
+    hat_table(tab, c);
+    const int i = blockIdx.x * CG_T + threadIdx.x + 1, cx0 = i / c;
     CHAIN_ENTER();
     LAUNDER(xH); LAUNDER(active);
-    if (active && !active[blockIdx.y]) return;
-    z += blockIdx.y * ldv;
-    xH += blockIdx.y * ldh;
-    const int m = g.m, c = g.c, w = g.N - 1;
-    const long long n = (long long)w * w;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(e % w) + 1, j = (int)(e / w) + 1;
-        const int cx0 = i / c, cy0 = j / c;
-        double sx = 0.0, sy = 0.0;
-        for (int b = 0; b < 2; b++) {
-            const int J = cy0 + b;
-            if (J < 1 || J > m) continue;
-            for (int a = 0; a < 2; a++) {
-                const int I = cx0 + a;
-                if (I < 1 || I > m) continue;
-                const int num = hat_num(i - c * I, j - c * J, c, g.diag);
-                if (num == 0) continue;
-                const double wt = (double)num / c;
-                const c2<T> u = xH[(I - 1) + (long long)(J - 1) * m];
-                sx = fma(wt, (double)u.x, sx);
-                sy = fma(wt, (double)u.y, sy);
+    if (active && !active[blockIdx.z]) return;
+    z += blockIdx.z * ldv;
+    xH += blockIdx.z * ldh;
+    if (i > w) return;
+    for (long long j0 = (long long)blockIdx.y * rpb; j0 < w; j0 += (long long)gridDim.y * rpb)
+        for (int j = (int)j0 + 1; j <= min(w, (int)j0 + rpb); j++) {
+            const int cy0 = j / c;
+            const long long e = (i - 1) + (long long)(j - 1) * w;
+            double2 o = make_double2(0.0, 0.0);
+            if (accumulate) o = z[e];
+            double sx = 0.0, sy = 0.0;
+#pragma unroll
+            for (int b = 0; b < 2; b++) {
+                const int J = cy0 + b;
+                if (J < 1 || J > m) continue;
+#pragma unroll
+                for (int a = 0; a < 2; a++) {
+                    const int I = cx0 + a;
+                    if (I < 1 || I > m) continue;
+                    const int num = hat_num(i - c * I, j - c * J, c, g.diag);
+                    if (num == 0) continue;
+                    const double wt = hat_weight(tab, num, c);
+                    const double2 u = widen_c(xH[(I - 1) + (long long)(J - 1) * m]);
+                    sx = fma(wt, u.x, sx);
+                    sy = fma(wt, u.y, sy);
+                }
             }
+            z[e] = accumulate ? make_double2(o.x + sx, o.y + sy) : make_double2(sx, sy);
         }
-        if (accumulate) {
-            double2 o = z[e];
-            o.x += sx;
-            o.y += sy;
-            z[e] = o;
-        } else {
-            z[e] = make_double2(sx, sy);
-        }
-    }
 }
 
 // One pass of the separable sine transform: out = (S · in)ᵀ, optionally scaled entrywise by
@@ -207,13 +229,16 @@ static int cg_grid(long long n) {
 template <typename T>
 void launch_cg_restrict(const CGrid &g, const double2 *v, c2<T> *vH, int nrhs, long long ldv, long long ldh,
                         const int *active, cudaStream_t s) {
-    launch_chained(k_cg_restrict<T>, dim3(cg_grid((long long)g.m * g.m), nrhs), 256, 0, s, g, v, vH, ldv, ldh, active);
+    const int rpb = 2;
+    launch_chained(k_cg_restrict<T>, dim3((g.m + CG_T - 1) / CG_T, std::min((g.m + rpb - 1) / rpb, 65535), nrhs), CG_T, 0, s, g,
+                   v, vH, ldv, ldh, active, rpb);
 }
 template <typename T>
 void launch_cg_prolong(const CGrid &g, const c2<T> *xH, double2 *z, int accumulate, int nrhs, long long ldv,
                        long long ldh, const int *active, cudaStream_t s) {
-    const long long n = (long long)(g.N - 1) * (g.N - 1);
-    launch_chained(k_cg_prolong<T>, dim3(cg_grid(n), nrhs), 256, 0, s, g, xH, z, accumulate, ldv, ldh, active);
+    const int w = g.N - 1, rpb = 4;
+    launch_chained(k_cg_prolong<T>, dim3((w + CG_T - 1) / CG_T, std::min((w + rpb - 1) / rpb, 65535), nrhs), CG_T, 0, s, g, xH,
+                   z, accumulate, ldv, ldh, active, rpb);
 }
 template <typename T>
 void launch_dst_pass(int m, const T *S, const T *Dinv, const c2<T> *in, c2<T> *out, int nrhs, long long ldh,

@@ -23,31 +23,6 @@ __device__ __forceinline__ float zw_f(int t) {
 }
 template <typename R> __device__ __forceinline__ R zw(int t) { return (R)zw_f(t); }
 
-// double -> R and R -> double.  A float conversion runs on the FP64 pipe, which holds a scheduler for
-// 64 clocks a warp whatever the operands; with FP32 vectors it is done on the bits instead (round to
-// nearest even; values that are no normal floats take the conversion).
-__device__ __forceinline__ float narrow_f(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned e = (hi >> 20) & 0x7ffu;
-    if (e - 897u < 254u) {                                // a normal float, up to rounding to infinity
-        const unsigned b = (hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
-        return __uint_as_float(b + (((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29));
-    }
-    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
-    return (float)x;
-}
-__device__ __forceinline__ double widen_f(float x) {
-    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
-    if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
-    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
-    return (double)x;
-}
-template <typename R> __device__ __forceinline__ c2<R> narrow_c(double2 v);
-template <> __device__ __forceinline__ c2<float> narrow_c<float>(double2 v) { return mk<float>(narrow_f(v.x), narrow_f(v.y)); }
-template <> __device__ __forceinline__ c2<double> narrow_c<double>(double2 v) { return v; }
-__device__ __forceinline__ double2 widen_c(float2 v) { return make_double2(widen_f(v.x), widen_f(v.y)); }
-__device__ __forceinline__ double2 widen_c(double2 v) { return v; }
-
 template <typename R> __device__ __forceinline__ c2<R> load_c(const c2<R> *p) { return *p; }
 
 // Row of a boundary node (impedance condition): Σ_q cf[q] v_q over the 7 stencil slots.
@@ -636,11 +611,38 @@ k_init_cycle(LocalArgs<R> a, InnerState<R> S, int restart, c2<R> *__restrict__ v
     publish(pr, 0, done ? 0 : 1);
 }
 
-// y = H(0:k,0:k)⁻¹ g(0:k) for task t, by one thread (k <= restart <= 64).
+// y = H(0:k,0:k)⁻¹ g(0:k) for task t (k <= restart <= 64), by one warp.  Up to 16 columns: H through
+// shared memory in one round of loads, lane 2r + c keeps component c of row r, and a step back
+// substitutes one entry for all rows above at once (one thread with its loads in a chain took 5 us).
+constexpr int SMALL_K = 16;
 template <typename R>
 __device__ void solve_small(const InnerState<R> &S, int restart, int t, int k, c2<R> *y) {
+    __shared__ c2<R> hs[SMALL_K * SMALL_K];
     const c2<R> *H = S.H + (long long)t * (restart + 1) * restart;
     const c2<R> *g = S.g + (long long)t * (restart + 1);
+    const int lane = threadIdx.x & 31;
+    if (k <= SMALL_K) {
+        const int row = lane >> 1, im = lane & 1;
+        R acc = row < k ? reinterpret_cast<const R *>(g)[lane] : (R)0;
+        for (int e = lane; e < k * SMALL_K; e += 32) {
+            const int l = e / SMALL_K, r = e % SMALL_K;
+            if (r <= l) hs[e] = H[(long long)l * (restart + 1) + r];
+        }
+        __syncwarp();
+        for (int r = k - 1; r >= 0; r--) {
+            const c2<R> d = hs[r * SMALL_K + r];
+            const R sx = shfl(acc, 2 * r), sy = shfl(acc, 2 * r + 1), den = d.x * d.x + d.y * d.y;
+            const R v = (im ? sy * d.x - sx * d.y : sx * d.x + sy * d.y) / den;
+            const R yx = shfl(v, 0), yy = shfl(v, 1);
+            if (lane == 0) y[r] = mk<R>(yx, yy);
+            if (row < r) {
+                const c2<R> h = hs[r * SMALL_K + row];
+                acc = fma(-h.x, im ? yy : yx, fma(im ? -h.y : h.y, im ? yx : yy, acc));
+            }
+        }
+        return;
+    }
+    if (lane) return;
     for (int r = k - 1; r >= 0; r--) {
         c2<R> sacc = g[r];
         for (int l = r + 1; l < k; l++) sacc = csub<R>(sacc, cmul<R>(H[(long long)l * (restart + 1) + r], y[l]));
@@ -657,6 +659,7 @@ template <typename R>
 __global__ void __launch_bounds__(LOCAL_THREADS)
 k_coarse_combine(LocalArgs<R> a, InnerState<R> S, int restart, const double2 *__restrict__ sbuf,
                  double2 *__restrict__ sc, const int *__restrict__ flag) {
+    __shared__ double2 yd[MAX_RESTART];
     __shared__ c2<R> y[MAX_RESTART];
     const Tile tl = a.ctiles[blockIdx.x];
     const Task T = a.tasks[tl.task];
@@ -664,16 +667,19 @@ k_coarse_combine(LocalArgs<R> a, InnerState<R> S, int restart, const double2 *__
     LAUNDER(sbuf); LAUNDER(flag);
     if (flag && !flag[tl.task]) return;
     const int k = S.kcols[tl.task];
-    if (threadIdx.x == 0) solve_small<R>(S, restart, tl.task, k, y);
+    if (threadIdx.x < 32) solve_small<R>(S, restart, tl.task, k, y);
+    __syncthreads();
+    if (threadIdx.x < k) yd[threadIdx.x] = widen_c(y[threadIdx.x]);
     __syncthreads();
     for (int e = threadIdx.x; e < tl.nr * T.mx; e += blockDim.x) {
         const long long idx = T.coff + (long long)tl.r0 * T.mx + e;
         double2 acc = sbuf[idx];
+#pragma unroll 4
         for (int l = 0; l < k; l++) {
             const double2 sv = sbuf[(long long)(l + 1) * a.ldc + idx];
-            const double yr = (double)y[l].x, yi = (double)y[l].y;
-            acc.x -= yr * sv.x - yi * sv.y;
-            acc.y -= yr * sv.y + yi * sv.x;
+            const double yr = yd[l].x, yi = yd[l].y;
+            acc.x = fma(-yr, sv.x, fma(yi, sv.y, acc.x));
+            acc.y = fma(-yr, sv.y, fma(-yi, sv.x, acc.y));
         }
         sc[idx] = acc;
     }
@@ -701,12 +707,10 @@ k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restr
     if (!flag[t]) return;
     const int k = S.kcols[t];
     const bool again = !S.conv[t] && S.its[t] < maxit;
-    if (threadIdx.x == 0) {
-        solve_small<R>(S, restart, t, k, y);
-        if (blockIdx.x == T.tile0) {
-            rs_out[t] = again ? 1 : 0;
-            its_out[t] = again ? ~S.its[t] : S.its[t];    // (the host's pinned memory)
-        }
+    if (threadIdx.x < 32) solve_small<R>(S, restart, t, k, y);
+    if (threadIdx.x == 32 && blockIdx.x == T.tile0) {
+        rs_out[t] = again ? 1 : 0;
+        its_out[t] = again ? ~S.its[t] : S.its[t];        // (the host's pinned memory)
     }
     const int maxc = prolong_max_cy(tl.nr);
     c2<R> *sc = reinterpret_cast<c2<R> *>(smem_raw);
@@ -721,6 +725,7 @@ k_finish(LocalArgs<R> a, InnerState<R> S, int restart, int first, c2<R> *__restr
         const bool own = gx >= T.ox0 && gx <= T.ox1 && gy >= T.oy0 && gy <= T.oy1;
         if (!again && !own) continue;
         c2<R> x = first ? mk<R>(0, 0) : u[base + e];
+#pragma unroll 4
         for (int l = 0; l < k; l++) caxpy<R>(x, y[l], V[(long long)l * a.ld + base + e]);
         if (again) {
             u[base + e] = x;
@@ -810,19 +815,6 @@ size_t step_smem_bytes(int max_nx, int max_ny, int C, int bytes_per_c) {
     const size_t a = (px > w ? px : w) + (size_t)nF * (max_nx + 3);
     const size_t e = (size_t)(nVz + nFz) * (max_nx + 3);
     return (a > e ? a : e) * bytes_per_c;
-}
-
-// sqrt(x² + y²) without overflow or underflow: for doubles scaled by a power of two (some 15 FP64
-// instructions, at 64 clocks each, where hypot takes several times that), hypot's own rounding kept
-// for what the scale does not reach
-__device__ __forceinline__ float hyp(float x, float y) { return hypotf(x, y); }
-__device__ __forceinline__ double hyp(double x, double y) {
-    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu, ey = ((unsigned)__double2hiint(y) >> 20) & 0x7ffu;
-    const unsigned e = ex > ey ? ex : ey;
-    if (e - 64u > 1900u) return hypot(x, y);
-    const double sc = __hiloint2double((int)((2046u - e) << 20), 0);
-    const double xs = x * sc, ys = y * sc;
-    return sqrt(fma(xs, xs, ys * ys)) * __hiloint2double((int)(e << 20), 0);
 }
 
 // Bound: with FP64 vectors by the FP64 pipe (64 clocks a warp instruction, whatever its lanes do),
@@ -1067,25 +1059,9 @@ k_arnoldi_step(StepArgs<R> a) {
             if (lane < 2) reinterpret_cast<R *>(hcs)[2 * l + lane] = o;
             x = mk<R>(shfl(o, 2), shfl(o, 3));
         }
-        // the new rotation of (x, ||w||): c = |x|/t, s = (x/|x|)·||w||/t, r = (x/|x|)·t
-        R c = 1;
-        c2<R> sv = mk<R>(0, 0), rr = x;
-        const R aa = hyp(x.x, x.y), bb = hn;
-        if (bb != (R)0) {
-            if (aa == (R)0) {
-                c = 0;
-                sv = mk<R>(1, 0);
-                rr = mk<R>(bb, 0);
-            } else {
-                const R tt = hyp(aa, bb);
-                const R qv = (second ? (im ? bb : aa) : (im ? x.y : x.x)) / (second ? tt : aa);
-                const c2<R> ph = mk<R>(shfl(qv, 0), shfl(qv, 1));
-                const R cb = shfl(qv, 3);
-                c = shfl(qv, 2);
-                sv = mk<R>(ph.x * cb, ph.y * cb);
-                rr = mk<R>(ph.x * tt, ph.y * tt);
-            }
-        }
+        R c;
+        c2<R> sv, rr;
+        rotation_warp<R>(x, hn, c, sv, rr);
         const c2<R> gi = g_s;
         const c2<R> gn = mk<R>(-(sv.x * gi.x + sv.y * gi.y), -(sv.x * gi.y - sv.y * gi.x));   // -conj(s) g_i
         const int its = its_s + 1;

@@ -608,18 +608,6 @@ __global__ void k_oreduce(OuterBatch B, const double2 *__restrict__ part, int nv
     if (lane == 0) out[(long long)r * B.ldp + l] = s;
 }
 
-__device__ void zgivens(double2 a, double2 b, double &c, double2 &s, double2 &r) {
-    double aa = hypot(a.x, a.y), bb = hypot(b.x, b.y);
-    if (bb == 0.0) { c = 1.0; s = make_double2(0.0, 0.0); r = a; return; }
-    if (aa == 0.0) { c = 0.0; s = make_double2(b.x / bb, -b.y / bb); r = make_double2(bb, 0.0); return; }
-    double t = hypot(aa, bb);
-    double2 ph = make_double2(a.x / aa, a.y / aa);
-    c = aa / t;
-    double2 cb = make_double2(b.x / t, -b.y / t);
-    s = cmul<double>(ph, cb);
-    r = make_double2(ph.x * t, ph.y * t);
-}
-
 // Outer Arnoldi column j of every active RHS (one CTA of OG threads each).  H keeps the
 // unrotated columns h = h1 + h2 (CGS2) with h_{j+1,j} = sqrt(Σ norm partials) below them; the
 // rotated entry that rotation j needs is formed without the sequential chain of the j earlier
@@ -628,13 +616,41 @@ __device__ void zgivens(double2 a, double2 b, double &c, double2 &s, double2 &r)
 // forms the triangular factor at the end of a cycle.  Then the g update; flag[r] = 1 while
 // |g_{j+1}| > tol·||f_r|| and h_{j+1,j} > 0; hist[r·hstride + it] records |g_{j+1}|/||f_r||.
 constexpr int OG = 128;
+// Eight sums over a CTA of OG threads, to every thread of warp 0: by halves across a warp's lanes,
+// then the four warps' parts side by side in one warp (FP64 additions cost 64 clocks a warp whatever
+// its lanes do: 11 instead of 9 for each sum).
+__device__ __forceinline__ void og_sums(double (&v)[8], double (*red)[8]) {
+    static_assert(OG == 128, "lane 4·value + warp");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int half = 4; half > 0; half >>= 1) {
+        const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+        for (int q = 0; q < half; q++) {
+            const double x = shfl_xor(up ? v[q] : v[q + half], 4 * half);
+            v[q] = (up ? v[q + half] : v[q]) + x;
+        }
+    }
+    v[0] += shfl_xor(v[0], 2);
+    v[0] += shfl_xor(v[0], 1);
+    if ((lane & 3) == 0) red[warp][lane >> 2] = v[0];
+    __syncthreads();
+    if (warp == 0) {
+        double x = red[lane & 3][lane >> 2];
+        x += shfl_xor(x, 1);
+        x += shfl_xor(x, 2);
+#pragma unroll
+        for (int q = 0; q < 8; q++) v[q] = shfl(x, 4 * q);
+    }
+}
+
 __global__ void __launch_bounds__(OG)
 k_ogivens(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double2 *__restrict__ sn,
           double2 *__restrict__ g, double2 *__restrict__ Wq, int j, const double2 *__restrict__ h1,
           const double2 *__restrict__ h2, const double *__restrict__ npart, const double *__restrict__ fnorm,
           double tol, double *__restrict__ hn_out, int *__restrict__ flag, double *__restrict__ hist,
           int hstride, int it) {
-    __shared__ double red[OG / 32], redx[OG / 32], redy[OG / 32];
+    __shared__ double red[OG / 32][8];
     __shared__ double c_s;
     __shared__ double2 s_s;
     const int r = blockIdx.x;
@@ -644,37 +660,33 @@ k_ogivens(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double
     g += (long long)r * (R + 1); Wq += (long long)r * (R + 1);
     h1 += (long long)r * B.ldp; h2 += (long long)r * B.ldp; npart += (long long)r * B.G;
     double2 *hc = H + (long long)j * (R + 1);
-    double s2 = 0.0;
-    for (int q = tid; q < B.G; q += OG) s2 += npart[q];
-    double dx = 0.0, dy = 0.0;
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};          // Σ norm partials, W·h
+    for (int q = tid; q < B.G; q += OG) v[0] += npart[q];
     for (int l = tid; l <= j; l += OG) {
         const double2 hv = make_double2(h1[l].x + h2[l].x, h1[l].y + h2[l].y);
         hc[l] = hv;
         const double2 wl = Wq[l];
-        dx = fma(wl.x, hv.x, fma(-wl.y, hv.y, dx));
-        dy = fma(wl.x, hv.y, fma(wl.y, hv.x, dy));
+        v[1] = fma(wl.x, hv.x, fma(-wl.y, hv.y, v[1]));
+        v[2] = fma(wl.x, hv.y, fma(wl.y, hv.x, v[2]));
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s2 += shfl_xor(s2, o); dx += shfl_xor(dx, o); dy += shfl_xor(dy, o);
-    }
-    if (lane == 0) { red[warp] = s2; redx[warp] = dx; redy[warp] = dy; }
-    __syncthreads();
-    if (tid == 0) {
-        double a = 0.0, bx = 0.0, by = 0.0;
-        for (int q = 0; q < OG / 32; q++) { a += red[q]; bx += redx[q]; by += redy[q]; }
-        const double hn = sqrt(a);
-        hc[j + 1] = make_double2(hn, 0.0);
+    og_sums(v, red);
+    if (warp == 0) {
+        const double hn = sqrt(v[0]);
         double c; double2 sr, rr;
-        zgivens(make_double2(bx, by), make_double2(hn, 0.0), c, sr, rr);
-        cs[j] = c; sn[j] = sr;
-        c_s = c; s_s = sr;
+        rotation_warp<double>(make_double2(v[1], v[2]), hn, c, sr, rr);
         const double2 gj = g[j];
-        g[j + 1] = make_double2(-(sr.x * gj.x + sr.y * gj.y), -(sr.x * gj.y - sr.y * gj.x));
-        g[j] = make_double2(c * gj.x, c * gj.y);
-        const double res = hypot(g[j + 1].x, g[j + 1].y);
-        hn_out[r] = hn;
-        hist[(long long)r * hstride + it] = res / fnorm[r];
-        flag[r] = (res > tol * fnorm[r] && hn > 0.0) ? 1 : 0;
+        const double2 g1 = make_double2(-(sr.x * gj.x + sr.y * gj.y), -(sr.x * gj.y - sr.y * gj.x));
+        const double res = hyp(g1.x, g1.y);
+        if (lane == 0) {
+            hc[j + 1] = make_double2(hn, 0.0);
+            cs[j] = c; sn[j] = sr;
+            c_s = c; s_s = sr;
+            g[j + 1] = g1;
+            g[j] = make_double2(c * gj.x, c * gj.y);
+            hn_out[r] = hn;
+            hist[(long long)r * hstride + it] = res / fnorm[r];
+            flag[r] = (res > tol * fnorm[r] && hn > 0.0) ? 1 : 0;
+        }
     }
     __syncthreads();
     const double c = c_s;
@@ -839,7 +851,7 @@ __device__ __forceinline__ void warp_dots2_df(const float2 *__restrict__ Vh, con
         }
         const int v = lane >> 4;
         if ((lane & 3) == 0 && l + v < nv)
-            reinterpret_cast<double *>((lane & 8 ? part2 : part1) + l + v)[(lane >> 2) & 1] = (double)h[0] + (double)q[0];
+            reinterpret_cast<double *>((lane & 8 ? part2 : part1) + l + v)[(lane >> 2) & 1] = widen_f(h[0]) + widen_f(q[0]);
     }
 }
 
@@ -869,10 +881,10 @@ k_odots2_df(OuterBatch B, int ng, const float2 *__restrict__ Vh, const float2 *_
         const float2 h = x1h[b + i], q = x1l[b + i];
         s1[i] = make_float4(h.x, q.x, h.y, q.y);
         const double2 x = w[b + i];
-        const float rh = (float)x.x, ih = (float)x.y;
-        s2[i] = make_float4(rh, (float)(x.x - (double)rh), ih, (float)(x.y - (double)ih));
+        const float2 re = df_split(x.x), im = df_split(x.y);
+        s2[i] = make_float4(re.x, re.y, im.x, im.y);
         m1 = fmaxf(m1, fmaxf(fabsf(h.x), fabsf(h.y)));
-        m2 = fmaxf(m2, fmaxf(fabsf(rh), fabsf(ih)));
+        m2 = fmaxf(m2, fmaxf(fabsf(re.x), fabsf(im.x)));
     }
     float xm1 = 0.f, xm2 = 0.f;
     if (BIAS) {
@@ -893,60 +905,6 @@ k_odots2_df(OuterBatch B, int ng, const float2 *__restrict__ Vh, const float2 *_
                         sh * (OT / 32) + (int)(threadIdx.x >> 5), ng * (OT / 32));
 }
 
-// Block reductions of the small per-RHS kernels (OG threads)
-__device__ __forceinline__ double og_sum(double v, double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int q = 0; q < OG / 32; q++) s += red[q];
-    return s;
-}
-
-// Rotation j of one RHS from the unrotated column hc (rows 0..j) and its subdiagonal hn: the
-// rotated entry (Q_jᵀ h)_j = W_j · h, then cs, sn, g and W_{j+1} (commit) or only the residual
-// estimate |g_{j+1}| (commit == false).  Returns |g_{j+1}| to every thread.
-__device__ double givens_step(const double2 *__restrict__ hc, double hn, int j, double *cs, double2 *sn,
-                              double2 *g, double2 *Wq, bool commit, double *red) {
-    __shared__ double c_s, res_s;
-    __shared__ double2 s_s;
-    double dx = 0.0, dy = 0.0;
-    for (int l = threadIdx.x; l <= j; l += OG) {
-        const double2 hv = hc[l], wl = Wq[l];
-        dx = fma(wl.x, hv.x, fma(-wl.y, hv.y, dx));
-        dy = fma(wl.x, hv.y, fma(wl.y, hv.x, dy));
-    }
-    const double bx = og_sum(dx, red), by = og_sum(dy, red);
-    if (threadIdx.x == 0) {
-        double c; double2 sr, rr;
-        zgivens(make_double2(bx, by), make_double2(hn, 0.0), c, sr, rr);
-        const double2 gj = g[j];
-        const double2 g1 = make_double2(-(sr.x * gj.x + sr.y * gj.y), -(sr.x * gj.y - sr.y * gj.x));
-        res_s = hypot(g1.x, g1.y);
-        c_s = c; s_s = sr;
-        if (commit) {
-            cs[j] = c; sn[j] = sr;
-            g[j + 1] = g1;
-            g[j] = make_double2(c * gj.x, c * gj.y);
-        }
-    }
-    __syncthreads();
-    const double res = res_s;
-    if (commit) {
-        const double c = c_s;
-        const double2 sr = s_s;
-        for (int l = threadIdx.x; l <= j; l += OG) {             // W_{j+1} = [-conj(s_j) W_j, c_j]
-            const double2 wl = Wq[l];
-            Wq[l] = make_double2(-(sr.x * wl.x + sr.y * wl.y), -(sr.x * wl.y - sr.y * wl.x));
-        }
-        if (threadIdx.x == 0) Wq[j + 1] = make_double2(c, 0.0);
-        __syncthreads();
-    }
-    return res;
-}
-
 // Delayed CGS2 coefficients of step j for every active RHS (one CTA each).  P1 = V^H ṽ_j and
 // P2 = V^H w over slots 0..j (reduced).  For j >= 1: column j-1 is completed (h += ν_j a,
 // subdiagonal ν_j σ) and its rotation committed (hist[it-1], the final residual estimate after
@@ -954,15 +912,18 @@ __device__ double givens_step(const double2 *__restrict__ hc, double hn, int j, 
 // stored in H.  err[0] is set if σ² <= d/4 (the pending vector lost more than half of its norm
 // to the basis, or is not finite): the delayed form then does not hold.  vmax[r·ldp + j] (the
 // largest |hi part| of slot j, recorded by the update of this step) is cleared.
+// Bound by the FP64 pipe's chain in one CTA: one pass, one reduction for all five sums (W·h of the
+// completed column is formed as the column is), divisions in lanes side by side: 16 -> 10.4 us at
+// j = 100, k_dcgs_tent 13.4 -> 11.
 __global__ void __launch_bounds__(OG)
 k_dcgs_col(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double2 *__restrict__ sn,
            double2 *__restrict__ g, double2 *__restrict__ Wq, int j, const double2 *__restrict__ P1,
            double2 *__restrict__ P2, const double *__restrict__ hn, double *__restrict__ invs,
            const double *__restrict__ fnorm, double *__restrict__ hist, int hstride, int it, int *__restrict__ err,
            unsigned *__restrict__ vmax) {
-    __shared__ double red[OG / 32];
-    __shared__ double2 hj_s;
-    const int r = blockIdx.x;
+    __shared__ double red[OG / 32][8];
+    __shared__ double2 s_s;
+    const int r = blockIdx.x, lane = threadIdx.x & 31;
     CHAIN_ENTER();
     LAUNDER(P1); LAUNDER(hn); LAUNDER(fnorm);
     if (B.active && !B.active[r]) return;
@@ -972,41 +933,60 @@ k_dcgs_col(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, doubl
     g += (long long)r * (R + 1); Wq += (long long)r * (R + 1);
     P1 += (long long)r * B.ldp; P2 += (long long)r * B.ldp;
     double2 *hcol = H + (long long)j * (R + 1);
-    if (j >= 1) {
-        double q2 = 0.0, abx = 0.0, aby = 0.0;
-        for (int l = threadIdx.x; l < j; l += OG) {
-            const double2 a = P1[l], bb = P2[l];
-            q2 = fma(a.x, a.x, fma(a.y, a.y, q2));
-            abx = fma(a.x, bb.x, fma(a.y, bb.y, abx));          // conj(a)·b
-            aby = fma(a.x, bb.y, fma(-a.y, bb.x, aby));
-        }
-        const double aa = og_sum(q2, red), sx = og_sum(abx, red), sy = og_sum(aby, red);
-        const double d = P1[j].x, s2 = d - aa;
+    if (j == 0) {
+        if (threadIdx.x == 0) hcol[0] = P2[0];
+        return;
+    }
+    const double nu = hn[r];
+    double2 *hp = H + (long long)(j - 1) * (R + 1);
+    // Σ|a|², a·b, and W·h of the completed column j-1, all in one pass and one reduction
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int l = threadIdx.x; l < j; l += OG) {
+        const double2 a = P1[l], bb = P2[l], wl = Wq[l], h0 = hp[l];
+        const double2 h = make_double2(fma(nu, a.x, h0.x), fma(nu, a.y, h0.y));
+        hp[l] = h;
+        hcol[l] = bb;
+        v[0] = fma(a.x, a.x, fma(a.y, a.y, v[0]));
+        v[1] = fma(a.x, bb.x, fma(a.y, bb.y, v[1]));              // conj(a)·b
+        v[2] = fma(a.x, bb.y, fma(-a.y, bb.x, v[2]));
+        v[3] = fma(wl.x, h.x, fma(-wl.y, h.y, v[3]));
+        v[4] = fma(wl.x, h.y, fma(wl.y, h.x, v[4]));
+    }
+    og_sums(v, red);
+    double c;
+    double2 sr, rr, g1;
+    if (threadIdx.x < 32) {
+        const double d = P1[j].x, s2 = d - v[0];
         const bool ok = s2 > 0.25 * d && isfinite(s2);
         const double sig = ok ? sqrt(s2) : 1.0;
-        const double nu = hn[r];
-        double2 *hp = H + (long long)(j - 1) * (R + 1);
-        for (int l = threadIdx.x; l < j; l += OG) {
-            const double2 a = P1[l];
-            hp[l] = make_double2(fma(nu, a.x, hp[l].x), fma(nu, a.y, hp[l].y));
+        const double2 p = P2[j];
+        const double q = (lane == 0 ? p.x - v[1] : lane == 1 ? p.y - v[2] : 1.0) / sig;
+        rotation_warp<double>(make_double2(v[3], v[4]), nu * sig, c, sr, rr);
+        const double2 gj = g[j - 1];
+        g1 = make_double2(-(sr.x * gj.x + sr.y * gj.y), -(sr.x * gj.y - sr.y * gj.x));
+        if (lane < 2) {
+            reinterpret_cast<double *>(P2 + j)[lane] = q;
+            reinterpret_cast<double *>(hcol + j)[lane] = q;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        if (lane == 2) invs[r] = q;
+        if (lane == 0) {
+            s_s = sr;
             hp[j] = make_double2(nu * sig, 0.0);
-            const double2 c = P2[j];
-            hj_s = make_double2((c.x - sx) / sig, (c.y - sy) / sig);
-            invs[r] = 1.0 / sig;
             if (!ok) atomicExch(err, 1);
+            cs[j - 1] = c; sn[j - 1] = sr;
+            g[j] = g1;
+            g[j - 1] = make_double2(c * gj.x, c * gj.y);
+            Wq[j] = make_double2(c, 0.0);
         }
-        __syncthreads();
-        const double res = givens_step(hp, nu * sig, j - 1, cs, sn, g, Wq, true, red);
-        if (threadIdx.x == 0) {
-            hist[(long long)r * hstride + it - 1] = res / fnorm[r];
-            P2[j] = hj_s;
-        }
-        __syncthreads();
     }
-    for (int l = threadIdx.x; l <= j; l += OG) hcol[l] = P2[l];
+    __syncthreads();
+    sr = s_s;
+    for (int l = threadIdx.x; l < j; l += OG) {                  // W_j = [-conj(s) W_{j-1}, c]
+        const double2 wl = Wq[l];
+        Wq[l] = make_double2(-(sr.x * wl.x + sr.y * wl.y), -(sr.x * wl.y - sr.y * wl.x));
+    }
+    if (threadIdx.x == 0) hist[(long long)r * hstride + it - 1] = hyp(g1.x, g1.y) / fnorm[r];
 }
 
 // Tentative stopping test of step j: ν_{j+1} = ||w'|| (gp partials per RHS) as the subdiagonal
@@ -1016,7 +996,7 @@ __global__ void __launch_bounds__(OG)
 k_dcgs_tent(OuterBatch B, double2 *__restrict__ H, double2 *__restrict__ g, double2 *__restrict__ Wq, int j,
             const double *__restrict__ npart, int gp, const double *__restrict__ fnorm, double tol,
             double *__restrict__ hn_out, int *__restrict__ flag, double *__restrict__ hist, int hstride, int it) {
-    __shared__ double red[OG / 32];
+    __shared__ double red[OG / 32][8];
     const int r = blockIdx.x;
     CHAIN_ENTER();
     LAUNDER(npart); LAUNDER(fnorm);
@@ -1024,11 +1004,24 @@ k_dcgs_tent(OuterBatch B, double2 *__restrict__ H, double2 *__restrict__ g, doub
     const int R = B.R;
     H += (long long)r * (R + 1) * R; g += (long long)r * (R + 1); Wq += (long long)r * (R + 1);
     npart += (long long)r * gp;
-    double s = 0.0;
-    for (int q = threadIdx.x; q < gp; q += OG) s += npart[q];
-    const double nu = sqrt(og_sum(s, red));
     double2 *hcol = H + (long long)j * (R + 1);
-    const double res = givens_step(hcol, nu, j, nullptr, nullptr, g, Wq, false, red);
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};      // Σ norm partials, W·h
+#pragma unroll 4
+    for (int q = threadIdx.x; q < gp; q += OG) v[0] += npart[q];
+#pragma unroll 2
+    for (int l = threadIdx.x; l <= j; l += OG) {
+        const double2 hv = hcol[l], wl = Wq[l];
+        v[1] = fma(wl.x, hv.x, fma(-wl.y, hv.y, v[1]));
+        v[2] = fma(wl.x, hv.y, fma(wl.y, hv.x, v[2]));
+    }
+    og_sums(v, red);
+    if (threadIdx.x >= 32) return;
+    const double nu = sqrt(v[0]);
+    double c;
+    double2 sr, rr;
+    rotation_warp<double>(make_double2(v[1], v[2]), nu, c, sr, rr);
+    const double2 gj = g[j];
+    const double res = hyp(sr.x * gj.x + sr.y * gj.y, sr.x * gj.y - sr.y * gj.x);
     if (threadIdx.x == 0) {
         hcol[j + 1] = make_double2(nu, 0.0);
         hn_out[r] = nu;
@@ -1042,14 +1035,40 @@ k_dcgs_tent(OuterBatch B, double2 *__restrict__ H, double2 *__restrict__ g, doub
 __global__ void __launch_bounds__(OG)
 k_dcgs_close(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double2 *__restrict__ sn,
              double2 *__restrict__ g, double2 *__restrict__ Wq, int j, const int *__restrict__ close) {
-    __shared__ double red[OG / 32];
+    __shared__ double red[OG / 32][8];
+    __shared__ double2 s_s;
     const int r = blockIdx.x;
     if (!close[r]) return;
     const int R = B.R;
     H += (long long)r * (R + 1) * R; cs += (long long)r * R; sn += (long long)r * R;
     g += (long long)r * (R + 1); Wq += (long long)r * (R + 1);
     const double2 *hcol = H + (long long)j * (R + 1);
-    givens_step(hcol, hcol[j + 1].x, j, cs, sn, g, Wq, true, red);
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int l = threadIdx.x; l <= j; l += OG) {
+        const double2 hv = hcol[l], wl = Wq[l];
+        v[0] = fma(wl.x, hv.x, fma(-wl.y, hv.y, v[0]));
+        v[1] = fma(wl.x, hv.y, fma(wl.y, hv.x, v[1]));
+    }
+    og_sums(v, red);
+    if (threadIdx.x < 32) {
+        double c;
+        double2 sr, rr;
+        rotation_warp<double>(make_double2(v[0], v[1]), hcol[j + 1].x, c, sr, rr);
+        if (threadIdx.x == 0) {
+            const double2 gj = g[j];
+            s_s = sr;
+            cs[j] = c; sn[j] = sr;
+            g[j + 1] = make_double2(-(sr.x * gj.x + sr.y * gj.y), -(sr.x * gj.y - sr.y * gj.x));
+            g[j] = make_double2(c * gj.x, c * gj.y);
+            Wq[j + 1] = make_double2(c, 0.0);
+        }
+    }
+    __syncthreads();
+    const double2 sr = s_s;
+    for (int l = threadIdx.x; l <= j; l += OG) {
+        const double2 wl = Wq[l];
+        Wq[l] = make_double2(-(sr.x * wl.x + sr.y * wl.y), -(sr.x * wl.y - sr.y * wl.x));
+    }
 }
 
 // Delayed CGS2 update of step j, one element pair per thread (as k_oupdate_df):
@@ -1230,9 +1249,11 @@ __global__ void k_oscale(OuterBatch B, double2 *__restrict__ out, float2 *__rest
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < B.n; i += (long long)gridDim.x * blockDim.x) {
         const double2 v = make_double2(w[i].x * inv, w[i].y * inv);
         out[i] = v;
-        const float2 hi = make_float2((float)v.x, (float)v.y);
-        if (out32) out32[i] = hi;
-        if (out32L) out32L[i] = make_float2((float)(v.x - (double)hi.x), (float)(v.y - (double)hi.y));
+        if (out32) {
+            const float2 re = df_split(v.x), im = df_split(v.y);
+            out32[i] = make_float2(re.x, im.x);
+            if (out32L) out32L[i] = make_float2(re.y, im.y);
+        }
         if (outD) outD[i] = v.x - v.y;
     }
 }
