@@ -55,7 +55,10 @@ struct FactorSet {            // banded FP64 factors of one matrix per shape, bl
     std::vector<int4> meta;         // host copy of Meta and the operators' length (for the spike matrices)
     long long mo = 0;
     bool spike_tried = false;       // the SPIKE plans were formed, or were not wanted at set-up
-    bool dense_on = false;          // the dense form pays for the tasks there are
+    bool dense_on = false;          // a product with explicit inverses pays for the tasks there are,
+    bool small_on = false;          // and it is the FP64 one
+    DevMem sinv, stab;              // FP64 inverses and their SmallShape, if they were formed
+    int small_m = 0;                // largest order
     int digits32 = 6;               // digits of the complex64 iteration
     struct Plan {
         DevMem sh, recs, tabs, tcoff, B, cs, ws, part;  // tabs: sunits, items, then tlist and tshape (ntask each)
@@ -63,7 +66,7 @@ struct FactorSet {            // banded FP64 factors of one matrix per shape, bl
         double bytes = 0, flops = 0;
         void clear() { sh.release(); recs.release(); tabs.release(); tcoff.release(); B.release(); cs.release(); ws.release(); part.release(); ntask = 0; }
     } plan[4];                      // {task table, doubled table} with 6 digits, with 7
-    void clear() { dA.release(); drs.release(); dop.clear(); for (auto &P : plan) P.clear(); meta.clear(); mo = 0; spike_tried = dense_on = false; G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
+    void clear() { dA.release(); drs.release(); dop.clear(); for (auto &P : plan) P.clear(); meta.clear(); mo = 0; spike_tried = dense_on = small_on = false; sinv.release(); stab.release(); small_m = 0; G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
                    M.release(); Mdf.release(); P.release(); Meta.release(); table.release(); h.clear(); fma_col.clear(); cfg = BlockSolveCfg{}; re2 = false; ready = false; }
 };
 
@@ -420,16 +423,21 @@ hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &met
 
 
 // ---- the coarse solve as a product with explicit inverses (kernels_dense.cu) ------------------
-// Whether it is the faster form for `per` tasks of each shape.  Dense: three kernels, about 12 us
-// where nothing else counts, and the operators' digits at 5.5 TB/s with the MMAs under them (28
-// products of nt columns per 16-column unit, nt/2 clocks each).  Banded: 0.77 us per 16-row block
-// and sweep (164 us for the 106 blocks of m = 1681), one chain per SM, or 1.7 times that for two
-// per SM.  Measured: four shapes, 64 tasks (k=200) 164 us against 45; 256 uneven shapes of
-// N = 1280 with 32 right-hand sides 15.2 ms against 2.3, while for one right-hand side the banded
-// form stays ahead (0.5 against 2 ms: every operator is read for one task); m = 64, 4 tasks, 15 us
-// against 17.
-bool dense_pays(const hdd_ctx *ctx, const FactorSet &F, const std::vector<int> &per) {
-    double bytes = 0, mma = 0, chain = 0, chains = 0;
+// Which form is the fastest for `per` tasks of each shape: 0 banded, 1 the product by digits on the
+// tensor cores, 2 the FP64 product.  Digits: three kernels, about 12 us where nothing else counts,
+// and the operators' digits at 5.5 TB/s with the MMAs under them (28 products of nt columns per
+// 16-column unit, nt/2 clocks each).  Banded: 0.77 us per 16-row block and sweep (164 us for the 106
+// blocks of m = 1681), one chain per SM, or 1.7 times that for two per SM.  Measured: four shapes, 64
+// tasks (k=200) 164 us against 45; 256 uneven shapes of N = 1280 with 32 right-hand sides 15.2 ms
+// against 2.3, while for one right-hand side the banded form stays ahead (0.5 against 2 ms: every
+// operator is read for one task); m = 64, 4 tasks, 15 us against 17.  FP64: one kernel, 6.5 us and its
+// products at the FP64 pipe's rate.  By events around a solve, banded / digits / FP64: m = 64, 4 or 16
+// tasks 13 / 15..17 / 7 us; m = 256, 4 tasks 31 / 16 / 7.6; m = 289, 4 complex 69 / 16 / 9.4; m = 576,
+// 4 tasks 62 / 16 / 11, 12 tasks 64 / 17 / 20; m = 441, 16 tasks 50 / 17 / 16.5; m = 1024, 4 tasks 107
+// / 16 / 22.  So measured the first two take 7 and 3.5 us more than the models above.
+int coarse_pays(const hdd_ctx *ctx, const FactorSet &F, const std::vector<int> &per) {
+    double bytes = 0, mma = 0, chain = 0, chains = 0, prod = 0;
+    int mmax = 0;
     for (size_t q = 0; q < F.h.size(); q++) {
         const int m = F.re2 ? F.h[q].m / 2 : F.h[q].m;
         const double units = (double)((m + 127) / 128) * ((m + 15) / 16) * (F.re2 ? 2 : 1);
@@ -437,10 +445,14 @@ bool dense_pays(const hdd_ctx *ctx, const FactorSet &F, const std::vector<int> &
         mma += units * 28.0 * 0.5 * std::max(16.0, 2.0 * per[q]);
         chain = std::max(chain, 2.0 * F.h[q].nblk * 0.77e-6);
         chains += (F.re2 ? 1.0 : 2.0) * per[q];
+        prod += (F.re2 ? 4.0 : 2.0) * per[q] * (double)m * m;
+        mmax = std::max(mmax, m);
     }
     const double td = 12e-6 + std::max(bytes / 5.5e12, mma / (ctx->nsm * 1.9e9));
     const double tb = chains <= ctx->nsm ? chain : 1.7 * chain * std::ceil(chains / (2.0 * ctx->nsm));
-    return td < 0.8 * tb;
+    const double ts = 6.5e-6 + prod / (2.0 * ctx->nsm * 1.9e9);
+    if (mmax <= SMALL_M && ts < std::min(td + 3.5e-6, tb + 7e-6)) return 2;
+    return td < 0.8 * tb ? 1 : 0;
 }
 
 std::vector<int> tasks_per_shape(const hdd_ctx *ctx) {
@@ -523,13 +535,15 @@ hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_
 
 // Explicit inverses of every shape as digits, where the product pays and fits (a quarter of the
 // free memory, 8192 operator columns, the set-up kernel's shared memory); else F.dop stays empty.
-hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
+hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, cudaStream_t s) {
     const int ns = (int)F.h.size();
     const int re2 = F.re2 ? 1 : 0, cw = std::max(F.cfg.cwx, F.cfg.cwy);
     if (ns > DENSE_MAXNS || inv_cols_smem(F.cfg.maxK, cw) > 226 * 1024) return HDD_OK;
     std::vector<FactorSet::DenseOp> op(ns);
     std::vector<long long> wsz(ns);
-    long long ao = 0, so = 0;
+    std::vector<SmallShape> ss(ns);
+    long long ao = 0, so = 0, sv = 0;
+    int sm = 0;
     for (int q = 0; q < ns; q++) {
         FactorSet::DenseOp &o = op[q];
         o.m = F.h[q].m / (re2 ? 2 : 1);
@@ -539,12 +553,21 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
         ao += (long long)o.mt * o.kc * DENSE_ABYTES;
         so += (long long)o.mt * 128;
         wsz[q] = (long long)o.kseg * 16 * F.h[q].nblk * BNB;       // 16 columns x all rows per column block
+        ss[q] = SmallShape{sv, o.m, (o.m + 7) & ~7};
+        sv += (long long)o.m * ss[q].ld;
+        sm = std::max(sm, o.m);
     }
     size_t fr = 0, tot = 0;
     CK(cudaMemGetInfo(&fr, &tot));
-    if ((size_t)ao > fr / 4) return HDD_OK;
-    CK(F.dA.ensure((size_t)ao));
-    CK(F.drs.ensure((size_t)so * sizeof(int)));
+    if ((small ? (size_t)sv * (re2 ? 16 : 8) : (size_t)ao) > fr / 4) return HDD_OK;
+    if (small) {
+        CK(F.sinv.ensure((size_t)sv * (re2 ? sizeof(double2) : sizeof(double))));
+        CK(F.stab.ensure(ns * sizeof(SmallShape)));
+        CK(cudaMemcpyAsync(F.stab.p, ss.data(), ns * sizeof(SmallShape), cudaMemcpyHostToDevice, s));
+    } else {
+        CK(F.dA.ensure((size_t)ao));
+        CK(F.drs.ensure((size_t)so * sizeof(int)));
+    }
     // shapes in groups of up to 1 GB of workspace
     DevMem W, jobs, shs, rmax;
     for (int q0 = 0; q0 < ns;) {
@@ -575,9 +598,14 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
         CK(cudaMemcpyAsync(shs.p, sh.data(), sh.size() * sizeof(InvShape), cudaMemcpyHostToDevice, s));
         CK(launch_inv(jobs.as<InvJob>(), (int)jb.size(), shs.as<InvShape>(), (int)sh.size(), mmax, kmax, tmax,
                       F.table.as<BlockFactor>(), F.M.as<double>(), F.P.as<int>(), F.Meta.as<int4>(), W.as<double>(),
-                      F.cfg.maxK, cw, re2, rmax.as<unsigned long long>(), F.drs.as<int>(), F.dA.as<uint8_t>(), s));
+                      F.cfg.maxK, cw, re2, rmax.as<unsigned long long>(), F.drs.as<int>(), F.dA.as<uint8_t>(),
+                      small ? F.stab.as<SmallShape>() + q0 : nullptr, F.sinv.as<double>(), s));
         CK(cudaStreamSynchronize(s));           // the tables and the workspace are used again
         q0 = q1;
+    }
+    if (small) {
+        F.small_m = sm;
+        return HDD_OK;
     }
     F.dop = op;
     // Against the exact inverse, 6 digits leave 1e-13 of the solution where the double-FP32 banded
@@ -590,6 +618,19 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
 
 // E⁻¹ in for the flagged tasks by the product; ds and which as in dense_plan.
 hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
+    if (F.small_on) {
+        const int nt = (int)ctx->h_tasks.size() * (which ? 2 : 1);
+        double by = 0, fl = 0;
+        for (const Task &T : ctx->h_tasks) {
+            const double m = F.h[T.shape].m / (F.re2 ? 2 : 1);
+            by += 32.0 * m;
+            fl += (F.re2 ? 8.0 : 4.0) * m * m;
+        }
+        KL(F_CDENSE, by * (which ? 2 : 1) + (double)F.sinv.bytes, fl * (which ? 2 : 1),
+           launch_small_solve(which ? ctx->d_tasks2.as<Task>() : ctx->d_tasks.as<Task>(), nt, F.stab.as<SmallShape>(), F.small_m,
+                              F.re2 ? 1 : 0, F.sinv.as<double>(), in, out, flag, s));
+        return HDD_OK;
+    }
     hdd_status st = dense_plan(ctx, F, ds, which, s);
     if (st != HDD_OK) return st;
     FactorSet::Plan &P = F.plan[which + (ds == 7 ? 2 : 0)];
@@ -620,12 +661,15 @@ hdd_status spike_build(hdd_ctx *ctx, FactorSet &F) {
 
 // The form the inner iteration's coarse solves take, chosen by the tasks there are: the product
 // with explicit inverses, or the banded kernels with their SPIKE plans.
+bool dense_built(const FactorSet &F) { return F.small_on ? F.small_m > 0 : !F.dop.empty(); }
 hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
     hdd_status st = HDD_OK;
-    F.dense_on = dense_pays(ctx, F, tasks_per_shape(ctx));
-    if (ctx->coarse_dense && F.dense_on && F.dop.empty()) st = dense_build(ctx, F, s);
+    const int form = coarse_pays(ctx, F, tasks_per_shape(ctx));
+    F.dense_on = form > 0;
+    F.small_on = form == 2;
+    if (ctx->coarse_dense && F.dense_on && !dense_built(F)) st = dense_build(ctx, F, F.small_on, s);
     if (!ctx->coarse_spike) F.spike_tried = true;
-    if (st == HDD_OK && !F.spike_tried && !(F.dense_on && !F.dop.empty())) {
+    if (st == HDD_OK && !F.spike_tried && !(F.dense_on && dense_built(F))) {
         CK(cudaStreamSynchronize(s));
         st = spike_build(ctx, F);
     }
@@ -634,7 +678,7 @@ hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
 
 // Whether the coarse solves of the inner iteration and of the training loss run as that product.
 bool use_dense(const hdd_ctx *ctx) {
-    return ctx->coarse_dense && ctx->coarse_la && ctx->E.dense_on && !ctx->E.dop.empty();
+    return ctx->coarse_dense && ctx->coarse_la && ctx->E.dense_on && dense_built(ctx->E);
 }
 
 // E_j (or A_j) factors for every distinct shape, FP64, on the device: banded LU with partial

@@ -445,6 +445,7 @@ struct InvShape {                            // one shape at set-up
     long long rows;                          // workspace rows per column block: 16·nblk
     int m, mt, kseg, kc, re2;                // order of E, row tiles, chunks per part and in all
 };
+struct SmallShape { long long off; int m, ld; };   // E⁻¹ in FP64: first entry, order, column stride
 struct DenseShape {                          // one shape of a solve plan
     long long aoff, soff, boff, acc0;        // operator (bytes), row exponents, right-hand-side digits (bytes), sums
     int m, mt, kseg, kc, re2;
@@ -471,7 +472,11 @@ struct DensePlanArgs {
 size_t inv_cols_smem(int maxK, int cw);
 cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns, int mmax, int ksegmax, int mtmax,
                        const BlockFactor *shapes, const double *Mall, const int *Pall, const int4 *Meta, double *W,
-                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, cudaStream_t s);
+                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, const SmallShape *ss,
+                       double *inv, cudaStream_t s);
+constexpr int SMALL_M = 2048;                // largest order of the FP64 product (its vector fits 48 KB of shared memory)
+void launch_small_solve(const Task *tasks, int ntask, const SmallShape *ss, int mmax, int re2, const double *inv,
+                        const double2 *in, double2 *out, const int *flag, cudaStream_t s);
 int dense_stages(int ds, int ns, int ntmax);
 cudaError_t dense_set_smem();
 void launch_dense_solve(int ds, const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s);

@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace hdd {
 
@@ -246,6 +247,94 @@ k_inv_slice(const InvShape *__restrict__ sh, const double *__restrict__ Wall,
             }
         }
     }
+}
+
+// ------------------------------------------------------------------------------------------
+// Small orders: E⁻¹ in FP64, column by column, and its product in one launch
+// ------------------------------------------------------------------------------------------
+// inv[off + c·ld + r] (or its complex entry): CTA (16 columns, 128 rows, shape), thread = row
+__global__ void __launch_bounds__(128)
+k_small_pack(const InvShape *__restrict__ sh, const SmallShape *__restrict__ ss, const double *__restrict__ Wall,
+             double *__restrict__ inv) {
+    const InvShape S = sh[blockIdx.z];
+    const SmallShape Q = ss[blockIdx.z];
+    const int i = blockIdx.y * 128 + threadIdx.x;
+    if (i >= Q.ld) return;
+    const double *W = Wall + S.woff;
+    for (int c = 0; c < 16; c++) {
+        const int j = blockIdx.x * 16 + c;
+        if (j >= S.m) break;
+        for (int part = 0; part <= S.re2; part++)
+            inv[((Q.off + (long long)j * Q.ld + i) << S.re2) + part] = i < S.m ? inv_entry(W, S.rows, S.re2, part, i, j) : 0.0;
+    }
+}
+
+// out = E⁻¹ in of a task's SM_R rows: lane = row x one of four columns, warps share the columns.
+// Bound by the FP64 pipe (a warp instruction is 64 clocks of its scheduler): m² · 2 products a task
+// (4 for complex E) over as many CTAs as there are blocks of rows; the matrix comes from L2, and the
+// first entries are loaded before the wait for the kernel in front.  m = 64, 4
+// tasks: 7 us by events around it where the banded sweeps take 13 and the three kernels of the
+// digits 15; m = 576: 11 us (62, 16).
+constexpr int SM_R = 8, SM_T = 256, SM_PRE = 4;
+template <bool RE2>
+__global__ void __launch_bounds__(SM_T)
+k_small_solve(const Task *__restrict__ tasks, const SmallShape *__restrict__ ss, const double *__restrict__ inv,
+              const double2 *__restrict__ in, double2 *__restrict__ out, const int *__restrict__ flag) {
+    using A = typename std::conditional<RE2, double2, double>::type;
+    extern __shared__ double2 xs[];
+    __shared__ double red[2 * SM_R][SM_T / 32];
+    const int t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Task T = tasks[t];
+    const SmallShape S = ss[T.shape];
+    const int r0 = blockIdx.x * SM_R, c0 = warp * 4 + (lane >> 3);
+    const bool mine = r0 < S.m;
+    const A *M = reinterpret_cast<const A *>(inv) + S.off + r0 + (lane & 7);
+    A pre[SM_PRE];
+    if (mine)
+#pragma unroll
+        for (int q = 0; q < SM_PRE; q++)
+            if (c0 + 32 * q < S.m) pre[q] = M[(long long)(c0 + 32 * q) * S.ld];
+    CHAIN_ENTER();
+    LAUNDER(in); LAUNDER(flag);
+    if (!mine || (flag && !flag[t])) return;
+    for (int i = tid; i < S.m; i += SM_T) xs[i] = in[T.coff + i];
+    __syncthreads();
+    double ax = 0.0, ay = 0.0;
+    auto add = [&](A a, double2 x) {
+        if constexpr (RE2) {
+            ax = fma(a.x, x.x, fma(-a.y, x.y, ax));
+            ay = fma(a.x, x.y, fma(a.y, x.x, ay));
+        } else {
+            ax = fma(a, x.x, ax);
+            ay = fma(a, x.y, ay);
+        }
+    };
+#pragma unroll
+    for (int q = 0; q < SM_PRE; q++)
+        if (c0 + 32 * q < S.m) add(pre[q], xs[c0 + 32 * q]);
+#pragma unroll 4
+    for (int c = c0 + 32 * SM_PRE; c < S.m; c += 32) add(M[(long long)c * S.ld], xs[c]);
+    const bool im = (lane & 8) != 0;                      // one component each after the first exchange
+    double v = (im ? ay : ax) + shfl_xor(im ? ax : ay, 8);
+    v += shfl_xor(v, 16);
+    if (lane < 16) red[lane][warp] = v;                   // lane = 8·component + row
+    __syncthreads();
+    if (tid < 16 * (SM_T / 32)) {
+        const int k = tid >> 3;
+        double s = red[k][tid & 7];
+        s += shfl_xor(s, 4);
+        s += shfl_xor(s, 2);
+        s += shfl_xor(s, 1);
+        const int r = r0 + (k & 7);
+        if ((tid & 7) == 0 && r < S.m) reinterpret_cast<double *>(out + T.coff + r)[k >> 3] = s;
+    }
+}
+void launch_small_solve(const Task *tasks, int ntask, const SmallShape *ss, int mmax, int re2, const double *inv,
+                        const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
+    const dim3 grid((mmax + SM_R - 1) / SM_R, ntask);
+    const size_t sm = (size_t)mmax * sizeof(double2);
+    if (re2) launch_chained(k_small_solve<true>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag);
+    else launch_chained(k_small_solve<false>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -691,13 +780,18 @@ size_t inv_cols_smem(int maxK, int cw) { return ((size_t)2 * BNB * maxK + (size_
 
 cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns, int mmax, int ksegmax, int mtmax,
                        const BlockFactor *shapes, const double *Mall, const int *Pall, const int4 *Meta, double *W,
-                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, cudaStream_t s) {
+                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, const SmallShape *ss,
+                       double *inv, cudaStream_t s) {
     const size_t smem = inv_cols_smem(maxK, cw);
     cudaError_t e = re2 ? cudaFuncSetAttribute(k_inv_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                         : cudaFuncSetAttribute(k_inv_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (re2) k_inv_cols<true><<<njobs, 256, smem, s>>>(jobs, shapes, Mall, Pall, Meta, W, maxK, cw);
     else k_inv_cols<false><<<njobs, 256, smem, s>>>(jobs, shapes, Mall, Pall, Meta, W, maxK, cw);
+    if (ss) {
+        k_small_pack<<<dim3(ksegmax, (mmax + 127 + SM_R) / 128, ns), 128, 0, s>>>(sh, ss, W, inv);
+        return cudaGetLastError();
+    }
     k_inv_rowmax<<<dim3((mmax + 127) / 128, (mmax + 15) / 16, ns), 128, 0, s>>>(sh, W, rmax);
     k_inv_slice<<<dim3(ksegmax, mtmax, ns), 128, 0, s>>>(sh, W, rmax, rexp, reinterpret_cast<uint4 *>(A));
     return cudaGetLastError();
