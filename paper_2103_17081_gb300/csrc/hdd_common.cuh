@@ -146,6 +146,26 @@ __device__ __forceinline__ double hyp(double x, double y) {
     return sqrt(fma(xs, xs, ys * ys)) * __hiloint2double((int)(e << 20), 0);
 }
 
+// (|x|, sqrt(|x|² + b²)) by a whole warp, lanes with `second` forming the other root: for doubles of
+// comparable size both roots in the time of one
+template <typename R> __device__ __forceinline__ c2<R> hyp2(c2<R> x, R b, bool second);
+template <> __device__ __forceinline__ float2 hyp2<float>(float2 x, float b, bool) {
+    const float a = hyp(x.x, x.y);
+    return make_float2(a, hyp(a, b));
+}
+template <> __device__ __forceinline__ double2 hyp2<double>(double2 x, double b, bool second) {
+    const unsigned ex = ((unsigned)__double2hiint(x.x) >> 20) & 0x7ffu, ey = ((unsigned)__double2hiint(x.y) >> 20) & 0x7ffu;
+    const unsigned ea = ex > ey ? ex : ey, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu, e = ea > eb ? ea : eb;
+    if (e - 64u > 1900u || ea + 400u < e) {
+        const double a = hyp(x.x, x.y);
+        return make_double2(a, hyp(a, b));
+    }
+    const double sc = __hiloint2double((int)((2046u - e) << 20), 0), up = __hiloint2double((int)(e << 20), 0);
+    const double xs = x.x * sc, ys = x.y * sc, bs = b * sc, aa = fma(xs, xs, ys * ys);
+    const double root = sqrt(second ? fma(bs, bs, aa) : aa) * up;
+    return make_double2(shfl(root, 0), shfl(root, 2));
+}
+
 // Givens rotation of (x, b) with b >= 0 real, by a whole warp: c = |x|/t, s = (x/|x|)·b/t,
 // r = (x/|x|)·t, t = sqrt(|x|² + b²); the four divisions in four lanes at once.
 template <typename R>
@@ -154,16 +174,16 @@ __device__ __forceinline__ void rotation_warp(c2<R> x, R b, R &c, c2<R> &s, c2<R
     c = 1;
     s = mk<R>(0, 0);
     r = x;
-    const R aa = hyp(x.x, x.y);
+    const bool second = (lane & 2) != 0, im = (lane & 1) != 0;
     if (b == (R)0) return;
+    const c2<R> at = hyp2<R>(x, b, second);
+    const R aa = at.x, t = at.y;
     if (aa == (R)0) {
         c = 0;
         s = mk<R>(1, 0);
         r = mk<R>(b, 0);
         return;
     }
-    const R t = hyp(aa, b);
-    const bool second = (lane & 2) != 0, im = (lane & 1) != 0;
     const R q = (second ? (im ? b : aa) : (im ? x.y : x.x)) / (second ? t : aa);
     const c2<R> ph = mk<R>(shfl(q, 0), shfl(q, 1));
     const R bt = shfl(q, 3);

@@ -629,11 +629,14 @@ __device__ void solve_small(const InnerState<R> &S, int restart, int t, int k, c
             if (r <= l) hs[e] = H[(long long)l * (restart + 1) + r];
         }
         __syncwarp();
+        // row r's lanes divide by its diagonal: q = num·(1/den), once corrected by its remainder
+        const c2<R> d = row < k ? hs[row * SMALL_K + row] : mk<R>(1, 0);
+        const R den = d.x * d.x + d.y * d.y, rden = (R)1 / den, di = im ? -d.y : d.y;
         for (int r = k - 1; r >= 0; r--) {
-            const c2<R> d = hs[r * SMALL_K + r];
-            const R sx = shfl(acc, 2 * r), sy = shfl(acc, 2 * r + 1), den = d.x * d.x + d.y * d.y;
-            const R v = (im ? sy * d.x - sx * d.y : sx * d.x + sy * d.y) / den;
-            const R yx = shfl(v, 0), yy = shfl(v, 1);
+            const R num = fma(acc, d.x, shfl_xor(acc, 1) * di);
+            R v = num * rden;
+            v = fma(fma(-v, den, num), rden, v);
+            const R yx = shfl(v, 2 * r), yy = shfl(v, 2 * r + 1);
             if (lane == 0) y[r] = mk<R>(yx, yy);
             if (row < r) {
                 const c2<R> h = hs[r * SMALL_K + row];
@@ -1087,15 +1090,19 @@ k_arnoldi_step(StepArgs<R> a) {
                 a.S.kcols[t] = i + 1;
                 if (conv || its >= a.maxit) a.S.conv[t] = 1;
                 a.act_out[t] = stop ? 0 : 1;
-                publish(a.pr, i + 1, stop ? 0 : 1);
             }
         }
     }
     __syncthreads();
-    if (stop_s) return;                           // the same decision in every CTA
+    const bool counts = rank == 0 && tid == 0;    // (the count's round trip overlaps what follows)
+    if (stop_s) {                                 // the same decision in every CTA
+        if (counts) publish(a.pr, i + 1, 0);
+        return;
+    }
     // ---- E: y = Zᵀ A v_{i+1} on coarse rows [c0, c1) ----
     cluster_barrier();                            // v_{i+1} of every CTA written and visible
     const int c0 = (int)(rank * my) / C, c1 = (int)((rank + 1) * my) / C;
+    if (counts && c1 <= c0) publish(a.pr, i + 1, 1);
     if (c1 <= c0) return;
     const int G0 = 2 * c0 - 1, G1 = 2 * (c1 - 1) + 3, nG = G1 - G0 + 1, nW = nG + 2, PE = nx + 3;
     c2<R> *vin = reinterpret_cast<c2<R> *>(smem_raw);                 // rows G0 - 1 .. G1 + 1
@@ -1106,6 +1113,7 @@ k_arnoldi_step(StepArgs<R> a) {
         const int q = e / 3, b = e - 3 * q;
         tt[q * PE + (b ? nx + b : 0)] = mk<R>(0, 0);
     }
+    if (counts) publish(a.pr, i + 1, 1);
     async_wait();
     __syncthreads();
 #pragma unroll 1

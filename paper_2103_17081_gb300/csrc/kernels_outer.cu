@@ -14,10 +14,12 @@ constexpr int OUTER_CTAS = 2 * 152;     // two CTAs per SM of a GB300 (minimum g
 constexpr int OT = 256;                 // threads per outer CTA
 constexpr int OCH = 1536;               // largest chunk one CTA owns (staged in shared memory)
 constexpr int OT2 = 512;                // threads of the memory-bound FP32 second pass (more loads in flight)
-// CTAs of the chunked reductions over a vector of n entries
+// CTAs of the chunked reductions over a vector of n entries (of at least a warp's 32: below that a
+// CTA's sums cost the same and only the partials grow, n = 961 8 us a reduction of 304,
+// 4.3 of 31)
 int outer_grid(long long n) {
-    long long g = (n + OCH - 1) / OCH;
-    return (int)(g > OUTER_CTAS ? g : OUTER_CTAS);
+    const long long g = (n + OCH - 1) / OCH, m = std::min<long long>(OUTER_CTAS, (n + 31) / 32);
+    return (int)std::max(g, m);
 }
 
 // y = A x (f == nullptr) or y = f - A x on the (N-1)² interior grid, zero Dirichlet values, or
@@ -155,6 +157,41 @@ __device__ __forceinline__ void warp_dots(const double2 *__restrict__ V, const d
                                           long long ld, int nv, const WStage &ws, long long b, int len,
                                           double2 *__restrict__ part, int ldp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // Short chunks, several vectors a warp: four at a time, their eight sums reduced by halves across
+    // the lanes (9 FP64 additions instead of 40, at 64 clocks each)
+    if (len <= 64 && nv > OT / 16) {
+        for (int l0 = 4 * warp; l0 < nv; l0 += OT / 8) {
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                double p = 0.0, q = 0.0, s = 0.0;
+                if (l0 + k < nv)
+                    for (int i = lane; i < len; i += 32) {
+                        const double2 x = V[(long long)(l0 + k) * ld + b + i];
+                        p = fma(D[(long long)(l0 + k) * ld + b + i], ws.a[i], p);
+                        q = fma(x.y, ws.p[i], q);
+                        s = fma(x.x, ws.m[i], s);
+                    }
+                v[2 * k] = p + q;
+                v[2 * k + 1] = p + s;
+            }
+#pragma unroll
+            for (int half = 4; half > 0; half >>= 1) {
+                const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+                for (int k = 0; k < half; k++) {
+                    const double x = shfl_xor(up ? v[k] : v[k + half], 4 * half);
+                    v[k] = (up ? v[k + half] : v[k]) + x;
+                }
+            }
+            v[0] += shfl_xor(v[0], 2);
+            v[0] += shfl_xor(v[0], 1);
+            const int l = l0 + (lane >> 3);
+            if ((lane & 3) == 0 && l < nv)
+                reinterpret_cast<double *>(part + (long long)blockIdx.x * ldp + l)[(lane >> 2) & 1] = v[0];
+        }
+        return;
+    }
     for (int l = warp; l < nv; l += OT / 32) {
         const double2 *vl = V + (long long)l * ld + b;
         const double *dl = D + (long long)l * ld + b;
@@ -183,6 +220,8 @@ k_odots(OuterBatch B, const double2 *__restrict__ V, int nv, const double2 *__re
         double2 *__restrict__ part) {
     __shared__ WStage ws;
     const int r = blockIdx.y;
+    CHAIN_ENTER();
+    LAUNDER(V); LAUNDER(w);
     if (B.active && !B.active[r]) return;
     V += r * B.n; w += r * B.n; part += (long long)r * B.G * B.ldp;
     const double *D = B.D + r * B.n;
@@ -368,6 +407,8 @@ k_oupdate(OuterBatch B, const double2 *__restrict__ V, int nv, const double2 *__
     __shared__ WStage ws;
     __shared__ double red[OT / 32];
     const int r = blockIdx.y;
+    CHAIN_ENTER();
+    LAUNDER(V); LAUNDER(h);
     if (B.active && !B.active[r]) return;
     V += r * B.n; w += r * B.n; h += (long long)r * B.ldp;
     const double *D = B.D + r * B.n;
@@ -654,6 +695,8 @@ k_ogivens(OuterBatch B, double2 *__restrict__ H, double *__restrict__ cs, double
     __shared__ double c_s;
     __shared__ double2 s_s;
     const int r = blockIdx.x;
+    CHAIN_ENTER();
+    LAUNDER(h1); LAUNDER(h2); LAUNDER(npart); LAUNDER(fnorm);
     if (B.active && !B.active[r]) return;
     const int R = B.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     H += (long long)r * (R + 1) * R; cs += (long long)r * R; sn += (long long)r * R;
@@ -1371,7 +1414,7 @@ void launch_build_rhs(const Stencil &st, int N, double h, int npts, const double
     k_build_rhs<<<grid_for(n, 256), 256, 0, s>>>(st, N, h, npts, pts, nb, bumps, f);
 }
 void launch_odots(const OuterBatch &B, const double2 *V, int nv, const double2 *w, double2 *part, cudaStream_t s) {
-    k_odots<<<dim3(B.G, B.nrhs), OT, 0, s>>>(B, V, nv, w, part);
+    launch_chained(k_odots, dim3(B.G, B.nrhs), OT, 0, s, B, V, nv, w, part);
 }
 void launch_odots_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int nv, const double2 *w,
                      double2 *part, cudaStream_t s) {
@@ -1379,7 +1422,7 @@ void launch_odots_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, in
 }
 void launch_oupdate(const OuterBatch &B, const double2 *V, int nv, const double2 *h, double2 *w,
                     double2 *part_dots, double *part_norm, cudaStream_t s) {
-    k_oupdate<<<dim3(B.G, B.nrhs), OT, (size_t)nv * 3 * sizeof(double), s>>>(B, V, nv, h, w, part_dots, part_norm);
+    launch_chained(k_oupdate, dim3(B.G, B.nrhs), OT, (size_t)nv * 3 * sizeof(double), s, B, V, nv, h, w, part_dots, part_norm);
 }
 // CTA size and grid of a one-element-pair-per-thread update kernel for vectors of n entries: of
 // the sizes 256, 224, ..., 128 threads the one whose grid leaves the least idle in the last wave
@@ -1535,7 +1578,7 @@ void launch_ogivens(const OuterBatch &B, double2 *H, double *cs, double2 *sn, do
                     const double2 *h1, const double2 *h2, const double *npart, const double *fnorm,
                     double tol, double *hn_out, int *flag, double *hist, int hstride, int it,
                     cudaStream_t s) {
-    k_ogivens<<<B.nrhs, OG, 0, s>>>(B, H, cs, sn, g, Wq, j, h1, h2, npart, fnorm, tol, hn_out, flag, hist,
+    launch_chained(k_ogivens, B.nrhs, OG, 0, s, B, H, cs, sn, g, Wq, j, h1, h2, npart, fnorm, tol, hn_out, flag, hist,
                                     hstride, it);
 }
 void launch_orotate(const OuterBatch &B, double2 *H, const double *cs, const double2 *sn, const int *kcols,
