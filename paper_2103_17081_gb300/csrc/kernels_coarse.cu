@@ -635,11 +635,9 @@ k_block_solve(const Task *__restrict__ tasks, const BlockFactor *__restrict__ sh
     extern __shared__ double sm[];
     constexpr int STR = RE2 ? 1 : 2;        // stride (doubles) of the solved real column
     const int t = RE2 ? (int)blockIdx.x : (int)(blockIdx.x >> 1), comp = RE2 ? 0 : (int)(blockIdx.x & 1);
+    if (flag && !flag[t]) return;
     const Task T = tasks[t];
     const BlockFactor F = shapes[T.shape];
-    CHAIN_ENTER();
-    LAUNDER(in); LAUNDER(flag);
-    if (flag && !flag[t]) return;
     const long long off = use_fine ? T.foff : T.coff;
     const int m = F.m, nbk = F.nblk;
     const int slot = BNB * maxK + BNB;
@@ -769,11 +767,9 @@ k_block_solve_la(const Task *__restrict__ tasks, const BlockFactor *__restrict__
     __shared__ int sw[RING];                  // panel width of the block in each ring slot
     constexpr int STR = RE2 ? 1 : 2;
     const int t = RE2 ? (int)blockIdx.x : (int)(blockIdx.x >> 1), comp = RE2 ? 0 : (int)(blockIdx.x & 1);
+    if (flag && !flag[t]) return;
     const Task T = tasks[t];
     const BlockFactor F = shapes[T.shape];
-    CHAIN_ENTER();
-    LAUNDER(in); LAUNDER(flag);
-    if (flag && !flag[t]) return;
     const long long off = use_fine ? T.foff : T.coff;
     const int m = F.m, nbk = F.nblk;
     const int slot = la_slot(maxK);
@@ -985,11 +981,9 @@ k_block_solve_la_df(const Task *__restrict__ tasks, const BlockFactor *__restric
     __shared__ int sw[RING];
     constexpr int STR = RE2 ? 1 : 2;
     const int t = RE2 ? (int)blockIdx.x : (int)(blockIdx.x >> 1), comp = RE2 ? 0 : (int)(blockIdx.x & 1);
+    if (flag && !flag[t]) return;
     const Task T = tasks[t];
     const BlockFactor F = shapes[T.shape];
-    CHAIN_ENTER();
-    LAUNDER(in); LAUNDER(flag);
-    if (flag && !flag[t]) return;
     const long long off = use_fine ? T.foff : T.coff;
     const int m = F.m, nbk = F.nblk;
     const int slot = la_slot(maxK);
@@ -1578,10 +1572,10 @@ static void la_launch(int grid, const BlockSolveCfg &c, const Task *tasks, const
                       const double *Mall, const float2 *Mdf, const int *Pall, const int4 *Meta, const double2 *in,
                       double2 *out, int use_fine, const int *flag, cudaStream_t s) {
     if (Mdf)
-        launch_chained(k_block_solve_la_df<RING, RE2>, grid, LAD_T, la_smem(c, RING), s, tasks, shapes, Mdf, Pall, Meta, in, out,
+        k_block_solve_la_df<RING, RE2><<<grid, LAD_T, la_smem(c, RING), s>>>(tasks, shapes, Mdf, Pall, Meta, in, out,
                                                                              use_fine, flag, c.maxK, c.cwy, c.cwx);
     else
-        launch_chained(k_block_solve_la<RING, RE2>, grid, LA_T, la_smem(c, RING), s, tasks, shapes, Mall, Pall, Meta, in, out,
+        k_block_solve_la<RING, RE2><<<grid, LA_T, la_smem(c, RING), s>>>(tasks, shapes, Mall, Pall, Meta, in, out,
                                                                           use_fine, flag, c.maxK, c.cwy, c.cwx);
 }
 
@@ -1619,18 +1613,18 @@ void launch_block_solve(const Task *tasks, int ntasks, const BlockFactor *shapes
     }
     if (re2) {
         if (c.ring == 4)
-            launch_chained(k_block_solve<4, true>, ntasks, BS_T, bs_smem(c, 4), s, tasks, shapes, Mall, Pall, Meta, in, out,
+            k_block_solve<4, true><<<ntasks, BS_T, bs_smem(c, 4), s>>>(tasks, shapes, Mall, Pall, Meta, in, out,
                                                                        use_fine, flag, c.maxK, c.cwy, c.cwx);
         else
-            launch_chained(k_block_solve<2, true>, ntasks, BS_T, bs_smem(c, 2), s, tasks, shapes, Mall, Pall, Meta, in, out,
+            k_block_solve<2, true><<<ntasks, BS_T, bs_smem(c, 2), s>>>(tasks, shapes, Mall, Pall, Meta, in, out,
                                                                        use_fine, flag, c.maxK, c.cwy, c.cwx);
         return;
     }
     if (c.ring == 4)
-        launch_chained(k_block_solve<4, false>, 2 * ntasks, BS_T, bs_smem(c, 4), s, tasks, shapes, Mall, Pall, Meta, in, out,
+        k_block_solve<4, false><<<2 * ntasks, BS_T, bs_smem(c, 4), s>>>(tasks, shapes, Mall, Pall, Meta, in, out,
                                                                         use_fine, flag, c.maxK, c.cwy, c.cwx);
     else
-        launch_chained(k_block_solve<2, false>, 2 * ntasks, BS_T, bs_smem(c, 2), s, tasks, shapes, Mall, Pall, Meta, in, out,
+        k_block_solve<2, false><<<2 * ntasks, BS_T, bs_smem(c, 2), s>>>(tasks, shapes, Mall, Pall, Meta, in, out,
                                                                         use_fine, flag, c.maxK, c.cwy, c.cwx);
 }
 

@@ -1413,8 +1413,14 @@ void launch_build_rhs(const Stencil &st, int N, double h, int npts, const double
     const long long w = st.bc ? N + 1 : N - 1, n = w * w;
     k_build_rhs<<<grid_for(n, 256), 256, 0, s>>>(st, N, h, npts, pts, nb, bumps, f);
 }
+// The FP64 passes over the basis are one wave of long CTAs, two per SM of the six that fit: started
+// while the kernel before them still runs they pile up on the SMs that are free first (k=200, 250
+// vectors: 607 ms for the plain launches, 798 chained).  Chunks of up to two elements a lane are
+// short and gain from the early start.
+static bool chunk_chained(const OuterBatch &B) { return B.n <= 64LL * B.G; }
 void launch_odots(const OuterBatch &B, const double2 *V, int nv, const double2 *w, double2 *part, cudaStream_t s) {
-    launch_chained(k_odots, dim3(B.G, B.nrhs), OT, 0, s, B, V, nv, w, part);
+    if (chunk_chained(B)) launch_chained(k_odots, dim3(B.G, B.nrhs), OT, 0, s, B, V, nv, w, part);
+    else k_odots<<<dim3(B.G, B.nrhs), OT, 0, s>>>(B, V, nv, w, part);
 }
 void launch_odots_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, int nv, const double2 *w,
                      double2 *part, cudaStream_t s) {
@@ -1422,7 +1428,9 @@ void launch_odots_df(const OuterBatch &B, const float2 *Vh, const float2 *Vl, in
 }
 void launch_oupdate(const OuterBatch &B, const double2 *V, int nv, const double2 *h, double2 *w,
                     double2 *part_dots, double *part_norm, cudaStream_t s) {
-    launch_chained(k_oupdate, dim3(B.G, B.nrhs), OT, (size_t)nv * 3 * sizeof(double), s, B, V, nv, h, w, part_dots, part_norm);
+    const size_t sm = (size_t)nv * 3 * sizeof(double);
+    if (chunk_chained(B)) launch_chained(k_oupdate, dim3(B.G, B.nrhs), OT, sm, s, B, V, nv, h, w, part_dots, part_norm);
+    else k_oupdate<<<dim3(B.G, B.nrhs), OT, sm, s>>>(B, V, nv, h, w, part_dots, part_norm);
 }
 // CTA size and grid of a one-element-pair-per-thread update kernel for vectors of n entries: of
 // the sizes 256, 224, ..., 128 threads the one whose grid leaves the least idle in the last wave
