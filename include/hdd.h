@@ -391,7 +391,8 @@ long long hdd_launch_count(const hdd_ctx *ctx);
 /* loss run as products with the explicit inverses of the distinct E_j on the tensor cores, in  */
 /* exact integer arithmetic on 56-bit fixed-point copies of the FP64 entries (1, the default,   */
 /* where the shapes and tasks make that the faster form; the inverses are formed at             */
-/* hdd_setup_deflation, or at hdd_setup_batch when the batch makes it pay) or by the banded     */
+/* hdd_setup_deflation, or at hdd_setup_batch when the batch makes it pay; small orders as one   */
+/* FP64 product with the inverse) or by the banded                                               */
 /* kernels the options 1, 6 and 7 describe (0).  hdd_local_op always applies the banded ones.   */
 /* With HDD_OPT_COARSE_LOOKAHEAD 0, or HDD_OPT_COARSE_DF 0 in complex64, the banded kernels run. */
 /* HDD_ERR_INVALID_ARG for an unknown key or a value other than 0 or 1.  Takes effect from the  */

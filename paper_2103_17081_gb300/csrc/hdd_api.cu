@@ -428,7 +428,7 @@ hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &met
 // and the operators' digits at 5.5 TB/s with the MMAs under them (28 products of nt columns per
 // 16-column unit, nt/2 clocks each).  Banded: 0.77 us per 16-row block and sweep (164 us for the 106
 // blocks of m = 1681), one chain per SM, or 1.7 times that for two per SM.  Measured: four shapes, 64
-// tasks (k=200) 164 us against 45; 256 uneven shapes of N = 1280 with 32 right-hand sides 15.2 ms
+// tasks (k=200) 164 us against 38; 256 uneven shapes of N = 1280 with 32 right-hand sides 15.2 ms
 // against 2.3, while for one right-hand side the banded form stays ahead (0.5 against 2 ms: every
 // operator is read for one task); m = 64, 4 tasks, 15 us against 17.  FP64: one kernel, 6.5 us and its
 // products at the FP64 pipe's rate.  By events around a solve, banded / digits / FP64: m = 64, 4 or 16

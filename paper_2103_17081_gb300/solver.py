@@ -266,9 +266,10 @@ class Solver:
         FP64 (0); "coarse_spike" those solves split over 2 or 4 SMs (SPIKE) when SMs are free (1)
         or not (0; takes effect at the next hdd_setup_deflation); "outer_dots_biased" the delayed
         CGS2 first-pass dot products with biased accumulators (1: half their FP32 instructions,
-        a few 1e-12 of Σ|v w|; the second pass removes what they leave) or with the two-sum (0); "coarse_dense" the inner iteration's coarse
-        solves as products with explicit inverses on the tensor cores where that is faster (1) or
-        by the banded kernels (0)."""
+        a few 1e-12 of Σ|v w|; the second pass removes what they leave) or with the two-sum (0);
+        "coarse_dense" the inner iteration's coarse solves as products with explicit inverses (on
+        the tensor cores, or in FP64 for small orders) where that is faster (1) or by the banded
+        kernels (0)."""
         self._check(self._L.hdd_set_option(self._h, self.OPTIONS[name], int(value)), "hdd_set_option")
         return self
 
