@@ -57,12 +57,14 @@ struct FactorSet {            // banded FP64 factors of one matrix per shape, bl
     bool spike_tried = false;       // the SPIKE plans were formed, or were not wanted at set-up
     bool dense_on = false;          // a product with explicit inverses pays for the tasks there are,
     bool small_on = false;          // and it is the FP64 one
+    bool by = false;                // the digits are kept as bytes, and `by_want`: should be
+    bool by_want = false;
     DevMem sinv, stab;              // FP64 inverses and their SmallShape, if they were formed
     int small_m = 0;                // largest order
     int digits32 = 6;               // digits of the complex64 iteration
     struct Plan {
         DevMem sh, recs, tabs, tcoff, B, cs, ws, part;  // tabs: sunits, items, then tlist and tshape (ntask each)
-        int ntask = 0, ntmax = 0, nst = 0, nitem = 0;
+        int ntask = 0, ntmax = 0, nst = 0, kb = 0, nitem = 0;
         double bytes = 0, flops = 0;
         void clear() { sh.release(); recs.release(); tabs.release(); tcoff.release(); B.release(); cs.release(); ws.release(); part.release(); ntask = 0; }
     } plan[4];                      // {task table, doubled table} with 6 digits, with 7
@@ -441,7 +443,7 @@ int coarse_pays(const hdd_ctx *ctx, const FactorSet &F, const std::vector<int> &
     for (size_t q = 0; q < F.h.size(); q++) {
         const int m = F.re2 ? F.h[q].m / 2 : F.h[q].m;
         const double units = (double)((m + 127) / 128) * ((m + 15) / 16) * (F.re2 ? 2 : 1);
-        bytes += units * DENSE_ABYTES;
+        bytes += units * dense_abytes(false);
         mma += units * 28.0 * 0.5 * std::max(16.0, 2.0 * per[q]);
         chain = std::max(chain, 2.0 * F.h[q].nblk * 0.77e-6);
         chains += (F.re2 ? 1.0 : 2.0) * per[q];
@@ -501,14 +503,14 @@ hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_
         }
         S.acc0 = wo;
         wo += (long long)S.mt * S.nct * 128 * S.nt;
-        units[q] = make_int4(S.mt * S.nct, S.kc, (ds * (4096 + 32 * S.nt) + 1023) / 1024, 0);
+        units[q] = make_int4(S.mt * S.nct, S.kc, (ds * ((F.by ? 2048 : 4096) + 32 * S.nt) + 1023) / 1024, 0);
         for (int t = 0; t < S.mt * S.nct; t++)
             for (int pr = 0; pr < S.nt / 2; pr += 8) items.push_back(make_int4(q, t, pr, 0));
         P.ntmax = std::max(P.ntmax, S.nt);
         P.bytes += (double)S.kc * 16 * S.m * 2 * ds;
         P.flops += 2.0 * (ds * (ds + 1) / 2) * S.kc * 16 * S.m * cols;
     }
-    P.nst = dense_stages(ds, ns, P.ntmax);
+    dense_stages(ds, F.by, ns, P.ntmax, P.kb, P.nst);
     CK(dense_set_smem());
     CK(P.sh.ensure(ns * sizeof(DenseShape)));
     P.nitem = (int)items.size();
@@ -535,7 +537,7 @@ hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_
 
 // Explicit inverses of every shape as digits, where the product pays and fits (a quarter of the
 // free memory, 8192 operator columns, the set-up kernel's shared memory); else F.dop stays empty.
-hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, cudaStream_t s) {
+hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStream_t s) {
     const int ns = (int)F.h.size();
     const int re2 = F.re2 ? 1 : 0, cw = std::max(F.cfg.cwx, F.cfg.cwy);
     if (ns > DENSE_MAXNS || inv_cols_smem(F.cfg.maxK, cw) > 226 * 1024) return HDD_OK;
@@ -550,7 +552,7 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, cudaStream_t s) {
         if (F.h[q].m > 8192) return HDD_OK;
         o.mt = (o.m + 127) / 128; o.kseg = (o.m + 15) / 16; o.kc = o.kseg * (re2 ? 2 : 1);
         o.aoff = ao; o.soff = so;
-        ao += (long long)o.mt * o.kc * DENSE_ABYTES;
+        ao += (long long)o.mt * o.kc * dense_abytes(by);
         so += (long long)o.mt * 128;
         wsz[q] = (long long)o.kseg * 16 * F.h[q].nblk * BNB;       // 16 columns x all rows per column block
         ss[q] = SmallShape{sv, o.m, (o.m + 7) & ~7};
@@ -598,7 +600,7 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, cudaStream_t s) {
         CK(cudaMemcpyAsync(shs.p, sh.data(), sh.size() * sizeof(InvShape), cudaMemcpyHostToDevice, s));
         CK(launch_inv(jobs.as<InvJob>(), (int)jb.size(), shs.as<InvShape>(), (int)sh.size(), mmax, kmax, tmax,
                       F.table.as<BlockFactor>(), F.M.as<double>(), F.P.as<int>(), F.Meta.as<int4>(), W.as<double>(),
-                      F.cfg.maxK, cw, re2, rmax.as<unsigned long long>(), F.drs.as<int>(), F.dA.as<uint8_t>(),
+                      F.cfg.maxK, cw, re2, rmax.as<unsigned long long>(), F.drs.as<int>(), F.dA.as<uint8_t>(), by,
                       small ? F.stab.as<SmallShape>() + q0 : nullptr, F.sinv.as<double>(), s));
         CK(cudaStreamSynchronize(s));           // the tables and the workspace are used again
         q0 = q1;
@@ -608,6 +610,8 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, cudaStream_t s) {
         return HDD_OK;
     }
     F.dop = op;
+    F.by = by;
+    for (FactorSet::Plan &P : F.plan) P.ntask = 0;        // (made for the other form of the digits)
     // Against the exact inverse, 6 digits leave 1e-13 of the solution where the double-FP32 banded
     // solve leaves 1e-12 to 2e-11 (36 geometries, m = 625 to 2401), but 5.5e-14 against 3.5e-14 at
     // m = 64, where nothing is gained by the shorter operator: 7 digits below 256
@@ -643,7 +647,7 @@ hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const doub
     a.tcoff = P.tcoff.as<long long>();
     a.A = F.dA.as<uint8_t>(); a.rexp = F.drs.as<int>();
     a.B = P.B.as<uint8_t>(); a.cexp = P.cs.as<int>(); a.ws = P.ws.as<unsigned long long>(); a.part = P.part.as<int2>();
-    a.ntmax = P.ntmax; a.nst = P.nst; a.grid = ctx->nsm;
+    a.ntmax = P.ntmax; a.nst = P.nst; a.kb = P.kb; a.by = F.by; a.grid = ctx->nsm;
     a.err = ctx->d_counter.as<int>();
     KL(F_CDENSE, P.bytes, P.flops, launch_dense_solve(ds, a, in, out, flag, s));
     ctx->prof.launches += 2;
@@ -661,13 +665,17 @@ hdd_status spike_build(hdd_ctx *ctx, FactorSet &F) {
 
 // The form the inner iteration's coarse solves take, chosen by the tasks there are: the product
 // with explicit inverses, or the banded kernels with their SPIKE plans.
-bool dense_built(const FactorSet &F) { return F.small_on ? F.small_m > 0 : !F.dop.empty(); }
+bool dense_built(const FactorSet &F) { return F.small_on ? F.small_m > 0 : !F.dop.empty() && F.by == F.by_want; }
 hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
     hdd_status st = HDD_OK;
-    const int form = coarse_pays(ctx, F, tasks_per_shape(ctx));
+    const std::vector<int> per = tasks_per_shape(ctx);
+    const int form = coarse_pays(ctx, F, per);
+    // Bytes halve what a chunk reads but cost the widening: faster up to 32 columns a shape (k=100 34
+    // -> 31 us, k=160 51 -> 45, complex k=60 x 4 45 -> 39), slower at 80 (k=200 38 -> 41)
+    F.by_want = 2 * *std::max_element(per.begin(), per.end()) <= DENSE_BYCOLS;
     F.dense_on = form > 0;
     F.small_on = form == 2;
-    if (ctx->coarse_dense && F.dense_on && !dense_built(F)) st = dense_build(ctx, F, F.small_on, s);
+    if (ctx->coarse_dense && F.dense_on && !dense_built(F)) st = dense_build(ctx, F, F.small_on, F.by_want, s);
     if (!ctx->coarse_spike) F.spike_tried = true;
     if (st == HDD_OK && !F.spike_tried && !(F.dense_on && dense_built(F))) {
         CK(cudaStreamSynchronize(s));

@@ -452,10 +452,13 @@ void launch_ops_to_df(long long n, const double *M, float2 *Mdf, cudaStream_t s)
 
 // ---- the coarse solve as a product with the explicit E⁻¹ (kernels_dense.cu) ----------------
 constexpr int DSL = 7;                       // base-256 digits per entry (56 bits)
-constexpr int DENSE_ABYTES = DSL * 128 * 16 * 2;   // operator digits of 128 rows x 16 columns
+// operator digits of 128 rows x 16 columns: a byte each, widened in the kernel, or BF16
+__host__ __device__ constexpr int dense_abytes(bool by) { return DSL * 128 * 16 * (by ? 1 : 2); }
+constexpr int DENSE_BYCOLS = 32;             // columns of a shape up to which the digits are kept as bytes
+constexpr int DENSE_NX = 3;                  // most stages of the operator digits widened to BF16 (two with two chunks each)
 // most columns of a column tile: 6 sums x 80, 7 sums x 64 of the 512 TMEM columns, 256 per MMA
 constexpr int dense_nt(int ds) { return ds == 6 ? 80 : 64; }
-constexpr int DENSE_MAXST = 7;               // stages of the shared-memory ring
+constexpr int DENSE_MAXST = 12;              // stages of the shared-memory ring
 constexpr int DENSE_MINU = 4;                // fewest units (16 operator columns) a CTA is given
 constexpr int DENSE_TILEW = 6;               // units that a tile's own cost is worth in the split of the work
 constexpr int DENSE_MAXNS = 1024;            // shapes the kernel's unit table takes
@@ -486,18 +489,19 @@ struct DensePlanArgs {
     const long long *tcoff;                  // task → its packed coarse offset
     const uint8_t *A; const int *rexp;       // operator digits, row exponents
     uint8_t *B; int *cexp; unsigned long long *ws; int2 *part;
-    int ntmax, nst, grid;
+    int ntmax, nst, kb, grid;                // kb: chunks per stage
+    bool by;                                 // operator digits as bytes
     int *err;
 };
 size_t inv_cols_smem(int maxK, int cw);
 cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns, int mmax, int ksegmax, int mtmax,
                        const BlockFactor *shapes, const double *Mall, const int *Pall, const int4 *Meta, double *W,
-                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, const SmallShape *ss,
-                       double *inv, cudaStream_t s);
+                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, bool by,
+                       const SmallShape *ss, double *inv, cudaStream_t s);
 constexpr int SMALL_M = 2048;                // largest order of the FP64 product (its vector fits 48 KB of shared memory)
 void launch_small_solve(const Task *tasks, int ntask, const SmallShape *ss, int mmax, int re2, const double *inv,
                         const double2 *in, double2 *out, const int *flag, cudaStream_t s);
-int dense_stages(int ds, int ns, int ntmax);
+void dense_stages(int ds, bool by, int ns, int ntmax, int &kb, int &nst);
 cudaError_t dense_set_smem();
 void launch_dense_solve(int ds, const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s);
 

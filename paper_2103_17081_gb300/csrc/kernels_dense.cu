@@ -26,7 +26,8 @@
 
 namespace hdd {
 
-constexpr int DE_T = 320;                        // 8 epilogue warps, a copy warp, an MMA warp
+constexpr int DE_G = 3;                          // groups of four widening warps
+__host__ __device__ constexpr int de_threads(bool by) { return 320 + (by ? 128 * DE_G : 0); }   // 8 epilogue warps, a copy warp, an MMA warp, the widening warps
 constexpr unsigned long long DE_LIMIT = 2000000000ull;   // ns after which a device wait gives up
 
 // v·2^(F-e) rounded to an integer, |v| < 2^e: at most 2^F (F <= 55).  On the significand, in
@@ -228,7 +229,7 @@ k_inv_slice(const InvShape *__restrict__ sh, const double *__restrict__ Wall,
     const bool ok = i < S.m && mx < INF_BITS;
     if (k == 0) rexp[S.soff + i] = mx < INF_BITS ? e : EXP_NAN;
     for (int part = 0; part <= S.re2; part++) {
-        uint4 *dst = A + S.aoff / 16 + ((size_t)rt * S.kc + part * S.kseg + k) * (DENSE_ABYTES / 16);
+        uint4 *dst = A + S.aoff / 16 + ((size_t)rt * S.kc + part * S.kseg + k) * (dense_abytes(false) / 16);
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             long long q[8];
@@ -246,6 +247,45 @@ k_inv_slice(const InvShape *__restrict__ sh, const double *__restrict__ Wall,
                                                                   bf16_pair(d[4], d[5]), bf16_pair(d[6], d[7]));
             }
         }
+    }
+}
+
+// The same as bytes: DSL slices of 128 records of 16 signed bytes.  The leading digit
+// of an entry at 0.996 of the row's power of two or above would be 128: such a row takes the next
+// power (its entries then still have 54 bits below the largest, as a row just above a power has).
+__global__ void __launch_bounds__(128)
+k_inv_slice_bytes(const InvShape *__restrict__ sh, const double *__restrict__ Wall,
+            const unsigned long long *__restrict__ rmax, int *__restrict__ rexp, uint4 *__restrict__ A) {
+    const InvShape S = sh[blockIdx.z];
+    const int k = blockIdx.x, rt = blockIdx.y;
+    if (k >= S.kseg || rt >= S.mt) return;
+    const double *W = Wall + S.woff;
+    const int i = rt * 128 + threadIdx.x;
+    const unsigned long long mx = i < S.m ? rmax[S.roff + i] : 0;
+    const int e = exp_of(mx) + (((mx >> 44) & 0xff) >= 0xfd ? 1 : 0);
+    const bool ok = i < S.m && mx < INF_BITS;
+    if (k == 0) rexp[S.soff + i] = mx < INF_BITS ? e : EXP_NAN;
+    for (int part = 0; part <= S.re2; part++) {
+        uint4 *dst = A + S.aoff / 16 + ((size_t)rt * S.kc + part * S.kseg + k) * (dense_abytes(true) / 16);
+        uint32_t w[DSL][4];
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            long long q[4];
+#pragma unroll
+            for (int x = 0; x < 4; x++) {
+                const int j = k * 16 + 4 * h + x;
+                q[x] = ok && j < S.m ? fixed_point<55>(inv_entry(W, S.rows, S.re2, part, i, j), e) : 0;
+            }
+#pragma unroll
+            for (int p = DSL - 1; p >= 0; p--) {
+                uint32_t v = 0;
+#pragma unroll
+                for (int x = 0; x < 4; x++) v |= (uint32_t)((p > 0 ? digit256(q[x]) : (int)q[x]) & 255) << (8 * x);
+                w[p][h] = v;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < DSL; p++) dst[p * 128 + threadIdx.x] = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
     }
 }
 
@@ -431,12 +471,28 @@ __device__ __forceinline__ bool epilogue_all(bool ok) {
     return r != 0;
 }
 
+// Four signed bytes to BF16: 128 + (b & 127) and 128 or 256 share their upper byte 0x43, and their
+// difference is b, exactly.
+__device__ __forceinline__ uint2 widen_digits(uint32_t b) {
+    auto two = [](uint32_t w) {
+        const uint32_t lo = w & 0xff7fff7fu, hi = w & 0xff80ff80u;
+        const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&lo),
+                                         *reinterpret_cast<const __nv_bfloat162 *>(&hi));
+        return *reinterpret_cast<const uint32_t *>(&r);
+    };
+    return make_uint2(two(__byte_perm(b, 0x43434343u, 0x4140)), two(__byte_perm(b, 0x43434343u, 0x4342)));
+}
+
 // out = E⁻¹ in for the flagged tasks.  Persistent, one CTA per SM.  The work is the list of
 // (tile of 128 rows, column tile, chunk of 16 operator columns) units of the shapes with a flagged
 // task, cut into gridDim.x ranges of equal bytes: a CTA's range is a few tiles, the first and last of them
 // shared with its neighbours.  One warp streams the operator's and the right-hand sides' digits
 // through a ring of shared-memory stages with bulk copies, one warp issues the MMAs, eight warps
-// put the DS sums together.  MMAs: the sums of weight s lie in TMEM columns s·nt.., the digits of
+// put the DS sums together.  Byte digits (BY): three groups of four warps take the stages in turn and
+// widen the operator's digits to BF16 in a second ring, a thread a row, 2 instructions a digit; half
+// the bytes are read, and a stage holds two chunks (k=100, 16 columns a tile, with the kernels around
+// it 33.9 -> 31.6 us; k=160 50.8 -> 45.0).  MMAs: the sums of weight s lie in TMEM columns
+// s·nt.., the digits of
 // the right-hand sides side by side in the operand, so operator digit p against digits 0..DS-1-p
 // is one product of (DS - p)·nt columns into the columns from p·nt on (cut at 256, the widest
 // MMA): the operator digit is read once for all of them.  The issuing loop is walked by a whole
@@ -447,30 +503,34 @@ __device__ __forceinline__ bool epilogue_all(bool ok) {
 // No CTA waits for another.
 // Every mbarrier wait is bounded; on a timeout the CTA sets *err and leaves (1; 2 if work it had
 // issued did not finish either, see kernels_cnn_tc.cu).
-template <int DS>
-__global__ void __launch_bounds__(DE_T, 1)
+template <int DS, bool BY>
+__global__ void __launch_bounds__(de_threads(BY), 1)
 k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ sunits,
             const int *__restrict__ tshape, const int *__restrict__ tlist, const long long *__restrict__ tcoff,
             const int *__restrict__ flag, int ntask, const uint8_t *__restrict__ A, const int *__restrict__ rexp,
             const uint8_t *__restrict__ B, const int *__restrict__ cexp, double2 *__restrict__ out,
-            unsigned long long *__restrict__ ws, int2 *__restrict__ part, int ntmax, int nst, int *__restrict__ err) {
+            unsigned long long *__restrict__ ws, int2 *__restrict__ part, int ntmax, int nst, int kbs, int *__restrict__ err) {
+    constexpr int T = de_threads(BY);
+    const int kb = BY ? kbs : 1;
     extern __shared__ __align__(128) uint8_t sm[];
-    __shared__ uint64_t full[DENSE_MAXST], empty[DENSE_MAXST], accf, acce, drain;
+    __shared__ uint64_t full[DENSE_MAXST], empty[DENSE_MAXST], xfull[DENSE_NX], accf, acce, drain;
     __shared__ uint32_t tbase;
     __shared__ volatile int bad;
     __shared__ long long ccoff[2][40];               // per column pair of a segment: its task's output, -1: none,
     __shared__ int2 ccexp[2][40];                    // and its columns' exponents
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int2 *pre = reinterpret_cast<int2 *>(sm);                  // ns + 1 offsets {units, weight}
-    uint8_t *ring = sm + (((size_t)(ns + 1) * 8 + 127) & ~(size_t)127);
-    constexpr uint32_t AB = DS * 4096u;                           // operator bytes per chunk used
-    const uint32_t stage = AB + 2u * DS * 16u * (uint32_t)ntmax;
+    uint8_t *wide = sm + (((size_t)(ns + 1) * 8 + 127) & ~(size_t)127);       // BF16 operator digits
+    constexpr uint32_t AB = DS * (BY ? 2048u : 4096u), XB = DS * 4096u;       // operator bytes per chunk used, and widened
+    const int nx = kb == 2 ? 2 : DENSE_NX;                        // (at most nst)
+    uint8_t *ring = wide + (BY ? (size_t)nx * kb * XB : 0);
+    const uint32_t stage = (uint32_t)kb * (AB + 2u * DS * 16u * (uint32_t)ntmax);
     // units and weight of the shapes with work: a unit weighs the bytes it streams, in KB, and a tile
     // DENSE_TILEW units more (the sums of the tile before it leave TMEM meanwhile)
-    for (int q = tid; q <= ns; q += DE_T) pre[q].x = flag ? 0 : 1;
+    for (int q = tid; q <= ns; q += T) pre[q].x = flag ? 0 : 1;
     __syncthreads();
     if (flag)
-        for (int t = tid; t < ntask; t += DE_T) {
+        for (int t = tid; t < ntask; t += T) {
             const int f = flag[t], q = tshape[t];
             if (f) pre[q].x = 1;
         }
@@ -498,7 +558,7 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
     const long long G = min((int)gridDim.x, max(1, U / DENSE_MINU));
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (blockIdx.x == 0) {                                     // for k_dense_finish
-        for (int q = tid; q <= ns; q += DE_T) part[q] = pre[q];
+        for (int q = tid; q <= ns; q += T) part[q] = pre[q];
         if (tid == 0) part[ns + 1] = make_int2((int)G, 0);
     }
     if (U == 0 || blockIdx.x >= G) {                 // (waits all the same: the end of this kernel is the end of those before)
@@ -526,6 +586,8 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
     if (warp == 0) umma::tmem_alloc(&tbase, 512);
     if (tid == 0) {
         for (int s = 0; s < nst; s++) { umma::mbar_init(&full[s], 1); umma::mbar_init(&empty[s], 1); }
+        if (BY)
+            for (int s = 0; s < nx; s++) umma::mbar_init(&xfull[s], 4);
         umma::mbar_init(&accf, 1);
         umma::mbar_init(&acce, 8);
         umma::mbar_init(&drain, 1);
@@ -564,18 +626,20 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
                     const Seg g = seg_at(u);
                     const DenseShape S = sh[g.q];
                     const uint32_t bb = 2u * DS * 16u * (uint32_t)S.nt;
-                    const uint8_t *a = A + S.aoff + ((size_t)g.rt * S.kc + g.k0) * DENSE_ABYTES;
+                    const uint8_t *a = A + S.aoff + ((size_t)g.rt * S.kc + g.k0) * dense_abytes(BY);
                     const uint8_t *b = B + S.boff + ((size_t)g.ct * S.kc + g.k0) * bb;
-                    for (int k = g.k0; k < g.k1 && (pass || it < nst); k++, it++, a += DENSE_ABYTES, b += bb) {
-                        const int st = it % nst, use = it / nst;
+                    for (int k = g.k0; k < g.k1 && (pass || it < nst); k += kb, it++) {
+                        const int st = it % nst, use = it / nst, n = min(kb, g.k1 - k);
                         uint8_t *d = ring + (size_t)st * stage;
                         if (use > 0 && !(ok = wait(&empty[st], (use - 1) & 1))) break;
                         if (!pass || it >= ahead) {
-                            umma::mbar_expect_tx(&full[st], AB + bb);
-                            umma::bulk_g2s(d, a, AB, &full[st]);
+                            umma::mbar_expect_tx(&full[st], (uint32_t)n * (AB + bb));
+                            for (int j = 0; j < n; j++) umma::bulk_g2s(d + j * AB, a + (size_t)j * dense_abytes(BY), AB, &full[st]);
                             issued++;
                         }
-                        if (pass) umma::bulk_g2s(d + AB, b, bb, &full[st]);
+                        if (pass) umma::bulk_g2s(d + kb * AB, b, (uint32_t)n * bb, &full[st]);
+                        a += (size_t)n * dense_abytes(BY);
+                        b += (size_t)n * bb;
                     }
                     u += g.k1 - g.k0;
                 }
@@ -588,11 +652,11 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
     } else if (warp == 9) {
         // the whole warp walks the loop, so that addresses stay in uniform registers; one lane issues
         const bool leader = umma::elect_one();
-        const uint32_t ring0 = umma::smem_u32(ring) >> 4, st16 = stage >> 4;
+        const uint32_t ring0 = umma::smem_u32(ring) >> 4, st16 = stage >> 4, wide0 = umma::smem_u32(wide) >> 4;
         const uint32_t ahi = (128u >> 4) | 0x4000u, alb = (2048u >> 4) << 16;
         bool ok = true;
-        int seg = 0, st = 0;
-        uint32_t par = 0;
+        int seg = 0, st = 0, sx = 0;
+        uint32_t par = 0, parx = 0;
         for (int u = ub; ok && u < ue; seg++) {
             const Seg g = seg_at(u);
             const uint32_t nt = (uint32_t)__shfl_sync(0xffffffffu, sh[g.q].nt, 0);
@@ -600,28 +664,64 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
             const uint32_t blb = (DS * nt) << 16;
             if (seg > 0 && !(ok = __all_sync(0xffffffffu, wait(&acce, (seg - 1) & 1)))) break;
             umma::fence_after_sync();
-            for (int k = 0; k < nk; k++) {
-                ok = __all_sync(0xffffffffu, wait(&full[st], par));
+            for (int k = 0; k < nk; k += kb) {
+                const int n = min(kb, nk - k);
+                ok = __all_sync(0xffffffffu, BY ? wait(&xfull[sx], parx) : wait(&full[st], par));   // (widened: the stage had arrived)
                 if (!ok) break;
                 umma::fence_after_sync();
                 if (leader) {
-                    const uint32_t a = ring0 + (uint32_t)st * st16;
-                    const uint32_t al = alb | a, bl = blb | (a + (AB >> 4));
+                    for (int j = 0; j < n; j++) {
+                        const uint32_t r = ring0 + (uint32_t)st * st16;
+                        const uint32_t al = alb | (BY ? wide0 + (uint32_t)(sx * kb + j) * (XB >> 4) : r + (uint32_t)j * (AB >> 4));
+                        const uint32_t bl = blb | (r + (uint32_t)kb * (AB >> 4) + (uint32_t)j * (2u * DS) * nt);
 #pragma unroll
-                    for (uint32_t p = 0; p < DS; p++) {
-                        const uint32_t cols = (DS - p) * nt, n0 = min(256u, cols), d = td + p * nt;
-                        umma::mma_bf16_lohi(d, al + p * 256u, bl, ahi, umma::idesc_bf16_f32(128, (int)n0), p > 0 || k > 0);
-                        if (cols > 256)
-                            umma::mma_bf16_lohi(d + 256u, al + p * 256u, bl + 256u, ahi,
-                                                umma::idesc_bf16_f32(128, (int)(cols - 256u)), p > 0 || k > 0);
+                        for (uint32_t p = 0; p < DS; p++) {
+                            const uint32_t cols = (DS - p) * nt, n0 = min(256u, cols), d = td + p * nt, acc = p > 0 || k + j > 0;
+                            umma::mma_bf16_lohi(d, al + p * 256u, bl, ahi, umma::idesc_bf16_f32(128, (int)n0), acc);
+                            if (cols > 256)
+                                umma::mma_bf16_lohi(d + 256u, al + p * 256u, bl + 256u, ahi,
+                                                    umma::idesc_bf16_f32(128, (int)(cols - 256u)), acc);
+                        }
                     }
                     umma::commit(&empty[st]);
                 }
                 __syncwarp();
                 if (++st == nst) { st = 0; par ^= 1u; }
+                if (++sx == nx) { sx = 0; parx ^= 1u; }
             }
             if (ok && leader) umma::commit(&accf);
             __syncwarp();
+            u += g.k1 - g.k0;
+        }
+    } else if (BY && warp >= 10) {
+        const int row = ((warp - 10) & 3) * 32 + lane, grp = (warp - 10) >> 2;
+        int it = 0;
+        bool ok = true;
+        for (int u = ub; ok && u < ue;) {
+            const Seg g = seg_at(u);
+            for (int k = g.k0; k < g.k1; k += kb, it++) {
+                if (it % DE_G != grp) continue;
+                const int st = it % nst, sx = it % nx, old = it - nx, n = min(kb, g.k1 - k);
+                if (old >= 0) ok = wait(&empty[old % nst], (old / nst) & 1);       // its place in the second ring is free
+                if (ok) ok = wait(&full[st], (it / nst) & 1);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                for (int j = 0; j < n; j++) {
+                    const uint4 *s = reinterpret_cast<const uint4 *>(ring + (size_t)st * stage + (size_t)j * AB) + row;
+                    uint4 *d = reinterpret_cast<uint4 *>(wide + (size_t)(sx * kb + j) * XB) + row;
+                    uint4 v[DS];
+#pragma unroll
+                    for (int p = 0; p < DS; p++) v[p] = s[p * 128];
+#pragma unroll
+                    for (int p = 0; p < DS; p++) {
+                        const uint2 a = widen_digits(v[p].x), b = widen_digits(v[p].y), c = widen_digits(v[p].z), e = widen_digits(v[p].w);
+                        d[(2 * p) * 128] = make_uint4(a.x, a.y, b.x, b.y);
+                        d[(2 * p + 1) * 128] = make_uint4(c.x, c.y, e.x, e.y);
+                    }
+                }
+                umma::fence_async_smem();
+                __syncwarp();
+                if (lane == 0) umma::mbar_arrive(&xfull[sx]);
+            }
             u += g.k1 - g.k0;
         }
     } else {
@@ -780,8 +880,8 @@ size_t inv_cols_smem(int maxK, int cw) { return ((size_t)2 * BNB * maxK + (size_
 
 cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns, int mmax, int ksegmax, int mtmax,
                        const BlockFactor *shapes, const double *Mall, const int *Pall, const int4 *Meta, double *W,
-                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, const SmallShape *ss,
-                       double *inv, cudaStream_t s) {
+                       int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, bool by,
+                       const SmallShape *ss, double *inv, cudaStream_t s) {
     const size_t smem = inv_cols_smem(maxK, cw);
     cudaError_t e = re2 ? cudaFuncSetAttribute(k_inv_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                         : cudaFuncSetAttribute(k_inv_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -793,38 +893,50 @@ cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns
         return cudaGetLastError();
     }
     k_inv_rowmax<<<dim3((mmax + 127) / 128, (mmax + 15) / 16, ns), 128, 0, s>>>(sh, W, rmax);
-    k_inv_slice<<<dim3(ksegmax, mtmax, ns), 128, 0, s>>>(sh, W, rmax, rexp, reinterpret_cast<uint4 *>(A));
+    if (by) k_inv_slice_bytes<<<dim3(ksegmax, mtmax, ns), 128, 0, s>>>(sh, W, rmax, rexp, reinterpret_cast<uint4 *>(A));
+    else k_inv_slice<<<dim3(ksegmax, mtmax, ns), 128, 0, s>>>(sh, W, rmax, rexp, reinterpret_cast<uint4 *>(A));
     return cudaGetLastError();
 }
 
-static size_t dense_smem(int ds, int ns, int ntmax, int nst) {
+static size_t dense_smem(int ds, bool by, int ns, int ntmax, int kb, int nst) {
     return (((size_t)(ns + 1) * 8 + 127) & ~(size_t)127) +
-           (size_t)nst * ((size_t)ds * 4096 + 2 * (size_t)ds * 16 * ntmax);
+           (size_t)kb * ((by ? (kb == 2 ? 2 : DENSE_NX) * (size_t)ds * 4096 : 0) +
+                         (size_t)nst * ((size_t)ds * (by ? 2048 : 4096) + 2 * (size_t)ds * 16 * ntmax));
 }
-int dense_stages(int ds, int ns, int ntmax) {
-    int nst = DENSE_MAXST;
-    while (nst > 2 && dense_smem(ds, ns, ntmax, nst) > 223 * 1024) nst--;
-    return nst;
+// Chunks per stage and stages.  A stage costs the issuing warp a wait and a commit, some 220 clocks
+// each, and the widening warps their waits and a proxy fence, where a chunk of 16 columns is 315
+// clocks of MMAs at nt = 16: two chunks a stage with byte digits where three such stages fit (up to 32
+// columns a tile).  With BF16 digits two a stage gave 1 % there and lost 1 % at 80 columns: one.
+void dense_stages(int ds, bool by, int ns, int ntmax, int &kb, int &nst) {
+    for (kb = by ? 2 : 1;; kb--) {
+        nst = by ? DENSE_MAXST : 7;
+        while (nst > (by ? 3 : 2) && dense_smem(ds, by, ns, ntmax, kb, nst) > 223 * 1024) nst--;
+        if (kb == 1 || dense_smem(ds, by, ns, ntmax, kb, nst) <= 223 * 1024) return;
+    }
 }
 cudaError_t dense_set_smem() {
-    const cudaError_t e = cudaFuncSetAttribute(k_dense_mma<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_dense_mma<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_dense_mma<6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_dense_mma<7, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_dense_mma<6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_dense_mma<7, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024);
 }
 template <int DS>
 static void dense_launch(const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
     launch_chained(k_dense_slice<DS>, dim3(p.ntask, DSPLIT), 128, 0, s, p.recs, in, reinterpret_cast<uint4 *>(p.B), p.cexp, flag);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.grid);
-    cfg.blockDim = dim3(DE_T);
-    cfg.dynamicSmemBytes = dense_smem(DS, p.ns, p.ntmax, p.nst);
+    cfg.blockDim = dim3(de_threads(p.by));
+    cfg.dynamicSmemBytes = dense_smem(DS, p.by, p.ns, p.ntmax, p.kb, p.nst);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_dense_mma<DS>, p.sh, p.ns, p.sunits, p.tshape, p.tlist, p.tcoff, flag, p.ntask, p.A, p.rexp,
-                       (const uint8_t *)p.B, (const int *)p.cexp, out, p.ws, p.part, p.ntmax, p.nst, p.err);
+    auto mma = p.by ? k_dense_mma<DS, true> : k_dense_mma<DS, false>;
+    cudaLaunchKernelEx(&cfg, mma, p.sh, p.ns, p.sunits, p.tshape, p.tlist, p.tcoff, flag, p.ntask, p.A, p.rexp,
+                       (const uint8_t *)p.B, (const int *)p.cexp, out, p.ws, p.part, p.ntmax, p.nst, p.kb, p.err);
     cfg.gridDim = dim3(std::min(p.nitem, 2 * p.grid));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
