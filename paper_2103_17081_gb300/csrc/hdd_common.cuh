@@ -458,6 +458,8 @@ constexpr int DENSE_BYCOLS = 32;             // columns of a shape up to which t
 constexpr int DENSE_NX = 3;                  // most stages of the operator digits widened to BF16 (two with two chunks each)
 // most columns of a column tile: 6 sums x 80, 7 sums x 64 of the 512 TMEM columns, 256 per MMA
 constexpr int dense_nt(int ds) { return ds == 6 ? 80 : 64; }
+// most chunks of 16 operator columns that go into one FP32 sum (even: whole stages; kernels_dense.cu)
+__host__ __device__ constexpr int dense_seg(int re2) { return re2 ? 32 : 64; }
 constexpr int DENSE_MAXST = 12;              // stages of the shared-memory ring
 constexpr int DENSE_MINU = 4;                // fewest units (16 operator columns) a CTA is given
 constexpr int DENSE_TILEW = 6;               // units that a tile's own cost is worth in the split of the work

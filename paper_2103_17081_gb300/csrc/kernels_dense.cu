@@ -10,12 +10,18 @@
 // multiples of 2^(ea-55); each column of y likewise (2^eb).  The 56-bit integers are written in
 // base 256 with DSL = 7 signed digits of at most 128, which BF16 holds exactly.  A product of two
 // digits has at most 14 bits, so the FP32 accumulators of the tensor cores hold the sums of
-// products of equal weight exactly up to 2^24 (about 30 standard deviations of a sum over 1700
-// columns; past it a sum rounds like any FP32 sum).  Sums of weight p + q < DS are kept, the rest
+// products of equal weight exactly up to 2^24.  On smooth data the leading digits add up instead of
+// cancelling (a constant against E⁻¹ at k = 4 reaches 1.45·2^24 over 4096 columns, where whole rows
+// in one sum then cost 1e-10 to 4e-8 of the solution), so a sum runs over at most dense_seg() chunks
+// before it moves to integers: 64 chunks of 16 columns, where the products of the leading digits stay
+// within 2^24 whatever the data (0.64·2^24 at most was seen for all of them together: constants,
+// half-sines, rows of E⁻¹ itself), 32 for complex E, whose rows can be constant to more
+// than a digit (impedance condition, small k).  Sums of weight p + q < DS are kept, the rest
 // lies below a 2^-8DS part of a column's and a row's largest entries: DS = 7 for the complex128
 // iteration, DS = 6 (48 bits, what the double-FP32 banded solve carries) for the complex64 one.
-// The DS sums are put together in 64-bit integers, so partial sums over column ranges add up to
-// the same bits in whatever order and split they come.
+// The DS sums are put together in 64-bit integers, in units of 2^13 of the last one's: a part of a
+// tile rounds its two last sums to such a unit (2^-60 of a full product), and the parts add up to
+// the same bits in whatever order they come.
 #include "hdd_common.cuh"
 #include "umma.cuh"
 
@@ -498,7 +504,7 @@ __device__ __forceinline__ uint2 widen_digits(uint32_t b) {
 // MMA): the operator digit is read once for all of them.  The issuing loop is walked by a whole
 // warp with one elected lane: from a single divergent lane the descriptors went through ordinary
 // registers and an MMA took 228 clocks to issue, twice what a 240-column one runs (120).
-// A tile that is not whole goes is added to
+// A tile that is not whole in one segment (a CTA's part of it, at most dense_seg() chunks) is added to
 // 64-bit integers in L2 (atomics; the order does not matter) and written out by k_dense_finish.
 // No CTA waits for another.
 // Every mbarrier wait is bounded; on a timeout the CTA sets *err and leaves (1; 2 if work it had
@@ -604,7 +610,13 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
         const int l = u - pre[lo].x, tile = l / kc;
         Seg g;
         g.q = lo; g.rt = tile / nct; g.ct = tile - g.rt * nct; g.k0 = l - tile * kc;
-        g.k1 = min(kc, g.k0 + (ue - u));
+        int n = min(kc - g.k0, ue - u);
+        const int cap = dense_seg(sh[lo].re2);
+        if (n > cap) {                               // in equal parts, of whole stages
+            const int parts = (n + cap - 1) / cap;
+            n = ((n + parts - 1) / parts + kb - 1) / kb * kb;
+        }
+        g.k1 = g.k0 + n;
         return g;
     };
     auto wait = [&](uint64_t *b, uint32_t par) {
@@ -859,10 +871,10 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
         const int2 p0 = part[it.x], p1 = part[it.x + 1];
         const unsigned G = (unsigned)part[ns + 1].x, Wt = (unsigned)part[ns].y;
         if (p1.x == p0.x) continue;                                              // no task of this shape
-        // the CTAs that hold the tile's first and last unit: one and the same wrote it out itself
+        // the CTAs that hold the tile's first and last unit: one and the same wrote a tile of one segment out itself
         const unsigned long long w0 = (unsigned)(p0.y + it.y * (n.y + DENSE_TILEW) * n.z + DENSE_TILEW * n.z),
                                  w1 = w0 + (unsigned)((n.y - 1) * n.z);
-        if (((w0 + 1) * G - 1) / Wt == ((w1 + 1) * G - 1) / Wt) continue;
+        if (n.y <= dense_seg(S.re2) && ((w0 + 1) * G - 1) / Wt == ((w1 + 1) * G - 1) / Wt) continue;
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const int pr = it.z + (tid >> 7) + 2 * e;
