@@ -357,10 +357,11 @@ static void emu_bwd_cols(const double *M, const int4 *meta, int J0, int J1, int 
 // both windows fit the kernel's staging (SPIKE_WMAX).  Gf_p[:, k] is the forward response of part
 // p to the unit value at row r_p - wf + k; Gb_p[:, k] the backward response of part p to the unit
 // value at row r_{p+1} + k (column-major, stored as (hi, lo) FP32 pairs).
-hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &meta, long long mo) {
+hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &meta, long long mo, cudaStream_t s) {
     const int ns = (int)F.h.size();
     std::vector<double> M((size_t)std::max(mo, 1LL));
-    CK(cudaMemcpy(M.data(), F.M.p, (size_t)mo * sizeof(double), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpyAsync(M.data(), F.M.p, (size_t)mo * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
     std::vector<SpikeInfo> tab((size_t)ns * SPIKE_LEVELS);
     std::vector<float2> Gall;
     auto put = [&](const std::vector<double> &Y, long long ybase, int W, long long r0, int np) {
@@ -412,14 +413,14 @@ hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &met
     for (int L = 0; L < SPIKE_LEVELS; L++) F.spike_levels_built += F.spike_level[L];
     if (F.spike_levels_built == 0) return HDD_OK;
     CK(F.G.ensure(std::max<size_t>(Gall.size(), 1) * sizeof(float2)));
-    CK(cudaMemcpy(F.G.p, Gall.data(), Gall.size() * sizeof(float2), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(F.G.p, Gall.data(), Gall.size() * sizeof(float2), cudaMemcpyHostToDevice, s));
     CK(F.spk.ensure(tab.size() * sizeof(SpikeInfo)));
     // level-major on the device: the table of level L is ns consecutive entries
     std::vector<SpikeInfo> dev(tab.size());
     for (int L = 0; L < SPIKE_LEVELS; L++)
         for (int q = 0; q < ns; q++) dev[(size_t)L * ns + q] = tab[(size_t)q * SPIKE_LEVELS + L];
-    CK(cudaMemcpy(F.spk.p, dev.data(), dev.size() * sizeof(SpikeInfo), cudaMemcpyHostToDevice));
-    (void)ctx;
+    CK(cudaMemcpyAsync(F.spk.p, dev.data(), dev.size() * sizeof(SpikeInfo), cudaMemcpyHostToDevice, s));
+    CK(cudaStreamSynchronize(s));
     return HDD_OK;
 }
 
@@ -522,14 +523,16 @@ hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_
     CK(P.cs.ensure(2 * (size_t)nt * sizeof(int)));
     CK(P.ws.ensure((size_t)wo * sizeof(unsigned long long)));
     CK(P.recs.ensure(recs.size() * sizeof(DenseTask)));
-    CK(cudaMemcpy(P.recs.p, recs.data(), recs.size() * sizeof(DenseTask), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(P.sh.p, sh.data(), ns * sizeof(DenseShape), cudaMemcpyHostToDevice));
+    // (on the stream of the solve that uses them: a copy on the default stream would not be ordered
+    // with a non-blocking one)
+    CK(cudaMemcpyAsync(P.recs.p, recs.data(), recs.size() * sizeof(DenseTask), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(P.sh.p, sh.data(), ns * sizeof(DenseShape), cudaMemcpyHostToDevice, s));
     char *tb = P.tabs.as<char>();
-    CK(cudaMemcpy(tb, units.data(), ns * sizeof(int4), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(tb + ns * sizeof(int4), items.data(), P.nitem * sizeof(int4), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(tb + b4, tlist.data(), b1, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(tb + b4 + b1, tshape.data(), b1, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(P.tcoff.p, tcoff.data(), tcoff.size() * sizeof(long long), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(tb, units.data(), ns * sizeof(int4), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(tb + ns * sizeof(int4), items.data(), P.nitem * sizeof(int4), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(tb + b4, tlist.data(), b1, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(tb + b4 + b1, tshape.data(), b1, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(P.tcoff.p, tcoff.data(), tcoff.size() * sizeof(long long), cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(P.ws.p, 0, P.ws.bytes, s));
     P.ntask = nt;
     return HDD_OK;
@@ -656,11 +659,11 @@ hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const doub
 
 // SPIKE plans of the coarse factors (their double-FP32 solves), where the host emulation that
 // forms the spike matrices stays cheap (about m·(wf² + wb²) multiply-adds per shape).
-hdd_status spike_build(hdd_ctx *ctx, FactorSet &F) {
+hdd_status spike_build(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
     F.spike_tried = true;
     double cost = 0.0;
     for (const BlockFactor &b : F.h) cost += (double)b.m * ((double)b.wl * b.wl + (double)b.wu * b.wu);
-    return cost <= 1.5e9 ? build_spikes(ctx, F, F.meta, F.mo) : HDD_OK;
+    return cost <= 1.5e9 ? build_spikes(ctx, F, F.meta, F.mo, s) : HDD_OK;
 }
 
 // The form the inner iteration's coarse solves take, chosen by the tasks there are: the product
@@ -678,8 +681,7 @@ hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
     if (ctx->coarse_dense && F.dense_on && !dense_built(F)) st = dense_build(ctx, F, F.small_on, F.by_want, s);
     if (!ctx->coarse_spike) F.spike_tried = true;
     if (st == HDD_OK && !F.spike_tried && !(F.dense_on && dense_built(F))) {
-        CK(cudaStreamSynchronize(s));
-        st = spike_build(ctx, F);
+        st = spike_build(ctx, F, s);
     }
     return st;
 }
@@ -786,7 +788,7 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     if (mo >= (1LL << 31)) FAIL(HDD_ERR_INVALID_ARG, "blocked factors exceed 2^31 doubles");
     CK(F.M.ensure((size_t)std::max(mo, 1LL) * sizeof(double)));
     CK(F.Meta.ensure(meta.size() * sizeof(int4)));
-    CK(cudaMemcpy(F.Meta.p, meta.data(), meta.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(F.Meta.p, meta.data(), meta.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
     for (int q = 0; q < ns; q++) lu[q].meta = F.h[q].meta_off;
     CK(cudaMemcpyAsync(dlu.p, lu.data(), ns * sizeof(LuShape), cudaMemcpyHostToDevice, s));
     launch_block_operators(dlu.as<LuShape>(), ns, max_m, AB.as<double>(), LP.as<double>(), F.Meta.as<int4>(),
@@ -1171,7 +1173,7 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     // both precisions), or the banded kernels; without coarse_df the complex64 iteration asks for those
     const bool dense = use_dense(ctx) && (cdf || sizeof(R) == 8);
     const int ds = sizeof(R) == 8 ? 7 : ctx->E.digits32;
-    if (!dense && cdf && ctx->coarse_spike && !ctx->E.spike_tried && (st = spike_build(ctx, ctx->E)) != HDD_OK) return st;
+    if (!dense && cdf && ctx->coarse_spike && !ctx->E.spike_tried && (st = spike_build(ctx, ctx->E, s)) != HDD_OK) return st;
     auto coarse = [&](const double2 *in, double2 *out, const int *flag, int n) -> hdd_status {
         if (dense) return dense_solve(ctx, ctx->E, ds, 0, in, out, flag, s);
         band_solve(ctx, ctx->E, in, out, false, flag, s, n, cdf);
@@ -1652,6 +1654,7 @@ hdd_status build_tasks(hdd_ctx *ctx, int nrhs) {
     CK(ctx->d_tasks2.ensure(2 * (size_t)nt * sizeof(Task)));
     CK(ctx->d_mask2.ensure(2 * (size_t)nt * sizeof(int)));
     CK(cudaMemcpy(ctx->d_tasks2.p, t2.data(), 2 * (size_t)nt * sizeof(Task), cudaMemcpyHostToDevice));
+    CK(cudaStreamSynchronize(0));                // the tables are there for any stream
     ctx->nrhs = nrhs;
     return HDD_OK;
 }
@@ -1760,6 +1763,7 @@ hdd_status hdd_assemble(hdd_ctx *ctx, const hdd_assemble_params *p) {
         CK(ctx->d_bmass.ensure(sizeof(bma)));
         CK(cudaMemcpy(ctx->d_bcoef.p, bco, sizeof(bco), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(ctx->d_bmass.p, bma, sizeof(bma), cudaMemcpyHostToDevice));
+        CK(cudaStreamSynchronize(0));            // there for any stream
         ctx->st.bcoef = ctx->d_bcoef.as<double2>();
         ctx->st.bmass = ctx->d_bmass.as<double>();
         ctx->cnn.ready = false;               // the warm start serves the Dirichlet problem only
@@ -2663,7 +2667,7 @@ hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void
     if (op == 3) {
         // the hook applies the banded kernels, whichever form the inner iteration takes
         if (prec == 64 && ctx->coarse_spike && !ctx->E.spike_tried) {
-            hdd_status st = spike_build(ctx, ctx->E);
+            hdd_status st = spike_build(ctx, ctx->E, s);
             if (st != HDD_OK) return st;
         }
         band_solve(ctx, ctx->E, in, out, false, nullptr, s, -1, prec == 64);
