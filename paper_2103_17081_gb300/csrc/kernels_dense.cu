@@ -387,19 +387,66 @@ void launch_small_solve(const Task *tasks, int ntask, const SmallShape *ss, int 
 // The solve
 // ------------------------------------------------------------------------------------------
 
-// Digits of the right-hand sides: CTA (task, share of its rows), the task's Re and Im columns of
+// Digits of the right-hand sides: CTA 1 + DSPLIT·task + share of its rows, the task's Re and Im columns of
 // the shape's product, each scaled by its own power of two (real factors), or both by one
 // (complex: columns [Re; -Im] and [Im; Re] against [Re E⁻¹ | Im E⁻¹]).  Layout per column tile and
 // chunk of 16 rows: 2 x DS x nt records of 8 BF16.  cexp: the column's exponent (EXP_NAN for a
 // column that is not finite, so that it stays visible).  Tasks not
 // flagged are left as they are: their columns are computed from whatever is there and not written
 // out.  Bound by latency (a column maximum, then one record per thread): four shares per task.
+// CTA 0 instead forms the table of units that k_dense_mma splits its work by, from the flags: those come from
+// the kernel in front of this one, whose results a kernel may read behind its own wait only, and
+// k_dense_mma's wait is for this one.
 constexpr int DSPLIT = 4;
+
+// part[q] = {units, weight} of the shapes before q that have a flagged task, q = 0..ns; part[ns + 1].x:
+// the CTAs that share them.  A unit weighs the bytes it streams, in KB, and a tile DENSE_TILEW units
+// more (the sums of the tile before it leave TMEM meanwhile).
+__device__ __forceinline__ void dense_units(int ns, const int4 *__restrict__ sunits, const int *__restrict__ tshape, int ntask,
+                                            const int *flag, int grid, int2 *__restrict__ part) {
+    __shared__ unsigned on[DENSE_MAXNS / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int q = tid; q < DENSE_MAXNS / 32; q += blockDim.x) on[q] = flag ? 0u : ~0u;
+    __syncthreads();
+    if (flag)
+#pragma unroll 4
+        for (int t = tid; t < ntask; t += blockDim.x) {
+            const int q = tshape[t];
+            if (flag[t]) atomicOr(&on[q >> 5], 1u << (q & 31));
+        }
+    __syncthreads();
+    if (tid >= 32) return;
+    int carry = 0, carryw = 0;
+    for (int q0 = 0; q0 <= ns; q0 += 32) {
+        const int q = q0 + lane;
+        const int4 n = q < ns ? sunits[q] : make_int4(0, 0, 1, 0);      // tiles, chunks, weight of a unit
+        const int has = q < ns && (on[q0 >> 5] >> lane & 1u), u = has ? n.x * n.y : 0, w = has ? n.x * (n.y + DENSE_TILEW) * n.z : 0;
+        int s = u, z = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, s, o), x = __shfl_up_sync(0xffffffffu, z, o);
+            if (lane >= o) { s += v; z += x; }
+        }
+        if (q <= ns) part[q] = make_int2(carry + s - u, carryw + z - w);
+        carry += __shfl_sync(0xffffffffu, s, 31);
+        carryw += __shfl_sync(0xffffffffu, z, 31);
+    }
+    if (lane == 0) part[ns + 1] = make_int2(min(grid, max(1, carry / DENSE_MINU)), 0);
+}
+
 template <int DS>
 __global__ void __launch_bounds__(128)
 k_dense_slice(const DenseTask *__restrict__ recs, const double2 *__restrict__ in, uint4 *__restrict__ B, int *__restrict__ cexp,
-              const int *__restrict__ flag) {
-    const int t = blockIdx.x, tid = threadIdx.x;
+              const int *__restrict__ flag, int ns, const int4 *__restrict__ sunits, const int *__restrict__ tshape, int ntask,
+              int grid, int2 *__restrict__ part) {
+    const int tid = threadIdx.x;
+    if (blockIdx.x == 0) {
+        CHAIN_ENTER();
+        LAUNDER(flag);
+        dense_units(ns, sunits, tshape, ntask, flag, grid, part);
+        return;
+    }
+    const int t = (blockIdx.x - 1) / DSPLIT, share = (blockIdx.x - 1) % DSPLIT;
     const DenseTask S = recs[t];
     CHAIN_ENTER();
     LAUNDER(in); LAUNDER(flag);
@@ -425,13 +472,13 @@ k_dense_slice(const DenseTask *__restrict__ recs, const double2 *__restrict__ in
     if (S.re2) mx = my = max(mx, my);
     const int ex = exp_of(mx), ey = exp_of(my);
     const bool okx = mx < INF_BITS, oky = my < INF_BITS;
-    if (tid == 0 && blockIdx.y == 0) {
+    if (tid == 0 && share == 0) {
         cexp[2 * t] = okx ? ex - 49 : EXP_NAN;
         cexp[2 * t + 1] = oky ? ey - 49 : EXP_NAN;
     }
     uint4 *Bt = B + S.b0;
     // items: records of 8 rows x {Re, Im}
-    for (int it = blockIdx.y * 128 + tid; it < 4 * S.kseg; it += DSPLIT * 128) {
+    for (int it = share * 128 + tid; it < 4 * S.kseg; it += DSPLIT * 128) {
         const int o = it >> 1, im = it & 1;
         const bool ok = im ? oky : okx;
         const int e = im ? ey : ex;
@@ -512,10 +559,10 @@ __device__ __forceinline__ uint2 widen_digits(uint32_t b) {
 template <int DS, bool BY>
 __global__ void __launch_bounds__(de_threads(BY), 1)
 k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ sunits,
-            const int *__restrict__ tshape, const int *__restrict__ tlist, const long long *__restrict__ tcoff,
-            const int *__restrict__ flag, int ntask, const uint8_t *__restrict__ A, const int *__restrict__ rexp,
+            const int *__restrict__ tlist, const long long *__restrict__ tcoff,
+            const int *__restrict__ flag, const uint8_t *__restrict__ A, const int *__restrict__ rexp,
             const uint8_t *__restrict__ B, const int *__restrict__ cexp, double2 *__restrict__ out,
-            unsigned long long *__restrict__ ws, int2 *__restrict__ part, int ntmax, int nst, int kbs, int *__restrict__ err) {
+            unsigned long long *__restrict__ ws, const int2 *__restrict__ part, int ntmax, int nst, int kbs, int *__restrict__ err) {
     constexpr int T = de_threads(BY);
     const int kb = BY ? kbs : 1;
     extern __shared__ __align__(128) uint8_t sm[];
@@ -531,46 +578,27 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
     const int nx = kb == 2 ? 2 : DENSE_NX;                        // (at most nst)
     uint8_t *ring = wide + (BY ? (size_t)nx * kb * XB : 0);
     const uint32_t stage = (uint32_t)kb * (AB + 2u * DS * 16u * (uint32_t)ntmax);
-    // units and weight of the shapes with work: a unit weighs the bytes it streams, in KB, and a tile
-    // DENSE_TILEW units more (the sums of the tile before it leave TMEM meanwhile)
-    for (int q = tid; q <= ns; q += T) pre[q].x = flag ? 0 : 1;
-    __syncthreads();
-    if (flag)
-        for (int t = tid; t < ntask; t += T) {
-            const int f = flag[t], q = tshape[t];
-            if (f) pre[q].x = 1;
-        }
-    __syncthreads();
-    if (warp == 0) {
-        int carry = 0, carryw = 0;
-        for (int q0 = 0; q0 <= ns; q0 += 32) {
-            const int q = q0 + lane;
-            const int4 n = q < ns ? sunits[q] : make_int4(0, 0, 1, 0);      // tiles, chunks, weight of a unit
-            const int on = q < ns && pre[q].x, u = on ? n.x * n.y : 0, w = on ? n.x * (n.y + DENSE_TILEW) * n.z : 0;
-            int s = u, z = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, s, o), x = __shfl_up_sync(0xffffffffu, z, o);
-                if (lane >= o) { s += v; z += x; }
-            }
-            if (q <= ns) pre[q] = make_int2(carry + s - u, carryw + z - w);
-            carry += __shfl_sync(0xffffffffu, s, 31);
-            carryw += __shfl_sync(0xffffffffu, z, 31);
-        }
+    if (warp == 0) umma::tmem_alloc(&tbase, 512);
+    if (tid == 0) {
+        for (int s = 0; s < nst; s++) { umma::mbar_init(&full[s], 1); umma::mbar_init(&empty[s], 1); }
+        if (BY)
+            for (int s = 0; s < nx; s++) umma::mbar_init(&xfull[s], 4);
+        umma::mbar_init(&accf, 1);
+        umma::mbar_init(&acce, 8);
+        umma::mbar_init(&drain, 1);
+        bad = 0;
     }
+    // units and weight of the shapes with work (dense_units)
+    CHAIN_ENTER();
+    LAUNDER(part); LAUNDER(cexp); LAUNDER(flag);
+    for (int q = tid; q <= ns; q += T) pre[q] = part[q];
+    const long long G = part[ns + 1].x;
+    umma::fence_before_sync();
     __syncthreads();
+    umma::fence_after_sync();
+    const uint32_t td = tbase;
     const int U = pre[ns].x;
     const long long Wt = pre[ns].y;
-    const long long G = min((int)gridDim.x, max(1, U / DENSE_MINU));
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    if (blockIdx.x == 0) {                                     // for k_dense_finish
-        for (int q = tid; q <= ns; q += T) part[q] = pre[q];
-        if (tid == 0) part[ns + 1] = make_int2((int)G, 0);
-    }
-    if (U == 0 || blockIdx.x >= G) {                 // (waits all the same: the end of this kernel is the end of those before)
-        asm volatile("griddepcontrol.wait;\n" ::: "memory");
-        return;
-    }
     // CTA b takes the units that start in [Wt·b/G, Wt·(b+1)/G) of the total weight
     auto shape_of = [&](int v, bool wt) {            // the last shape whose offset is at most v
         int lo = 0, hi = ns;
@@ -589,20 +617,6 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
         return pre[q].x + t * n.y + (k > 0 ? (k + n.z - 1) / n.z : 0);
     };
     const int ub = unit_from(blockIdx.x), ue = unit_from(blockIdx.x + 1);
-    if (warp == 0) umma::tmem_alloc(&tbase, 512);
-    if (tid == 0) {
-        for (int s = 0; s < nst; s++) { umma::mbar_init(&full[s], 1); umma::mbar_init(&empty[s], 1); }
-        if (BY)
-            for (int s = 0; s < nx; s++) umma::mbar_init(&xfull[s], 4);
-        umma::mbar_init(&accf, 1);
-        umma::mbar_init(&acce, 8);
-        umma::mbar_init(&drain, 1);
-        bad = 0;
-    }
-    umma::fence_before_sync();
-    __syncthreads();
-    umma::fence_after_sync();
-    const uint32_t td = tbase;
     struct Seg { int q, rt, ct, k0, k1; };
     auto seg_at = [&](int u) {
         const int lo = shape_of(u, false);
@@ -627,38 +641,26 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
     int issued = 0;
     if (warp == 8) {
         if (lane == 0) {
-            // the right-hand sides' digits come from the kernel before this one in the stream, which
-            // may still be running (programmatic dependent launch): the first stages take their
-            // operator digits ahead of it, then wait for it once
             bool ok = true;
-            int ahead = 0;
-            for (int pass = 0; ok && pass < 2; pass++) {
-                int it = 0;
-                for (int u = ub; ok && u < ue && (pass || it < nst);) {
-                    const Seg g = seg_at(u);
-                    const DenseShape S = sh[g.q];
-                    const uint32_t bb = 2u * DS * 16u * (uint32_t)S.nt;
-                    const uint8_t *a = A + S.aoff + ((size_t)g.rt * S.kc + g.k0) * dense_abytes(BY);
-                    const uint8_t *b = B + S.boff + ((size_t)g.ct * S.kc + g.k0) * bb;
-                    for (int k = g.k0; k < g.k1 && (pass || it < nst); k += kb, it++) {
-                        const int st = it % nst, use = it / nst, n = min(kb, g.k1 - k);
-                        uint8_t *d = ring + (size_t)st * stage;
-                        if (use > 0 && !(ok = wait(&empty[st], (use - 1) & 1))) break;
-                        if (!pass || it >= ahead) {
-                            umma::mbar_expect_tx(&full[st], (uint32_t)n * (AB + bb));
-                            for (int j = 0; j < n; j++) umma::bulk_g2s(d + j * AB, a + (size_t)j * dense_abytes(BY), AB, &full[st]);
-                            issued++;
-                        }
-                        if (pass) umma::bulk_g2s(d + kb * AB, b, (uint32_t)n * bb, &full[st]);
-                        a += (size_t)n * dense_abytes(BY);
-                        b += (size_t)n * bb;
-                    }
-                    u += g.k1 - g.k0;
+            int it = 0;
+            for (int u = ub; ok && u < ue;) {
+                const Seg g = seg_at(u);
+                const DenseShape S = sh[g.q];
+                const uint32_t bb = 2u * DS * 16u * (uint32_t)S.nt;
+                const uint8_t *a = A + S.aoff + ((size_t)g.rt * S.kc + g.k0) * dense_abytes(BY);
+                const uint8_t *b = B + S.boff + ((size_t)g.ct * S.kc + g.k0) * bb;
+                for (int k = g.k0; k < g.k1; k += kb, it++) {
+                    const int st = it % nst, use = it / nst, n = min(kb, g.k1 - k);
+                    uint8_t *d = ring + (size_t)st * stage;
+                    if (use > 0 && !(ok = wait(&empty[st], (use - 1) & 1))) break;
+                    umma::mbar_expect_tx(&full[st], (uint32_t)n * (AB + bb));
+                    for (int j = 0; j < n; j++) umma::bulk_g2s(d + j * AB, a + (size_t)j * dense_abytes(BY), AB, &full[st]);
+                    umma::bulk_g2s(d + kb * AB, b, (uint32_t)n * bb, &full[st]);
+                    issued++;
+                    a += (size_t)n * dense_abytes(BY);
+                    b += (size_t)n * bb;
                 }
-                if (!pass) {
-                    ahead = it;
-                    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-                }
+                u += g.k1 - g.k0;
             }
         }
     } else if (warp == 9) {
@@ -737,7 +739,6 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
             u += g.k1 - g.k0;
         }
     } else {
-        asm volatile("griddepcontrol.wait;\n" ::: "memory");
         int seg = 0;
         for (int u = ub; u < ue; seg++) {
             const Seg g = seg_at(u);
@@ -827,7 +828,7 @@ k_dense_mma(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict__ 
 }
 
 // The outputs of the tiles that were shared between CTAs, and their sums back to zero.  Item: 8
-// column pairs of one tile; its shape's offsets and the number of CTAs come from k_dense_mma.  In
+// column pairs of one tile; its shape's offsets and the number of CTAs come from k_dense_slice.  In
 // the CTA that added a tile's last part this took 12 k clocks with the other SMs idle (6 us at
 // k=200); over all SMs, launched ahead and waiting, about 2 us.
 __global__ void __launch_bounds__(256)
@@ -838,7 +839,7 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
     const int tid = threadIdx.x, row = tid & 127;
     bool waited = false;
     for (int b = blockIdx.x; b < nitem; b += gridDim.x) {
-        // everything but the sums and exponents is there before the products are done
+        // everything but the flags, sums and exponents is there before the products are done
         const int4 it = items[b];                                                // shape, tile (rt·nct + ct), first pair
         const DenseShape S = sh[it.x];
         const int4 n = sunits[it.x];
@@ -850,12 +851,11 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
         for (int e = 0; e < 4; e++) {
             const int task = ct * (S.nt / 2) + it.z + (tid >> 7) + 2 * e;
             t[e] = task < S.ntask && i < S.m ? tlist[S.t0 + task] : -1;
-            if (t[e] >= 0 && flag && !flag[t[e]]) t[e] = -1;
             o[e] = t[e] >= 0 ? tcoff[t[e]] + i : 0;
         }
         if (!waited) {
-            asm volatile("griddepcontrol.wait;\n" ::: "memory");
-            asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+            CHAIN_ENTER();
+            LAUNDER(flag); LAUNDER(cexp); LAUNDER(part);
             waited = true;
         }
         unsigned long long *acc = ws + S.acc0 + (size_t)it.y * 128 * S.nt + row;
@@ -867,6 +867,7 @@ k_dense_finish(const DenseShape *__restrict__ sh, int ns, const int4 *__restrict
             x[2 * e] = __ldcg(acc + (size_t)(2 * pr) * 128);
             x[2 * e + 1] = __ldcg(acc + (size_t)(2 * pr + 1) * 128);
             ce[e] = t[e] >= 0 ? make_int2(cexp[2 * t[e]], cexp[2 * t[e] + 1]) : make_int2(0, 0);
+            if (t[e] >= 0 && flag && !flag[t[e]]) t[e] = -1;
         }
         const int2 p0 = part[it.x], p1 = part[it.x + 1];
         const unsigned G = (unsigned)part[ns + 1].x, Wt = (unsigned)part[ns].y;
@@ -935,7 +936,8 @@ cudaError_t dense_set_smem() {
 }
 template <int DS>
 static void dense_launch(const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
-    launch_chained(k_dense_slice<DS>, dim3(p.ntask, DSPLIT), 128, 0, s, p.recs, in, reinterpret_cast<uint4 *>(p.B), p.cexp, flag);
+    launch_chained(k_dense_slice<DS>, dim3(1 + p.ntask * DSPLIT), 128, 0, s, p.recs, in, reinterpret_cast<uint4 *>(p.B), p.cexp,
+                   flag, p.ns, p.sunits, p.tshape, p.ntask, p.grid, p.part);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.grid);
     cfg.blockDim = dim3(de_threads(p.by));
@@ -947,8 +949,8 @@ static void dense_launch(const DensePlanArgs &p, const double2 *in, double2 *out
     cfg.attrs = at;
     cfg.numAttrs = 1;
     auto mma = p.by ? k_dense_mma<DS, true> : k_dense_mma<DS, false>;
-    cudaLaunchKernelEx(&cfg, mma, p.sh, p.ns, p.sunits, p.tshape, p.tlist, p.tcoff, flag, p.ntask, p.A, p.rexp,
-                       (const uint8_t *)p.B, (const int *)p.cexp, out, p.ws, p.part, p.ntmax, p.nst, p.kb, p.err);
+    cudaLaunchKernelEx(&cfg, mma, p.sh, p.ns, p.sunits, p.tlist, p.tcoff, flag, p.A, p.rexp,
+                       (const uint8_t *)p.B, (const int *)p.cexp, out, p.ws, (const int2 *)p.part, p.ntmax, p.nst, p.kb, p.err);
     cfg.gridDim = dim3(std::min(p.nitem, 2 * p.grid));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
