@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -68,7 +69,13 @@ struct FactorSet {            // banded FP64 factors of one matrix per shape, bl
         double bytes = 0, flops = 0;
         void clear() { sh.release(); recs.release(); tabs.release(); tcoff.release(); B.release(); cs.release(); ws.release(); part.release(); ntask = 0; }
     } plan[4];                      // {task table, doubled table} with 6 digits, with 7
-    void clear() { dA.release(); drs.release(); dop.clear(); for (auto &P : plan) P.clear(); meta.clear(); mo = 0; spike_tried = dense_on = small_on = false; sinv.release(); stab.release(); small_m = 0; G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
+    bool inverses() const { return dA.p || sinv.p; }
+    void drop_inverses() {          // (the next change of the batch may form them again)
+        dop.clear(); small_m = 0; dense_on = small_on = false;
+        for (auto &P : plan) P.clear();
+        dA.release(); drs.release(); sinv.release(); stab.release();
+    }
+    void clear() { drop_inverses(); meta.clear(); mo = 0; spike_tried = false; G.release(); spk.release(); spike_level[0] = spike_level[1] = 0; spike_levels_built = 0;
                    M.release(); Mdf.release(); P.release(); Meta.release(); table.release(); h.clear(); fma_col.clear(); cfg = BlockSolveCfg{}; re2 = false; ready = false; }
 };
 
@@ -539,7 +546,8 @@ hdd_status dense_plan(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_
 }
 
 // Explicit inverses of every shape as digits, where the product pays and fits (a quarter of the
-// free memory, 8192 operator columns, the set-up kernel's shared memory); else F.dop stays empty.
+// free memory, half of it with the workspace, 8192 operator columns, the set-up kernel's shared
+// memory); else, or if an allocation fails all the same, there are none and the banded kernels serve.
 hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStream_t s) {
     const int ns = (int)F.h.size();
     const int re2 = F.re2 ? 1 : 0, cw = std::max(F.cfg.cwx, F.cfg.cwy);
@@ -564,17 +572,39 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStre
     }
     size_t fr = 0, tot = 0;
     CK(cudaMemGetInfo(&fr, &tot));
-    if ((small ? (size_t)sv * (re2 ? 16 : 8) : (size_t)ao) > fr / 4) return HDD_OK;
+    const size_t need = small ? (size_t)sv * (re2 ? 16 : 8) : (size_t)ao;
+    const long long wmax = *std::max_element(wsz.begin(), wsz.end()),
+                    wtot = std::max(wmax, std::min(std::accumulate(wsz.begin(), wsz.end(), 0LL), 1LL << 27));
+    if (need > fr / 4 || need + (size_t)wtot * sizeof(double) > fr / 2) return HDD_OK;
+    // from here on the operator is not there until the last group is: no solve may find the old
+    // tables beside new or missing digits
+    if (small) F.small_m = 0;
+    else F.dop.clear();
+    DevMem W, jobs, shs, rmax;
+    bool room = true;
+    auto ensure = [&](DevMem &m, size_t bytes) {
+        const cudaError_t e = room ? m.ensure(bytes) : cudaSuccess;
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+        room = false;
+        return cudaSuccess;
+    };
+    auto give_up = [&]() {
+        if (small) { F.sinv.release(); F.stab.release(); }
+        else { F.dA.release(); F.drs.release(); }
+        return HDD_OK;
+    };
     if (small) {
-        CK(F.sinv.ensure((size_t)sv * (re2 ? sizeof(double2) : sizeof(double))));
-        CK(F.stab.ensure(ns * sizeof(SmallShape)));
+        CK(ensure(F.sinv, need));
+        CK(ensure(F.stab, ns * sizeof(SmallShape)));
+        if (!room) return give_up();
         CK(cudaMemcpyAsync(F.stab.p, ss.data(), ns * sizeof(SmallShape), cudaMemcpyHostToDevice, s));
     } else {
-        CK(F.dA.ensure((size_t)ao));
-        CK(F.drs.ensure((size_t)so * sizeof(int)));
+        CK(ensure(F.dA, need));
+        CK(ensure(F.drs, (size_t)so * sizeof(int)));
+        if (!room) return give_up();
     }
     // shapes in groups of up to 1 GB of workspace
-    DevMem W, jobs, shs, rmax;
     for (int q0 = 0; q0 < ns;) {
         int q1 = q0;
         long long w = 0;
@@ -594,10 +624,11 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStre
         std::stable_sort(jb.begin(), jb.end(), [&](const InvJob &a, const InvJob &b) {
             return op[a.shape].kseg - a.jc > op[b.shape].kseg - b.jc;
         });
-        CK(W.ensure((size_t)w * sizeof(double)));
-        CK(jobs.ensure(jb.size() * sizeof(InvJob)));
-        CK(shs.ensure(sh.size() * sizeof(InvShape)));
-        CK(rmax.ensure((size_t)so * sizeof(unsigned long long)));
+        CK(ensure(W, (size_t)w * sizeof(double)));
+        CK(ensure(jobs, jb.size() * sizeof(InvJob)));
+        CK(ensure(shs, sh.size() * sizeof(InvShape)));
+        CK(ensure(rmax, (size_t)so * sizeof(unsigned long long)));
+        if (!room) return give_up();
         if (q0 == 0) CK(cudaMemsetAsync(rmax.p, 0, (size_t)so * sizeof(unsigned long long), s));
         CK(cudaMemcpyAsync(jobs.p, jb.data(), jb.size() * sizeof(InvJob), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(shs.p, sh.data(), sh.size() * sizeof(InvShape), cudaMemcpyHostToDevice, s));
@@ -623,6 +654,17 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStre
     return HDD_OK;
 }
 
+// The product's plan, ahead of the solves that use it; dense becomes false if there is no room for it.
+hdd_status dense_ready(hdd_ctx *ctx, FactorSet &F, int ds, int which, cudaStream_t s, bool &dense) {
+    if (!dense || F.small_on) return HDD_OK;
+    const hdd_status st = dense_plan(ctx, F, ds, which, s);
+    if (st != HDD_ERR_OOM) return st;
+    cudaGetLastError();
+    F.plan[which + (ds == 7 ? 2 : 0)].clear();
+    dense = false;
+    return HDD_OK;
+}
+
 // E⁻¹ in for the flagged tasks by the product; ds and which as in dense_plan.
 hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
     if (F.small_on) {
@@ -638,7 +680,7 @@ hdd_status dense_solve(hdd_ctx *ctx, FactorSet &F, int ds, int which, const doub
                               F.re2 ? 1 : 0, F.sinv.as<double>(), in, out, flag, s));
         return HDD_OK;
     }
-    hdd_status st = dense_plan(ctx, F, ds, which, s);
+    const hdd_status st = dense_plan(ctx, F, ds, which, s);     // (formed by dense_ready)
     if (st != HDD_OK) return st;
     FactorSet::Plan &P = F.plan[which + (ds == 7 ? 2 : 0)];
     DensePlanArgs a;
@@ -1021,8 +1063,10 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     float2 *Rr = reinterpret_cast<float2 *>(C.Rr.as<float>());
     double2 *Yc = C.Yc.as<double2>(), *Sc = C.Sc.as<double2>();
     hdd_status st = HDD_OK;
+    bool dense = use_dense(ctx);
+    if ((st = dense_ready(ctx, ctx->E, 7, 0, s, dense)) != HDD_OK) return st;
     auto coarse = [&](const double2 *in, double2 *out) -> hdd_status {
-        if (use_dense(ctx)) return dense_solve(ctx, ctx->E, 7, 0, in, out, nullptr, s);
+        if (dense) return dense_solve(ctx, ctx->E, 7, 0, in, out, nullptr, s);
         band_solve(ctx, ctx->E, in, out, false, nullptr, s);
         return HDD_OK;
     };
@@ -1171,8 +1215,10 @@ hdd_status inner_ras(hdd_ctx *ctx, const double2 *v, double2 *z, const hdd_solve
     const bool cdf = sizeof(R) == 4 && ctx->coarse_df;
     // E⁻¹ in for the flagged tasks: the product with explicit inverses (FP64 accuracy, so it serves
     // both precisions), or the banded kernels; without coarse_df the complex64 iteration asks for those
-    const bool dense = use_dense(ctx) && (cdf || sizeof(R) == 8);
+    bool dense = use_dense(ctx) && (cdf || sizeof(R) == 8);
     const int ds = sizeof(R) == 8 ? 7 : ctx->E.digits32;
+    if ((st = dense_ready(ctx, ctx->E, ds, 0, s, dense)) != HDD_OK) return st;
+    if (prm->warm_start && ctx->cnn.ready && (st = dense_ready(ctx, ctx->E, ds, 1, s, dense)) != HDD_OK) return st;
     if (!dense && cdf && ctx->coarse_spike && !ctx->E.spike_tried && (st = spike_build(ctx, ctx->E, s)) != HDD_OK) return st;
     auto coarse = [&](const double2 *in, double2 *out, const int *flag, int n) -> hdd_status {
         if (dense) return dense_solve(ctx, ctx->E, ds, 0, in, out, flag, s);
