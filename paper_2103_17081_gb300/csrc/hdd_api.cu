@@ -1728,6 +1728,19 @@ void wr_le32(unsigned char *p, uint32_t v) {
 }
 }  // namespace
 
+namespace {
+// The coarse inverses are an option that costs no call its memory: one that runs out of it while
+// they are held runs once more without them (with the banded kernels; the next hdd_setup_batch or
+// hdd_setup_deflation may form them again).
+template <typename Call> hdd_status with_room(hdd_ctx *ctx, Call call) {
+    const hdd_status st = call();
+    if (st != HDD_ERR_OOM || !ctx->E.inverses()) return st;
+    cudaGetLastError();
+    ctx->E.drop_inverses();
+    return call();
+}
+}  // namespace
+
 // ===========================================================================================
 // C ABI
 // ===========================================================================================
@@ -1962,7 +1975,7 @@ hdd_status hdd_setup_deflation(hdd_ctx *ctx, void *stream) {
     return build_factors(ctx, ctx->E, true, (cudaStream_t)stream);
 }
 
-hdd_status hdd_setup_exact(hdd_ctx *ctx, void *stream) {
+static hdd_status setup_exact_once(hdd_ctx *ctx, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->dd) FAIL(HDD_ERR_STATE, "hdd_setup_dd first");
@@ -1970,7 +1983,7 @@ hdd_status hdd_setup_exact(hdd_ctx *ctx, void *stream) {
     return build_factors(ctx, ctx->Aex, false, (cudaStream_t)stream);
 }
 
-hdd_status hdd_setup_coarse_grid(hdd_ctx *ctx, int c, void *stream) {
+static hdd_status setup_coarse_grid_once(hdd_ctx *ctx, int c, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->assembled) FAIL(HDD_ERR_STATE, "hdd_assemble first");
@@ -2025,7 +2038,7 @@ long long hdd_coarse_grid_size(const hdd_ctx *ctx) {
     return (long long)ctx->cg.m * ctx->cg.m;
 }
 
-hdd_status hdd_coarse_grid_op(hdd_ctx *ctx, int stages, int prec, const void *in_dev, void *out_dev,
+static hdd_status coarse_grid_op_once(hdd_ctx *ctx, int stages, int prec, const void *in_dev, void *out_dev,
                               void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
@@ -2044,7 +2057,7 @@ hdd_status hdd_coarse_grid_op(hdd_ctx *ctx, int stages, int prec, const void *in
     return HDD_OK;
 }
 
-hdd_status hdd_ras_apply(hdd_ctx *ctx, const void *v_dev, void *z_dev, const hdd_solve_params *prm,
+static hdd_status ras_apply_once(hdd_ctx *ctx, const void *v_dev, void *z_dev, const hdd_solve_params *prm,
                          int *inner_its, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
@@ -2063,7 +2076,7 @@ hdd_status hdd_ras_apply(hdd_ctx *ctx, const void *v_dev, void *z_dev, const hdd
     return HDD_OK;
 }
 
-hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_solve_params *prm,
+static hdd_status solve_once(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_solve_params *prm,
                      hdd_solve_stats *stats, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
@@ -2375,7 +2388,7 @@ hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_sol
     return result;
 }
 
-hdd_status hdd_autotune(hdd_ctx *ctx, const hdd_solve_params *prm, void *stream, int *fine_rows,
+static hdd_status autotune_once(hdd_ctx *ctx, const hdd_solve_params *prm, void *stream, int *fine_rows,
                         int *coarse_rows, double *best_ms) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
@@ -2435,7 +2448,7 @@ hdd_status hdd_autotune(hdd_ctx *ctx, const hdd_solve_params *prm, void *stream,
     return HDD_OK;
 }
 
-hdd_status hdd_setup_batch(hdd_ctx *ctx, int nrhs) {
+static hdd_status setup_batch_once(hdd_ctx *ctx, int nrhs) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->dd) FAIL(HDD_ERR_STATE, "hdd_setup_dd first");
@@ -2484,7 +2497,7 @@ long long hdd_launch_count(const hdd_ctx *ctx) { return ctx ? ctx->prof.launches
 
 int hdd_cnn_num_params(void) { return CNN_NPARAM; }
 
-hdd_status hdd_cnn_set_params(hdd_ctx *ctx, const float *params) {
+static hdd_status cnn_set_params_once(hdd_ctx *ctx, const float *params) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->dd) FAIL(HDD_ERR_STATE, "hdd_setup_dd first");
@@ -2568,7 +2581,7 @@ hdd_status hdd_cnn_get_params(hdd_ctx *ctx, float *params) {
     return HDD_OK;
 }
 
-hdd_status hdd_cnn_forward(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
+static hdd_status cnn_forward_once(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->cnn.ready) FAIL(HDD_ERR_STATE, "hdd_cnn_set_params first");
@@ -2586,7 +2599,7 @@ hdd_status hdd_cnn_forward(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *
     return HDD_OK;
 }
 
-hdd_status hdd_cnn_infer(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
+static hdd_status cnn_infer_once(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->cnn.ready) FAIL(HDD_ERR_STATE, "hdd_cnn_set_params first");
@@ -2604,7 +2617,7 @@ hdd_status hdd_cnn_infer(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *st
     return cnn_check_err(ctx, s);
 }
 
-hdd_status hdd_cnn_loss_grad(hdd_ctx *ctx, const void *f_dev, double *loss, float *grad) {
+static hdd_status cnn_loss_grad_once(hdd_ctx *ctx, const void *f_dev, double *loss, float *grad) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->cnn.ready) FAIL(HDD_ERR_STATE, "hdd_cnn_set_params first");
@@ -2617,7 +2630,7 @@ hdd_status hdd_cnn_loss_grad(hdd_ctx *ctx, const void *f_dev, double *loss, floa
     return HDD_OK;
 }
 
-hdd_status hdd_cnn_train_step(hdd_ctx *ctx, const void *f_dev, float lr, double *loss, void *stream) {
+static hdd_status cnn_train_step_once(hdd_ctx *ctx, const void *f_dev, float lr, double *loss, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->cnn.ready) FAIL(HDD_ERR_STATE, "hdd_cnn_set_params first");
@@ -2696,7 +2709,7 @@ hdd_status hdd_apply_PA_noalloc(hdd_ctx *ctx, const void *in_dev, void *out_dev,
     return HDD_OK;
 }
 
-hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void *out_dev, void *stream) {
+static hdd_status local_op_once(hdd_ctx *ctx, int op, int prec, const void *in_dev, void *out_dev, void *stream) {
     if (!ctx) return HDD_ERR_INVALID_ARG;
     if (ctx->poisoned) FAIL(HDD_ERR_TIMEOUT, "context lost: a device wait and its drain timed out earlier");
     if (!ctx->dd) FAIL(HDD_ERR_STATE, "hdd_setup_dd first");
@@ -2767,6 +2780,62 @@ hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void
         return HDD_OK;
     };
     return prec == 64 ? run(float{}) : run(double{});
+}
+
+// ---- entries that allocate (with_room) -------------------------------------------------------
+hdd_status hdd_setup_exact(hdd_ctx *ctx, void *stream) {
+    return with_room(ctx, [&] { return setup_exact_once(ctx, stream); });
+}
+
+hdd_status hdd_setup_coarse_grid(hdd_ctx *ctx, int c, void *stream) {
+    return with_room(ctx, [&] { return setup_coarse_grid_once(ctx, c, stream); });
+}
+
+hdd_status hdd_ras_apply(hdd_ctx *ctx, const void *v_dev, void *z_dev, const hdd_solve_params *prm,
+                         int *inner_its, void *stream) {
+    return with_room(ctx, [&] { return ras_apply_once(ctx, v_dev, z_dev, prm, inner_its, stream); });
+}
+
+hdd_status hdd_solve(hdd_ctx *ctx, const void *f_dev, void *x_dev, const hdd_solve_params *prm,
+                     hdd_solve_stats *stats, void *stream) {
+    return with_room(ctx, [&] { return solve_once(ctx, f_dev, x_dev, prm, stats, stream); });
+}
+
+hdd_status hdd_cnn_set_params(hdd_ctx *ctx, const float *params) {
+    return with_room(ctx, [&] { return cnn_set_params_once(ctx, params); });
+}
+
+hdd_status hdd_cnn_forward(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
+    return with_room(ctx, [&] { return cnn_forward_once(ctx, f_dev, x0_dev, stream); });
+}
+
+hdd_status hdd_cnn_infer(hdd_ctx *ctx, const void *f_dev, void *x0_dev, void *stream) {
+    return with_room(ctx, [&] { return cnn_infer_once(ctx, f_dev, x0_dev, stream); });
+}
+
+hdd_status hdd_cnn_loss_grad(hdd_ctx *ctx, const void *f_dev, double *loss, float *grad) {
+    return with_room(ctx, [&] { return cnn_loss_grad_once(ctx, f_dev, loss, grad); });
+}
+
+hdd_status hdd_cnn_train_step(hdd_ctx *ctx, const void *f_dev, float lr, double *loss, void *stream) {
+    return with_room(ctx, [&] { return cnn_train_step_once(ctx, f_dev, lr, loss, stream); });
+}
+
+hdd_status hdd_coarse_grid_op(hdd_ctx *ctx, int stages, int prec, const void *in_dev, void *out_dev, void *stream) {
+    return with_room(ctx, [&] { return coarse_grid_op_once(ctx, stages, prec, in_dev, out_dev, stream); });
+}
+
+hdd_status hdd_autotune(hdd_ctx *ctx, const hdd_solve_params *prm, void *stream, int *fine_rows,
+                        int *coarse_rows, double *best_ms) {
+    return with_room(ctx, [&] { return autotune_once(ctx, prm, stream, fine_rows, coarse_rows, best_ms); });
+}
+
+hdd_status hdd_setup_batch(hdd_ctx *ctx, int nrhs) {
+    return with_room(ctx, [&] { return setup_batch_once(ctx, nrhs); });
+}
+
+hdd_status hdd_local_op(hdd_ctx *ctx, int op, int prec, const void *in_dev, void *out_dev, void *stream) {
+    return with_room(ctx, [&] { return local_op_once(ctx, op, prec, in_dev, out_dev, stream); });
 }
 
 }  // extern "C"

@@ -45,3 +45,45 @@ def test_no_room_for_the_products_plan_takes_the_banded_kernels():
     assert "coarse_solve_dense" in families()
     s.profile(False)
     assert float(torch.linalg.vector_norm(z - ref)) <= 1e-4 * float(torch.linalg.vector_norm(ref))
+
+
+def test_a_solve_that_needs_the_inverses_memory_runs_without_them():
+    """A solve whose Krylov basis fits the free memory only together with half of what the inverses
+    hold: it runs with the banded kernels, to the result it has with them from the start."""
+    torch = pytest.importorskip("torch")
+    from paper_2103_17081_gb300 import Solver
+
+    def solver():
+        return Solver(0).assemble(100.0, 320).setup_dd(4, 4, 2)
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    twin = solver()
+    before = free()
+    twin.set_option("coarse_dense", 0).setup_deflation()
+    banded = before - free()
+    f = torch.from_numpy(W.random_complex_fast(twin.n, 8)).cuda()
+    x, opt = twin.empty(), dict(outer_maxit=60, outer_restart=60, outer_tol=1e-10, raise_on_error=False)
+    before = free()
+    _, st = twin.solve(f, out=x, **opt)
+    need = before - free()
+    twin.close()
+    s = solver()
+    before = free()
+    s.setup_deflation()
+    held = before - free() - banded
+    assert held > 40 << 20 and need > 200 << 20
+    y = s.empty()
+    s.profile(True)
+    rest = _fill(torch, need - held // 2)
+    try:
+        _, st2 = s.solve(f, out=y, **opt)
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    assert "coarse_solve_dense" not in {d["name"] for d in s.profile_stats() if d["launches"]}
+    assert st2["status_code"] == st["status_code"] and st2["outer_its"] == st["outer_its"]
+    assert torch.equal(x, y)
