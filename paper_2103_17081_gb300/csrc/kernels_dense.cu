@@ -320,19 +320,20 @@ k_small_pack(const InvShape *__restrict__ sh, const SmallShape *__restrict__ ss,
 // (4 for complex E) over as many CTAs as there are blocks of rows; the matrix comes from L2, and the
 // first entries are loaded before the wait for the kernel in front.  m = 64, 4
 // tasks: 7 us by events around it where the banded sweeps take 13 and the three kernels of the
-// digits 15; m = 576: 11 us (62, 16).
+// digits 15; m = 576: 11 us (62, 16).  CTA task·nb + block of rows: in the grid's first dimension, as
+// a batch may have more tasks than the others hold.
 constexpr int SM_R = 8, SM_T = 256, SM_PRE = 4;
 template <bool RE2>
 __global__ void __launch_bounds__(SM_T)
 k_small_solve(const Task *__restrict__ tasks, const SmallShape *__restrict__ ss, const double *__restrict__ inv,
-              const double2 *__restrict__ in, double2 *__restrict__ out, const int *__restrict__ flag) {
+              const double2 *__restrict__ in, double2 *__restrict__ out, const int *__restrict__ flag, int nb) {
     using A = typename std::conditional<RE2, double2, double>::type;
     extern __shared__ double2 xs[];
     __shared__ double red[2 * SM_R][SM_T / 32];
-    const int t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int t = blockIdx.x / nb, rb = blockIdx.x - t * nb, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Task T = tasks[t];
     const SmallShape S = ss[T.shape];
-    const int r0 = blockIdx.x * SM_R, c0 = warp * 4 + (lane >> 3);
+    const int r0 = rb * SM_R, c0 = warp * 4 + (lane >> 3);
     const bool mine = r0 < S.m;
     const A *M = reinterpret_cast<const A *>(inv) + S.off + r0 + (lane & 7);
     A pre[SM_PRE];
@@ -377,10 +378,11 @@ k_small_solve(const Task *__restrict__ tasks, const SmallShape *__restrict__ ss,
 }
 void launch_small_solve(const Task *tasks, int ntask, const SmallShape *ss, int mmax, int re2, const double *inv,
                         const double2 *in, double2 *out, const int *flag, cudaStream_t s) {
-    const dim3 grid((mmax + SM_R - 1) / SM_R, ntask);
+    const int nb = (mmax + SM_R - 1) / SM_R;
+    const dim3 grid((unsigned)nb * (unsigned)ntask);
     const size_t sm = (size_t)mmax * sizeof(double2);
-    if (re2) launch_chained(k_small_solve<true>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag);
-    else launch_chained(k_small_solve<false>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag);
+    if (re2) launch_chained(k_small_solve<true>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag, nb);
+    else launch_chained(k_small_solve<false>, grid, SM_T, sm, s, tasks, ss, inv, in, out, flag, nb);
 }
 
 // ------------------------------------------------------------------------------------------
