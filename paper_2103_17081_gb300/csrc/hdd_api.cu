@@ -976,7 +976,7 @@ hdd_status cnn_tc_buffers(hdd_ctx *ctx, cudaStream_t s) {
     if (!C.pad_ready || grow) {
         CK(cudaMemsetAsync(C.Ba.p, 0, act, s)); CK(cudaMemsetAsync(C.Bb.p, 0, act, s));
         CK(cudaMemsetAsync(C.err.p, 0, sizeof(int), s));
-        CK(set_conv_tc_smem(ctx->tc_wmax));
+        CK(set_conv_tc_smem());
         C.pad_ready = true;
     }
     return HDD_OK;
@@ -1058,7 +1058,7 @@ hdd_status cnn_loss_grad(hdd_ctx *ctx, const c2<R> *f, double *loss, cudaStream_
     //   P f̂, r = f̂ - A y, q = P r, Pᵀ q = q - Z E⁻¹ Zᵀ A q; dL/dy_t = scale_t · A Pᵀ q
     LocalArgs<float> a = local_args<float>(ctx);
     const size_t lsm = local_max_dynamic_smem(ctx->max_nx, (int)sizeof(float2), ctx->frows, ctx->crows);
-    if (lsm > 48 * 1024) CK(set_local_smem_limits<float>(lsm));
+    if (lsm > 48 * 1024) CK(set_local_smem_limits<float>());
     float2 *Fh = C.Fh.as<float2>(), *Q = C.Q.as<float2>(), *T2 = C.T2.as<float2>();
     float2 *Rr = reinterpret_cast<float2 *>(C.Rr.as<float>());
     double2 *Yc = C.Yc.as<double2>(), *Sc = C.Sc.as<double2>();
@@ -1137,7 +1137,7 @@ template <typename R> hdd_status ensure_inner(hdd_ctx *ctx, int R_) {
     CK(W.ints.ensure(7 * nt * sizeof(int)));
     W.restart = R_;
     size_t smem = local_max_dynamic_smem(ctx->max_nx, (int)cs, ctx->frows, ctx->crows);
-    if (smem > 48 * 1024) CK(set_local_smem_limits<R>(smem));
+    if (smem > 48 * 1024) CK(set_local_smem_limits<R>());
     return HDD_OK;
 }
 
@@ -2146,7 +2146,7 @@ static hdd_status solve_once(hdd_ctx *ctx, const void *f_dev, void *x_dev, const
     CK(O.hist.ensure((size_t)nr * (prm->outer_maxit + 1) * sizeof(double)));
     const size_t osm = (size_t)(R + 1) * 3 * sizeof(double);   // dynamic: h (update), y (axpy, trisolve)
     if (osm + 40 * 1024 > 227 * 1024) FAIL(HDD_ERR_INVALID_ARG, "outer restart %d too long", R);
-    CK(set_outer_smem_limits(osm));
+    CK(set_outer_smem_limits());
     double2 *V = O.V.as<double2>(), *Zb = O.Z.as<double2>(), *w = O.w.as<double2>(), *rv = O.r.as<double2>();
     const double2 *f = (const double2 *)f_dev;
     double2 *x = (double2 *)x_dev;
@@ -2693,7 +2693,7 @@ hdd_status hdd_apply_PA_noalloc(hdd_ctx *ctx, const void *in_dev, void *out_dev,
     cudaStream_t s = (cudaStream_t)stream;
     LocalArgs<double> a = local_args<double>(ctx);
     const size_t smem = local_max_dynamic_smem(ctx->max_nx, (int)sizeof(double2), ctx->frows, ctx->crows);
-    if (smem > 48 * 1024) CK(set_local_smem_limits<double>(smem));
+    if (smem > 48 * 1024) CK(set_local_smem_limits<double>());
     double2 *y = scratch, *sc = scratch + HDD_NOALLOC_MAX_COARSE;
     const double2 *in = (const double2 *)in_dev;
     double2 *out = (double2 *)out_dev;
@@ -2740,7 +2740,7 @@ static hdd_status local_op_once(hdd_ctx *ctx, int op, int prec, const void *in_d
         using R = decltype(tag);
         LocalArgs<R> a = local_args<R>(ctx);
         size_t smem = local_max_dynamic_smem(ctx->max_nx, (int)sizeof(c2<R>), ctx->frows, ctx->crows);
-        if (smem > 48 * 1024) CK(set_local_smem_limits<R>(smem));
+        if (smem > 48 * 1024) CK(set_local_smem_limits<R>());
         CK(ctx->tmp_a.ensure(std::max(ld, ldc) * sizeof(c2<R>)));
         CK(ctx->tmp_b.ensure(std::max(ld, ldc) * sizeof(c2<R>)));
         CK(ctx->tmp_c.ensure((std::max(ld, ldc) + 64) * sizeof(double2)));

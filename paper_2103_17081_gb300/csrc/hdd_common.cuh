@@ -222,6 +222,19 @@ inline cudaError_t launch_chained(void (*kern)(KA...), dim3 grid, dim3 block, si
     return cudaLaunchKernelEx(&cfg, kern, (KA)args...);
 }
 
+// Opens a kernel to all the dynamic shared memory a CTA can have beside its static part.  The limit
+// belongs to the kernel in the process, and contexts of other host threads launch it too: it is the
+// same whatever the problem, so none takes away what another is about to launch with.
+template <typename K>
+inline cudaError_t allow_smem(K kern) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, kern);
+    if (e != cudaSuccess) return e;
+    const int most = 227 * 1024 - (int)a.sharedSizeBytes;
+    if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Progress of an inner cycle: slot i counts the tasks that have decided about step i (high word) and
 // those that run it (low word).  The task that comes last writes the count to the host's pinned
 // memory (-2 if a dense coarse solve has reported an error), where the host waits for it: no copy
@@ -394,7 +407,7 @@ template <typename R> void launch_finish(const LocalArgs<R> &a, const InnerState
                                          c2<R> *u, const c2<R> *V, const double2 *sc, const int *flag,
                                          int *rs_out, int *its_out, int maxit, long long nglob, double2 *glob,
                                          cudaStream_t s);
-template <typename R> cudaError_t set_local_smem_limits(size_t bytes);
+template <typename R> cudaError_t set_local_smem_limits();
 template <typename R> void launch_set_ref(const LocalArgs<R> &a, const InnerState<R> &S, const c2<R> *p3,
                                           const int *flag, cudaStream_t s);
 template <typename R> void launch_coarse_combine(const LocalArgs<R> &a, const InnerState<R> &S,
@@ -633,7 +646,7 @@ void launch_oinit(const OuterBatch &B, const double2 *rv, const double *npart, d
                   float2 *V32L, double *D, double2 *g, double2 *Wq, double *beta_out, cudaStream_t s);
 void launch_orotate(const OuterBatch &B, double2 *H, const double *cs, const double2 *sn, const int *kcols,
                     int kmax, cudaStream_t s);
-cudaError_t set_outer_smem_limits(size_t bytes);
+cudaError_t set_outer_smem_limits();
 
 // tensor-core inference of the warm-start network (kernels_cnn_tc.cu)
 void launch_cnn_l1_bf16(const Task *tasks, const Tile *tiles, int ntiles, const __nv_bfloat16 *W, const float *b,
@@ -641,7 +654,7 @@ void launch_cnn_l1_bf16(const Task *tasks, const Tile *tiles, int ntiles, const 
 void launch_cnn_tc_weights(const __nv_bfloat16 *Wb, __nv_bfloat16 *img2, __nv_bfloat16 *img3,
                            __nv_bfloat16 *img4, cudaStream_t s);
 size_t conv_tc_smem(int nco, int wmax);
-cudaError_t set_conv_tc_smem(int wmax);
+cudaError_t set_conv_tc_smem();
 void launch_conv_tc(int nco, int grid, const Task *tasks, const int2 *tct, int ntct, const uint4 *X, long long ptot,
                     const uint4 *Wimg, const float *bias, uint4 *Y, float2 *A4, int wmax, int *err, cudaStream_t s);
 

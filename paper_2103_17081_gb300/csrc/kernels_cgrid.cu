@@ -245,7 +245,7 @@ void launch_dst_pass(int m, const T *S, const T *Dinv, const c2<T> *in, c2<T> *o
                      const int *active, cudaStream_t s) {
     const int t = (m + DT - 1) / DT;
     static_assert((size_t)DGROUPS * DT * (DT + 1) * sizeof(c2<T>) <= dst_smem<T>(), "the groups' sums fit");
-    cudaFuncSetAttribute(k_dst_pass<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dst_smem<T>());
+    allow_smem(k_dst_pass<T>);
     launch_chained(k_dst_pass<T>, dim3(t, t, nrhs), DTHREADS, dst_smem<T>(), s, m, ldh, S, Dinv, in, out, active);
 }
 void launch_cg_widen(long long n, const float2 *in, double2 *out, cudaStream_t s) {

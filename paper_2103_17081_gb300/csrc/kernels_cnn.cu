@@ -558,7 +558,7 @@ static void conv32(const Task *tasks, const Tile *tiles, int ntiles, int max_nx,
     while (sr > 1 && smem(sr) > 220 * 1024) sr--;
     // (narrower boxes, or fewer rows, may have a larger stride than their size by the padding)
     const size_t sm = smem(sr) + 32 * 32 * sizeof(float);
-    cudaFuncSetAttribute(k_conv32<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (allow_smem(k_conv32<BWD>) != cudaSuccess) return;          // (the error stays for the caller to find)
     k_conv32<BWD><<<std::min(ntiles, sm_count()), CONV_T, sm, s>>>(tasks, tiles, ntiles, W, b, X, mask, Y, sr);
 }
 void launch_conv_fwd(int layer, const Task *tasks, const Tile *tiles, int ntiles, int max_nx, int frows,
@@ -588,7 +588,7 @@ static void bwd_w(const Task *tasks, const Tile *tiles, int ntiles, int max_nx, 
     const size_t rows = (size_t)4 * (max_nx + 2) * CIN + (size_t)2 * max_nx * COUT;
     const size_t sums = NSEG > 1 ? (size_t)NSEG * (COUT * 9 * CIN + COUT) : 0;
     const size_t sm = std::max(rows, sums) * sizeof(float);
-    cudaFuncSetAttribute(k_conv_bwd_w<CIN, COUT, CPT, NSEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (allow_smem(k_conv_bwd_w<CIN, COUT, CPT, NSEG>) != cudaSuccess) return;
     k_conv_bwd_w<CIN, COUT, CPT, NSEG><<<conv_bwd_w_parts(ntiles), CT, sm, s>>>(tasks, tiles, ntiles, dY, act_out, X,
                                                                                part, max_nx);
 }

@@ -232,11 +232,9 @@ void launch_cnn_tc_weights(const __nv_bfloat16 *Wb, __nv_bfloat16 *img2, __nv_bf
                                                      img4);
 }
 
-cudaError_t set_conv_tc_smem(int wmax) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)conv_tc_smem(32, wmax));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_conv_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_tc_smem(16, wmax));
+cudaError_t set_conv_tc_smem() {
+    const cudaError_t e = allow_smem(k_conv_tc<32>);
+    return e != cudaSuccess ? e : allow_smem(k_conv_tc<16>);
 }
 
 void launch_conv_tc(int nco, int grid, const Task *tasks, const int2 *tct, int ntct, const uint4 *X, long long ptot,

@@ -1531,7 +1531,7 @@ cudaError_t launch_band_lu(const LuShape *sh, int ns, int max_kl, int max_ku, do
                            cudaStream_t s) {
     const size_t sm = lu_cluster_smem(max_kl, max_ku);
     if (sm <= 200 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_band_lu_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        const cudaError_t e = allow_smem(k_band_lu_cluster);
         if (e != cudaSuccess) return e;
         k_band_lu_cluster<<<ns * LUC, LUT, sm, s>>>(sh, AB, PIV, info);
     } else {
@@ -1547,7 +1547,7 @@ void launch_ops_to_df(long long n, const double *M, float2 *Mdf, cudaStream_t s)
 cudaError_t launch_factor_prepare(const LuShape *sh, int ns, int max_m, const double *AB, const int *PIV, double *LP,
                                   int *LEXT, int *UEXT, int *PERM, int *err, cudaStream_t s) {
     const int ints = std::min(2 * max_m, 48 * 1024);
-    const cudaError_t e = cudaFuncSetAttribute(k_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, ints * (int)sizeof(int));
+    const cudaError_t e = allow_smem(k_perm);
     if (e != cudaSuccess) return e;
     k_perm<<<ns, 256, ints * sizeof(int), s>>>(sh, PIV, PERM, ints);
     k_lperm<<<dim3((max_m + 127) / 128, ns), 128, 0, s>>>(sh, AB, PIV, LP, LEXT, err);
@@ -1675,25 +1675,21 @@ bool launch_block_solve_spike(int P, const Task *tasks, int ntasks, const BlockF
     return e == cudaSuccess;
 }
 
-template <int RING, bool RE2> static cudaError_t spk_attr(size_t lim, size_t &static_bytes) {
+template <int RING, bool RE2> static cudaError_t spk_attr(size_t &static_bytes) {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_block_solve_spike_df<RING, RE2>);
     if (e != cudaSuccess) return e;
     static_bytes = std::max(static_bytes, a.sharedSizeBytes);
-    return cudaFuncSetAttribute(k_block_solve_spike_df<RING, RE2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(lim - a.sharedSizeBytes));
+    return allow_smem(k_block_solve_spike_df<RING, RE2>);
 }
-template <int RING, bool RE2> static cudaError_t la_attr(size_t lim, size_t &static_bytes) {
+template <int RING, bool RE2> static cudaError_t la_attr(size_t &static_bytes) {
     cudaFuncAttributes a, b;
     cudaError_t e = cudaFuncGetAttributes(&a, k_block_solve_la<RING, RE2>);
     if (e != cudaSuccess) return e;
     if ((e = cudaFuncGetAttributes(&b, k_block_solve_la_df<RING, RE2>)) != cudaSuccess) return e;
     static_bytes = std::max(static_bytes, std::max(a.sharedSizeBytes, b.sharedSizeBytes));
-    if ((e = cudaFuncSetAttribute(k_block_solve_la<RING, RE2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(lim - a.sharedSizeBytes))) != cudaSuccess)
-        return e;
-    return cudaFuncSetAttribute(k_block_solve_la_df<RING, RE2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(lim - b.sharedSizeBytes));
+    if ((e = allow_smem(k_block_solve_la<RING, RE2>)) != cudaSuccess) return e;
+    return allow_smem(k_block_solve_la_df<RING, RE2>);
 }
 
 // Ring depth 4 if its shared memory fits the per-CTA limit, else 2; error if not even that fits.
@@ -1712,32 +1708,28 @@ cudaError_t set_block_solve_smem(BlockSolveCfg &c) {
     const size_t lim2 = lim - std::max(a2.sharedSizeBytes, b2.sharedSizeBytes);
     c.ring = bs_smem(c, 4) <= lim4 ? 4 : 2;
     if (bs_smem(c, c.ring) > (c.ring == 4 ? lim4 : lim2)) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(k_block_solve<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim4)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_block_solve<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim2)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_block_solve<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim4)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_block_solve<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim2)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(k_block_solve<4, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_block_solve<2, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_block_solve<4, true>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_block_solve<2, true>)) != cudaSuccess) return e;
     size_t st = 0;
-    if ((e = la_attr<6, false>(lim, st)) != cudaSuccess) return e;
-    if ((e = la_attr<4, false>(lim, st)) != cudaSuccess) return e;
-    if ((e = la_attr<3, false>(lim, st)) != cudaSuccess) return e;
-    if ((e = la_attr<6, true>(lim, st)) != cudaSuccess) return e;
-    if ((e = la_attr<4, true>(lim, st)) != cudaSuccess) return e;
-    if ((e = la_attr<3, true>(lim, st)) != cudaSuccess) return e;
+    if ((e = la_attr<6, false>(st)) != cudaSuccess) return e;
+    if ((e = la_attr<4, false>(st)) != cudaSuccess) return e;
+    if ((e = la_attr<3, false>(st)) != cudaSuccess) return e;
+    if ((e = la_attr<6, true>(st)) != cudaSuccess) return e;
+    if ((e = la_attr<4, true>(st)) != cudaSuccess) return e;
+    if ((e = la_attr<3, true>(st)) != cudaSuccess) return e;
     c.la_ring = 0;
     for (int r : {6, 4, 3})
         if (la_smem(c, r) + st <= lim) { c.la_ring = r; break; }
     // the SPIKE kernels (one CTA per SM): the deepest ring of 6, 4, 3 that fits (spike_ok = ring)
     size_t sst = 0;
-    if ((e = spk_attr<6, false>(lim, sst)) != cudaSuccess) return e;
-    if ((e = spk_attr<6, true>(lim, sst)) != cudaSuccess) return e;
-    if ((e = spk_attr<4, false>(lim, sst)) != cudaSuccess) return e;
-    if ((e = spk_attr<4, true>(lim, sst)) != cudaSuccess) return e;
-    if ((e = spk_attr<3, false>(lim, sst)) != cudaSuccess) return e;
-    if ((e = spk_attr<3, true>(lim, sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<6, false>(sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<6, true>(sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<4, false>(sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<4, true>(sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<3, false>(sst)) != cudaSuccess) return e;
+    if ((e = spk_attr<3, true>(sst)) != cudaSuccess) return e;
     c.spike_ok = 0;
     for (int r : {6, 4, 3})
         if (la_smem(c, r) + sst <= lim) { c.spike_ok = r; break; }

@@ -898,8 +898,7 @@ cudaError_t launch_inv(const InvJob *jobs, int njobs, const InvShape *sh, int ns
                        int maxK, int cw, int re2, unsigned long long *rmax, int *rexp, uint8_t *A, bool by,
                        const SmallShape *ss, double *inv, cudaStream_t s) {
     const size_t smem = inv_cols_smem(maxK, cw);
-    cudaError_t e = re2 ? cudaFuncSetAttribute(k_inv_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                        : cudaFuncSetAttribute(k_inv_cols<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = re2 ? allow_smem(k_inv_cols<true>) : allow_smem(k_inv_cols<false>);
     if (e != cudaSuccess) return e;
     if (re2) k_inv_cols<true><<<njobs, 256, smem, s>>>(jobs, shapes, Mall, Pall, Meta, W, maxK, cw);
     else k_inv_cols<false><<<njobs, 256, smem, s>>>(jobs, shapes, Mall, Pall, Meta, W, maxK, cw);
@@ -931,10 +930,10 @@ void dense_stages(int ds, bool by, int ns, int ntmax, int &kb, int &nst) {
 }
 cudaError_t dense_set_smem() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_dense_mma<6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_dense_mma<7, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_dense_mma<6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_dense_mma<7, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 223 * 1024);
+    if ((e = allow_smem(k_dense_mma<6, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_dense_mma<7, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_dense_mma<6, true>)) != cudaSuccess) return e;
+    return allow_smem(k_dense_mma<7, true>);
 }
 template <int DS>
 static void dense_launch(const DensePlanArgs &p, const double2 *in, double2 *out, const int *flag, cudaStream_t s) {

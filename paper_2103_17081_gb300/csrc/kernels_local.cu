@@ -1278,9 +1278,9 @@ cudaError_t launch_arnoldi_step(const LocalArgs<R> &la, int C, int i, int restar
 // co-schedule (0 on error); sets the kernels' dynamic shared-memory limit to `smem` first.
 template <typename R> int arnoldi_step_max_cluster(size_t smem, int C) {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_arnoldi_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = allow_smem(k_arnoldi_step<R, false>)) != cudaSuccess)
         return 0;
-    if ((e = cudaFuncSetAttribute(k_arnoldi_step<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = allow_smem(k_arnoldi_step<R, true>)) != cudaSuccess)
         return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C);
@@ -1322,16 +1322,16 @@ size_t local_max_dynamic_smem(int max_nx, int bytes_per_c, int frows, int crows)
     return ps > zt ? ps : zt;
 }
 
-template <typename R> cudaError_t set_local_smem_limits(size_t bytes) {
+template <typename R> cudaError_t set_local_smem_limits() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_prolong_stencil<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_prolong_stencil<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_zt<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_zt<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_z<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_finish<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_local_A<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_local_A<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_prolong_stencil<R, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_prolong_stencil<R, true>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_zt<R, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_zt<R, true>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_z<R>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_finish<R>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_local_A<R, false>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_local_A<R, true>)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -1346,7 +1346,7 @@ template <typename R> cudaError_t set_local_smem_limits(size_t bytes) {
     template void launch_givens_normalize<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const c2<R> *, const c2<R> *, const int *, int *, const Progress &, R, int, cudaStream_t); \
     template void launch_init_cycle<R>(const LocalArgs<R> &, const InnerState<R> &, int, c2<R> *, const c2<R> *, const int *, int *, const Progress &, R, int, int, cudaStream_t); \
     template void launch_finish<R>(const LocalArgs<R> &, const InnerState<R> &, int, int, c2<R> *, const c2<R> *, const double2 *, const int *, int *, int *, int, long long, double2 *, cudaStream_t); \
-    template cudaError_t set_local_smem_limits<R>(size_t); \
+    template cudaError_t set_local_smem_limits<R>(); \
     template void launch_coarse_combine<R>(const LocalArgs<R> &, const InnerState<R> &, int, const double2 *, double2 *, const int *, cudaStream_t); \
     template void launch_set_ref<R>(const LocalArgs<R> &, const InnerState<R> &, const c2<R> *, const int *, cudaStream_t); \
     template cudaError_t launch_arnoldi_step<R>(const LocalArgs<R> &, int, int, int, c2<R> *, const double2 *, double2 *, const InnerState<R> &, const int *, int *, const Progress &, R, int, size_t, cudaStream_t); \

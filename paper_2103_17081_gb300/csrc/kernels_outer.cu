@@ -1517,22 +1517,13 @@ cudaError_t launch_odots2_df(const OuterBatch &B0, const float2 *Vh, const float
     odots2_plan(B0, nv, B.G, ng);
     const long long chunk = (B.n + B.G - 1) / B.G;
     const size_t smem = (size_t)(2 * chunk) * sizeof(float4) + (bias ? (size_t)nv * sizeof(float) : 0);
-    // the largest dynamic shared memory requested so far, per device and variant (the attribute
-    // is set on the current device)
-    constexpr int MAXDEV = 64;
-    static size_t set[MAXDEV][2];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= MAXDEV) return cudaErrorInvalidDevice;
     bias = bias ? 1 : 0;
     void (*const kern[2])(OuterBatch, int, const float2 *, const float2 *, int, const float2 *, const float2 *,
                           const double2 *, double2 *, double2 *, const unsigned *) = {k_odots2_df<false>,
                                                                                       k_odots2_df<true>};
-    if (smem > 47 * 1024 && smem > set[dev][bias]) {         // (48 KB with the kernel's static part)
-        e = cudaFuncSetAttribute(kern[bias], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 47 * 1024) {                                  // (48 KB with the kernel's static part)
+        const cudaError_t e = allow_smem(kern[bias]);
         if (e != cudaSuccess) return e;
-        set[dev][bias] = smem;
     }
     launch_chained(kern[bias], dim3(B.G * ng, B.nrhs), OT, smem, s, B, ng, Vh, Vl, nv, x1h, x1l, w, part1, part2, vmax);
     launch_chained(k_oreduce, dim3((nv + 7) / 8, B.nrhs, 2), 256, 0, s, B, part1, nv, out1, part2, out2);
@@ -1609,16 +1600,16 @@ void launch_oinit(const OuterBatch &B, const double2 *rv, const double *npart, d
                   float2 *V32L, double *D, double2 *g, double2 *Wq, double *beta_out, cudaStream_t s) {
     k_oinit<<<dim3(grid_for(B.n, 256), B.nrhs), 256, 0, s>>>(B, rv, npart, V, V32, V32L, D, g, Wq, beta_out);
 }
-cudaError_t set_outer_smem_limits(size_t bytes) {
+cudaError_t set_outer_smem_limits() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_oupdate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oupdate_dcgs<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_otrisolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_oaxpy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate2)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate_df)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate_dcgs<1>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate_dcgs<2>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oupdate_dcgs<4>)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_otrisolve)) != cudaSuccess) return e;
+    if ((e = allow_smem(k_oaxpy)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
