@@ -1459,7 +1459,7 @@ static void pair_plan(K kern, PairPlan &c, long long n, int &threads, int &grid)
     threads = c.threads;
     grid = c.grid;
 }
-static PairPlan plan_udf, plan_dcgs;
+static thread_local PairPlan plan_udf, plan_dcgs;      // (contexts run in several host threads)
 int oupdate_df_grid(long long n) {
     int t = 0, g = 0;
     pair_plan(k_oupdate_df, plan_udf, n, t, g);
