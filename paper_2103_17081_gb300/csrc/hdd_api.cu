@@ -721,8 +721,7 @@ hdd_status coarse_forms(hdd_ctx *ctx, FactorSet &F, cudaStream_t s) {
     F.dense_on = form > 0;
     F.small_on = form == 2;
     if (ctx->coarse_dense && F.dense_on && !dense_built(F)) st = dense_build(ctx, F, F.small_on, F.by_want, s);
-    if (!ctx->coarse_spike) F.spike_tried = true;
-    if (st == HDD_OK && !F.spike_tried && !(F.dense_on && dense_built(F))) {
+    if (st == HDD_OK && ctx->coarse_spike && !F.spike_tried && !(F.dense_on && dense_built(F))) {
         st = spike_build(ctx, F, s);
     }
     return st;
@@ -850,6 +849,7 @@ hdd_status build_factors(hdd_ctx *ctx, FactorSet &F, bool coarse, cudaStream_t s
     if (coarse) {
         F.meta = std::move(meta);
         F.mo = mo;
+        F.spike_tried = !ctx->coarse_spike;          // (the option counts at the set-up of the factors)
         hdd_status dst = coarse_forms(ctx, F, s);
         if (dst != HDD_OK) return dst;
     }
