@@ -389,11 +389,14 @@ long long hdd_launch_count(const hdd_ctx *ctx);
 /* first pass left) or the two-sum for both (0).                                              */
 /* HDD_OPT_COARSE_DENSE (9): the coarse solves E_j⁻¹ of the inner iteration and of the training */
 /* loss run as products with the explicit inverses of the distinct E_j on the tensor cores, in  */
-/* exact integer arithmetic on 56-bit fixed-point copies of the FP64 entries (1, the default,   */
-/* where the shapes and tasks make that the faster form; the inverses are formed at             */
-/* hdd_setup_deflation, or at hdd_setup_batch when the batch makes it pay; small orders as one   */
-/* FP64 product with the inverse) or by the banded                                               */
+/* integer arithmetic on 56-bit (complex64: 48-bit) fixed-point copies of the FP64 entries, to   */
+/* the accuracy of the banded FP64 solves (1, the default, where the shapes and tasks make that  */
+/* the faster form; the inverses are formed at hdd_setup_deflation, or at hdd_setup_batch when   */
+/* the batch makes it pay; small orders as one FP64 product with the inverse) or by the banded   */
 /* kernels the options 1, 6 and 7 describe (0).  hdd_local_op always applies the banded ones.   */
+/* The inverses take at most a quarter of the device memory that is free when they are formed    */
+/* (and a workspace of up to 1 GB meanwhile); a batch that asks for the other form has both.  A  */
+/* call that runs out of memory gives them up and runs with the banded kernels.                  */
 /* With HDD_OPT_COARSE_LOOKAHEAD 0, or HDD_OPT_COARSE_DF 0 in complex64, the banded kernels run. */
 /* HDD_ERR_INVALID_ARG for an unknown key or a value other than 0 or 1.  Takes effect from the  */
 /* next call that solves.                                                                       */

@@ -196,8 +196,8 @@ struct hdd_ctx {
     DevMem d_alist;                            // active tasks of a SPIKE coarse solve, compacted
     int *h_counter = nullptr;                  // pinned copy of the error flag
     int *h_pub = nullptr;                      // pinned, written by the kernels: tasks before step i (-1: not known yet)
-    DevMem d_counter;                          // error flag of the dense solves, then the steps' progress
-                                               // before each inner step of a cycle and after it (CNT_*)
+    DevMem d_counter;                          // error flag of the dense solves, then the progress counts
+                                               // (Progress::slot) before each step of an inner cycle and after the last
     int *h_its = nullptr;                      // pinned: step counts of the tasks
     size_t h_its_n = 0;
     std::vector<double> hist;
@@ -436,10 +436,11 @@ hdd_status build_spikes(hdd_ctx *ctx, FactorSet &F, const std::vector<int4> &met
 // Which form is the fastest for `per` tasks of each shape: 0 banded, 1 the product by digits on the
 // tensor cores, 2 the FP64 product.  Digits: three kernels, about 12 us where nothing else counts,
 // and the operators' digits at 5.5 TB/s with the MMAs under them (28 products of nt columns per
-// 16-column unit, nt/2 clocks each).  Banded: 0.77 us per 16-row block and sweep (164 us for the 106
+// 16-column unit, nt/2 clocks each; counted as BF16 digits and for complex128, so that few columns, kept as
+// bytes, and complex64, with 21 products, are faster than that).  Banded: 0.77 us per 16-row block and sweep (164 us for the 106
 // blocks of m = 1681), one chain per SM, or 1.7 times that for two per SM.  Measured: four shapes, 64
 // tasks (k=200) 164 us against 38; 256 uneven shapes of N = 1280 with 32 right-hand sides 15.2 ms
-// against 2.3, while for one right-hand side the banded form stays ahead (0.5 against 2 ms: every
+// against 2.3, while for one right-hand side the banded form stays ahead (0.5 against 2 ms with BF16 digits: every
 // operator is read for one task); m = 64, 4 tasks, 15 us against 17.  FP64: one kernel, 6.5 us and its
 // products at the FP64 pipe's rate.  By events around a solve, banded / digits / FP64: m = 64, 4 or 16
 // tasks 13 / 15..17 / 7 us; m = 256, 4 tasks 31 / 16 / 7.6; m = 289, 4 complex 69 / 16 / 9.4; m = 576,
@@ -647,8 +648,9 @@ hdd_status dense_build(hdd_ctx *ctx, FactorSet &F, bool small, bool by, cudaStre
     F.by = by;
     for (FactorSet::Plan &P : F.plan) P.ntask = 0;        // (made for the other form of the digits)
     // Against the exact inverse, 6 digits leave 1e-13 of the solution where the double-FP32 banded
-    // solve leaves 1e-12 to 2e-11 (36 geometries, m = 625 to 2401), but 5.5e-14 against 3.5e-14 at
-    // m = 64, where nothing is gained by the shorter operator: 7 digits below 256
+    // solve leaves 1e-12 to 2e-11 (36 geometries, m = 625 to 2401; up to 2e-12 where E is worse
+    // conditioned, as the FP64 banded solve does), but 5.5e-14 against 3.5e-14 at m = 64, where
+    // nothing is gained by the shorter operator: 7 digits below 256
     F.digits32 = 6;
     for (const FactorSet::DenseOp &o : op) if (o.m < 256) F.digits32 = 7;
     return HDD_OK;
